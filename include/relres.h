@@ -565,8 +565,9 @@ relres_status relres_get_timings(relres_ctx* ctx, double* ms, long long* counts,
  * own allocator and loads this library as a plug-in, or a loop in which the
  * device synchronisation of cudaMalloc/cudaFree is not allowed.  No context
  * is needed and nothing is allocated on the device: the scratch memory (the
- * type-pair table and per-block partial sums) is one file-scope static device
- * array, present on every GPU that loads the library until the process exits.
+ * type-pair table, packed atoms and per-block partial sums, 0.5 MB) is one
+ * file-scope static device array, present on every GPU that loads the
+ * library until the process exits.
  *   p              parameters as for relres_create (only the pair terms are used).
  *   n_atoms        1..RELRES_STATIC_MAX_ATOMS, else RELRES_ERR_ARG.
  *   d_type         [n_atoms] device atom types.

@@ -6,15 +6,15 @@
 // cudaFree (which may synchronise the device) are not allowed.  For them this
 // entry point evaluates the RelRes pair forces, energy and virial of a small
 // system by an all-pairs FP64 sum, with every piece of scratch memory (the
-// type-pair table and the per-block partial sums) in one file-scope static
-// device array of fixed size.  The caller provides only inputs and outputs.
+// type-pair table, packed atoms and per-block partial sums: 0.5 MB) in one
+// file-scope static device array of fixed size.  The caller provides only inputs and outputs.
 //
 // Limits and sharing: at most RELRES_STATIC_MAX_ATOMS atoms and
 // RELRES_MAX_TYPES types.  The array exists once per GPU that loads the
 // library and stays allocated until the process exits.  All calls on a GPU
 // share it: calls whose work overlaps on the GPU (different streams, or
 // several host threads) race on it and must be serialised by the caller.
-// Each call rewrites the table and every partial sum it reads, and clears the
+// Each call rewrites the table, atoms and partial sums it reads, and clears the
 // bad-type flag before its kernels run, so stale contents from an earlier
 // call are never used.
 //
@@ -22,6 +22,15 @@
 // skips every pair whose type index is outside [0, n_types) (no table read
 // with it), writes NaN forces for such an atom and raises a flag in the static
 // array, and the reduction then writes NaN energy and virial.
+//
+// How a call works: k_pack_static reduces every position into the box once and
+// packs it as FP32 with a type code; k_allpairs_static gives each atom one
+// warp, which rejects partners by their FP32 distance (32 a pass) and queues
+// the others; full queues are evaluated in FP64, one pair a lane.  The FP32
+// radius is widened by more than the rounding of the packed coordinates, so
+// every pair inside its interaction range is evaluated, from the caller's own
+// FP64 positions.  Energy and virial are summed in a fixed order from one
+// partial sum per block.
 //
 // Set-up: the first call on each device (with that device current) looks up
 // the array's device address with cudaGetSymbolAddress.
@@ -34,13 +43,19 @@
 namespace relres {
 namespace {
 
-constexpr int kStaticThreads = 256;
-constexpr int kStaticMaxBlocks = (RELRES_STATIC_MAX_ATOMS + kStaticThreads - 1) / kStaticThreads;
+constexpr int kStaticThreads = 128;  // four atoms (warps) per block
+constexpr int kStaticMaxBlocks = RELRES_STATIC_MAX_ATOMS / (kStaticThreads / 32);
 constexpr int kMaxDevices = 64;
+// Type codes of packed atoms past the valid types: an atom whose type is out
+// of range (no pair with it is evaluated) and one with a non-finite coordinate
+// (every pair with it is, so that the non-finite value reaches the results).
+constexpr int kCodeBadType = RELRES_MAX_TYPES, kCodeNonfinite = RELRES_MAX_TYPES + 1;
+constexpr int kCodes = RELRES_MAX_TYPES + 2;
 
 struct StaticScratch {
   PairTab<double> tab[RELRES_MAX_TYPES * RELRES_MAX_TYPES];
-  long long partial[kStaticMaxBlocks][kNQ];
+  float4 atom[RELRES_STATIC_MAX_ATOMS];  // position in [0, L] and type code
+  double partial[kNQ][kStaticMaxBlocks];
   unsigned bad_type;  // set when an atom type was outside [0, n_types)
 };
 
@@ -49,6 +64,11 @@ static __device__ __align__(256) StaticScratch g_static_scratch;
 // host-side cache of the array's device address, per device (several host
 // threads may look it up at once; each finds the same address)
 static std::atomic<StaticScratch*> s_scratch_ptr[kMaxDevices];
+
+// squared FP32 distances from which a pair of types is certainly out of range
+struct StaticReach {
+  float r2[RELRES_MAX_TYPES * RELRES_MAX_TYPES];
+};
 
 __device__ __forceinline__ double poly5(const double* g, double d) {
   return (((g[4] * d + g[3]) * d + g[2]) * d + g[1]) * d + g[0];
@@ -93,100 +113,159 @@ __device__ __forceinline__ void relres_pair(const PairTab<double>& T, double r2,
   *u = e;
 }
 
-// One thread per atom, all partners j != i through shared-memory tiles.
-__global__ void __launch_bounds__(kStaticThreads)
-    k_allpairs_static(int n, int nt, const double* __restrict__ pos, const int* __restrict__ type,
-                      double l0, double l1, double l2, const int* __restrict__ eoff,
-                      const int* __restrict__ eidx, int with_excl, double* __restrict__ forces,
-                      StaticScratch* scratch) {
-  __shared__ double sx[kStaticThreads], sy[kStaticThreads], sz[kStaticThreads];
-  __shared__ int stype[kStaticThreads];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool live = i < n;
-  double xi = 0.0, yi = 0.0, zi = 0.0;
-  int ti = 0, e0 = 0, e1 = 0;
-  bool bad_i = false;
-  if (live) {
-    xi = pos[3 * i];
-    yi = pos[3 * i + 1];
-    zi = pos[3 * i + 2];
-    ti = type[i];
-    bad_i = ti < 0 || ti >= nt;
-    if (bad_i) {
-      ti = 0;
-      atomicOr(&scratch->bad_type, 1u);
-    }
-    if (with_excl) {
-      e0 = eoff[i];
-      e1 = eoff[i + 1];
-    }
-  }
-  double fx = 0.0, fy = 0.0, fz = 0.0;
-  double acc[kNQ];
-#pragma unroll
-  for (int q = 0; q < kNQ; ++q) acc[q] = 0.0;
-  for (int base = 0; base < n; base += kStaticThreads) {
-    const int jl = base + threadIdx.x;
-    if (jl < n) {
-      sx[threadIdx.x] = pos[3 * jl];
-      sy[threadIdx.x] = pos[3 * jl + 1];
-      sz[threadIdx.x] = pos[3 * jl + 2];
-      stype[threadIdx.x] = type[jl];
-    }
-    __syncthreads();
-    const int m = min(kStaticThreads, n - base);
-    if (live) {
-      for (int k = 0; k < m; ++k) {
-        const int j = base + k;
-        const int tj = stype[k];
-        if (j == i || bad_i || tj < 0 || tj >= nt) continue;  // out-of-range types: no table read
-        bool ex = false;
-        for (int e = e0; e < e1; ++e) ex |= eidx[e] == j;
-        if (ex) continue;
-        double dx = xi - sx[k], dy = yi - sy[k], dz = zi - sz[k];
-        dx -= l0 * rint(dx / l0);
-        dy -= l1 * rint(dy / l1);
-        dz -= l2 * rint(dz / l2);
-        double fr, u;
-        relres_pair(scratch->tab[ti * nt + tj], dx * dx + dy * dy + dz * dz, &fr, &u);
-        fx += fr * dx;
-        fy += fr * dy;
-        fz += fr * dz;
-        acc[0] += u;
-        acc[1] += fr * dx * dx;
-        acc[2] += fr * dy * dy;
-        acc[3] += fr * dz * dz;
-        acc[4] += fr * dx * dy;
-        acc[5] += fr * dx * dz;
-        acc[6] += fr * dy * dz;
-      }
-    }
-    __syncthreads();
-  }
-  if (live) {
-    const double nan = __longlong_as_double(0x7ff8000000000000LL);
-    forces[3 * i] = bad_i ? nan : fx;
-    forces[3 * i + 1] = bad_i ? nan : fy;
-    forces[3 * i + 2] = bad_i ? nan : fz;
-  }
-  __shared__ double sh[(kStaticThreads / 32) * kNQ];
-  block_sum<double, kNQ>(acc, sh);
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int q = 0; q < kNQ; ++q) scratch->partial[blockIdx.x][q] = to_fix_sum(0.5 * acc[q]);
+// x reduced into [0, L] (FP32; the quotient is exact for any image that FP64
+// tells apart from its neighbours).
+__device__ __forceinline__ float into_box(double x, double l, double il) {
+  const float f = float(fma(-floor(x * il), l, x));
+  return fminf(fmaxf(f, 0.f), float(l));
 }
 
-__global__ void k_allpairs_static_reduce(int nblocks, const StaticScratch* scratch, double* energy,
-                                         int with_energy, double* virial, int with_virial) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  long long tot[kNQ] = {0, 0, 0, 0, 0, 0, 0};
-  for (int b = 0; b < nblocks; ++b)
-    for (int q = 0; q < kNQ; ++q) tot[q] += scratch->partial[b][q];
-  const bool bad = scratch->bad_type != 0u;
-  const double nan = __longlong_as_double(0x7ff8000000000000LL);
-  if (with_energy) energy[0] = bad ? nan : double(tot[0]) / kFix;
-  if (with_virial)
-    for (int q = 1; q < kNQ; ++q) virial[q - 1] = bad ? nan : double(tot[q]) / kFix;
+__global__ void __launch_bounds__(kThreads) k_pack_static(int n, int nt, const double* __restrict__ pos,
+                                                          const int* __restrict__ type, double l0, double l1,
+                                                          double l2, StaticScratch* scratch) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  bool bad = false;
+  if (i < n) {
+    const double x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2];
+    const int t = type[i];
+    bad = t < 0 || t >= nt;
+    const bool fin = isfinite(x) && isfinite(y) && isfinite(z);
+    const int code = bad ? kCodeBadType : (fin ? t : kCodeNonfinite);
+    scratch->atom[i] =
+        make_float4(into_box(x, l0, 1.0 / l0), into_box(y, l1, 1.0 / l1), into_box(z, l2, 1.0 / l2), __int_as_float(code));
+  }
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&scratch->bad_type, 1u);
+}
+
+// distance along one axis to the nearest image, both coordinates in [0, l]
+__device__ __forceinline__ float nearest(float a, float b, float l) {
+  const float d = fabsf(a - b);
+  return fminf(d, l - d);
+}
+
+// d - l rint(d / l).  The quotient is rounded by adding and subtracting
+// 1.5 2^52; d * il may round to the other side of a half integer where d / l
+// does not, which only exchanges two images at half the box, out of range.
+__device__ __forceinline__ double min_image(double d, double l, double il) {
+  const double t = fma(d, il, 6755399441055744.0);
+  return fma(-l, t - 6755399441055744.0, d);
+}
+
+struct StaticSums {
+  double f[3] = {0.0, 0.0, 0.0};
+  double q[kNQ] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+};
+
+// One queued pair (i, j): excluded partners are skipped here, where few
+// candidates are left.
+__device__ __forceinline__ void static_pair(const double* __restrict__ pos, const int* __restrict__ type, double xi,
+                                            double yi, double zi, int ti, int nt, int j, double l0, double l1,
+                                            double l2, double il0, double il1, double il2, const int* __restrict__ eidx,
+                                            int e0, int e1, const PairTab<double>* tab, StaticSums& S) {
+  for (int e = e0; e < e1; ++e)
+    if (eidx[e] == j) return;
+  const double dx = min_image(xi - pos[3 * j], l0, il0), dy = min_image(yi - pos[3 * j + 1], l1, il1),
+               dz = min_image(zi - pos[3 * j + 2], l2, il2);
+  double fr, u;
+  relres_pair(tab[ti * nt + type[j]], dx * dx + dy * dy + dz * dz, &fr, &u);
+  const double fx = fr * dx, fy = fr * dy, fz = fr * dz;
+  S.f[0] += fx;
+  S.f[1] += fy;
+  S.f[2] += fz;
+  S.q[0] += u;
+  S.q[1] += fx * dx;
+  S.q[2] += fy * dy;
+  S.q[3] += fz * dz;
+  S.q[4] += fx * dy;
+  S.q[5] += fx * dz;
+  S.q[6] += fy * dz;
+}
+
+// One warp per atom.  The FP32 test of a partner is ~20 instructions (n^2 of
+// them: the floor of large n); the FP64 evaluation of the few percent that
+// pass runs with full lanes from the queue, at the FP64 rate (1.66 FMA per
+// clock and SM).  Against one thread per atom evaluating every partner in
+// FP64: 18.5 -> 0.14 ms per call at 3993 propane-like atoms, where 16 blocks
+// of 256 had left most SMs without work and 95 % of the FP64 arithmetic went
+// to pairs out of range.
+__global__ void __launch_bounds__(kStaticThreads)
+    k_allpairs_static(int n, int nt, const double* __restrict__ pos, const int* __restrict__ type, double l0,
+                      double l1, double l2, const int* __restrict__ eoff, const int* __restrict__ eidx, int with_excl,
+                      StaticReach reach, double* __restrict__ forces, StaticScratch* scratch) {
+  constexpr int kWarps = kStaticThreads / 32;
+  __shared__ float s_reach[kWarps][kCodes];
+  __shared__ int s_queue[kWarps][64];
+  __shared__ double s_sum[kWarps * kNQ];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i = blockIdx.x * kWarps + w;
+  StaticSums S;
+  if (i < n) {
+    const float4 ai = scratch->atom[i];
+    const int ci = __float_as_int(ai.w);
+    const bool bad_i = ci == kCodeBadType;
+    if (!bad_i) {
+      const int ti = type[i];
+      if (lane < kCodes) {
+        // partners by type code: never, always, or by the widened distance
+        // (always for a non-finite atom i)
+        float r2 = lane < nt ? (ci == kCodeNonfinite ? __int_as_float(0x7f800000) : reach.r2[ti * nt + lane]) : -1.f;
+        if (lane == kCodeNonfinite) r2 = __int_as_float(0x7f800000);
+        s_reach[w][lane] = r2;
+      }
+      __syncwarp();
+      const double xi = pos[3 * i], yi = pos[3 * i + 1], zi = pos[3 * i + 2];
+      const double il0 = 1.0 / l0, il1 = 1.0 / l1, il2 = 1.0 / l2;
+      const int e0 = with_excl ? eoff[i] : 0, e1 = with_excl ? eoff[i + 1] : 0;
+      const float fl0 = float(l0), fl1 = float(l1), fl2 = float(l2);
+      int waiting = 0;
+      for (int base = 0; base < n; base += 32) {
+        const int j = base + lane;
+        bool near = false;
+        if (j < n && j != i) {
+          const float4 aj = scratch->atom[j];
+          const float dx = nearest(ai.x, aj.x, fl0), dy = nearest(ai.y, aj.y, fl1), dz = nearest(ai.z, aj.z, fl2);
+          near = dx * dx + dy * dy + dz * dz < s_reach[w][__float_as_int(aj.w)];
+        }
+        const unsigned b = __ballot_sync(0xffffffffu, near);
+        if (b == 0u) continue;
+        if (near) s_queue[w][waiting + __popc(b & ((1u << lane) - 1u))] = j;
+        waiting += __popc(b);
+        __syncwarp();
+        if (waiting >= 32) {
+          waiting -= 32;
+          const int jq = s_queue[w][waiting + lane];
+          __syncwarp();
+          static_pair(pos, type, xi, yi, zi, ti, nt, jq, l0, l1, l2, il0, il1, il2, eidx, e0, e1, scratch->tab, S);
+        }
+      }
+      if (lane < waiting)
+        static_pair(pos, type, xi, yi, zi, ti, nt, s_queue[w][lane], l0, l1, l2, il0, il1, il2, eidx, e0, e1,
+                    scratch->tab, S);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) S.f[q] = warp_sum(S.f[q]);
+    if (lane < 3)
+      forces[3 * i + lane] =
+          bad_i ? __longlong_as_double(0x7ff8000000000000LL) : (lane == 0 ? S.f[0] : (lane == 1 ? S.f[1] : S.f[2]));
+  }
+  block_sum<double, kNQ>(S.q, s_sum);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int q = 0; q < kNQ; ++q) scratch->partial[q][blockIdx.x] = 0.5 * S.q[q];
+}
+
+// Block q sums the q-th of the energy and virial partial sums (fixed order).
+__global__ void __launch_bounds__(1024) k_allpairs_static_out(int nblocks, const StaticScratch* scratch, double* energy,
+                                                              int with_energy, double* virial, int with_virial) {
+  __shared__ double sh[32];
+  const int q = blockIdx.x;
+  double v[1] = {0.0};
+  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v[0] += scratch->partial[q][b];
+  block_sum<double, 1>(v, sh);
+  if (threadIdx.x != 0) return;
+  if (scratch->bad_type != 0u) v[0] = __longlong_as_double(0x7ff8000000000000LL);
+  if (q == 0 && with_energy) energy[0] = v[0];
+  if (q > 0 && with_virial) virial[q - 1] = v[0];
 }
 
 }  // namespace
@@ -210,6 +289,7 @@ extern "C" relres_status relres_pair_forces_static(const relres_params* p, int n
   if (ps != RELRES_OK) return ps;
   const int nt = p->n_types;
   double rmax = 0.0;
+  StaticReach reach{};
   PairTab<double> tabs[RELRES_MAX_TYPES * RELRES_MAX_TYPES];
   std::memset(tabs, 0, sizeof(tabs));
   for (int k = 0; k < nt * nt; ++k) {
@@ -243,7 +323,12 @@ extern "C" relres_status relres_pair_forces_static(const relres_params* p, int n
     for (int m = 1; m < 5; ++m) t.cgod[m - 1] = m * o[18 + m];
     t.gam_cm = o[23];
     t.e_cg_close = o[13] - o[23];
-    rmax = std::fmax(rmax, std::fmax(o[5], o[2] > 0.0 ? o[7] : 0.0));
+    const double rk = std::fmax(o[5], o[2] > 0.0 ? o[7] : 0.0);
+    rmax = std::fmax(rmax, rk);
+    // beyond rk the pair's force and energy are exactly zero; widened by more
+    // than the rounding of two packed coordinates and their difference
+    const double wide = rk * (1.0 + 1e-5) + 1e-6 * std::fmax(box[0], std::fmax(box[1], box[2])) + 1e-3;
+    reach.r2[k] = float(wide * wide * (1.0 + 1e-5));
   }
   // minimum image needs every interaction range below half the box
   if (!(rmax < 0.5 * std::fmin(box[0], std::fmin(box[1], box[2])))) return RELRES_ERR_BOX;
@@ -263,7 +348,6 @@ extern "C" relres_status relres_pair_forces_static(const relres_params* p, int n
                       stream) != cudaSuccess)
     return RELRES_ERR_CUDA;
   if (cudaMemsetAsync(&scratch->bad_type, 0, sizeof(unsigned), stream) != cudaSuccess) return RELRES_ERR_CUDA;
-  int nblocks = (n_atoms + kStaticThreads - 1) / kStaticThreads;
   int with_excl = d_excl_offsets ? 1 : 0;
   // cudaLaunchKernel returns the status of this launch only: an earlier
   // error of unrelated work is neither reported as this call's nor cleared
@@ -271,18 +355,23 @@ extern "C" relres_status relres_pair_forces_static(const relres_params* p, int n
   double l0 = box[0], l1 = box[1], l2 = box[2];
   const int* eoff = with_excl ? d_excl_offsets : d_type;
   const int* eidx = with_excl ? d_excl_index : d_type;
+  void* args0[] = {&n, &ntt, const_cast<double**>(&d_pos), const_cast<int**>(&d_type), &l0, &l1, &l2, &scratch};
+  if (cudaLaunchKernel(reinterpret_cast<const void*>(&k_pack_static), dim3((n_atoms + kThreads - 1) / kThreads),
+                       dim3(kThreads), args0, 0, stream) != cudaSuccess)
+    return RELRES_ERR_CUDA;
   void* args1[] = {&n, &ntt, const_cast<double**>(&d_pos), const_cast<int**>(&d_type), &l0, &l1, &l2,
-                   const_cast<int**>(&eoff), const_cast<int**>(&eidx), &with_excl, &d_forces, &scratch};
-  if (cudaLaunchKernel(reinterpret_cast<const void*>(&k_allpairs_static), dim3(nblocks), dim3(kStaticThreads),
-                       args1, 0, stream) != cudaSuccess)
+                   const_cast<int**>(&eoff), const_cast<int**>(&eidx), &with_excl, &reach, &d_forces, &scratch};
+  int nblocks = (n_atoms + kStaticThreads / 32 - 1) / (kStaticThreads / 32);
+  if (cudaLaunchKernel(reinterpret_cast<const void*>(&k_allpairs_static), dim3(nblocks), dim3(kStaticThreads), args1,
+                       0, stream) != cudaSuccess)
     return RELRES_ERR_CUDA;
   const StaticScratch* cscratch = scratch;
   double* e_out = d_energy ? d_energy : d_forces;
   double* w_out = d_virial ? d_virial : d_forces;
   int with_e = d_energy ? 1 : 0, with_w = d_virial ? 1 : 0;
   void* args2[] = {&nblocks, &cscratch, &e_out, &with_e, &w_out, &with_w};
-  if (cudaLaunchKernel(reinterpret_cast<const void*>(&k_allpairs_static_reduce), dim3(1), dim3(1), args2, 0,
-                       stream) != cudaSuccess)
+  if (cudaLaunchKernel(reinterpret_cast<const void*>(&k_allpairs_static_out), dim3((with_e || with_w) ? kNQ : 1),
+                       dim3(1024), args2, 0, stream) != cudaSuccess)
     return RELRES_ERR_CUDA;
   return RELRES_OK;
 }
