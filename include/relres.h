@@ -172,7 +172,9 @@ typedef struct relres_stats {
   long long n_steps;             /* MD steps since create (also the thermostat counter) */
   int has_cg;                    /* 1 if any hybrid pair has eps^CG > 0 */
   long long n_launches;          /* CUDA kernels this context has launched */
-  int pair_tpa, pair_block;      /* forces-only pair kernel: threads per atom, block size */
+  int pair_tpa, pair_block;      /* forces-only pair kernel: threads per atom and block size of its launch
+                                    configuration (small FP32 systems left to configuration -1 run
+                                    configuration 0 with several lanes per atom, the same force bits) */
   double prune_delta;            /* pruning margin in Angstrom (0: pruning off) */
   long long n_prunes;            /* pruning passes since create (each build is followed by one) */
   double mean_fg_pruned, mean_cg_pruned;  /* mean pruned list length over all passes */
@@ -417,10 +419,8 @@ relres_status relres_get_list(relres_ctx* ctx, int which, int* h_i, int* h_j, lo
  * bits as without pruning when one thread walks each list (pair launch
  * configurations 0-2 of relres_set_pair_config) and the force sums are
  * running sums (RELRES_ACC_FP32, RELRES_ACC_FP64); the default compensated
- * sums add the entries four at a time, so there they agree to rounding, as do
- * the pair energies of the FP32 path (summed in an order that follows the
- * lists walked).  delta <= 0 turns pruning
- * off (the pair kernels then walk the full lists and the second pair of lists
+ * sums add the entries four at a time, so there they agree to rounding.
+ * delta <= 0 turns pruning off (the pair kernels then walk the full lists and the second pair of lists
  * is freed).  Default: delta = 0.5 A.  Rebuilds the lists at the current
  * positions if they exist.  Synchronous.  Errors: RELRES_ERR_ARG (null
  * context, non-finite delta).
@@ -517,7 +517,9 @@ void relres_batch_destroy(relres_batch* batch);
  * list (1, 2, 4, 8) x block size -- on the context's own lists and keep the
  * fastest (systems under 20 000 atoms keep configuration 0; with list pruning
  * on only the one-thread configurations 0-2 are timed, since the others need a
- * separate pruning pass); config 0..6
+ * separate pruning pass; with compensated sums a system of up to 40 000 list
+ * owners runs configuration 0 with 4 or 8 lanes per list, which gives the
+ * same force bits); config 0..6
  * fixes one (0: one thread per atom, 256 per block; 1, 2: one thread per
  * atom, 128, 512 per block; 3-6: 2, 4, 8, 2 threads per atom).  The choice is reported
  * in relres_stats.  Results agree within rounding (the summation order of an

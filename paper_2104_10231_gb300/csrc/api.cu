@@ -274,6 +274,15 @@ relres_status forces_now(relres_ctx* c, int ev_mode, double* d_forces, double* d
   return RELRES_OK;
 }
 
+// the launch configuration of the pair kernels back to its start; the next
+// evaluation chooses again (captured graphs hold the old one)
+void untune(relres_ctx* c) {
+  c->tuned = false;
+  c->pair_cfg = 0;
+  c->pair_lanes = 0;
+  ++c->buf_gen;
+}
+
 size_t force_bytes(const relres_ctx* c) { return size_t(c->n) * (c->fp64 ? 24 : 16); }
 
 
@@ -307,6 +316,7 @@ relres_status relres_create(relres_ctx** out, const relres_params* p, void* cuda
   c->fp64 = p->precision == RELRES_PREC_FP64;
   c->stream = static_cast<cudaStream_t>(cuda_stream);
   build_kernel_tables(c->recs, &c->tab_f, &c->tab_d);
+  pack_pair_rows(c->tab_f, c->tab_d, &c->rows_f, &c->rows_e);
   for (const PairRecord& r : c->recs) {
     c->rlist_fg_cut = std::max(c->rlist_fg_cut, r.rsp);
     if (r.eps_cg > 0.0) {
@@ -316,17 +326,15 @@ relres_status relres_create(relres_ctx** out, const relres_params* p, void* cuda
   }
   for (int t = 0; t < c->n_types; ++t)
     if (c->has_cg && c->is_hybrid[t]) c->hyb_mask |= 1 << t;
-  const size_t tb = c->fp64 ? sizeof(PairTab<double>) * c->tab_d.size()
-                            : sizeof(PairTab<float>) * c->tab_f.size();
+  const size_t tb = c->fp64 ? sizeof(PairTab<double>) * c->tab_d.size() : sizeof(PairRowF) * c->rows_f.size();
   cudaError_t ce = cudaMalloc(&c->d_tab, tb);
   if (ce == cudaSuccess)
     ce = cudaMemcpy(c->d_tab, c->fp64 ? static_cast<const void*>(c->tab_d.data())
-                                      : static_cast<const void*>(c->tab_f.data()),
+                                      : static_cast<const void*>(c->rows_f.data()),
                     tb, cudaMemcpyHostToDevice);
-  if (ce == cudaSuccess) ce = cudaMalloc(&c->d_tabd, sizeof(PairTab<double>) * c->tab_d.size());
+  if (ce == cudaSuccess) ce = cudaMalloc(&c->d_tabe, sizeof(PairRowE) * c->rows_e.size());
   if (ce == cudaSuccess)
-    ce = cudaMemcpy(c->d_tabd, c->tab_d.data(), sizeof(PairTab<double>) * c->tab_d.size(),
-                    cudaMemcpyHostToDevice);
+    ce = cudaMemcpy(c->d_tabe, c->rows_e.data(), sizeof(PairRowE) * c->rows_e.size(), cudaMemcpyHostToDevice);
   build_basis_tables(c->recs, p->shift, &c->basis_f, &c->basis_d);
   const size_t bb = c->fp64 ? sizeof(BasisTab<double>) * c->basis_d.size()
                             : sizeof(BasisTab<float>) * c->basis_f.size();
@@ -676,6 +684,7 @@ relres_status relres_set_topology(relres_ctx* c, const relres_topology* t) {
   c->have_topo = true;
   c->have_lists = false;
   c->consts_dt = 0.0;  // masses may have changed
+  if (c->tune_mode < 0) untune(c);  // the pair launches go with the size
   c->forces_valid = false;
   c->cap_fg = c->cap_cg = 0;
   return RELRES_OK;
@@ -748,6 +757,11 @@ relres_status relres_compute(relres_ctx* c, const double* d_pos, double* d_force
 // force scratch, which the next evaluation overwrites.
 static relres_status autotune_pairs(relres_ctx* c) {
   c->tuned = true;
+  if (c->tune_mode < 0 && !c->fp64 && fp32_lanes(c, false) > 1) {  // configuration 0 over several lanes
+    c->pair_cfg = 0;
+    c->pair_lanes = fp32_lanes(c, false);
+    return RELRES_OK;
+  }
   if (c->tune_mode >= 0 || c->fp64 || c->n < 20000) {
     c->pair_cfg = c->tune_mode >= 0 ? c->tune_mode : 0;
     return RELRES_OK;
@@ -852,6 +866,7 @@ relres_status relres_set_force_accumulation(relres_ctx* c, int mode) {
     return fail(c, RELRES_ERR_ARG, "unknown force accumulation mode");
   CK(cudaStreamSynchronize(c->stream));
   c->force_acc = mode;
+  if (c->tune_mode < 0) untune(c);  // the lanes of small systems go with the accumulation
   drop_step_graph(c);
   ++c->buf_gen;  // batch graphs bake the launches in too
   return RELRES_OK;
@@ -860,7 +875,7 @@ relres_status relres_set_force_accumulation(relres_ctx* c, int mode) {
 relres_status relres_set_pair_config(relres_ctx* c, int config) {
   if (!c || config < -1 || config >= kNPairConfigs) return RELRES_ERR_ARG;
   c->tune_mode = config;
-  c->tuned = false;
+  untune(c);
   c->pair_cfg = config >= 0 ? config : 0;
   return RELRES_OK;
 }
@@ -1116,17 +1131,18 @@ relres_status relres_set_params(relres_ctx* c, const relres_params* p) {
   c->eps_fg.assign(p->eps_fg, p->eps_fg + p->n_types);
   c->sig_fg.assign(p->sig_fg, p->sig_fg + p->n_types);
   build_kernel_tables(c->recs, &c->tab_f, &c->tab_d);
+  pack_pair_rows(c->tab_f, c->tab_d, &c->rows_f, &c->rows_e);
   build_basis_tables(c->recs, p->shift, &c->basis_f, &c->basis_d);
   if (c->fp64) {
     CK(cudaMemcpy(c->d_tab, c->tab_d.data(), sizeof(PairTab<double>) * c->tab_d.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->d_basis, c->basis_d.data(), sizeof(BasisTab<double>) * c->basis_d.size(),
                   cudaMemcpyHostToDevice));
   } else {
-    CK(cudaMemcpy(c->d_tab, c->tab_f.data(), sizeof(PairTab<float>) * c->tab_f.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(c->d_tab, c->rows_f.data(), sizeof(PairRowF) * c->rows_f.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(c->d_tabe, c->rows_e.data(), sizeof(PairRowE) * c->rows_e.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->d_basis, c->basis_f.data(), sizeof(BasisTab<float>) * c->basis_f.size(),
                   cudaMemcpyHostToDevice));
   }
-  CK(cudaMemcpy(c->d_tabd, c->tab_d.data(), sizeof(PairTab<double>) * c->tab_d.size(), cudaMemcpyHostToDevice));
   c->forces_valid = false;
   return RELRES_OK;
 }
@@ -1394,7 +1410,7 @@ struct relres_batch {
   int mode = -1;                 // relres_batch_set_mode
   std::vector<int> shared;       // replicas in the shared launches of the captured graph
   std::vector<char> is_shared;   // [nrep]
-  BatchLaunch bl_pair, bl_drift, bl_sum;
+  BatchLaunch bl_pair, bl_pair_ev, bl_drift, bl_sum;
   RebuildBatch rebuild;
   DevState** d_states = nullptr;  // [nrep]
 };
@@ -1523,7 +1539,7 @@ static relres_status capture_shared(relres_batch* b, const std::vector<relres_ct
       c0->stream = own;
       if (s != RELRES_OK) b->err = "shared rebuild node (capture): " + c0->err;
     }
-    if (e == cudaSuccess && s == RELRES_OK) e = launch_pairs_batch(b->stream, fp64, acc, ev_step, b->bl_pair, ns);
+    if (e == cudaSuccess && s == RELRES_OK) e = launch_pairs_batch(b->stream, fp64, acc, ev_step, ev_step ? b->bl_pair_ev : b->bl_pair, ns);
     if (e == cudaSuccess && s == RELRES_OK) e = launch_sum_batch(b->stream, fp64, k, b->bl_sum, ns);
   }
   if (s == RELRES_OK && e != cudaSuccess) s = batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
@@ -1562,7 +1578,7 @@ static relres_status batch_graph(relres_batch* b, const std::vector<StepParams>&
   // device tables of the shared launches, uploaded before the capture
   cudaError_t e = cudaSuccess;
   if (ns > 0) {
-    e = prepare_pairs_batch(cs, &b->bl_pair);
+    e = prepare_pairs_batch(cs, &b->bl_pair, &b->bl_pair_ev);
     if (e == cudaSuccess) e = prepare_drift_batch(cs, ssp, svel.data(), &b->bl_drift);
     if (e == cudaSuccess) e = prepare_sum_batch(cs, ssp, svel.data(), &b->bl_sum);
     if (e == cudaSuccess) e = prepare_rebuild_batch(cs, &b->rebuild);
@@ -1766,6 +1782,7 @@ void relres_batch_destroy(relres_batch* b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   batch_drop_graph(b);
   free_batch(&b->bl_pair);
+  free_batch(&b->bl_pair_ev);
   free_batch(&b->bl_drift);
   free_batch(&b->bl_sum);
   free_rebuild_batch(&b->rebuild);
@@ -1915,7 +1932,7 @@ void relres_destroy(relres_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->body_stream) cudaStreamDestroy(c->body_stream);
   dfree(c->d_tab);
-  dfree(c->d_tabd);
+  dfree(c->d_tabe);
   dfree(c->d_cdt);
   dfree(c->d_mass);
   dfree(c->d_type);

@@ -1645,7 +1645,7 @@ static cudaError_t prepare_drift_batch_t(const std::vector<relres_ctx*>& cs, con
     smem = std::max(smem, drift_seg_smem<R>(cs[r]));
   }
   b->nblk = off.back();
-  b->smem = b->smem_ev = smem;
+  b->smem = smem;
   return upload_batch(b, args.data(), sizeof(DriftSegArgs<R>) * args.size(), off);
 }
 
@@ -1682,7 +1682,7 @@ static cudaError_t prepare_sum_batch_t(const std::vector<relres_ctx*>& cs, const
     off[r + 1] = off[r] + sum_blocks(cs[r]);
   }
   b->nblk = off.back();
-  b->smem = b->smem_ev = 0;
+  b->smem = 0;
   return upload_batch(b, args.data(), sizeof(SumArgs<R>) * args.size(), off);
 }
 

@@ -219,6 +219,27 @@ void build_kernel_tables(const std::vector<PairRecord>& recs, std::vector<PairTa
   }
 }
 
+void pack_pair_rows(const std::vector<PairTab<float>>& tf, const std::vector<PairTab<double>>& td,
+                    std::vector<PairRowF>* rows, std::vector<PairRowE>* rows_e) {
+  rows->resize(tf.size());
+  rows_e->resize(td.size());
+  for (size_t k = 0; k < tf.size(); ++k) {
+    const PairTab<float>& t = tf[k];
+    const float f[20] = {t.fgd[3], t.rsp2,   t.f12f, t.f6f, t.rsm,   t.fgd[0], t.fgd[1],  t.fgd[2],  t.rsp2,    t.rcp2,
+                         t.rsm,    t.rcm,    t.ond3, t.ond4, t.f12c, t.f6c,    t.cgod[0], t.cgod[1], t.cgod[2], t.cgod[3]};
+    std::memcpy((*rows)[k].v, f, sizeof f);
+    const PairTab<double>& d = td[k];
+    const double e[23] = {d.c12f, d.c6f, d.e_fg_shift, d.rsm, d.fg[0], d.fg[1], d.fg[2], d.fg[3], d.fg[4],
+                          d.c12c, d.c6c, d.gam_cm, d.rsm, d.rcm, d.on0, d.on3, d.on4, d.e_cg_close,
+                          d.cgo[0], d.cgo[1], d.cgo[2], d.cgo[3], d.cgo[4]};
+    for (int m = 0; m < 23; ++m) {
+      const float hi = float(e[m]);
+      (*rows_e)[k].v[2 * m] = hi;
+      (*rows_e)[k].v[2 * m + 1] = float(e[m] - double(hi));
+    }
+  }
+}
+
 namespace {
 // r^-k and its first two derivatives
 void powk3(double r, int k, double* u, double* du, double* d2u) {

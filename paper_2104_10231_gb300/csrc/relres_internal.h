@@ -50,6 +50,16 @@ struct PairTab {
 };
 static_assert(sizeof(PairTab<float>) % 8 == 4, "odd row length in words");
 
+// One type pair of the FP32 pair kernels as they read it (see pair.cuh): the
+// words of its force coefficients, and of its energy constants as float-float
+// values (energy steps).
+struct PairRowF {
+  float v[20];
+};
+struct PairRowE {
+  float v[46];
+};
+
 // Basis form of one type pair for the differentiable path.  Every smoothing
 // coefficient (Eq. 17, Eq. 18) and shift (Eq. 19) is linear in the potential,
 // so each part of Eq. 20 is C12 phi12(r) - C6 phi6(r), with phik the same
@@ -69,6 +79,8 @@ void build_basis_tables(const std::vector<PairRecord>& recs, int shift, std::vec
                         std::vector<BasisTab<double>>* td);
 void build_kernel_tables(const std::vector<PairRecord>& recs, std::vector<PairTab<float>>* tf,
                          std::vector<PairTab<double>>* td);
+void pack_pair_rows(const std::vector<PairTab<float>>& tf, const std::vector<PairTab<double>>& td,
+                    std::vector<PairRowF>* rows, std::vector<PairRowE>* rows_e);
 void mix_pair(int mixing, double ea, double sa, double eb, double sb, double* e, double* s);
 bool sum_rule(int nt, const double* eps, const double* sig, int mixing, const int* ci,
               const int* cj, double* eps_cg, double* sig_cg);
@@ -184,6 +196,8 @@ struct relres_ctx {
   bool fp64 = false;
   std::vector<relres::PairRecord> recs;
   std::vector<relres::PairTab<float>> tab_f;
+  std::vector<relres::PairRowF> rows_f;
+  std::vector<relres::PairRowE> rows_e;
   std::vector<relres::PairTab<double>> tab_d;
   double rlist_fg_cut = 0, rlist_cg_cut = 0;  // max r_s+, max r_c+ over pairs
   cudaStream_t stream = nullptr;
@@ -203,8 +217,8 @@ struct relres_ctx {
   int grad_n = 0;             // atoms the gradient buffers were allocated for
 
   // device tables
-  void* d_tab = nullptr;  // PairTab<float or double>[n_types^2]
-  void* d_tabd = nullptr; // PairTab<double>[n_types^2] (energies of the FP32 path)
+  void* d_tab = nullptr;  // PairRowF (FP32) or PairTab<double> [n_types^2]
+  void* d_tabe = nullptr; // PairRowE[n_types^2] (energies of the FP32 path)
   double* d_cdt = nullptr;   // per type: (dt/2m) * ftm2v  (set per step call)
   float2* d_cdt_ff = nullptr;  // the same as float-float (FP32 path)
   float* d_kec = nullptr;      // per type: m / 2 in kcal/mol per (A/fs)^2, FP32
@@ -349,6 +363,9 @@ struct relres_ctx {
   // the device displacement trigger.  Everything below is baked into the
   // instantiated graph; it is re-captured when any of it changes.
   int pair_cfg = 0;        // index into kPairConfigs
+  // threads per slot of forces-only launches that keep the force bits of one
+  // (pair_lanes.cu): the choice of small systems, 0 elsewhere (pair_cfg's kernel)
+  int pair_lanes = 0;
   int force_acc = RELRES_ACC_DEFAULT;  // relres_accumulation of the FP32 pair kernels
   int tune_mode = -1;      // -1: autotune on the first relres_step; >= 0: fixed configuration
   bool tuned = false;
@@ -459,12 +476,14 @@ struct BatchLaunch {
   size_t args_bytes = 0;
   int n_off = 0;
   int nblk = 0;
-  size_t smem = 0, smem_ev = 0;
+  size_t smem = 0;
+  int nt = 1;     // pair launches: most types of any replica
+  int lanes = 0;  // pair launches: threads per slot of pair_lanes.cu (0: k_pair_batch)
 };
 // (re)allocates the device tables of b as needed and copies args and off in (synchronous)
 cudaError_t upload_batch(BatchLaunch* b, const void* args, size_t bytes, const std::vector<int>& off);
 void free_batch(BatchLaunch* b);
-cudaError_t prepare_pairs_batch(const std::vector<relres_ctx*>& cs, BatchLaunch* b);
+cudaError_t prepare_pairs_batch(const std::vector<relres_ctx*>& cs, BatchLaunch* b, BatchLaunch* b_ev);
 cudaError_t launch_pairs_batch(cudaStream_t s, bool fp64, int acc, bool ev, const BatchLaunch& b, int nrep);
 cudaError_t prepare_drift_batch(const std::vector<relres_ctx*>& cs, const std::vector<StepParams>& sp,
                                 double* const* d_vel, BatchLaunch* b);
@@ -494,15 +513,39 @@ constexpr long long kRebuildKernels = 7;
 // MD steps take the segmented drift + bonded kernel and k_sum
 inline bool step_segments(const relres_ctx* c) { return c->seg_ok && c->use_seg; }
 
+constexpr int kPartSMs = 152;
+
+// slots of both lists
+inline long long pair_slots(const relres_ctx* c) {
+  return (long long)c->n + ((c->has_cg && c->n_h > 0) ? c->n_h : 0);
+}
+
+// Threads per slot of FP32 launches with compensated sums by the slots of the
+// launch (1: one thread per slot), for energy launches and for the forces-only
+// launches left to the library.  Measured on neopentane-like liquids (1.2
+// slots an atom), us per MD step forces only / with energies every step:
+//   atoms      8 lanes        4 lanes        1 thread
+//    1 715   26.2 /  38.2   27.4 /  44.5   32.0 /  82.2
+//   10 000   30.2 /  48.6   30.1 /  52.8   34.9 /  90.4
+//   20 000   36.8 /  57.0   33.6 /  56.4   36.4 /  94.2
+//   30 000   42.2 /  66.1   38.1 /  62.6   40.7 /  94.2
+//   40 000   48.1 /  72.9   44.4 /  67.5   42.3 /  94.8
+//   90 000   68.7 / 118.4   58.6 / 102.7   52.5 / 115.1
+//  160 000   98.8 / 180.9   79.6 / 149.5   73.2 / 147.7
+inline int fp32_lanes_for(long long slots, int acc, bool ev) {
+  if (acc != RELRES_ACC_COMPENSATED) return 1;
+  if (ev) return slots <= 20000 ? 8 : (slots <= 150000 ? 4 : 1);
+  return slots <= 12000 ? 8 : (slots <= 40000 ? 4 : 1);
+}
+inline int fp32_lanes(const relres_ctx* c, bool ev) { return fp32_lanes_for(pair_slots(c), c->force_acc, ev); }
+
 // FP64 forces-only pair launches: 32-thread blocks for a system with fewer
 // 256-slot blocks than SMs, else 256; eight threads per slot (walk_ordered)
 // for one whose slots fill fewer than four warps per SM with one thread each
-constexpr int kPartSMs = 152;
 constexpr int kFp64SmallTpa = 8;
 inline int fp64_pair_block(const relres_ctx* c) { return (c->n + 255) / 256 < kPartSMs ? 32 : 256; }
 inline int fp64_pair_tpa(const relres_ctx* c) {
-  const long long slots = (long long)c->n + ((c->has_cg && c->n_h > 0) ? c->n_h : 0);
-  return slots < 4LL * 32 * kPartSMs ? kFp64SmallTpa : 1;
+  return pair_slots(c) < 4LL * 32 * kPartSMs ? kFp64SmallTpa : 1;
 }
 
 // the lists the pair kernels walk: the pruned ones when pruning is on

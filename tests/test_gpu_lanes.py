@@ -1,0 +1,111 @@
+"""FP32 pair launches with several lanes per list (systems too small to fill the
+GPU with one thread per list) and the FP32 energy steps: the force bits of one
+thread per list, energies and virial that do not depend on the launch, and
+pruned lists with the same entries in the same order."""
+import numpy as np
+import pytest
+
+from paper_2104_10231_gb300 import relres as R
+from paper_2104_10231_gb300 import systems as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch as T
+
+    assert T.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2104_10231_gb300.build import build_library
+
+    build_library()
+    R.load()
+    return T
+
+
+def _dev(torch, a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+
+# list owners (atoms + hybrids) around the changes of the rule: 12 000 and
+# 40 000 for forces, 20 000 and 150 000 for energies; the FG reference (one
+# list) and propane in its smallest box have the longest and shortest lists
+SYSTEMS = {
+    "propane_648": lambda: S.propane(),
+    "fg_only_1250": lambda: S.fg_only(S.neopentane(n_mol=250, seed=6)),
+    "neopentane_10000": lambda: S.neopentane(n_mol=2000, seed=7),
+    "neopentane_10005": lambda: S.neopentane(n_mol=2001, density=0.5, seed=8),
+    "neopentane_16670": lambda: S.neopentane(n_mol=3334, density=0.5, seed=9),
+    "neopentane_33330": lambda: S.neopentane(n_mol=6666, seed=10),
+}
+
+
+@pytest.mark.parametrize("name", list(SYSTEMS))
+def test_lanes_keep_the_bits_of_one_thread(torch, name):
+    s = SYSTEMS[name]()
+    out = []
+    for config in (-1, 0):
+        ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP32), R.topology_for(s))
+        ctx.set_pair_config(config)
+        p, v = _dev(torch, s.pos), _dev(torch, s.vel)
+        ctx.build_neighbors(p, s.box)
+        th = torch.zeros((6, R.RELRES_THERMO_COLS), dtype=torch.float64, device="cuda")
+        ctx.step(60, s.dt, p, v, t_target=s.temperature, tau_fs=100.0, seed=3, thermo_every=10, d_thermo=th)
+        torch.cuda.synchronize()
+        lists = [ctx.get_list(w) for w in ((2, 3) if s.n_hybrid else (2,))]
+        out.append((p.cpu().numpy(), v.cpu().numpy(), th.cpu().numpy(), ctx.stats()["n_prunes"], lists))
+        ctx.close()
+    (p0, v0, t0, n0, l0), (p1, v1, t1, n1, l1) = out
+    assert np.array_equal(p0, p1) and np.array_equal(v0, v1)
+    assert np.array_equal(t0, t1)
+    assert n0 == n1 and n0 > 2
+    for a, b in zip(l0, l1):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("acc", [R.RELRES_ACC_FP32, R.RELRES_ACC_COMPENSATED, R.RELRES_ACC_FP64])
+@pytest.mark.parametrize("prune", [0.5, 0.0])
+def test_energies_and_virial_do_not_depend_on_accumulation_or_pruning(torch, acc, prune):
+    from oracle import core as O
+
+    s = S.neopentane(n_mol=400, seed=12)
+    ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP32), R.topology_for(s))
+    ctx.set_force_accumulation(acc)
+    ctx.set_prune(prune)
+    p = _dev(torch, s.pos)
+    ctx.build_neighbors(p, s.box)
+    f = torch.empty_like(p)
+    e, w = torch.zeros(4, dtype=torch.float64, device="cuda"), torch.zeros(6, dtype=torch.float64, device="cuda")
+    ctx.compute(p, f, e, w)
+    torch.cuda.synchronize()
+    ctx.close()
+    _, e0, w0 = O.pair_forces(s.pos, s.box, s.types, O.table_for(s), s.n_types, s.excl)
+    e, w = e.cpu().numpy(), w.cpu().numpy()
+    assert abs(e[0] + e[1] - e0) <= 1e-7 * abs(e0)
+    # FP32 products of each pair, summed exactly: a few 2^-24 of the largest component
+    assert np.abs(w - w0).max() <= 2e-6 * np.abs(w0[:3]).max()
+    key = (e.tobytes(), w.tobytes())
+    seen = test_energies_and_virial_do_not_depend_on_accumulation_or_pruning.__dict__.setdefault("seen", key)
+    assert seen == key
+
+
+def test_overlapping_atoms_keep_their_energy(torch):
+    """A pair whose energy and virial are past the range of the FP32 conversion
+    to fixed point (2^20 kcal/mol)."""
+    from oracle import core as O
+
+    s = S.propane()
+    pos = s.pos.copy()
+    pos[3] = pos[0] + np.array([0.5, 0.6, 0.4])  # atoms of two molecules, 0.88 A apart
+    ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP32), R.make_topology(s.types, s.mass_by_type, s.excl, None))
+    p = _dev(torch, pos)
+    ctx.build_neighbors(p, s.box)
+    f = torch.empty_like(p)
+    e, w = torch.zeros(4, dtype=torch.float64, device="cuda"), torch.zeros(6, dtype=torch.float64, device="cuda")
+    ctx.compute(p, f, e, w)
+    torch.cuda.synchronize()
+    ctx.close()
+    _, e0, w0 = O.pair_forces(pos, s.box, s.types, O.table_for(s), s.n_types, s.excl)
+    assert abs(e0) > 2.0 ** 20
+    assert abs(float(e[3]) - e0) <= 1e-7 * abs(e0)
+    assert np.abs(w.cpu().numpy() - w0).max() <= 1e-5 * np.abs(w0).max()
