@@ -632,6 +632,8 @@ relres_status relres_set_topology(relres_ctx* c, const relres_topology* t) {
   CK(dalloc(&c->d_cell_cg, size_t(n)));
   CK(dalloc(&c->d_slot_fg, size_t(n)));
   CK(dalloc(&c->d_slot_cg, size_t(n)));
+  CK(dalloc(&c->d_order_fg, size_t(n)));
+  CK(dalloc(&c->d_order_cg, size_t(nh)));
   CK(dalloc(&c->d_perm_fg, size_t(n)));
   CK(dalloc(&c->d_rank_fg, size_t(n)));
   CK(dalloc(&c->d_perm_cg, size_t(nh)));
@@ -1406,7 +1408,7 @@ struct relres_batch {
   std::string err;
   // single-launch path: one drift, one pair and one force-sum launch per step
   // for every replica (argument tables in device memory), and the list
-  // rebuilds of the replicas that need one in seven launches for all of them
+  // rebuilds of the replicas that need one in six launches for all of them
   int mode = -1;                 // relres_batch_set_mode
   std::vector<int> shared;       // replicas in the shared launches of the captured graph
   std::vector<char> is_shared;   // [nrep]
@@ -1495,7 +1497,7 @@ static void batch_drop_graph(relres_batch* b) {
 // The shared-launch part of one block of steps, captured on the batch stream
 // (tables uploaded beforehand): per replica the rollback snapshot and the
 // thermostat draws, then per step the batched drift, the work list of
-// replicas whose trigger fired with one conditional node holding the seven
+// replicas whose trigger fired with one conditional node holding the six
 // batched rebuild kernels, the batched pair kernel and the batched force sum.
 static relres_status capture_shared(relres_batch* b, const std::vector<relres_ctx*>& cs,
                                     const std::vector<StepParams>& sp, const std::vector<double*>& vel, int blk,
@@ -1964,6 +1966,8 @@ void relres_destroy(relres_ctx* c) {
   dfree(c->d_cell_cg);
   dfree(c->d_slot_fg);
   dfree(c->d_slot_cg);
+  dfree(c->d_order_fg);
+  dfree(c->d_order_cg);
   dfree(c->d_perm_fg);
   dfree(c->d_rank_fg);
   dfree(c->d_perm_cg);

@@ -12,8 +12,8 @@
 // the position gathers of the pair kernel local in L1/L2.
 //
 // Rebuild sequence: k_bin (cell of every atom, counts) -> k_scan (exclusive
-// scan per grid) -> k_scatter (slot = start + arrival rank) -> k_sort_cells
-// (atom order inside each cell, so lists are deterministic) -> k_pack (sorted
+// scan per grid) -> k_scatter (each cell's atoms, in arrival order) -> k_order
+// (slots in atom order inside each cell, so lists are deterministic: sorted
 // positions, ranks, reference positions for the displacement trigger) ->
 // k_list (FG and CG lists in one launch).  Every kernel can be gated on the
 // device rebuild flag, so the whole sequence can sit inside a CUDA graph step.
@@ -210,12 +210,12 @@ __device__ __forceinline__ void scatter_body(int bid, int nblk, int n, const uns
                                             const int* __restrict__ fstart, int with_cg,
                                             const int* __restrict__ cstart, const int* __restrict__ cell_fg,
                                             const int* __restrict__ slot_fg, const int* __restrict__ cell_cg,
-                                            const int* __restrict__ slot_cg, int* __restrict__ perm_fg,
-                                            int* __restrict__ perm_cg) {
+                                            const int* __restrict__ slot_cg, int* __restrict__ order_fg,
+                                            int* __restrict__ order_cg) {
   if (gate_closed(gate)) return;
   for (int i = bid * blockDim.x + threadIdx.x; i < n; i += nblk * blockDim.x) {
-    perm_fg[fstart[cell_fg[i]] + slot_fg[i]] = i;
-    if (with_cg && ((hyb_mask >> type[i]) & 1)) perm_cg[cstart[cell_cg[i]] + slot_cg[i]] = i;
+    order_fg[fstart[cell_fg[i]] + slot_fg[i]] = i;
+    if (with_cg && ((hyb_mask >> type[i]) & 1)) order_cg[cstart[cell_cg[i]] + slot_cg[i]] = i;
   }
 }
 
@@ -223,77 +223,67 @@ __global__ void k_scatter(int n, const unsigned* gate, const int* __restrict__ t
                           const int* __restrict__ fstart, int with_cg, const int* __restrict__ cstart,
                           const int* __restrict__ cell_fg, const int* __restrict__ slot_fg,
                           const int* __restrict__ cell_cg, const int* __restrict__ slot_cg,
-                          int* __restrict__ perm_fg, int* __restrict__ perm_cg) {
+                          int* __restrict__ order_fg, int* __restrict__ order_cg) {
   scatter_body(blockIdx.x, gridDim.x, n, gate, type, hyb_mask, fstart, with_cg, cstart, cell_fg, slot_fg, cell_cg,
-               slot_cg, perm_fg, perm_cg);
+               slot_cg, order_fg, order_cg);
 }
 
-// One thread per cell: the cell's atoms put in index order (the scatter order
-// is arbitrary) by an insertion sort in place; cells hold ~5 atoms.
-__device__ __forceinline__ void sort_body(int bid, int nblk, const unsigned* gate, int fn, const int* fstart, int cn,
-                                         const int* cstart, int* __restrict__ perm_fg, int* __restrict__ perm_cg) {
+// The slots of the atoms, cell by cell: `width` lanes (a power of two, at most
+// 32) take one cell.  An atom's slot is the cell's start plus the number of
+// the cell's atoms with a smaller index (k_scatter left them in arrival
+// order); its sorted position, ranks and reference position are written at
+// once.  Lanes per cell: 8 where cells hold few atoms (x-slabs), else 32.
+// Against one thread per cell with an insertion sort (13 us at 20 000 atoms,
+// 75 us at 250 000 atoms of the FG reference, 110 us for a batch of small
+// boxes with whole cells) and a packing pass: 12 us less per rebuild at 20 000
+// atoms, 120 us less at 250 000, 4.97 -> 4.63 ms per 25 steps of 24 replicas.
+struct OrderGrid {
+  int ncell;  // 0: no such list
+  const int* start;
+  const int* order;
+  int* perm;
+  int* rank;
+  int4* pos;
+  Pos64* pos64;
+};
+
+__device__ __forceinline__ void order_body(int bid, int nblk, const unsigned* gate, const OrderGrid& fg,
+                                          const OrderGrid& cg, const unsigned long long* __restrict__ xfx,
+                                          const int* __restrict__ type, int fp64, int4* __restrict__ ref, int width) {
   if (gate_closed(gate)) return;
-  for (int t = bid * blockDim.x + threadIdx.x; t < fn + cn; t += nblk * blockDim.x) {
-    const bool fg = t < fn;
-    const int c = fg ? t : t - fn;
-    const int* const start = fg ? fstart : cstart;
-    int* const perm = fg ? perm_fg : perm_cg;
-    const int lo = start[c], hi = start[c + 1];
-    for (int k = lo + 1; k < hi; ++k) {
-      const int v = perm[k];
-      int q = k - 1;
-      int u = perm[q];
-      while (u > v) {
-        perm[q + 1] = u;
-        if (--q < lo) break;
-        u = perm[q];
-      }
-      perm[q + 1] = v;
+  const int lane = threadIdx.x & (width - 1), per = blockDim.x / width;
+  const int total = fg.ncell + cg.ncell;
+  for (int c = bid * per + threadIdx.x / width; c < total; c += nblk * per) {
+    const bool is_fg = c < fg.ncell;
+    const int k = is_fg ? c : c - fg.ncell;
+    const int* const start = is_fg ? fg.start : cg.start;
+    const int* const order = is_fg ? fg.order : cg.order;
+    int* const perm = is_fg ? fg.perm : cg.perm;
+    int* const rank = is_fg ? fg.rank : cg.rank;
+    int4* const pos = is_fg ? fg.pos : cg.pos;
+    Pos64* const pos64 = is_fg ? fg.pos64 : cg.pos64;
+    const int lo = start[k], hi = start[k + 1];
+    for (int q = lo + lane; q < hi; q += width) {
+      const int i = order[q];
+      int s = lo;
+      for (int m = lo; m < hi; ++m) s += order[m] < i ? 1 : 0;
+      const unsigned long long x = xfx[3 * i], y = xfx[3 * i + 1], z = xfx[3 * i + 2];
+      const int t = type[i];
+      const int4 h = make_int4(hi32(x), hi32(y), hi32(z), t);
+      perm[s] = i;
+      rank[i] = s;
+      pos[s] = h;
+      if (fp64) pos64[s] = Pos64{(long long)x, (long long)y, (long long)z, t};
+      if (is_fg) ref[i] = h;
     }
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_sort_cells(const unsigned* gate, int fn, const int* fstart, int cn,
-                                                         const int* cstart, int* __restrict__ perm_fg,
-                                                         int* __restrict__ perm_cg) {
-  sort_body(blockIdx.x, gridDim.x, gate, fn, fstart, cn, cstart, perm_fg, perm_cg);
-}
-
-__device__ __forceinline__ void pack_body(int bid, int nblk, int n, int n_h, const unsigned* gate,
-                                         const unsigned long long* __restrict__ xfx, const int* __restrict__ type,
-                                         const int* __restrict__ perm_fg, const int* __restrict__ perm_cg,
-                                         int* __restrict__ rank_fg, int* __restrict__ rank_cg,
-                                         int4* __restrict__ pos_fg, int4* __restrict__ pos_cg,
-                                         Pos64* __restrict__ pos_fg64, Pos64* __restrict__ pos_cg64, int fp64,
-                                         int4* __restrict__ ref) {
-  if (gate_closed(gate)) return;
-  for (int s = bid * blockDim.x + threadIdx.x; s < n; s += nblk * blockDim.x) {
-    const int i = perm_fg[s];
-    const unsigned long long x = xfx[3 * i], y = xfx[3 * i + 1], z = xfx[3 * i + 2];
-    const int t = type[i];
-    rank_fg[i] = s;
-    const int4 h = make_int4(hi32(x), hi32(y), hi32(z), t);
-    pos_fg[s] = h;
-    ref[i] = h;
-    if (fp64) pos_fg64[s] = Pos64{(long long)x, (long long)y, (long long)z, t};
-    if (s < n_h) {
-      const int j = perm_cg[s];
-      const unsigned long long xj = xfx[3 * j], yj = xfx[3 * j + 1], zj = xfx[3 * j + 2];
-      rank_cg[j] = s;
-      pos_cg[s] = make_int4(hi32(xj), hi32(yj), hi32(zj), type[j]);
-      if (fp64) pos_cg64[s] = Pos64{(long long)xj, (long long)yj, (long long)zj, type[j]};
-    }
-  }
-}
-
-__global__ void k_pack(int n, int n_h, const unsigned* gate, const unsigned long long* __restrict__ xfx,
-                       const int* __restrict__ type, const int* __restrict__ perm_fg,
-                       const int* __restrict__ perm_cg, int* __restrict__ rank_fg,
-                       int* __restrict__ rank_cg, int4* __restrict__ pos_fg,
-                       int4* __restrict__ pos_cg, Pos64* __restrict__ pos_fg64,
-                       Pos64* __restrict__ pos_cg64, int fp64, int4* __restrict__ ref) {
-  pack_body(blockIdx.x, gridDim.x, n, n_h, gate, xfx, type, perm_fg, perm_cg, rank_fg, rank_cg, pos_fg, pos_cg,
-            pos_fg64, pos_cg64, fp64, ref);
+__global__ void __launch_bounds__(kThreads) k_order(const unsigned* gate, OrderGrid fg, OrderGrid cg,
+                                                    const unsigned long long* __restrict__ xfx,
+                                                    const int* __restrict__ type, int fp64, int4* __restrict__ ref,
+                                                    int width) {
+  order_body(blockIdx.x, gridDim.x, gate, fg, cg, xfx, type, fp64, ref, width);
 }
 
 struct ListArgs {
@@ -620,16 +610,16 @@ static int blocks_for(int n) {
 }
 
 // ---- batches (relres_batch_step): the list rebuild of every replica whose
-// displacement trigger fired, in seven launches for the whole batch.  After the
+// displacement trigger fired, in six launches for the whole batch.  After the
 // drift, k_worklist lists those replicas and, per kernel class, the prefix
 // sums of the blocks each of them takes in its own rebuild (the same counts as
 // launch_rebuild / launch_lists); each batched kernel then walks the work
 // items (replica, block) with a fixed grid, so a step in which few replicas
-// rebuild costs seven short launches, and one in which none does, seven empty ones.
+// rebuild costs six short launches, and one in which none does, none.
 
 // Everything one replica's rebuild kernels take.
 struct BuildArgs {
-  int n, n_h_pack, hyb_mask, fp64;
+  int n, hyb_mask, fp64;
   const unsigned* gate;
   const unsigned long long* xfx;
   const int* type;
@@ -639,21 +629,17 @@ struct BuildArgs {
   int* cell_cg;
   int* slot_cg;
   unsigned* flags;
-  int* perm_fg;
-  int* perm_cg;
-  int* rank_fg;
-  int* rank_cg;
-  int4* pos_fg;
-  int4* pos_cg;
-  Pos64* p64f;
-  Pos64* p64c;
+  int* order_fg;
+  int* order_cg;
+  OrderGrid ofg, ocg;
+  int order_width;
   int4* ref;
   DevState* st;
   ListArgs lfg, lcg;
   int ncell_cg;
 };
 
-enum { kRbBin = 0, kRbScanTiles, kRbScanAdd, kRbScatter, kRbSort, kRbPack, kRbList, kRbClasses };
+enum { kRbBin = 0, kRbScanTiles, kRbScanAdd, kRbScatter, kRbOrder, kRbList, kRbClasses };
 
 // one block: wl[0] = number of rebuilding replicas, wl[1 .. nrep] their
 // indices, then per class k the prefix sums pre_k[0 .. count] at
@@ -764,24 +750,15 @@ __global__ void __launch_bounds__(kThreads, 6) k_scatter_batch(const BuildArgs* 
                                 const int* __restrict__ nbt, int nrep) {
   RELRES_BATCH_LOOP(kRbScatter)
   scatter_body(b, nb, sa.n, sa.gate, sa.type, sa.hyb_mask, sa.gf.start, sa.gc.valid, sa.gc.start, sa.cell_fg,
-               sa.slot_fg, sa.cell_cg, sa.slot_cg, sa.perm_fg, sa.perm_cg);
+               sa.slot_fg, sa.cell_cg, sa.slot_cg, sa.order_fg, sa.order_cg);
   RELRES_BATCH_END
 }
 
-__global__ void __launch_bounds__(kThreads, 6) k_sort_batch(const BuildArgs* __restrict__ args,
-                                                         const int* __restrict__ wl, const int* __restrict__ nbt,
-                                                         int nrep) {
-  RELRES_BATCH_LOOP(kRbSort)
-  sort_body(b, nb, sa.gate, sa.gf.ncell, sa.gf.start, sa.gc.valid ? sa.gc.ncell : 0, sa.gc.start, sa.perm_fg,
-            sa.perm_cg);
-  RELRES_BATCH_END
-}
-
-__global__ void __launch_bounds__(kThreads, 6) k_pack_batch(const BuildArgs* __restrict__ args, const int* __restrict__ wl,
-                             const int* __restrict__ nbt, int nrep) {
-  RELRES_BATCH_LOOP(kRbPack)
-  pack_body(b, nb, sa.n, sa.n_h_pack, sa.gate, sa.xfx, sa.type, sa.perm_fg, sa.perm_cg, sa.rank_fg, sa.rank_cg,
-            sa.pos_fg, sa.pos_cg, sa.p64f, sa.p64c, sa.fp64, sa.ref);
+__global__ void __launch_bounds__(kThreads, 6) k_order_batch(const BuildArgs* __restrict__ args,
+                                                             const int* __restrict__ wl, const int* __restrict__ nbt,
+                                                             int nrep) {
+  RELRES_BATCH_LOOP(kRbOrder)
+  order_body(b, nb, sa.gate, sa.ofg, sa.ocg, sa.xfx, sa.type, sa.fp64, sa.ref, sa.order_width);
   RELRES_BATCH_END
 }
 
@@ -810,7 +787,6 @@ static BuildArgs build_args(relres_ctx* c, const unsigned* gate) {
     b.gc.valid = 0;
   }
   b.n = c->n;
-  b.n_h_pack = b.gc.valid ? c->n_h : 0;
   b.hyb_mask = c->hyb_mask;
   b.fp64 = c->fp64 ? 1 : 0;
   b.gate = gate;
@@ -821,14 +797,16 @@ static BuildArgs build_args(relres_ctx* c, const unsigned* gate) {
   b.cell_cg = c->d_cell_cg;
   b.slot_cg = c->d_slot_cg;
   b.flags = &c->d_state->flags;
-  b.perm_fg = c->d_perm_fg;
-  b.perm_cg = c->d_perm_cg;
-  b.rank_fg = c->d_rank_fg;
-  b.rank_cg = c->d_rank_cg;
-  b.pos_fg = c->d_pos_fg;
-  b.pos_cg = c->d_pos_cg;
-  b.p64f = c->fp64 ? c->d_pos_fg64 : static_cast<Pos64*>(c->d_dummy);
-  b.p64c = c->fp64 ? c->d_pos_cg64 : static_cast<Pos64*>(c->d_dummy);
+  b.order_fg = c->d_order_fg;
+  b.order_cg = c->d_order_cg;
+  b.ofg = OrderGrid{c->gfg.ncell, c->gfg.d_start, c->d_order_fg, c->d_perm_fg, c->d_rank_fg, c->d_pos_fg,
+                    c->fp64 ? c->d_pos_fg64 : static_cast<Pos64*>(c->d_dummy)};
+  b.ocg = b.ofg;  // stand-in without a CG list
+  b.ocg.ncell = 0;
+  if (b.gc.valid)
+    b.ocg = OrderGrid{c->gcg.ncell, c->gcg.d_start, c->d_order_cg, c->d_perm_cg, c->d_rank_cg, c->d_pos_cg,
+                      c->fp64 ? c->d_pos_cg64 : static_cast<Pos64*>(c->d_dummy)};
+  b.order_width = c->n > 12LL * c->gfg.ncell ? 32 : 8;
   b.ref = c->d_ref;
   b.st = c->d_state;
   b.lfg = list_args_fg(c);
@@ -840,7 +818,9 @@ static BuildArgs build_args(relres_ctx* c, const unsigned* gate) {
 
 // list-kernel blocks: persistent, one wave walks the cells (a closed gate costs one small launch)
 static int list_blocks(const BuildArgs& b) { return std::min(b.ncell_cg + b.gf.ncell_full, 152 * 8); }
-static int sort_cells_of(const BuildArgs& b) { return b.gf.ncell + (b.gc.valid ? b.gc.ncell : 0); }
+static int order_blocks(const BuildArgs& b) {
+  return blocks_for(int(std::min(1LL << 30, (long long)(b.ofg.ncell + b.ocg.ncell) * b.order_width)));
+}
 
 cudaError_t launch_rebuild(relres_ctx* c, const unsigned* gate) {
   if (gate == nullptr) gate = c->d_open;
@@ -860,14 +840,10 @@ cudaError_t launch_rebuild(relres_ctx* c, const unsigned* gate) {
   RELRES_LAUNCHED(c);
   k_scatter<<<nb, kThreads, 0, c->stream>>>(c->n, gate, c->d_type, c->hyb_mask, gf.start, gc.valid, gc.start,
                                             c->d_cell_fg, c->d_slot_fg, c->d_cell_cg, c->d_slot_cg,
-                                            c->d_perm_fg, c->d_perm_cg);
+                                            c->d_order_fg, c->d_order_cg);
   RELRES_LAUNCHED(c);
-  k_sort_cells<<<blocks_for(sort_cells_of(b)), kThreads, 0, c->stream>>>(
-      gate, gf.ncell, gf.start, gc.valid ? gc.ncell : 0, gc.start, c->d_perm_fg, c->d_perm_cg);
-  RELRES_LAUNCHED(c);
-  k_pack<<<nb, kThreads, 0, c->stream>>>(c->n, b.n_h_pack, gate, c->d_xfx, c->d_type, c->d_perm_fg, c->d_perm_cg,
-                                         c->d_rank_fg, c->d_rank_cg, c->d_pos_fg, c->d_pos_cg, b.p64f, b.p64c,
-                                         b.fp64, c->d_ref);
+  k_order<<<order_blocks(b), kThreads, 0, c->stream>>>(gate, b.ofg, b.ocg, c->d_xfx, c->d_type, b.fp64, c->d_ref,
+                                                       b.order_width);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
@@ -884,8 +860,7 @@ cudaError_t prepare_rebuild_batch(const std::vector<relres_ctx*>& cs, RebuildBat
     nbt[kRbScanTiles * nr + r] = ntiles;
     nbt[kRbScanAdd * nr + r] = ntiles;
     nbt[kRbScatter * nr + r] = blocks_for(c->n);
-    nbt[kRbSort * nr + r] = blocks_for(sort_cells_of(args[r]));
-    nbt[kRbPack * nr + r] = blocks_for(c->n);
+    nbt[kRbOrder * nr + r] = order_blocks(args[r]);
     nbt[kRbList * nr + r] = list_blocks(args[r]);
   }
   const std::vector<int> off{0, nr};
@@ -916,8 +891,7 @@ cudaError_t launch_rebuild_batch(cudaStream_t s, const RebuildBatch& rb, int nre
   k_scan_tiles_batch<<<152, kScanTile / 4, 0, s>>>(args, wl, nbt, nrep);
   k_scan_add_batch<<<152, kScanTile / 4, 0, s>>>(args, wl, nbt, nrep);
   k_scatter_batch<<<152 * 4, kThreads, 0, s>>>(args, wl, nbt, nrep);
-  k_sort_batch<<<152 * 4, kThreads, 0, s>>>(args, wl, nbt, nrep);
-  k_pack_batch<<<152 * 4, kThreads, 0, s>>>(args, wl, nbt, nrep);
+  k_order_batch<<<152 * 4, kThreads, 0, s>>>(args, wl, nbt, nrep);
   k_list_batch<<<152 * 8, kListThreads, 0, s>>>(args, wl, nbt, nrep);
   return cudaGetLastError();
 }

@@ -267,6 +267,8 @@ struct relres_ctx {
   int* d_cell_cg = nullptr;
   int* d_slot_fg = nullptr;             // arrival rank of the atom inside its cell
   int* d_slot_cg = nullptr;
+  int* d_order_fg = nullptr;            // each cell's atoms in arrival order
+  int* d_order_cg = nullptr;
   int* d_perm_fg = nullptr;             // FG slot -> atom
   int* d_rank_fg = nullptr;             // atom -> FG slot
   int* d_perm_cg = nullptr;             // CG slot -> atom
@@ -492,7 +494,7 @@ cudaError_t prepare_sum_batch(const std::vector<relres_ctx*>& cs, const std::vec
                               double* const* d_vel, BatchLaunch* b);
 cudaError_t launch_sum_batch(cudaStream_t s, bool fp64, int k, const BatchLaunch& b, int nrep);
 // the list rebuild of every replica whose displacement trigger fired (d_states[r]->flags & F_REBUILD):
-// a work-list kernel and seven batched rebuild kernels (neighbor.cu)
+// a work-list kernel and six batched rebuild kernels (neighbor.cu)
 struct RebuildBatch {
   BatchLaunch args;  // BuildArgs per replica
   BatchLaunch nbt;   // blocks of each kernel class per replica
@@ -503,12 +505,12 @@ cudaError_t prepare_rebuild_batch(const std::vector<relres_ctx*>& cs, RebuildBat
 // the work list of this step; sets `any` (a graph conditional) iff some replica rebuilds
 cudaError_t launch_worklist(cudaStream_t s, const RebuildBatch& rb, DevState* const* d_states, int nrep,
                             cudaGraphConditionalHandle any);
-// the seven batched rebuild kernels over the work list
+// the six batched rebuild kernels over the work list
 cudaError_t launch_rebuild_batch(cudaStream_t s, const RebuildBatch& rb, int nrep);
 void free_rebuild_batch(RebuildBatch* rb);
 // kernels of one list rebuild: k_bin, k_scan_tiles, k_scan_add, k_scatter,
-// k_sort_cells, k_pack, k_list
-constexpr long long kRebuildKernels = 7;
+// k_order, k_list
+constexpr long long kRebuildKernels = 6;
 
 // MD steps take the segmented drift + bonded kernel and k_sum
 inline bool step_segments(const relres_ctx* c) { return c->seg_ok && c->use_seg; }
