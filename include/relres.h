@@ -373,10 +373,9 @@ relres_status relres_backward(relres_ctx* ctx, const double* d_pos, const double
 /*
  * Step execution mode (an implementation choice; the paper has no
  * counterpart).  enable != 0 (the default) runs relres_step as one CUDA graph
- * per block of up to 100 steps: the list rebuild of every step is a
- * conditional node that a one-thread kernel opens only when the device-side
- * displacement trigger fired, so steps without a rebuild launch no binning or
- * list kernels.  The graph is captured on first use and reused while the
+ * per block of up to 100 steps: the list rebuild of every step is one
+ * cooperative kernel that returns at once unless the device-side displacement
+ * trigger fired.  The graph is captured on first use and reused while the
  * step arguments, the timing mode and the context's buffers stay the same
  * (re-captured otherwise).  enable == 0 launches the kernels on the stream
  * one by one, the rebuild kernels gated on the device flag.  Both modes give
@@ -542,8 +541,8 @@ relres_status relres_set_force_accumulation(relres_ctx* ctx, int mode);
  * relres_timing_class and accumulate the elapsed times; enable == 0 stops it.
  * On the stream path the gated rebuild kernels are timed also when they find
  * nothing to do; in graph mode (relres_set_graphs) RELRES_T_REBUILD times the
- * decision kernel plus the conditional rebuild node (binning and both lists)
- * and RELRES_T_LISTS stays empty.  relres_set_timing always clears the totals.
+ * rebuild kernel (binning, both lists and a separate pruning pass)
+ * and RELRES_T_LISTS and RELRES_T_PRUNE stay empty.  relres_set_timing always clears the totals.
  * relres_get_timings writes, for the first n classes, the total milliseconds
  * (ms[k]) and the number of timed launches (counts[k]; either may be NULL).
  */

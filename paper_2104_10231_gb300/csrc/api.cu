@@ -98,7 +98,7 @@ relres_status setup_grid(relres_ctx* c, Grid* g, double rlist) {
   CK(dalloc(&g->d_rank_of, size_t(nc)));
   CK(dalloc(&g->d_start, size_t(nc) + 1));
   CK(dalloc(&g->d_count, size_t(nc)));
-  CK(dalloc(&g->d_tile, size_t(g->ntile)));
+  CK(dalloc(&g->d_tile, size_t((nc + kScanTileMin - 1) / kScanTileMin)));
   CK(cudaMemcpy(g->d_rank_of, rank.data(), sizeof(int) * nc, cudaMemcpyHostToDevice));
   CK(cudaMemset(g->d_count, 0, sizeof(int) * nc));
   CK(cudaMemset(g->d_start, 0, sizeof(int) * (nc + 1)));
@@ -354,6 +354,8 @@ relres_status relres_create(relres_ctx** out, const relres_params* p, void* cuda
   if (ce == cudaSuccess) ce = cudaMemset(c->d_acc, 0, sizeof(long long) * kNAcc);
   if (ce == cudaSuccess) ce = cudaMalloc(&c->d_draws, sizeof(double) * 2 * kBlockSteps);
   if (ce == cudaSuccess) ce = cudaMemset(c->d_draws, 0, sizeof(double) * 2 * kBlockSteps);
+  if (ce == cudaSuccess) ce = cudaMalloc(&c->d_bar, 2 * sizeof(unsigned));
+  if (ce == cudaSuccess) ce = cudaMemset(c->d_bar, 0, 2 * sizeof(unsigned));
   if (ce == cudaSuccess) ce = cudaMalloc(&c->d_open, sizeof(unsigned));
   if (ce == cudaSuccess) {
     const unsigned open = F_REBUILD;
@@ -883,8 +885,9 @@ relres_status relres_set_pair_config(relres_ctx* c, int config) {
 }
 
 // ---- relres_step: one block of steps, recorded either on the stream (the
-// rebuild kernels gated on the device flag) or into a CUDA graph (the
-// rebuild of each step behind a conditional node).
+// rebuild kernels gated on the device flag) or into a CUDA graph (the rebuild
+// of each step as one gated kernel; behind a conditional node on the branches
+// of a batch graph).
 
 static void drop_one_graph(relres_ctx::StepGraph& g) {
   if (g.exec) cudaGraphExecDestroy(g.exec);
@@ -958,7 +961,9 @@ static relres_status add_rebuild_node(relres_ctx* c, cudaGraphConditionalHandle*
 // those steps (graph: a conditional node; stream: a launch gated on the flags).
 static relres_status record_pairs(relres_ctx* c, bool ev, bool graph, cudaGraphConditionalHandle hp) {
   if (c->prune_on && !pairs_prune(c)) {
-    if (graph) {
+    if (graph && c->use_fused) {
+      // pruned with the rebuild
+    } else if (graph) {
       const bool t_ = timed_now(c, RELRES_T_PRUNE);
       if (t_) CK(tic(c, RELRES_T_PRUNE));
       relres_status s = add_conditional(c, hp, [c]() { return launch_prune(c, c->d_open); });
@@ -991,8 +996,12 @@ static relres_status record_block(relres_ctx* c, const StepParams& sp, double* d
     if (graph) {
       const bool t_ = timed_now(c, RELRES_T_REBUILD);
       if (t_) CK(tic(c, RELRES_T_REBUILD));
-      relres_status s = add_rebuild_node(c, &hp);
-      if (s != RELRES_OK) return s;
+      if (c->use_fused) {
+        CK(launch_rebuild_fused(c, c->prune_on && !pairs_prune(c)));
+      } else {
+        relres_status s = add_rebuild_node(c, &hp);
+        if (s != RELRES_OK) return s;
+      }
       if (t_) CK(toc(c));
     } else {
       TIMED(RELRES_T_REBUILD, launch_rebuild(c, gate));
@@ -1078,8 +1087,9 @@ static relres_status step_graph(relres_ctx* c, const StepParams& sp, double* d_v
   }
   // kernels: per step the rebuild body holds kRebuildKernels (binning stages +
   // lists), the pruning body 1, and the decide kernel sits in the parent
-  g.k_body = kRebuildKernels;
-  g.k_prune = (c->prune_on && !pairs_prune(c)) ? 1 : 0;
+  // (none of them where the rebuild is one kernel of the parent)
+  g.k_body = c->use_fused ? 0 : kRebuildKernels;
+  g.k_prune = (!c->use_fused && c->prune_on && !pairs_prune(c)) ? 1 : 0;
   g.k_parent = captured - (g.k_body + g.k_prune) * blk;
   g.valid = true;
   g.blk = blk;
@@ -1327,6 +1337,12 @@ static relres_status block_end(relres_ctx* c, double* d_pos, double* d_vel, doub
   }
   const unsigned fl = c->h_state->flags;
   if (fl & F_BADCELL) return fail(c, RELRES_ERR_CUDA, "cell binning produced an out-of-range index");
+  if (fl & F_BARRIER) {
+    CK(launch_flags_and(c, ~(unsigned)F_BARRIER));
+    CK(cudaMemsetAsync(c->d_bar, 0, 2 * sizeof(unsigned), c->stream));
+    c->have_lists = false;  // left unfinished
+    return fail(c, RELRES_ERR_CUDA, "the list rebuild's grid-wide barrier timed out");
+  }
   if (fl & (F_OVERFLOW_FG | F_OVERFLOW_CG | F_NONFINITE)) {
     s = rollback_block(c, d_vel);
     if (s != RELRES_OK) return s;
@@ -1607,15 +1623,17 @@ static relres_status batch_graph(relres_batch* b, const std::vector<StepParams>&
     e = cudaStreamWaitEvent(b->fork[r], b->ev_fork, 0);
     if (e != cudaSuccess) break;
     const cudaStream_t own = c->stream;
-    const bool timing = c->timing, pdl = c->use_pdl;
+    const bool timing = c->timing, pdl = c->use_pdl, fused = c->use_fused;
     const long long n0 = c->n_launches;
     c->stream = b->fork[r];
     c->timing = false;  // per-class timing is not recorded in batches
     // no programmatic dependent launches on branches: a kernel waiting for its
     // predecessor would hold SM resources that other branches' kernels can use
     c->use_pdl = false;
+    c->use_fused = false;  // nor blocks that wait for one another beside other branches
     s = record_block(c, sp[r], d_vel[r], blk, done, true);
     c->use_pdl = pdl;
+    c->use_fused = fused;
     if (s != RELRES_OK) b->err = "replica " + std::to_string(r) + " (capture): " + c->err;
     const long long kpr = (c->prune_on && !pairs_prune(c)) ? 1 : 0;
     b->k_parent[r] = (c->n_launches - n0) - (kRebuildKernels + kpr) * blk;
@@ -2011,6 +2029,7 @@ void relres_destroy(relres_ctx* c) {
   dfree(c->d_snap_f);
   dfree(c->d_snap_state);
   dfree(c->d_dummy);
+  dfree(c->d_bar);
   dfree(c->d_open);
   if (c->h_state) cudaFreeHost(c->h_state);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);

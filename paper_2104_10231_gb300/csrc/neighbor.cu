@@ -54,9 +54,8 @@ __device__ __forceinline__ void bin_body(int bid, int nblk, int n, const unsigne
                                         const unsigned long long* __restrict__ xfx, const int* __restrict__ type,
                                         int hyb_mask, int f0, int f1, int f2, const int* __restrict__ frank,
                                         int* fcount, int with_cg, int c0, int c1, int c2,
-                                        const int* __restrict__ crank, int* ccount, int* __restrict__ cell_fg,
-                                        int* __restrict__ slot_fg, int* __restrict__ cell_cg,
-                                        int* __restrict__ slot_cg, unsigned* flags) {
+                                        const int* __restrict__ crank, int* ccount, int* cell_fg, int* slot_fg,
+                                        int* cell_cg, int* slot_cg, unsigned* flags) {
   if (gate_closed(gate)) return;
   const int nf = f0 * f1 * f2, nc = c0 * c1 * c2;
   bool bad = false;
@@ -99,8 +98,8 @@ __global__ void k_bin(int n, const unsigned* gate, const unsigned long long* __r
 }
 
 // Exclusive scan of the cell counts into start[0..ncell] in two passes over
-// tiles of kScanTile cells: scan_tile_body scans one tile locally (4 cells per
-// thread of 1024, warp shuffles, then the warp totals), writes the tile total
+// tiles of four cells per thread of a block (kScanTile in blocks of 1024):
+// scan_tile_body scans one tile locally (warp shuffles, then the warp totals), writes the tile total
 // and resets the counts to zero for the next build; scan_add_body adds the sum
 // of the tile totals before its tile.  Tile t of a build: the tiles of the FG
 // grid, then those of the CG grid.
@@ -135,7 +134,7 @@ __device__ __forceinline__ void scan_tile_body(int t, const unsigned* gate, cons
   pick_scan(g0, g1, t, &g, &tile);
   __shared__ int sh[kScanTile / 4 / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int c0 = tile * kScanTile + 4 * threadIdx.x;
+  const int c0 = 4 * (tile * int(blockDim.x) + int(threadIdx.x));
   int v[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) v[q] = c0 + q < g.ncell ? g.count[c0 + q] : 0;
@@ -184,7 +183,7 @@ __device__ __forceinline__ void scan_add_body(int t, const unsigned* gate, const
   __syncthreads();
   int off = 0;
   for (int w = 0; w < nw; ++w) off += sh[w];
-  const int c0 = tile * kScanTile + 4 * threadIdx.x;
+  const int c0 = 4 * (tile * int(blockDim.x) + int(threadIdx.x));
 #pragma unroll
   for (int q = 0; q < 4; ++q)
     if (c0 + q < g.ncell) g.start[c0 + q] += off;
@@ -206,12 +205,9 @@ __host__ __device__ __forceinline__ ScanGrid scan_grid(const GridArgs& g) {
 }
 
 __device__ __forceinline__ void scatter_body(int bid, int nblk, int n, const unsigned* gate,
-                                            const int* __restrict__ type, int hyb_mask,
-                                            const int* __restrict__ fstart, int with_cg,
-                                            const int* __restrict__ cstart, const int* __restrict__ cell_fg,
-                                            const int* __restrict__ slot_fg, const int* __restrict__ cell_cg,
-                                            const int* __restrict__ slot_cg, int* __restrict__ order_fg,
-                                            int* __restrict__ order_cg) {
+                                            const int* __restrict__ type, int hyb_mask, const int* fstart,
+                                            int with_cg, const int* cstart, const int* cell_fg, const int* slot_fg,
+                                            const int* cell_cg, const int* slot_cg, int* order_fg, int* order_cg) {
   if (gate_closed(gate)) return;
   for (int i = bid * blockDim.x + threadIdx.x; i < n; i += nblk * blockDim.x) {
     order_fg[fstart[cell_fg[i]] + slot_fg[i]] = i;
@@ -249,7 +245,7 @@ struct OrderGrid {
 
 __device__ __forceinline__ void order_body(int bid, int nblk, const unsigned* gate, const OrderGrid& fg,
                                           const OrderGrid& cg, const unsigned long long* __restrict__ xfx,
-                                          const int* __restrict__ type, int fp64, int4* __restrict__ ref, int width) {
+                                          const int* __restrict__ type, int fp64, int4* ref, int width) {
   if (gate_closed(gate)) return;
   const int lane = threadIdx.x & (width - 1), per = blockDim.x / width;
   const int total = fg.ncell + cg.ncell;
@@ -1005,32 +1001,137 @@ __global__ void __launch_bounds__(kPruneThreads) k_prune(const unsigned* gate, P
   }
 }
 
-cudaError_t launch_prune(relres_ctx* c, const unsigned* gate) {
-  if (!c->prune_on) return cudaSuccess;
-  if (gate == nullptr) gate = c->d_open;
-  const float s0 = float(c->box[0] / 4294967296.0), s1 = float(c->box[1] / 4294967296.0),
-              s2 = float(c->box[2] / 4294967296.0);
+static PruneArgs prune_args(const relres_ctx* c) {
   DevState* st = c->d_state;
   const double rf = c->rlist_fg_cut + c->prune_delta + kPruneSlack;
   PruneArgs a;
-  a.fg = PruneList{c->n, c->d_pos_fg, c->d_nbr_fg, c->d_cnt_fg, c->d_nbr_fg_in, c->d_cnt_fg_in,
-                   float(rf * rf), &st->tot_in_fg};
+  a.fg = PruneList{c->n, c->d_pos_fg, c->d_nbr_fg, c->d_cnt_fg, c->prune_on ? c->d_nbr_fg_in : c->d_nbr_fg,
+                   c->prune_on ? c->d_cnt_fg_in : c->d_cnt_fg, float(rf * rf), &st->tot_in_fg};
   a.cg = a.fg;  // stand-in when there is no CG list (no CG blocks are launched)
   a.nblk_cg = 0;
-  if (c->has_cg && c->n_h > 0) {
+  if (c->prune_on && c->has_cg && c->n_h > 0) {
     const double rc = c->rlist_cg_cut + c->prune_delta + kPruneSlack;
     a.cg = PruneList{c->n_h, c->d_pos_cg, c->d_nbr_cg, c->d_cnt_cg, c->d_nbr_cg_in, c->d_cnt_cg_in,
                      float(rc * rc), &st->tot_in_cg};
     a.nblk_cg = (c->n_h + kPruneThreads - 1) / kPruneThreads;
   }
-  a.sx = s0;
-  a.sy = s1;
-  a.sz = s2;
+  a.sx = float(c->box[0] / 4294967296.0);
+  a.sy = float(c->box[1] / 4294967296.0);
+  a.sz = float(c->box[2] / 4294967296.0);
   a.perm_fg = c->d_perm_fg;
   a.ref_p = c->d_ref_p;
   a.st = st;
+  return a;
+}
+
+cudaError_t launch_prune(relres_ctx* c, const unsigned* gate) {
+  if (!c->prune_on) return cudaSuccess;
+  if (gate == nullptr) gate = c->d_open;
+  const PruneArgs a = prune_args(c);
   const int nb = a.nblk_cg + (c->n + kPruneThreads - 1) / kPruneThreads;
   k_prune<<<nb, kPruneThreads, 0, c->stream>>>(gate, a);
+  RELRES_LAUNCHED(c);
+  return cudaGetLastError();
+}
+
+// ---- the whole rebuild as one kernel (step graphs of one system).  A
+// conditional graph node costs 8-9 us in every step in which it stays closed,
+// plus the kernel that sets it; a kernel that finds the gate closed costs 2 us.
+// The phases are those of the separate kernels, with a grid-wide barrier
+// between them, so the launch is cooperative (every block resident; as many
+// blocks as fit, which the list phase needs).  us per MD step with the
+// conditional node / as one kernel (neopentane-like, FP32): 25.7 / 17.8 at
+// 1 715 atoms, 28.5 / 21.2 at 10 000, 40.3 / 35.1 at 40 000, 70.7 / 64.5 at
+// 160 000, 282 / 276 at 1 000 000.
+
+// Grid-wide barrier: bar[0] counts arrivals, bar[1] is the generation.  The
+// wait is bounded (about a second); a block that gives up sets F_BARRIER, and
+// every block leaves at its next barrier.  Returns whether to go on.
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned* flags) {
+  __shared__ int s_go;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned gen = *(volatile unsigned*)(bar + 1);
+    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+      *(volatile unsigned*)bar = 0u;
+      __threadfence();
+      atomicAdd(bar + 1, 1u);
+    } else {
+      int spin = 0;
+      while (*(volatile unsigned*)(bar + 1) == gen && ++spin < (1 << 21)) {
+      }
+      if (*(volatile unsigned*)(bar + 1) == gen) atomicOr(flags, F_BARRIER);
+    }
+    __threadfence();
+    s_go = (*(volatile unsigned*)flags & F_BARRIER) == 0u;
+  }
+  __syncthreads();
+  return s_go != 0;
+}
+
+__global__ void __launch_bounds__(kListThreads) k_rebuild(const unsigned* gate, const __grid_constant__ BuildArgs b,
+                                                          const __grid_constant__ PruneArgs p, int prune,
+                                                          unsigned* bar) {
+  const unsigned f = *(volatile const unsigned*)gate;
+  const int bid = blockIdx.x, nblk = gridDim.x;
+  if (f & F_REBUILD) {
+    bin_body(bid, nblk, b.n, gate, b.xfx, b.type, b.hyb_mask, b.gf.n0, b.gf.n1, b.gf.n2, b.gf.rank_of, b.gf.count,
+             b.gc.valid, b.gc.n0, b.gc.n1, b.gc.n2, b.gc.rank_of, b.gc.count, b.cell_fg, b.slot_fg, b.cell_cg,
+             b.slot_cg, b.flags);
+    if (!grid_barrier(bar, b.flags)) return;
+    ScanGrid sf = scan_grid(b.gf), sc = scan_grid(b.gc);
+    sf.ntile = (sf.ncell + 4 * kListThreads - 1) / (4 * kListThreads);
+    sc.ntile = sc.valid ? (sc.ncell + 4 * kListThreads - 1) / (4 * kListThreads) : 0;
+    for (int t = bid; t < sf.ntile + sc.ntile; t += nblk) scan_tile_body(t, gate, sf, sc, b.st);
+    if (!grid_barrier(bar, b.flags)) return;
+    for (int t = bid; t < sf.ntile + sc.ntile; t += nblk) scan_add_body(t, gate, sf, sc);
+    if (!grid_barrier(bar, b.flags)) return;
+    scatter_body(bid, nblk, b.n, gate, b.type, b.hyb_mask, b.gf.start, b.gc.valid, b.gc.start, b.cell_fg, b.slot_fg,
+                 b.cell_cg, b.slot_cg, b.order_fg, b.order_cg);
+    if (!grid_barrier(bar, b.flags)) return;
+    order_body(bid, nblk, gate, b.ofg, b.ocg, b.xfx, b.type, b.fp64, b.ref, b.order_width);
+    if (!grid_barrier(bar, b.flags)) return;
+    const int ncell = b.ncell_cg + b.lfg.g.ncell_full;
+    for (int c = bid; c < ncell; c += nblk) list_cell(b.lfg, b.lcg, b.ncell_cg, c);
+  }
+  // the pruning pass of launches that do not prune as they walk
+  if (prune && (f & (F_REBUILD | F_PRUNE))) {
+    if ((f & F_REBUILD) && !grid_barrier(bar, b.flags)) return;
+    const int n_cg = p.nblk_cg > 0 ? p.cg.nslots : 0;
+    unsigned long long kept_cg = 0ull, kept_fg = 0ull;
+    for (int s = bid * kListThreads + threadIdx.x; s < n_cg + p.fg.nslots; s += nblk * kListThreads) {
+      if (s < n_cg) {
+        kept_cg += prune_slot(p.cg, s, p.sx, p.sy, p.sz);
+      } else {
+        const int sf = s - n_cg;
+        kept_fg += prune_slot(p.fg, sf, p.sx, p.sy, p.sz);
+        p.ref_p[p.perm_fg[sf]] = p.fg.pos[sf];
+      }
+    }
+    kept_cg = warp_sum(kept_cg);
+    kept_fg = warp_sum(kept_fg);
+    if ((threadIdx.x & 31) == 0) {
+      if (kept_cg) atomicAdd(p.cg.total, kept_cg);
+      if (kept_fg) atomicAdd(p.fg.total, kept_fg);
+    }
+    if (bid == 0 && threadIdx.x == 0) atomicAdd(&p.st->n_prunes, 1ull);
+  }
+}
+
+cudaError_t launch_rebuild_fused(relres_ctx* c, bool prune) {
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rebuild, kListThreads, 0);
+  if (e != cudaSuccess) return e;
+  BuildArgs b = build_args(c, &c->d_state->flags);
+  PruneArgs p = prune_args(c);
+  const unsigned* gate = &c->d_state->flags;
+  int with_prune = prune ? 1 : 0;
+  void* args[] = {&gate, &b, &p, &with_prune, &c->d_bar};
+  const int nb = std::max(1, std::min(b.ncell_cg + b.gf.ncell_full, kPartSMs * per_sm));
+  e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_rebuild), dim3(nb),
+                                  dim3(kListThreads), args, 0, c->stream);
+  if (e != cudaSuccess) return e;
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }

@@ -95,6 +95,7 @@ enum : unsigned {
   F_DIRTY = 16u,        // incoming positions differ from the cached state
   F_BADCELL = 32u,      // a computed cell index was out of range (access skipped)
   F_PRUNE = 64u,        // an atom moved more than delta/2 since the last pruning pass
+  F_BARRIER = 256u,     // a grid-wide barrier of the fused rebuild ran out of time
   F_VDIRTY = 128u,      // incoming velocities differ from the ones returned last
 };
 
@@ -181,6 +182,7 @@ struct Grid {
   int* d_tile = nullptr;     // [ntile] per-tile cell counts of the scan
 };
 constexpr int kScanTile = 4096;  // cells per block of the two-pass cell scan
+constexpr int kScanTileMin = 512;  // the same in the fused rebuild's smaller blocks
 
 // ------------------------------------------------------------------ context
 }  // namespace relres
@@ -331,6 +333,10 @@ struct relres_ctx {
   long long* d_acc = nullptr;
   double* d_draws = nullptr;  // CSVR random numbers of the current block of steps, 2 per step
   relres::DevState* d_state = nullptr;
+  unsigned* d_bar = nullptr;   // grid-wide barrier of the fused rebuild: arrivals, generation
+  // step graphs rebuild in one kernel (else behind a conditional node: the
+  // concurrent branches of a batch graph)
+  bool use_fused = true;
   unsigned* d_open = nullptr;  // device word that always reads F_REBUILD (un-gated launches)
   void* d_dummy = nullptr;     // valid target for pointer arguments a kernel does not use
   relres::DevState* h_state = nullptr;  // pinned mirror
@@ -361,8 +367,8 @@ struct relres_ctx {
   size_t ev_used = 0;
 
   // CUDA graph of one block of MD steps (relres_step): the list rebuild of
-  // each step is a conditional node whose flag a one-thread kernel sets from
-  // the device displacement trigger.  Everything below is baked into the
+  // each step is one kernel that returns at once unless the device
+  // displacement trigger fired.  Everything below is baked into the
   // instantiated graph; it is re-captured when any of it changes.
   int pair_cfg = 0;        // index into kPairConfigs
   // threads per slot of forces-only launches that keep the force bits of one
@@ -424,6 +430,8 @@ cudaError_t launch_rebuild(relres_ctx* c, const unsigned* gate);
 cudaError_t launch_decide(relres_ctx* c, cudaGraphConditionalHandle h, cudaGraphConditionalHandle hp,
                           int with_prune);
 cudaError_t launch_lists(relres_ctx* c, const unsigned* gate);
+// a step's rebuild (and separate pruning pass) as one gated kernel
+cudaError_t launch_rebuild_fused(relres_ctx* c, bool prune);
 // pruning pass: inner lists from the full ones at the current positions
 // (gate: runs if F_REBUILD or F_PRUNE is set)
 cudaError_t launch_prune(relres_ctx* c, const unsigned* gate);
