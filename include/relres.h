@@ -475,7 +475,7 @@ relres_status relres_measure_rates(void* d_scratch, size_t scratch_bytes, void* 
  *                   Newton-Raphson step (results below the smallest normal
  *                   float are 0);
  *   d_out64[k]    = 1/x in FP64, and d_out64[n + k] = 1/sqrt(x): FP32
- *                   estimate plus one FP64 Newton-Raphson step.
+ *                   estimate plus one FP64 third-order step.
  * d_out32 holds n floats, d_out64 2n doubles (device, caller-owned).
  * Errors: RELRES_ERR_ARG (null pointer, n < 0), RELRES_ERR_CUDA.
  */

@@ -257,7 +257,7 @@ relres_status forces_now(relres_ctx* c, int ev_mode, double* d_forces, double* d
     s = autotune_pairs(c);
     if (s != RELRES_OK) return s;
   }
-  CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAcc, c->stream));
+  CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAccAll, c->stream));
   TIMED(ev_mode == 1 ? RELRES_T_PAIR_EV : RELRES_T_PAIR, launch_pairs(c, ev_mode == 1));
   TIMED(RELRES_T_FINISH, launch_finish(c, ev_mode == 1, d_forces, nullptr));
   if (ev_mode == 1) TIMED(RELRES_T_THERMO, launch_reduce_out(c, d_energy, d_virial));
@@ -350,8 +350,8 @@ relres_status relres_create(relres_ctx** out, const relres_params* p, void* cuda
   if (ce == cudaSuccess) ce = cudaMallocHost(&c->h_state, sizeof(DevState));
   if (ce == cudaSuccess) ce = cudaMalloc(&c->d_dummy, 256);
   if (ce == cudaSuccess) ce = cudaMemset(c->d_dummy, 0, 256);
-  if (ce == cudaSuccess) ce = cudaMalloc(&c->d_acc, sizeof(long long) * kNAcc);
-  if (ce == cudaSuccess) ce = cudaMemset(c->d_acc, 0, sizeof(long long) * kNAcc);
+  if (ce == cudaSuccess) ce = cudaMalloc(&c->d_acc, sizeof(long long) * kNAccAll);
+  if (ce == cudaSuccess) ce = cudaMemset(c->d_acc, 0, sizeof(long long) * kNAccAll);
   if (ce == cudaSuccess) ce = cudaMalloc(&c->d_draws, sizeof(double) * 2 * kBlockSteps);
   if (ce == cudaSuccess) ce = cudaMemset(c->d_draws, 0, sizeof(double) * 2 * kBlockSteps);
   if (ce == cudaSuccess) ce = cudaMalloc(&c->d_bar, 2 * sizeof(unsigned));
@@ -1305,7 +1305,7 @@ static relres_status step_begin(relres_ctx* c, int n_steps, double dt_fs, double
     fresh = true;
   }
   CK(upload_type_consts(c, dt_fs));
-  CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAcc, c->stream));
+  CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAccAll, c->stream));
   // Everything that follows runs on the context stream, after these launches.
   // Without a force evaluation above, the state read at the start is still
   // current for the block accounting (the set-up above changes no count), so
@@ -1867,8 +1867,8 @@ relres_status relres_get_stats(relres_ctx* c, relres_stats* o) {
   std::memset(o, 0, sizeof(*o));
   o->n_atoms = c->n;
   o->n_hybrid = c->n_h;
-  o->pair_tpa = c->fp64 ? fp64_pair_tpa(c) : kPairConfigs[c->pair_cfg].tpa;
-  o->pair_block = c->fp64 ? fp64_pair_block(c) : kPairConfigs[c->pair_cfg].bs;
+  o->pair_tpa = c->fp64 ? fp64_lanes(c) : kPairConfigs[c->pair_cfg].tpa;
+  o->pair_block = c->fp64 ? kFp64Block : kPairConfigs[c->pair_cfg].bs;
   o->cap_fg = c->cap_fg;
   o->cap_cg = c->cap_cg;
   o->max_fg = c->h_state->max_fg;

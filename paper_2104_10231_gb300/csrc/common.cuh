@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include "fbits.h"
 #include "relres_internal.h"
 
 // Every launcher counts its kernels.  Building with -DRELRES_DEBUG_SYNC also
@@ -224,6 +225,14 @@ __device__ __forceinline__ ff ff_fixed_diff32(int a, int b, ff s) {
 
 // Integer accumulators: a block's FP64 sum is converted to 64-bit fixed point
 // and added with an integer atomic (exact, independent of order).
+// The accumulator kNAcc places on takes what the first rounding left, in units
+// 2^30 finer (acc_add_fine; zero where acc_add is used).
+__device__ __forceinline__ void acc_add_fine(long long* acc, double v) {
+  const long long hi = to_fix_sum(v);
+  const double rest = fma(v, kFix, -double(hi)) * kFixFine;
+  atomicAdd(reinterpret_cast<unsigned long long*>(acc), (unsigned long long)hi);
+  atomicAdd(reinterpret_cast<unsigned long long*>(acc + kNAcc), (unsigned long long)__double2ll_rn(rest));
+}
 __device__ __forceinline__ void acc_add(long long* acc, double v) {
   atomicAdd(reinterpret_cast<unsigned long long*>(acc), (unsigned long long)to_fix_sum(v));
 }
@@ -245,16 +254,20 @@ __device__ __forceinline__ float rcp_nr(float x) {
   return fmaf(y, fmaf(-x, y, 1.f), y);
 }
 
-// FP64 1/x and 1/sqrt(x) from the FP32 hardware estimate plus one Newton
-// step (relative error ~1e-13; FP64 division and square root are many times
-// slower on this part).
-__device__ __forceinline__ double rcp_d(double x) {
-  const double y = double(rcp_approx(float(x)));
-  return y * fma(-x, y, 2.0);
+// FP64 1/x and 1/sqrt(x) from the FP32 estimate of a nearby FP32 value xf (to
+// ~1e-6 of x) and one third-order step: with e = 1 - x y (or 1 - x y^2),
+// y (1 + e + e^2) and y (1 + e / 2 + 3 e^2 / 8) leave e^3 (FP64 division and
+// square root are many times slower on this part).  The estimate is widened
+// with integer operations: conversion instructions run at half the FP64 rate.
+__device__ __forceinline__ double rcp_d(double x, float xf) {
+  const double y = double_of_float(rcp_approx(xf));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
-__device__ __forceinline__ double rsqrt_d(double x) {
-  const double y = double(rsqrtf(float(x)));
-  return y * fma(-0.5 * x * y, y, 1.5);
+__device__ __forceinline__ double rsqrt_d(double x, float xf) {
+  const double y = double_of_float(rsqrtf(xf));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y, e * fma(e, 0.375, 0.5), y);
 }
 
 }  // namespace relres

@@ -968,6 +968,11 @@ __global__ void k_csvr_draws(double n_f, unsigned long long seed, int count, con
   draws[2 * k + 1] = s;
 }
 
+// total of an accumulator and the finer one beside it
+__device__ __forceinline__ double acc_value(long long hi, long long fine) {
+  return (double(hi) + double(fine) / kFixFine) / kFix;
+}
+
 // End of a step (one thread): thermostat factor from the kinetic energy,
 // thermo row on energy steps, counters, and the accumulators cleared for the
 // next step.  `draw` points at this step's (r1, s).  The accumulators are read
@@ -987,16 +992,17 @@ __device__ void end_of_step(volatile long long* acc, const StepParams& sp, DevSt
   double* thermo = sp.thermo;
   if (ev && sp.thermo_every > 0) {
     double* row = thermo + (size_t)st->thermo_row * RELRES_THERMO_COLS;
-    row[0] = double(acc[kAccFg]) / kFix;
-    row[1] = double(acc[kAccCg]) / kFix;
+    row[0] = acc_value(acc[kAccFg], acc[kNAcc + kAccFg]);
+    row[1] = acc_value(acc[kAccCg], acc[kNAcc + kAccCg]);
     row[2] = double(acc[kAccEb]) / kFix;
     row[3] = ke * alpha * alpha;
 #pragma unroll
-    for (int q = 1; q < kNQ; ++q) row[3 + q] = double(acc[kAccFg + q] + acc[kAccCg + q]) / kFix;
+    for (int q = 1; q < kNQ; ++q)
+      row[3 + q] = acc_value(acc[kAccFg + q] + acc[kAccCg + q], acc[kNAcc + kAccFg + q] + acc[kNAcc + kAccCg + q]);
     st->thermo_row += 1;
   }
 #pragma unroll
-  for (int q = 0; q < kNAcc; ++q) acc[q] = 0;
+  for (int q = 0; q < (ev ? kNAccAll : kNAcc); ++q) acc[q] = 0;
   st->local_step += 1;
   st->step += 1;
   if (st->flags & F_REBUILD) {
@@ -1154,7 +1160,7 @@ __global__ void __launch_bounds__(kThreads) k_sum_batch(const SumArgs<R>* __rest
 
 // Energies and virial of relres_compute (one thread); clears the accumulators.
 __global__ void k_reduce_out(long long* acc, double* energy, int with_e, double* virial, int with_w) {
-  const double efg = double(acc[kAccFg]) / kFix, ecg = double(acc[kAccCg]) / kFix;
+  const double efg = acc_value(acc[kAccFg], acc[kNAcc + kAccFg]), ecg = acc_value(acc[kAccCg], acc[kNAcc + kAccCg]);
   const double eb = double(acc[kAccEb]) / kFix;
   if (with_e) {
     energy[0] = efg;
@@ -1164,9 +1170,11 @@ __global__ void k_reduce_out(long long* acc, double* energy, int with_e, double*
   }
   if (with_w)
 #pragma unroll
-    for (int q = 1; q < kNQ; ++q) virial[q - 1] = double(acc[kAccFg + q] + acc[kAccCg + q]) / kFix;
+    for (int q = 1; q < kNQ; ++q)
+      virial[q - 1] =
+          acc_value(acc[kAccFg + q] + acc[kAccCg + q], acc[kNAcc + kAccFg + q] + acc[kNAcc + kAccCg + q]);
 #pragma unroll
-  for (int q = 0; q < kNAcc; ++q) acc[q] = 0;
+  for (int q = 0; q < kNAccAll; ++q) acc[q] = 0;
 }
 
 // Start of a relres_step call: its step and thermo-row counters, and (unless

@@ -1,105 +1,15 @@
-// Device code shared by the pair kernels (pair.cu, pair_lanes.cu): positions,
-// the FG and CG terms of one pair, launch arguments and force accumulators.
+// Device code shared by the FP32 pair kernels (pair.cu, pair_lanes.cu): the FG
+// and CG terms of one pair, launch arguments and force accumulators.
 #pragma once
-
-#include <type_traits>
 
 #include "common.cuh"
 
 namespace relres {
 
-template <typename R>
-struct PosOf;
-template <>
-struct PosOf<float> {
-  using T = int4;
-};
-template <>
-struct PosOf<double> {
-  using T = Pos64;
-};
-
-template <typename R>
-using ForceOut = typename std::conditional<std::is_same<R, float>::value, float4, double>::type;
-
-__device__ __forceinline__ void delta(const int4& a, const int4& b, float sx, float sy, float sz,
-                                      float& dx, float& dy, float& dz) {
-  dx = dfix32(a.x, b.x, sx);
-  dy = dfix32(a.y, b.y, sy);
-  dz = dfix32(a.z, b.z, sz);
-}
-__device__ __forceinline__ void delta(const Pos64& a, const Pos64& b, double sx, double sy,
-                                      double sz, double& dx, double& dy, double& dz) {
-  dx = dfix64(a.x, b.x, sx);
-  dy = dfix64(a.y, b.y, sy);
-  dz = dfix64(a.z, b.z, sz);
-}
-__device__ __forceinline__ int ptype(const int4& p) { return p.w; }
-__device__ __forceinline__ int ptype(const Pos64& p) { return int(p.t); }
-
 __device__ __forceinline__ int4 load_pos(const int4* p, int j) { return __ldg(p + j); }
-__device__ __forceinline__ Pos64 load_pos(const Pos64* p, int j) { return p[j]; }
-
-__device__ __forceinline__ float recip(float x) { return rcp_nr(x); }
-__device__ __forceinline__ double recip(double x) { return rcp_d(x); }
-__device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsq(double x) { return rsqrt_d(x); }
 
 __device__ __forceinline__ void store_force(float4* f, int i, float x, float y, float z) {
   f[i] = make_float4(x, y, z, 0.f);
-}
-__device__ __forceinline__ void store_force(double* f, int i, double x, double y, double z) {
-  f[3 * i] = x;
-  f[3 * i + 1] = y;
-  f[3 * i + 2] = z;
-}
-
-// FG part for one entry (FP64 path and FP64 energies).  Returns false outside r_s+.
-template <typename R, bool EV>
-__device__ __forceinline__ bool fg_term(const PairTab<R>& T, R r2, R& fr, R& ep) {
-  if (!(r2 < T.rsp2)) return false;
-  if (r2 < T.rsm2) {
-    const R r2i = recip(r2);
-    const R r6i = r2i * r2i * r2i;
-    fr = r6i * (T.f12f * r6i - T.f6f) * r2i;
-    if (EV) ep = r6i * (T.c12f * r6i - T.c6f) - T.e_fg_shift;
-  } else {
-    const R ri = rsq(r2);
-    const R d = r2 * ri - T.rsm;
-    const R fp = ((T.fgd[3] * d + T.fgd[2]) * d + T.fgd[1]) * d + T.fgd[0];
-    fr = -fp * ri;
-    if (EV) ep = ((((T.fg[4] * d + T.fg[3]) * d + T.fg[2]) * d + T.fg[1]) * d + T.fg[0]) - T.e_fg_shift;
-  }
-  return true;
-}
-
-// CG part for one entry (FP64 path and FP64 energies).  Returns false outside r_c+.
-template <typename R, bool EV>
-__device__ __forceinline__ bool cg_term(const PairTab<R>& T, R r2, R& fr, R& ep) {
-  if (!(r2 < T.rcp2)) return false;
-  if (r2 < T.rsm2) {  // constant: f_{s+}(0) - Gamma_{c-}, no force
-    fr = R(0);
-    if (EV) ep = T.e_cg_close;
-    return true;
-  }
-  const R ri = rsq(r2);
-  if (r2 < T.rsp2) {  // switching on
-    const R d = r2 * ri - T.rsm;
-    const R d2 = d * d;
-    fr = -(d2 * (T.ond4 * d + T.ond3)) * ri;
-    if (EV) ep = T.on0 + d2 * d * (T.on4 * d + T.on3) - T.gam_cm;
-  } else if (r2 < T.rcm2) {  // CG LJ
-    const R r2i = ri * ri;
-    const R r6i = r2i * r2i * r2i;
-    fr = r6i * (T.f12c * r6i - T.f6c) * r2i;
-    if (EV) ep = r6i * (T.c12c * r6i - T.c6c) - T.gam_cm;
-  } else {  // switching off
-    const R d = r2 * ri - T.rcm;
-    const R fp = ((T.cgod[3] * d + T.cgod[2]) * d + T.cgod[1]) * d + T.cgod[0];
-    fr = -fp * ri;
-    if (EV) ep = ((((T.cgo[4] * d + T.cgo[3]) * d + T.cgo[2]) * d + T.cgo[1]) * d + T.cgo[0]) - T.gam_cm;
-  }
-  return true;
 }
 
 // FP32 force coefficients of one type pair for 16-byte shared-memory loads
@@ -211,44 +121,41 @@ __device__ __forceinline__ float4 cg_radii2(const CgRow& T) {
 }
 
 
-template <typename R>
 struct ListWalk {
   int nslots;
-  const typename PosOf<R>::T* pos;
+  const int4* pos;
   const int* nbr;  // the list walked (pruned when pruning is on)
   const int* cnt;
   const int* perm;
-  ForceOut<R>* f_out;
+  float4* f_out;
   long long* acc;  // kNQ accumulators of this list (energy, six virial components)
   // pruning launches (PRN): walk the full list and write the pruned one
   const int* nbr_full;
   const int* cnt_full;
   int* nbr_in;
   int* cnt_in;
-  R rp2;  // (interaction cutoff + delta + slack)^2
+  float rp2;  // (interaction cutoff + delta + slack)^2
   unsigned long long* tot_in;
 };
 
-template <typename R>
 struct PairLaunch {
   int nblk_cg;  // blocks [0, nblk_cg) walk the CG list, the rest the FG list
-  ListWalk<R> fg, cg;
-  const void* tab;  // PairRow[nt^2] (FP32) or PairTab<double>[nt^2]
-  const PairRowEnergy* tabe;  // FP32 path: energy constants
+  ListWalk fg, cg;
+  const PairRow* tab;          // [nt^2]
+  const PairRowEnergy* tabe;   // energy steps
   int nt;
-  R sx, sy, sz;
-  float sxl, syl, szl;  // FP32 path: lo parts of L / 2^32 (float-float energies)
+  float sx, sy, sz;
+  float sxl, syl, szl;  // lo parts of L / 2^32 (float-float energies)
   const unsigned* gate;  // device flag word of the step
-  int prune_on;          // prune on this launch if F_REBUILD or F_PRUNE is set (TPA = 1 only)
+  int prune_on;          // prune on this launch if F_REBUILD or F_PRUNE is set
   int4* ref_p;  // PRN: positions of this pruning pass, caller order (FG walk)
   DevState* st;
 };
 
 // type-pair tables in shared memory
 struct SmemTabs {
-  const void* tab;             // PairTab<double>
-  const PairRow* row;          // FP32
-  const PairRowEnergy* rowe;   // FP32 energy steps
+  const PairRow* row;
+  const PairRowEnergy* rowe;  // energy steps
 };
 
 // copies n words from global to shared memory with the whole block
@@ -263,19 +170,16 @@ __device__ __forceinline__ void copy_words(void* dst, const void* src, int n) {
 // added to a float-float total (fx + cx, ...) with an error-free two-sum; or
 // FP64 running sums (dfx, ...), one conversion and FP64 add per entry.  The
 // members a variant does not use are removed by the compiler.
-template <typename R>
 struct Acc {
-  R fx = R(0), fy = R(0), fz = R(0);
+  float fx = 0.f, fy = 0.f, fz = 0.f;
   float kx = 0.f, ky = 0.f, kz = 0.f;
   float cx = 0.f, cy = 0.f, cz = 0.f;
   double dfx = 0.0, dfy = 0.0, dfz = 0.0;
-  R w[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};  // FP64 path: virial and energy
-  R e = R(0);
 };
 
 // The FMAs are explicit: every kernel that sums a chunk rounds it alike.
 template <int ACC>
-__device__ __forceinline__ void acc_force(Acc<float>& A, float fr, float dx, float dy, float dz) {
+__device__ __forceinline__ void acc_force(Acc& A, float fr, float dx, float dy, float dz) {
   if constexpr (ACC == RELRES_ACC_COMPENSATED) {
     A.kx = fmaf(fr, dx, A.kx);
     A.ky = fmaf(fr, dy, A.ky);
@@ -294,7 +198,7 @@ __device__ __forceinline__ void acc_force(Acc<float>& A, float fr, float dx, flo
 // end of a list chunk: the compensated variant moves the chunk sum into its
 // float-float total
 template <int ACC>
-__device__ __forceinline__ void acc_chunk(Acc<float>& A) {
+__device__ __forceinline__ void acc_chunk(Acc& A) {
   if constexpr (ACC == RELRES_ACC_COMPENSATED) {
     const ff sx = ff_two_sum(A.fx, A.kx), sy = ff_two_sum(A.fy, A.ky), sz = ff_two_sum(A.fz, A.kz);
     A.fx = sx.hi;
@@ -306,12 +210,10 @@ __device__ __forceinline__ void acc_chunk(Acc<float>& A) {
     A.kx = A.ky = A.kz = 0.f;
   }
 }
-template <int ACC>
-__device__ __forceinline__ void acc_chunk(Acc<double>&) {}
 
 // the owner's force sum rounded to FP32 (the width of the force buffers)
 template <int ACC>
-__device__ __forceinline__ void acc_final(Acc<float>& A) {
+__device__ __forceinline__ void acc_final(Acc& A) {
   if constexpr (ACC == RELRES_ACC_COMPENSATED) {
     A.fx = __fadd_rn(A.fx, A.cx);
     A.fy = __fadd_rn(A.fy, A.cy);
@@ -322,30 +224,30 @@ __device__ __forceinline__ void acc_final(Acc<float>& A) {
     A.fz = float(A.dfz);
   }
 }
-template <int ACC>
-__device__ __forceinline__ void acc_final(Acc<double>&) {}
 
 // One FP32 pair: squared distance (past every cutoff for a padding entry),
 // force factor -u'(r)/r and coordinate difference.
 template <bool CG>
 __device__ __forceinline__ float pair_term(const int4& pi, const int4& pj, bool valid, const PairRow& T, float sx,
                                            float sy, float sz, float& fr, float& dx, float& dy, float& dz) {
-  delta(pi, pj, sx, sy, sz, dx, dy, dz);
+  dx = dfix32(pi.x, pj.x, sx);
+  dy = dfix32(pi.y, pj.y, sy);
+  dz = dfix32(pi.z, pj.z, sz);
   float r2 = dx * dx + dy * dy + dz * dz;
   r2 = valid ? r2 : 3.0e38f;
   fr = CG ? cg_force(T.cg, r2) : fg_force(T.fg, r2);
   return r2;
 }
 
-__device__ __forceinline__ int4 ref_of(const int4& p) { return p; }
-__device__ __forceinline__ int4 ref_of(const Pos64& p) {
-  return make_int4(int(p.x >> 32), int(p.y >> 32), int(p.z >> 32), int(p.t));
-}
-
 // ---- pair_lanes.cu: FP32 launches of kLaneThreads-thread blocks, `lanes`
 // threads per slot (1, 4 or 8; forces only: 4 or 8)
 constexpr int kLaneThreads = 128;
-void launch_pairs_lanes(cudaStream_t s, int acc, const PairLaunch<float>& a, bool ev, int lanes, int grid);
+void launch_pairs_lanes(cudaStream_t s, int acc, const PairLaunch& a, bool ev, int lanes, int grid);
 void launch_pairs_lanes_batch(cudaStream_t s, int acc, bool ev, const BatchLaunch& b, int nrep);
+
+// ---- pair64.cu: FP64 contexts
+cudaError_t launch_pairs_f64(relres_ctx* c, bool ev, int which);
+cudaError_t prepare_pairs_batch_f64(const std::vector<relres_ctx*>& cs, BatchLaunch* b, BatchLaunch* b_ev);
+void launch_pairs_batch_f64(cudaStream_t s, bool ev, const BatchLaunch& b, int nrep);
 
 }  // namespace relres

@@ -1,0 +1,392 @@
+// RelRes pair launches of FP64 contexts: the terms of pair.cu in double, from
+// 64-bit fixed-point positions.
+//
+// FP64 runs at 1.66 FMA per clock and SM on this part, 70 times below FP32, so
+// the FP64 instructions a warp issues are what a launch costs.  One thread per
+// list entry by entry issues every region's arithmetic for every entry (the
+// lanes of a warp hold entries of all regions, and a quarter of the entries of
+// a pruned list is past the cutoff): ~48 FP64 instructions an entry.  Here a
+// warp takes 128 list entries at a time (T lanes per slot, four entries per
+// lane), decides each one's region from its FP32 distance, and sorts the
+// entries inside the cutoff by region in shared memory; full warps then
+// evaluate 32 of them at a time, nearly always of one region, ~22 FP64
+// instructions each.  Against one thread per list entry by entry, and eight
+// per slot with the pruning as a pass of its own below 20 000 slots: 200 ->
+// 163 us per step at 25 000 neopentane-like atoms, 65 -> 44 us at 648
+// propane-like ones (185 -> 16 us the launch with energies).  The potential is C2 at the region limits, so a pair that
+// FP32 puts on the other side of one (1e-7 of r^2) changes nothing above 1e-13.
+//
+// The terms of a slot are stored by their rank in its list and added in list
+// order, one rounded product after the other.  Entries past the cutoff are no
+// terms, so the forces (and, per slot, energy and virial) are the same bits
+// for every T, with and without pruning.
+#include "common.cuh"
+#include "fbits.h"
+#include "pair.cuh"
+
+namespace relres {
+
+struct Walk64 {
+  int nslots;
+  const Pos64* pos;
+  const int4* pos32;  // the same positions, upper 32 bits and type
+  const int* nbr;     // the list walked (pruned when pruning is on)
+  const int* cnt;
+  const int* perm;
+  double* f_out;
+  long long* acc;  // kNQ accumulators of this list (energy, six virial components)
+  // pruning launches: walk the full list and write the pruned one
+  const int* nbr_full;
+  const int* cnt_full;
+  int* nbr_in;
+  int* cnt_in;
+  float rp2;  // (interaction cutoff + delta + slack)^2
+  unsigned long long* tot_in;
+};
+
+struct Launch64 {
+  int nblk_cg;  // blocks [0, nblk_cg) walk the CG list, the rest the FG list
+  Walk64 fg, cg;
+  const PairTab<double>* tab;  // [nt^2]
+  int nt;
+  double sx, sy, sz;  // L / 2^64
+  float fx, fy, fz;   // L / 2^32
+  const unsigned* gate;
+  int prune_on;
+  int4* ref_p;
+  DevState* st;
+};
+
+// regions, in the order the entries are sorted by
+enum { kCore = 0, kShell = 1, kFgRegions = 2 };                      // FG: LJ below r_s-, switching off
+enum { kLj = 0, kOff = 1, kOn = 2, kClose = 3, kCgRegions = 4 };     // CG: kClose has an energy only
+
+// values of a term: force, then (energy steps) energy and virial
+constexpr int kTermF = 3, kTermEv = 3 + kNQ;
+
+template <bool EV>
+struct WarpTerms {
+  double v[EV ? kTermEv : kTermF][128];  // by 4 T (slot in the warp) + rank in the slot's list
+  long long px[32], py[32], pz[32];      // the slots' positions and first type-pair rows
+  int row0[32];
+  int j[128];  // the sorted entries: partner, FP32 squared distance, place in v
+  float r2[128];
+  unsigned short at[128];
+};
+
+// -u'(r)/r (and u) of one pair in the given region
+template <bool CG, bool EV>
+__device__ __forceinline__ void term64(int region, const PairTab<double>& T, double r2, float r2f, double& fr,
+                                       double& e) {
+  if (CG && region == kClose) {
+    fr = 0.0;
+    e = T.e_cg_close;
+    return;
+  }
+  if (region == (CG ? int(kLj) : int(kCore))) {
+    const double r2i = rcp_d(r2, r2f);
+    const double r6i = r2i * r2i * r2i;
+    fr = r6i * ((CG ? T.f12c : T.f12f) * r6i - (CG ? T.f6c : T.f6f)) * r2i;
+    if (EV) e = r6i * ((CG ? T.c12c : T.c12f) * r6i - (CG ? T.c6c : T.c6f)) - (CG ? T.gam_cm : T.e_fg_shift);
+    return;
+  }
+  const double ri = rsqrt_d(r2, r2f);
+  if (CG && region == kOn) {
+    const double d = r2 * ri - T.rsm, d2 = d * d;
+    fr = -(d2 * (T.ond4 * d + T.ond3)) * ri;
+    if (EV) e = T.on0 + d2 * d * (T.on4 * d + T.on3) - T.gam_cm;
+    return;
+  }
+  const double* g = CG ? T.cgo : T.fg;
+  const double* gd = CG ? T.cgod : T.fgd;
+  const double d = r2 * ri - (CG ? T.rcm : T.rsm);
+  fr = -(((gd[3] * d + gd[2]) * d + gd[1]) * d + gd[0]) * ri;
+  if (EV) e = ((((g[4] * d + g[3]) * d + g[2]) * d + g[1]) * d + g[0]) - (CG ? T.gam_cm : T.e_fg_shift);
+}
+
+// One warp's walk over the lists of its 32 / T slots.  thr: FP32 squared radii
+// (r_s-, r_s+, r_c-, r_c+) per type pair.  Returns the entries this lane kept
+// (pruning launches).
+template <bool CG, bool EV, int T, bool PRN>
+__device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0, const PairTab<double>* tab,
+                                                     const float4* thr, WarpTerms<EV>& W, const Launch64& a) {
+  constexpr int NV = EV ? kTermEv : kTermF;
+  constexpr int NL = (NV + T - 1) / T;  // values summed by one lane: q, q + T, ...
+  constexpr int NR = CG ? (EV ? int(kCgRegions) : int(kClose)) : int(kFgRegions);
+  const int lane = threadIdx.x & 31, sl = lane / T, q = lane % T;
+  const int s = slot0 + sl;
+  const bool own = s < L.nslots;
+  const int ss = own ? s : 0;  // a valid slot for the loads of the other lanes
+  const int4 pi = L.pos32[ss];
+  const int m = own ? (PRN ? L.cnt_full[s] : L.cnt[s]) : 0;
+  const int nch = (m + 3) >> 2;
+  const int4* nb4 = reinterpret_cast<const int4*>(PRN ? L.nbr_full : L.nbr) + ss;
+  int4 jj = make_int4(ss, ss, ss, ss);
+  if (q < nch) jj = __ldcs(nb4 + size_t(q) * L.nslots);
+  if (q == 0) {
+    const Pos64 p = L.pos[ss];
+    W.px[sl] = p.x;
+    W.py[sl] = p.y;
+    W.pz[sl] = p.z;
+    W.row0[sl] = pi.w * a.nt;
+  }
+  const int rounds = __reduce_max_sync(0xffffffffu, (nch + T - 1) / T);
+  const int row0 = pi.w * a.nt;
+  const unsigned below = (1u << lane) - 1u;
+  const unsigned slot_mask = (T == 32 ? 0xffffffffu : ((1u << T) - 1u)) << (sl * T), before = slot_mask & below;
+  double f[NL];
+#pragma unroll
+  for (int k = 0; k < NL; ++k) f[k] = 0.0;
+  int kept = 0;
+  for (int r = 0; r < rounds; ++r) {
+    const int ch = r * T + q;
+    int4 jn = jj;
+    if (ch + T < nch) jn = __ldcs(nb4 + size_t(ch + T) * L.nslots);
+    const int rem = m - 4 * ch;  // <= 0 past the list
+    const int j[4] = {rem > 0 ? jj.x : ss, rem > 1 ? jj.y : ss, rem > 2 ? jj.z : ss, rem > 3 ? jj.w : ss};
+    float r2[4];
+    int region[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int4 p = __ldg(L.pos32 + j[e]);
+      const float dx = dfix32(pi.x, p.x, a.fx), dy = dfix32(pi.y, p.y, a.fy), dz = dfix32(pi.z, p.z, a.fz);
+      r2[e] = rem > e ? dx * dx + dy * dy + dz * dz : 3.0e38f;
+      const float4 t = thr[row0 + p.w];
+      if (CG)
+        region[e] = !(r2[e] < t.w) ? -1 : (r2[e] < t.x ? (EV ? int(kClose) : -1)
+                                                        : (r2[e] < t.y ? int(kOn) : (r2[e] < t.z ? int(kLj) : int(kOff))));
+      else
+        region[e] = !(r2[e] < t.y) ? -1 : (r2[e] < t.x ? int(kCore) : int(kShell));
+    }
+    // rank of each term in its slot's list order, and place in the sorted entries
+    unsigned in[4];
+    int rank = 0, terms = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      in[e] = __ballot_sync(0xffffffffu, region[e] >= 0);
+      rank += __popc(in[e] & before);
+      terms += __popc(in[e] & slot_mask);
+    }
+    int total = 0, place[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int c = 0; c < NR; ++c)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const unsigned b = __ballot_sync(0xffffffffu, region[e] == c);
+        if (region[e] == c) place[e] = total + __popc(b & below);
+        total += __popc(b);
+      }
+    __syncwarp();  // the sums of the last round have been read
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (region[e] >= 0) {
+        W.j[place[e]] = j[e];
+        W.r2[place[e]] = r2[e];
+        W.at[place[e]] = (unsigned short)((region[e] << 8) | (4 * T * sl + rank));
+        ++rank;
+      }
+    __syncwarp();
+    for (int k = lane; k < total; k += 32) {
+      const int at = W.at[k] & 0xff, from = at / (4 * T);
+      const Pos64 p = L.pos[W.j[k]];
+      const double dx = dfix64(W.px[from], p.x, a.sx), dy = dfix64(W.py[from], p.y, a.sy),
+                   dz = dfix64(W.pz[from], p.z, a.sz);
+      double fr, en = 0.0;
+      term64<CG, EV>(W.at[k] >> 8, tab[W.row0[from] + int(p.t)], fma(dz, dz, fma(dy, dy, dx * dx)), W.r2[k], fr, en);
+      const double tx = fr * dx, ty = fr * dy, tz = fr * dz;
+      W.v[0][at] = tx;
+      W.v[1][at] = ty;
+      W.v[2][at] = tz;
+      if constexpr (EV) {
+        W.v[3][at] = en;
+        W.v[4][at] = tx * dx;
+        W.v[5][at] = ty * dy;
+        W.v[6][at] = tz * dz;
+        W.v[7][at] = tx * dy;
+        W.v[8][at] = tx * dz;
+        W.v[9][at] = ty * dz;
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int v = 0; v < NL; ++v)
+      if (q + v * T < NV)
+        for (int k = 0; k < terms; ++k) f[v] += W.v[q + v * T][4 * T * sl + k];
+    if constexpr (PRN) {
+      int at = kept;
+      unsigned b[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        b[e] = __ballot_sync(0xffffffffu, r2[e] < L.rp2);
+        at += __popc(b[e] & before);
+        kept += __popc(b[e] & slot_mask);
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (r2[e] < L.rp2) {
+          L.nbr_in[(size_t(at >> 2) * L.nslots + s) * 4 + (at & 3)] = j[e];
+          ++at;
+        }
+    }
+    jj = jn;
+  }
+  if (own) {
+    const int i = L.perm[s];
+#pragma unroll
+    for (int v = 0; v < NL; ++v)
+      if (q + v * T < kTermF) L.f_out[3 * size_t(i) + q + v * T] = f[v];
+    if (PRN && q == 0) {
+      L.cnt_in[s] = kept;
+      if (!CG) a.ref_p[i] = pi;
+    }
+  }
+  if constexpr (EV) {
+    // the warp's slots added in slot order, then to the accumulators (full
+    // lists: every pair was visited from both ends)
+    __syncwarp();
+#pragma unroll
+    for (int v = 0; v < NL; ++v)
+      if (q + v * T < NV) W.v[q + v * T][sl] = own ? f[v] : 0.0;
+    __syncwarp();
+    if (lane < kNQ) {
+      double t = 0.0;
+      for (int k = 0; k < 32 / T; ++k) t += W.v[kTermF + lane][k];
+      acc_add_fine(L.acc + lane, 0.5 * t);
+    }
+  }
+  return own && q == 0 ? (unsigned long long)kept : 0ull;
+}
+
+// shared memory of a block (one warp): tables, FP32 radii, terms
+template <bool EV>
+static size_t smem64(int nt) {
+  return (sizeof(PairTab<double>) + sizeof(float4)) * size_t(nt) * nt + sizeof(WarpTerms<EV>);
+}
+
+template <bool EV, int T>
+__device__ __forceinline__ void block64(const Launch64& a, int bid) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nrow = a.nt * a.nt;
+  float4* const thr = reinterpret_cast<float4*>(smem_raw);
+  PairTab<double>* const tab = reinterpret_cast<PairTab<double>*>(thr + nrow);
+  WarpTerms<EV>& terms = *reinterpret_cast<WarpTerms<EV>*>(tab + nrow);
+  copy_words(tab, a.tab, nrow * int(sizeof(PairTab<double>) / sizeof(int)));
+  for (int k = threadIdx.x; k < nrow; k += kFp64Block)
+    thr[k] = make_float4(float(a.tab[k].rsm2), float(a.tab[k].rsp2), float(a.tab[k].rcm2), float(a.tab[k].rcp2));
+  __syncwarp();
+  const bool cg = bid < a.nblk_cg;
+  const int slot0 = (cg ? bid : bid - a.nblk_cg) * (32 / T);
+  if (a.prune_on && (*(volatile const unsigned*)a.gate & (F_REBUILD | F_PRUNE)) != 0u) {
+    const unsigned long long kept = warp_sum(cg ? walk64<true, EV, T, true>(a.cg, slot0, tab, thr, terms, a)
+                                                : walk64<false, EV, T, true>(a.fg, slot0, tab, thr, terms, a));
+    if (threadIdx.x == 0) {
+      atomicAdd(cg ? a.cg.tot_in : a.fg.tot_in, kept);
+      if (bid == 0) atomicAdd(&a.st->n_prunes, 1ull);
+    }
+  } else if (cg) {
+    walk64<true, EV, T, false>(a.cg, slot0, tab, thr, terms, a);
+  } else {
+    walk64<false, EV, T, false>(a.fg, slot0, tab, thr, terms, a);
+  }
+}
+
+template <bool EV, int T>
+__global__ void __launch_bounds__(kFp64Block) k_pair64(Launch64 a) {
+  grid_dependents_launch();  // as k_pair
+  block64<EV, T>(a, blockIdx.x);
+}
+
+template <bool EV, int T>
+__global__ void __launch_bounds__(kFp64Block)
+    k_pair64_batch(const Launch64* __restrict__ args, const int* __restrict__ off, int nrep) {
+  const int r = batch_replica(off, nrep, blockIdx.x);
+  block64<EV, T>(args[r], int(blockIdx.x) - off[r]);
+}
+
+static int make_launch64(const relres_ctx* c, int which, int per, bool prune, Launch64* out) {
+  Launch64 a{};
+  a.sx = c->box[0] / 18446744073709551616.0;
+  a.sy = c->box[1] / 18446744073709551616.0;
+  a.sz = c->box[2] / 18446744073709551616.0;
+  a.fx = float(c->box[0] / 4294967296.0);
+  a.fy = float(c->box[1] / 4294967296.0);
+  a.fz = float(c->box[2] / 4294967296.0);
+  a.nt = c->n_types;
+  a.tab = static_cast<const PairTab<double>*>(c->d_tab);
+  a.gate = &c->d_state->flags;
+  a.ref_p = c->d_ref_p;
+  a.st = c->d_state;
+  const bool do_fg = (which & 1) != 0;
+  const bool do_cg = (which & 2) && c->has_cg && c->n_h > 0;
+  const float rf = float(c->rlist_fg_cut + c->prune_delta + kPruneSlack);
+  a.fg = Walk64{c->n, c->d_pos_fg64, c->d_pos_fg, walk_nbr_fg(c), walk_cnt_fg(c), c->d_perm_fg,
+                static_cast<double*>(c->d_f_fg), c->d_acc + kAccFg, c->d_nbr_fg, c->d_cnt_fg, c->d_nbr_fg_in,
+                c->d_cnt_fg_in, rf * rf, &c->d_state->tot_in_fg};
+  a.cg = a.fg;  // a stand-in without a CG list
+  if (do_cg) {
+    const float rc = float(c->rlist_cg_cut + c->prune_delta + kPruneSlack);
+    a.cg = Walk64{c->n_h, c->d_pos_cg64, c->d_pos_cg, walk_nbr_cg(c), walk_cnt_cg(c), c->d_perm_cg,
+                  static_cast<double*>(c->d_f_cg), c->d_acc + kAccCg, c->d_nbr_cg, c->d_cnt_cg, c->d_nbr_cg_in,
+                  c->d_cnt_cg_in, rc * rc, &c->d_state->tot_in_cg};
+  }
+  a.prune_on = prune ? 1 : 0;
+  a.nblk_cg = do_cg ? (c->n_h + per - 1) / per : 0;
+  *out = a;
+  return a.nblk_cg + (do_fg ? (c->n + per - 1) / per : 0);
+}
+
+cudaError_t launch_pairs_f64(relres_ctx* c, bool ev, int which) {
+  const int lanes = fp64_lanes(c);
+  Launch64 a;
+  const int grid = make_launch64(c, which, kFp64Block / lanes, pairs_prune(c), &a);
+  if (grid == 0) return cudaSuccess;
+  const size_t smem = ev ? smem64<true>(a.nt) : smem64<false>(a.nt);
+  if (lanes == kFp64LanesSmall) {
+    if (ev)
+      k_pair64<true, kFp64LanesSmall><<<grid, kFp64Block, smem, c->stream>>>(a);
+    else
+      k_pair64<false, kFp64LanesSmall><<<grid, kFp64Block, smem, c->stream>>>(a);
+  } else if (ev) {
+    k_pair64<true, kFp64Lanes><<<grid, kFp64Block, smem, c->stream>>>(a);
+  } else {
+    k_pair64<false, kFp64Lanes><<<grid, kFp64Block, smem, c->stream>>>(a);
+  }
+  RELRES_LAUNCHED(c);
+  return cudaGetLastError();
+}
+
+// ---- batches (see pair.cu)
+cudaError_t prepare_pairs_batch_f64(const std::vector<relres_ctx*>& cs, BatchLaunch* b, BatchLaunch* b_ev) {
+  long long slots = 0;
+  for (const relres_ctx* c : cs) slots += pair_slots(c);
+  const int lanes = fp64_lanes_for(slots);
+  std::vector<Launch64> args(cs.size());
+  std::vector<int> off(cs.size() + 1, 0);
+  b->nt = 1;
+  for (size_t r = 0; r < cs.size(); ++r) {
+    off[r + 1] = off[r] + make_launch64(cs[r], 3, kFp64Block / lanes, cs[r]->prune_on, &args[r]);
+    b->nt = std::max(b->nt, cs[r]->n_types);
+  }
+  b->nblk = b_ev->nblk = off.back();
+  b->lanes = b_ev->lanes = lanes;
+  b_ev->nt = b->nt;
+  const cudaError_t e = upload_batch(b, args.data(), sizeof(Launch64) * args.size(), off);
+  return e != cudaSuccess ? e : upload_batch(b_ev, args.data(), sizeof(Launch64) * args.size(), off);
+}
+
+void launch_pairs_batch_f64(cudaStream_t s, bool ev, const BatchLaunch& b, int nrep) {
+  const auto* args = static_cast<const Launch64*>(b.d_args);
+  const size_t smem = ev ? smem64<true>(b.nt) : smem64<false>(b.nt);
+  if (b.lanes == kFp64LanesSmall) {
+    if (ev)
+      k_pair64_batch<true, kFp64LanesSmall><<<b.nblk, kFp64Block, smem, s>>>(args, b.d_off, nrep);
+    else
+      k_pair64_batch<false, kFp64LanesSmall><<<b.nblk, kFp64Block, smem, s>>>(args, b.d_off, nrep);
+  } else if (ev) {
+    k_pair64_batch<true, kFp64Lanes><<<b.nblk, kFp64Block, smem, s>>>(args, b.d_off, nrep);
+  } else {
+    k_pair64_batch<false, kFp64Lanes><<<b.nblk, kFp64Block, smem, s>>>(args, b.d_off, nrep);
+  }
+}
+
+}  // namespace relres

@@ -25,7 +25,7 @@ namespace relres {
 // float-float energy of one pair inside the cutoff from its exact 32-bit
 // coordinate differences
 template <bool CG>
-__device__ __forceinline__ ff pair_energy_ff(const int4& d, const SmemTabs& S, const PairLaunch<float>& a) {
+__device__ __forceinline__ ff pair_energy_ff(const int4& d, const SmemTabs& S, const PairLaunch& a) {
   const ff ex = ff_fixed_diff32(d.x, 0, ff{a.sx, a.sxl});
   const ff ey = ff_fixed_diff32(d.y, 0, ff{a.sy, a.syl});
   const ff ez = ff_fixed_diff32(d.z, 0, ff{a.sz, a.szl});
@@ -46,7 +46,7 @@ struct PairTotals {
 
 // energy and virial of one queued pair added to the thread's totals
 template <bool CG>
-__device__ __forceinline__ void add_pair(const int4& d, float fr, const SmemTabs& S, const PairLaunch<float>& a,
+__device__ __forceinline__ void add_pair(const int4& d, float fr, const SmemTabs& S, const PairLaunch& a,
                                          PairTotals* tot) {
   const ff e = pair_energy_ff<CG>(d, S, a);
   const float x = float(d.x) * a.sx, y = float(d.y) * a.sy, z = float(d.z) * a.sz;
@@ -74,8 +74,8 @@ struct PairQueue {
 
 // One warp's walk over the lists of its 32 / T slots.
 template <bool CG, bool EV, int T, bool PRN, int ACC>
-__device__ __forceinline__ void walk_lanes(const ListWalk<float>& L, int blk, const SmemTabs& S, float4* stage,
-                                           PairQueue* queue, PairTotals* tot, const PairLaunch<float>& a,
+__device__ __forceinline__ void walk_lanes(const ListWalk& L, int blk, const SmemTabs& S, float4* stage,
+                                           PairQueue* queue, PairTotals* tot, const PairLaunch& a,
                                            bool first_block) {
   static_assert(T == 1 || (T >= 4 && 32 % T == 0 && ACC == RELRES_ACC_COMPENSATED), "three lanes add the chunk sums");
   const int s = (blk * kLaneThreads + threadIdx.x) / T, q = threadIdx.x % T;
@@ -91,7 +91,7 @@ __device__ __forceinline__ void walk_lanes(const ListWalk<float>& L, int blk, co
   const int rounds = __reduce_max_sync(0xffffffffu, (nch + T - 1) / T);
   const int row0 = pi.w * a.nt;
   __syncthreads();  // the type-pair tables
-  Acc<float> A;
+  Acc A;
   int kept = 0;
   int4 buf = make_int4(ss, ss, ss, ss);
   int waiting = 0;
@@ -236,7 +236,7 @@ static size_t lanes_smem(int nt) {
 }
 
 template <bool EV, int T, int ACC>
-__device__ __forceinline__ void lanes_block(const PairLaunch<float>& a, int bid) {
+__device__ __forceinline__ void lanes_block(const PairLaunch& a, int bid) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nrow = a.nt * a.nt;
   size_t off = 0;
@@ -277,26 +277,26 @@ __device__ __forceinline__ void lanes_block(const PairLaunch<float>& a, int bid)
 
 // energy steps: 80 registers a thread (six blocks per SM), forces only: 64
 template <bool EV, int T, int ACC>
-__global__ void __launch_bounds__(kLaneThreads, EV ? 6 : 8) k_pair_lanes(PairLaunch<float> a) {
+__global__ void __launch_bounds__(kLaneThreads, EV ? 6 : 8) k_pair_lanes(PairLaunch a) {
   grid_dependents_launch();  // as k_pair
   lanes_block<EV, T, ACC>(a, blockIdx.x);
 }
 
 template <bool EV, int T, int ACC>
 __global__ void __launch_bounds__(kLaneThreads, EV ? 6 : 8)
-    k_pair_lanes_batch(const PairLaunch<float>* __restrict__ args, const int* __restrict__ off, int nrep) {
+    k_pair_lanes_batch(const PairLaunch* __restrict__ args, const int* __restrict__ off, int nrep) {
   const int r = batch_replica(off, nrep, blockIdx.x);
   lanes_block<EV, T, ACC>(args[r], int(blockIdx.x) - off[r]);
 }
 
 template <bool EV, int T, int ACC>
-static void launch_one(cudaStream_t s, const PairLaunch<float>& a, int grid) {
+static void launch_one(cudaStream_t s, const PairLaunch& a, int grid) {
   k_pair_lanes<EV, T, ACC><<<grid, kLaneThreads, lanes_smem<EV, T>(a.nt), s>>>(a);
 }
 template <bool EV, int T, int ACC>
 static void launch_batch(cudaStream_t s, const BatchLaunch& b, int nrep) {
   k_pair_lanes_batch<EV, T, ACC><<<b.nblk, kLaneThreads, lanes_smem<EV, T>(b.nt), s>>>(
-      static_cast<const PairLaunch<float>*>(b.d_args), b.d_off, nrep);
+      static_cast<const PairLaunch*>(b.d_args), b.d_off, nrep);
 }
 
 // F<EV, T, ACC>(...) for the accumulation and the lanes of a launch
@@ -319,7 +319,7 @@ static void launch_batch(cudaStream_t s, const BatchLaunch& b, int nrep) {
     F<true, 1, RELRES_ACC_FP64>(__VA_ARGS__);                     \
   }
 
-void launch_pairs_lanes(cudaStream_t s, int acc, const PairLaunch<float>& a, bool ev, int lanes, int grid) {
+void launch_pairs_lanes(cudaStream_t s, int acc, const PairLaunch& a, bool ev, int lanes, int grid) {
   RELRES_LANES(launch_one, s, a, grid)
 }
 

@@ -70,8 +70,8 @@ __global__ void k_eval_recip(const double* __restrict__ x, float* __restrict__ o
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const double v = x[k];
     out32[k] = rcp_nr(float(v));
-    out64[k] = rcp_d(v);
-    out64[n + k] = rsqrt_d(v);
+    out64[k] = rcp_d(v, float(v));
+    out64[n + k] = rsqrt_d(v, float(v));
   }
 }
 

@@ -119,9 +119,11 @@ struct DevState {
 // Energy / virial partial sums are 64-bit fixed point (value * 2^32): exact,
 // order-independent integer reductions.
 constexpr double kFix = 4294967296.0;
+constexpr double kFixFine = 1073741824.0;  // the second accumulators' units per 2^-32
 constexpr int kNQ = 7;  // E, Wxx, Wyy, Wzz, Wxy, Wxz, Wyz
 // accumulator slots: FG pair sums, CG pair sums, kinetic energy, bonded energy
 constexpr int kAccFg = 0, kAccCg = kNQ, kAccKe = 2 * kNQ, kAccEb = 2 * kNQ + 1, kNAcc = 2 * kNQ + 2;
+constexpr int kNAccAll = 2 * kNAcc;  // with the second accumulators (acc_add_fine)
 constexpr int kBlockSteps = 100;  // steps between host status checks in relres_step
 #ifndef RELRES_SEG_ATOMS
 #define RELRES_SEG_ATOMS 256
@@ -329,7 +331,7 @@ struct relres_ctx {
   bool use_seg = true;  // the fused kernel where segments exist (relres_set_option)
   // force sum and drift as programmatic dependent launches (untimed steps)
   bool use_pdl = true;
-  // reductions: 64-bit fixed-point accumulators (kNAcc), cleared by their reader
+  // reductions: 64-bit fixed-point accumulators (kNAccAll), cleared by their reader
   long long* d_acc = nullptr;
   double* d_draws = nullptr;  // CSVR random numbers of the current block of steps, 2 per step
   relres::DevState* d_state = nullptr;
@@ -549,14 +551,15 @@ inline int fp32_lanes_for(long long slots, int acc, bool ev) {
 }
 inline int fp32_lanes(const relres_ctx* c, bool ev) { return fp32_lanes_for(pair_slots(c), c->force_acc, ev); }
 
-// FP64 forces-only pair launches: 32-thread blocks for a system with fewer
-// 256-slot blocks than SMs, else 256; eight threads per slot (walk_ordered)
-// for one whose slots fill fewer than four warps per SM with one thread each
-constexpr int kFp64SmallTpa = 8;
-inline int fp64_pair_block(const relres_ctx* c) { return (c->n + 255) / 256 < kPartSMs ? 32 : 256; }
-inline int fp64_pair_tpa(const relres_ctx* c) {
-  return pair_slots(c) < 4LL * 32 * kPartSMs ? kFp64SmallTpa : 1;
-}
+// FP64 pair launches (pair64.cu): threads per slot, and one warp per block (a
+// launch is a few blocks per SM long, and the last ones decide: 152.7 against
+// 163.1 us per step with 128-thread blocks at 25 000 neopentane-like atoms).
+// Eight threads per slot below four warps of them per SM; us per step there
+// and above with 16 / 8 / 4 / 2 threads: 10 000 atoms - / 87 / - / -, 20 000
+// atoms 158 / - / 117 / 134, 40 000 atoms 244 / - / 202 / 211.
+constexpr int kFp64LanesSmall = 8, kFp64Lanes = 4, kFp64Block = 32;
+inline int fp64_lanes_for(long long slots) { return slots < 4LL * 32 * kPartSMs ? kFp64LanesSmall : kFp64Lanes; }
+inline int fp64_lanes(const relres_ctx* c) { return fp64_lanes_for(pair_slots(c)); }
 
 // the lists the pair kernels walk: the pruned ones when pruning is on
 inline const int* walk_nbr_fg(const relres_ctx* c) { return c->prune_on ? c->d_nbr_fg_in : c->d_nbr_fg; }

@@ -109,3 +109,35 @@ def test_overlapping_atoms_keep_their_energy(torch):
     assert abs(e0) > 2.0 ** 20
     assert abs(float(e[3]) - e0) <= 1e-7 * abs(e0)
     assert np.abs(w.cpu().numpy() - w0).max() <= 1e-5 * np.abs(w0).max()
+
+
+def test_fp64_batch_keeps_the_bits_of_each_replica_alone(torch):
+    """FP64 replicas that alone take eight lanes per list and together four."""
+    systems = [S.neopentane(n_mol=1000, seed=31), S.propane(n_mol=1000, box=53.0, seed=32),
+               S.neopentane(n_mol=2000, seed=33), S.neopentane(n_mol=400, seed=34)]
+    temps, seeds = [s.temperature for s in systems], [5, 6, 7, 8]
+
+    def make():
+        out = []
+        for s in systems:
+            ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP64), R.topology_for(s))
+            p, v = _dev(torch, s.pos), _dev(torch, s.vel)
+            ctx.build_neighbors(p, s.box)
+            out.append((ctx, p, v))
+        return out
+
+    alone = make()
+    for (c, p, v), t, sd in zip(alone, temps, seeds):
+        assert c.stats()["pair_tpa"] == 8
+        c.step(60, 1.0, p, v, t_target=t, tau_fs=100.0, seed=sd)
+    both = make()
+    batch = R.Batch([c for c, _, _ in both])
+    batch.step(60, 1.0, [p for _, p, _ in both], [v for _, _, v in both], temps, 100.0, seeds)
+    torch.cuda.synchronize()
+    assert batch.n_shared() == 4 and sum(s.n_atoms + s.n_hybrid for s in systems) > 19456
+    for (c1, p1, v1), (c2, p2, v2) in zip(alone, both):
+        assert np.array_equal(p1.cpu().numpy(), p2.cpu().numpy())
+        assert np.array_equal(v1.cpu().numpy(), v2.cpu().numpy())
+    batch.close()
+    for c, _, _ in alone + both:
+        c.close()
