@@ -558,14 +558,16 @@ relres_status relres_set_topology(relres_ctx* c, const relres_topology* t) {
     if (size_t(std::max(1, seg_slots)) * slot_bytes + 24 * size_t(kSegAtoms) > kSegSmemMax) seg_ok = false;
   }
   std::vector<double> bp(2 * size_t(std::max(1, t->n_bond_types)), 0.0),
-      ap(2 * size_t(std::max(1, t->n_angle_types)), 0.0), dp(4 * size_t(std::max(1, t->n_dihedral_types)), 0.0);
+      ap(4 * size_t(std::max(1, t->n_angle_types)), 0.0), dp(4 * size_t(std::max(1, t->n_dihedral_types)), 0.0);
   for (int k = 0; k < t->n_bond_types && t->n_bonds; ++k) {
     bp[2 * k] = t->bond_k[k];
     bp[2 * k + 1] = t->bond_r0[k];
   }
   for (int k = 0; k < t->n_angle_types && t->n_angles; ++k) {
-    ap[2 * k] = t->angle_k[k];
-    ap[2 * k + 1] = t->angle_theta0[k];
+    ap[4 * k] = t->angle_k[k];
+    ap[4 * k + 1] = t->angle_theta0[k];
+    ap[4 * k + 2] = std::cos(t->angle_theta0[k]);
+    ap[4 * k + 3] = std::sin(t->angle_theta0[k]);
   }
   for (int k = 0; k < 4 * t->n_dihedral_types && t->n_dihedrals; ++k) dp[k] = t->dihedral_k[k];
 
@@ -606,15 +608,15 @@ relres_status relres_set_topology(relres_ctx* c, const relres_topology* t) {
   CK(dalloc(&c->d_bond_par, bp.size()));
   CK(dalloc(&c->d_angle_par, ap.size()));
   CK(dalloc(&c->d_dih_par, dp.size()));
-  std::vector<float> bfp(4 * (bp.size() / 2), 0.f), afp(8 * (ap.size() / 2), 0.f);
+  std::vector<float> bfp(4 * (bp.size() / 2), 0.f), afp(8 * (ap.size() / 4), 0.f);
   for (size_t k = 0; k < bp.size() / 2; ++k) {
     bfp[4 * k] = float(bp[2 * k]);
     bfp[4 * k + 1] = float(bp[2 * k + 1]);
     bfp[4 * k + 2] = float(bp[2 * k + 1] - double(bfp[4 * k + 1]));
   }
-  for (size_t k = 0; k < ap.size() / 2; ++k) {
-    const double t0 = ap[2 * k + 1], c0 = std::cos(t0), s0 = std::sin(t0);
-    afp[8 * k] = float(ap[2 * k]);
+  for (size_t k = 0; k < ap.size() / 4; ++k) {
+    const double t0 = ap[4 * k + 1], c0 = std::cos(t0), s0 = std::sin(t0);
+    afp[8 * k] = float(ap[4 * k]);
     afp[8 * k + 1] = float(t0);
     afp[8 * k + 2] = float(c0);
     afp[8 * k + 3] = float(c0 - double(afp[8 * k + 2]));

@@ -248,7 +248,7 @@ struct relres_ctx {
   int4* d_dihs = nullptr;       // i, j, k, l
   int* d_dih_type = nullptr;
   double* d_bond_par = nullptr;   // k, r0 per type
-  double* d_angle_par = nullptr;  // k, theta0 per type
+  double* d_angle_par = nullptr;  // k, theta0, cos theta0, sin theta0 per type
   double* d_dih_par = nullptr;    // K1..K4 per type
   float* d_bond_fpar = nullptr;   // FP32 path: k, r0 hi, r0 lo, 0 per type
   float* d_angle_fpar = nullptr;  // FP32 path: k, theta0, cos hi/lo, sin hi/lo, 0, 0 per type
