@@ -480,7 +480,7 @@ relres_status relres_set_topology(relres_ctx* c, const relres_topology* t) {
   // bonded + force-sum kernel gives one block to each segment; without a valid
   // segmentation (a molecule larger than a segment) the two-kernel path runs.
   std::vector<int> seg;
-  int seg_slots = 0;
+  int seg_slots = 0, seg_atoms = 1, seg_terms = 0;
   bool seg_ok = true;
   {
     std::vector<int> cross(size_t(n) + 2, 0);  // > 0: a term spans the boundary before atom a
@@ -501,19 +501,26 @@ relres_status relres_set_topology(relres_ctx* c, const relres_topology* t) {
       }
       return lo;
     };
+    const int want = seg_atoms_for(n);
     int a0 = 0;
     while (a0 < n && seg_ok) {
-      int a1 = std::min(n, a0 + kSegAtoms);
+      int a1 = std::min(n, a0 + want);
       while (a1 > a0 && a1 < n && cross[a1] > 0) --a1;
-      if (a1 == a0) {
-        seg_ok = false;
-        break;
+      if (a1 == a0) {  // a molecule longer than `want`
+        a1 = std::min(n, a0 + want);
+        while (a1 < n && cross[a1] > 0) ++a1;
+        if (a1 - a0 > kSegAtoms) {
+          seg_ok = false;
+          break;
+        }
       }
       const int b0 = first_ge(hb, t->n_bonds, 0, a0), b1 = first_ge(hb, t->n_bonds, 0, a1);
       const int g0 = first_ge(ha, t->n_angles, 1, a0), g1 = first_ge(ha, t->n_angles, 1, a1);
       const int d0 = first_ge(hd, t->n_dihedrals, 2, a0), d1 = first_ge(hd, t->n_dihedrals, 2, a1);
       seg.insert(seg.end(), {a0, a1, b0, b1, g0, g1, d0, d1, a0});
       seg_slots = std::max(seg_slots, 2 * (b1 - b0) + 3 * (g1 - g0) + 4 * (d1 - d0));
+      seg_atoms = std::max(seg_atoms, a1 - a0);
+      seg_terms = std::max(seg_terms, (b1 - b0) + (g1 - g0) + (d1 - d0));
       a0 = a1;
     }
     // Prototypes: a segment whose term records and incident-term lists, taken
@@ -555,7 +562,7 @@ relres_status relres_set_topology(relres_ctx* c, const relres_topology* t) {
     // shared memory of the segment kernels: term slots (float4 or 3 doubles)
     // plus the segment's positions in the drift kernel
     const size_t slot_bytes = c->fp64 ? 24 : 16;
-    if (size_t(std::max(1, seg_slots)) * slot_bytes + 24 * size_t(kSegAtoms) > kSegSmemMax) seg_ok = false;
+    if (size_t(std::max(1, seg_slots)) * slot_bytes + 24 * size_t(seg_atoms) > kSegSmemMax) seg_ok = false;
   }
   std::vector<double> bp(2 * size_t(std::max(1, t->n_bond_types)), 0.0),
       ap(4 * size_t(std::max(1, t->n_angle_types)), 0.0), dp(4 * size_t(std::max(1, t->n_dihedral_types)), 0.0);
@@ -681,6 +688,8 @@ relres_status relres_set_topology(relres_ctx* c, const relres_topology* t) {
   c->seg_ok = seg_ok && !seg.empty();
   c->n_seg = int(seg.size() / kSegRec);
   c->seg_slots = std::max(1, seg_slots);
+  c->seg_atoms = seg_atoms;
+  c->seg_block = std::min(kSegAtoms, (std::max(seg_atoms, seg_terms) + 31) / 32 * 32);
   if (c->seg_ok) {
     CK(dalloc(&c->d_seg, seg.size()));
     CK(cudaMemcpy(c->d_seg, seg.data(), sizeof(int) * seg.size(), cudaMemcpyHostToDevice));

@@ -848,14 +848,20 @@ struct DriftSegArgs {
   const int* inc;
   ForceT<R>* f_bond;  // caller order
   long long* acc;
+  int seg_atoms;  // atoms of the largest segment
 };
+
+// shared memory of a segment's positions (the term slots follow, 16-byte aligned)
+__host__ __device__ __forceinline__ size_t seg_pos_bytes(int atoms) {
+  return (sizeof(unsigned long long) * 3 * size_t(atoms) + 15) / 16 * 16;
+}
 
 // The work of block `bid` (segment bid) of one system's drift launch.
 template <typename R, bool EV>
 __device__ __forceinline__ void drift_seg_block(const DriftSegArgs<R>& a, int bid) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned long long* sx = reinterpret_cast<unsigned long long*>(smem_raw);  // [kSegAtoms][3]
-  ForceT<R>* slot = reinterpret_cast<ForceT<R>*>(smem_raw + sizeof(unsigned long long) * 3 * kSegAtoms);
+  unsigned long long* sx = reinterpret_cast<unsigned long long*>(smem_raw);  // [seg_atoms][3], then the term slots
+  ForceT<R>* slot = reinterpret_cast<ForceT<R>*>(smem_raw + seg_pos_bytes(a.seg_atoms));
   const int* g = a.seg + kSegRec * bid;
   const int a0 = g[0], a1 = g[1], b0 = g[2], b1 = g[3], g0 = g[4], g1 = g[5], d0 = g[6], d1 = g[7], base = g[8];
   const int nb = b1 - b0, na = g1 - g0, nd = d1 - d0;
@@ -864,7 +870,7 @@ __device__ __forceinline__ void drift_seg_block(const DriftSegArgs<R>& a, int bi
   const int ip = base + threadIdx.x;  // the prototype's atom (its incident terms)
   // loads that do not depend on the drift, issued before it: the records of
   // this thread's first two bond/angle terms and its atom's incident-term range
-  const int q0 = threadIdx.x, q1 = threadIdx.x + kSegAtoms;
+  const int q0 = threadIdx.x, q1 = threadIdx.x + blockDim.x;
   const int4 rec0 = q0 < nb ? a.B.bonds[b0 + q0] : (q0 < nb + na ? a.B.angles[g0 + q0 - nb] : make_int4(0, 0, 0, 0));
   const int4 rec1 = q1 < nb ? a.B.bonds[b0 + q1] : (q1 < nb + na ? a.B.angles[g0 + q1 - nb] : make_int4(0, 0, 0, 0));
   const int e0 = i < a1 ? a.inc_off[ip] : 0, e1 = i < a1 ? a.inc_off[ip + 1] : 0;
@@ -1467,9 +1473,9 @@ static cudaError_t launch_finish_seg_t(relres_ctx* c, bool ev, double* d_forces_
   a.st = c->d_state;
   const size_t smem = size_t(c->seg_slots) * (std::is_same<R, float>::value ? 16 : 24);
   if (ev)
-    k_finish_seg<R, true><<<c->n_seg, kThreads, smem, c->stream>>>(a);
+    k_finish_seg<R, true><<<c->n_seg, c->seg_block, smem, c->stream>>>(a);
   else
-    k_finish_seg<R, false><<<c->n_seg, kThreads, smem, c->stream>>>(a);
+    k_finish_seg<R, false><<<c->n_seg, c->seg_block, smem, c->stream>>>(a);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
@@ -1558,12 +1564,13 @@ static DriftSegArgs<R> drift_seg_args(relres_ctx* c, const StepParams& sp, doubl
   a.inc = c->d_inc;
   a.f_bond = static_cast<ForceT<R>*>(c->d_f_bond);
   a.acc = c->d_acc;
+  a.seg_atoms = c->seg_atoms;
   return a;
 }
 
 template <typename R>
 static size_t drift_seg_smem(const relres_ctx* c) {
-  return sizeof(unsigned long long) * 3 * kSegAtoms + size_t(c->seg_slots) * (std::is_same<R, float>::value ? 16 : 24);
+  return seg_pos_bytes(c->seg_atoms) + size_t(c->seg_slots) * (std::is_same<R, float>::value ? 16 : 24);
 }
 
 // A launch that may overlap the tail of the previous kernel of the stream
@@ -1596,8 +1603,8 @@ static cudaError_t launch_drift_t(relres_ctx* c, const StepParams& sp, double* d
     const size_t smem = drift_seg_smem<R>(c);
     // after the force sum of the previous step: overlap its tail
     const bool pdl = after_sum && pdl_ok(c);
-    const cudaError_t e = ev ? launch_pdl(pdl, k_drift_seg<R, true>, c->n_seg, kSegAtoms, smem, c->stream, a)
-                             : launch_pdl(pdl, k_drift_seg<R, false>, c->n_seg, kSegAtoms, smem, c->stream, a);
+    const cudaError_t e = ev ? launch_pdl(pdl, k_drift_seg<R, true>, c->n_seg, c->seg_block, smem, c->stream, a)
+                             : launch_pdl(pdl, k_drift_seg<R, false>, c->n_seg, c->seg_block, smem, c->stream, a);
     if (e != cudaSuccess) return e;
   } else {
     k_drift<R><<<(c->n + kThreads - 1) / kThreads, kThreads, 0, c->stream>>>(drift_args<R>(c, sp, d_vel));
@@ -1691,12 +1698,15 @@ static cudaError_t prepare_drift_batch_t(const std::vector<relres_ctx*>& cs, con
   std::vector<DriftSegArgs<R>> args(cs.size());
   std::vector<int> off(cs.size() + 1, 0);
   size_t smem = 0;
+  int threads = 32;
   for (size_t r = 0; r < cs.size(); ++r) {
     args[r] = drift_seg_args<R>(cs[r], sp[r], d_vel[r]);
     off[r + 1] = off[r] + cs[r]->n_seg;
     smem = std::max(smem, drift_seg_smem<R>(cs[r]));
+    threads = std::max(threads, cs[r]->seg_block);
   }
   b->nblk = off.back();
+  b->threads = threads;
   b->smem = smem;
   return upload_batch(b, args.data(), sizeof(DriftSegArgs<R>) * args.size(), off);
 }
@@ -1710,9 +1720,9 @@ template <typename R>
 static void launch_drift_batch_t(cudaStream_t s, bool ev, const BatchLaunch& b, int nrep) {
   const auto* args = static_cast<const DriftSegArgs<R>*>(b.d_args);
   if (ev)
-    k_drift_seg_batch<R, true><<<b.nblk, kSegAtoms, b.smem, s>>>(args, b.d_off, nrep);
+    k_drift_seg_batch<R, true><<<b.nblk, b.threads, b.smem, s>>>(args, b.d_off, nrep);
   else
-    k_drift_seg_batch<R, false><<<b.nblk, kSegAtoms, b.smem, s>>>(args, b.d_off, nrep);
+    k_drift_seg_batch<R, false><<<b.nblk, b.threads, b.smem, s>>>(args, b.d_off, nrep);
 }
 
 cudaError_t launch_drift_batch(cudaStream_t s, bool fp64, bool ev, const BatchLaunch& b, int nrep) {

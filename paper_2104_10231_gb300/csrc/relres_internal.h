@@ -128,7 +128,15 @@ constexpr int kBlockSteps = 100;  // steps between host status checks in relres_
 #ifndef RELRES_SEG_ATOMS
 #define RELRES_SEG_ATOMS 256
 #endif
-constexpr int kSegAtoms = RELRES_SEG_ATOMS;  // atoms per segment (one block of the segment kernels)
+constexpr int kSegAtoms = RELRES_SEG_ATOMS;  // most atoms of a segment (one block of the segment kernels)
+// Atoms per segment aimed at (more where one molecule has more): a drift block
+// lasts as long as its segment, so small systems take segments that leave each
+// SM one or two of them, with a thread per term where that is more than a
+// thread per atom.  us per MD step with segments of up to 256 atoms / by this
+// rule (neopentane-like, FP32): 18.1 / 16.9 at 1 715 atoms, 21.8 / 20.6 at
+// 10 000, 27.2 / 26.1 at 20 000, 31.2 / 30.4 at 30 000; at a million atoms
+// segments of 128 gain 3 % of the drift and are not taken.
+inline int seg_atoms_for(int n) { return n <= 2 * 64 * 152 ? 64 : (n <= 2 * 128 * 152 ? 128 : kSegAtoms); }
 // A segment record: atoms [a0, a1), then the bond, angle and dihedral ranges
 // and the first atom of its prototype (a segment whose terms and incident-term
 // lists are those of this one shifted by a0 - base; base = a0 where none).
@@ -327,6 +335,8 @@ struct relres_ctx {
   // ranges, the prototype's first atom
   int* d_seg = nullptr;
   int n_seg = 0, seg_slots = 0, n_seg_proto = 0;
+  int seg_atoms = 1;          // atoms of the largest segment
+  int seg_block = relres::kSegAtoms;  // threads of a segment's block: one per atom and, up to kSegAtoms, per term
   bool seg_ok = false;
   bool use_seg = true;  // the fused kernel where segments exist (relres_set_option)
   // force sum and drift as programmatic dependent launches (untimed steps)
@@ -489,6 +499,7 @@ struct BatchLaunch {
   int n_off = 0;
   int nblk = 0;
   size_t smem = 0;
+  int threads = 0;  // drift launches: threads per block
   int nt = 1;     // pair launches: most types of any replica
   int lanes = 0;  // pair launches: threads per slot of pair_lanes.cu (0: k_pair_batch)
 };
