@@ -145,6 +145,13 @@ relres_status alloc_lists(relres_ctx* c) {
   return RELRES_OK;
 }
 
+relres_status barrier_timeout(relres_ctx* c) {
+  CK(launch_flags_and(c, ~(unsigned)F_BARRIER));
+  CK(cudaMemsetAsync(c->d_bar, 0, 2 * sizeof(unsigned), c->stream));
+  c->have_lists = false;  // left unfinished
+  return fail(c, RELRES_ERR_CUDA, "the list rebuild's grid-wide barrier timed out");
+}
+
 // Rebuild both lists at the current fixed-point positions, growing capacity
 // until everything fits.
 relres_status host_rebuild(relres_ctx* c) {
@@ -164,7 +171,12 @@ relres_status host_rebuild(relres_ctx* c) {
       c->last_mean_cg = c->n_h ? double(h.tot_cg) / c->n_h : 0.0;
       c->have_lists = true;
       c->n_builds += 1;
-      CK(launch_prune(c, nullptr));  // pruned lists at the same positions
+      // the pruning pass: by the next pair launch as it walks, where it can
+      c->prune_pending = pairs_prune(c);
+      if (c->prune_pending)
+        CK(launch_flags_or(c, F_PRUNE));
+      else
+        CK(launch_prune(c, nullptr));
       return RELRES_OK;
     }
     if (of) c->cap_fg = round_cap(h.max_fg * 1.2 + 8, c->n);
@@ -230,45 +242,84 @@ static bool timed_now(const relres_ctx* c, int cls) {
     if (t_) CK(toc(c));                      \
   } while (0)
 
-// Lists valid at the positions already converted into d_xfx: a rebuild if an
-// atom moved more than skin/2 since the last build, else a pruning pass if an
-// atom moved more than delta/2 since the last one.
-relres_status refresh_lists(relres_ctx* c) {
-  if (c->h_state->flags & F_REBUILD) return host_rebuild(c);
-  if (c->h_state->flags & F_PRUNE) {
-    CK(launch_prune(c, nullptr));
-    CK(launch_flags_and(c, ~(unsigned)F_PRUNE));
+// The pruning pass left over by the last host build, for a reader of the
+// pruned lists other than a pair launch (at the current positions).
+relres_status finish_prune(relres_ctx* c) {
+  if (!c->prune_pending) return RELRES_OK;
+  CK(launch_prune(c, nullptr));
+  CK(launch_flags_and(c, ~(unsigned)F_PRUNE));
+  c->prune_pending = false;
+  return RELRES_OK;
+}
+
+// Lists valid at the positions already converted into d_xfx, without a host
+// round trip: one gated kernel rebuilds them if an atom moved more than skin/2
+// since the last build, and prunes them (`prune`; else the pair launch that
+// follows does) if one moved more than delta/2 since the last pass.
+relres_status refresh_lists(relres_ctx* c, bool prune) {
+  CK(launch_rebuild_fused(c, prune && c->prune_on));
+  return RELRES_OK;
+}
+
+// After an evaluation: what the kernels reported, in h_state.  A list that did
+// not fit is rebuilt with more room (*retry = true: evaluate again).
+relres_status check_evaluation(relres_ctx* c, bool* retry) {
+  *retry = false;
+  const unsigned fl = c->h_state->flags;
+  if (fl & F_BADCELL) return fail(c, RELRES_ERR_CUDA, "cell binning produced an out-of-range index");
+  if (fl & F_BARRIER) return barrier_timeout(c);
+  if (fl & F_NONFINITE) {
+    CK(launch_flags_and(c, ~(unsigned)(F_NONFINITE | F_BADPOS)));
+    c->forces_valid = false;
+    return fail(c, RELRES_ERR_NONFINITE, (fl & F_BADPOS) ? "non-finite position" : "non-finite force");
+  }
+  if (fl & (F_OVERFLOW_FG | F_OVERFLOW_CG)) {
+    if (fl & F_OVERFLOW_FG) c->cap_fg = round_cap(c->h_state->max_fg * 1.2 + 8, c->n);
+    if (fl & F_OVERFLOW_CG) c->cap_cg = round_cap(c->h_state->max_cg * 1.2 + 8, c->n_h);
+    relres_status s = alloc_lists(c);
+    if (s == RELRES_OK) s = host_rebuild(c);
+    if (s != RELRES_OK) return s;
+    *retry = true;
   }
   return RELRES_OK;
+}
+
+// whether autotune_pairs times launches (else it goes by size)
+bool tunes_by_timing(const relres_ctx* c) {
+  return c->tune_mode < 0 && !c->fp64 && fp32_lanes(c, false) == 1 && c->n >= 20000;
 }
 
 // Forces at the positions already converted into d_xfx (F_tot, FP64 copy optional).
 relres_status forces_now(relres_ctx* c, int ev_mode, double* d_forces, double* d_energy,
                          double* d_virial) {
-  relres_status s = read_state(c);
-  if (s != RELRES_OK) return s;
-  if (c->h_state->flags & F_NONFINITE) {
-    CK(launch_flags_and(c, ~(unsigned)F_NONFINITE));
-    return fail(c, RELRES_ERR_NONFINITE, "non-finite position");
-  }
-  s = refresh_lists(c);
-  if (s != RELRES_OK) return s;
-  if (!c->tuned) {
-    s = autotune_pairs(c);
+  if (!c->tuned && tunes_by_timing(c)) {  // on lists that are ready
+    relres_status s = refresh_lists(c, true);
+    if (s != RELRES_OK) return s;
+    CK(launch_close_call(c));
+    c->prune_pending = false;
+    s = read_state(c);
+    bool retry;
+    if (s == RELRES_OK) s = check_evaluation(c, &retry);
     if (s != RELRES_OK) return s;
   }
-  CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAccAll, c->stream));
-  TIMED(ev_mode == 1 ? RELRES_T_PAIR_EV : RELRES_T_PAIR, launch_pairs(c, ev_mode == 1));
-  TIMED(RELRES_T_FINISH, launch_finish(c, ev_mode == 1, d_forces, nullptr));
-  if (ev_mode == 1) TIMED(RELRES_T_THERMO, launch_reduce_out(c, d_energy, d_virial));
-  s = read_state(c);
-  if (s != RELRES_OK) return s;
-  s = flush_timing(c);
-  if (s != RELRES_OK) return s;
-  if (c->h_state->flags & F_NONFINITE) {
-    CK(launch_flags_and(c, ~(unsigned)F_NONFINITE));
-    c->forces_valid = false;
-    return fail(c, RELRES_ERR_NONFINITE, "non-finite force");
+  if (!c->tuned) {
+    const relres_status s = autotune_pairs(c);
+    if (s != RELRES_OK) return s;
+  }
+  for (bool retry = true; retry;) {
+    relres_status s = refresh_lists(c, !pairs_prune(c));
+    if (s != RELRES_OK) return s;
+    CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAccAll, c->stream));
+    TIMED(ev_mode == 1 ? RELRES_T_PAIR_EV : RELRES_T_PAIR, launch_pairs(c, ev_mode == 1));
+    TIMED(RELRES_T_FINISH, launch_finish(c, ev_mode == 1, d_forces, nullptr, true));
+    if (ev_mode == 1) TIMED(RELRES_T_THERMO, launch_reduce_out(c, d_energy, d_virial));
+    c->prune_pending = false;
+    s = read_state(c);
+    if (s != RELRES_OK) return s;
+    s = flush_timing(c);
+    if (s != RELRES_OK) return s;
+    s = check_evaluation(c, &retry);
+    if (s != RELRES_OK) return s;
   }
   c->forces_valid = true;
   return RELRES_OK;
@@ -748,7 +799,7 @@ relres_status relres_build_neighbors(relres_ctx* c, const double* d_pos, const d
   s = read_state(c);
   if (s != RELRES_OK) return s;
   if (c->h_state->flags & F_NONFINITE) {
-    CK(launch_flags_and(c, ~(unsigned)F_NONFINITE));
+    CK(launch_flags_and(c, ~(unsigned)(F_NONFINITE | F_BADPOS)));
     return fail(c, RELRES_ERR_NONFINITE, "non-finite position");
   }
   c->forces_valid = false;
@@ -777,10 +828,12 @@ static relres_status autotune_pairs(relres_ctx* c) {
     c->pair_lanes = fp32_lanes(c, false);
     return RELRES_OK;
   }
-  if (c->tune_mode >= 0 || c->fp64 || c->n < 20000) {
+  if (!tunes_by_timing(c)) {
     c->pair_cfg = c->tune_mode >= 0 ? c->tune_mode : 0;
     return RELRES_OK;
   }
+  const relres_status s = finish_prune(c);
+  if (s != RELRES_OK) return s;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
@@ -832,6 +885,10 @@ relres_status relres_get_list(relres_ctx* c, int which, int* h_i, int* h_j, long
   if (!c->have_lists) return fail(c, RELRES_ERR_STATE, "relres_build_neighbors first");
   const bool cg = (which & 1) != 0, pruned = which >= 2;
   if (pruned && !c->prune_on) return fail(c, RELRES_ERR_STATE, "pruning is off");
+  if (pruned) {
+    const relres_status s = finish_prune(c);
+    if (s != RELRES_OK) return s;
+  }
   const int nslots = cg ? ((c->has_cg && c->n_h > 0) ? c->n_h : 0) : c->n;
   *n_pairs = 0;
   if (nslots == 0) return RELRES_OK;
@@ -1023,7 +1080,7 @@ static relres_status record_block(relres_ctx* c, const StepParams& sp, double* d
     if (step_segments(c)) {  // bonded forces came with the drift; thermostat in k_sum's last block
       TIMED(RELRES_T_FINISH, launch_end_of_step(c, sp, k, ev_step, d_vel));
     } else {
-      TIMED(RELRES_T_FINISH, launch_finish(c, ev_step, nullptr, d_vel));
+      TIMED(RELRES_T_FINISH, launch_finish(c, ev_step, nullptr, d_vel, false));
       TIMED(RELRES_T_THERMO, launch_thermo(c, sp, k));
     }
   }
@@ -1215,15 +1272,6 @@ relres_status relres_backward(relres_ctx* c, const double* d_pos, const double* 
   if (!d_pos || !std::isfinite(grad_energy)) return fail(c, RELRES_ERR_ARG, "invalid backward arguments");
   // positions into the device state (lists rebuilt if an atom moved too far)
   c->io_valid = false;
-  CK(launch_convert(c, d_pos));
-  relres_status s = read_state(c);
-  if (s != RELRES_OK) return s;
-  if (c->h_state->flags & F_NONFINITE) {
-    CK(launch_flags_and(c, ~(unsigned)F_NONFINITE));
-    return fail(c, RELRES_ERR_NONFINITE, "non-finite position");
-  }
-  s = refresh_lists(c);
-  if (s != RELRES_OK) return s;
   c->forces_valid = false;
   // gradient buffers (allocated on first use)
   if (c->grad_n != c->n) {
@@ -1237,10 +1285,21 @@ relres_status relres_backward(relres_ctx* c, const double* d_pos, const double* 
     CK(cudaMemsetAsync(c->d_zero_n3, 0, sizeof(double) * 3 * c->n, c->stream));
     c->grad_n = c->n;
   }
-  CK(launch_pair_grad(c, d_grad_forces, grad_energy, d_grad_pos));
+  // positions into the device state, lists rebuilt and pruned as needed
+  CK(launch_convert(c, d_pos));
   std::vector<double> gc(4 * c->recs.size());
-  CK(cudaMemcpyAsync(gc.data(), c->d_gc, sizeof(double) * gc.size(), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  for (bool retry = true; retry;) {
+    relres_status s = refresh_lists(c, true);
+    if (s != RELRES_OK) return s;
+    CK(launch_pair_grad(c, d_grad_forces, grad_energy, d_grad_pos));
+    CK(launch_close_call(c));
+    c->prune_pending = false;
+    CK(cudaMemcpyAsync(gc.data(), c->d_gc, sizeof(double) * gc.size(), cudaMemcpyDeviceToHost, c->stream));
+    s = read_state(c);
+    if (s != RELRES_OK) return s;
+    s = check_evaluation(c, &retry);
+    if (s != RELRES_OK) return s;
+  }
   if (grad_c) std::copy(gc.begin(), gc.end(), grad_c);
   chain_params(c, gc.data(), d_eps_fg, d_sig_fg, d_eps_cg, d_sig_cg);
   return RELRES_OK;
@@ -1348,12 +1407,7 @@ static relres_status block_end(relres_ctx* c, double* d_pos, double* d_vel, doub
   }
   const unsigned fl = c->h_state->flags;
   if (fl & F_BADCELL) return fail(c, RELRES_ERR_CUDA, "cell binning produced an out-of-range index");
-  if (fl & F_BARRIER) {
-    CK(launch_flags_and(c, ~(unsigned)F_BARRIER));
-    CK(cudaMemsetAsync(c->d_bar, 0, 2 * sizeof(unsigned), c->stream));
-    c->have_lists = false;  // left unfinished
-    return fail(c, RELRES_ERR_CUDA, "the list rebuild's grid-wide barrier timed out");
-  }
+  if (fl & F_BARRIER) return barrier_timeout(c);
   if (fl & (F_OVERFLOW_FG | F_OVERFLOW_CG | F_NONFINITE)) {
     s = rollback_block(c, d_vel);
     if (s != RELRES_OK) return s;
@@ -1739,6 +1793,7 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
     for (int r = 0; r < nr; ++r) {
       builds0[r] = b->ctx[r]->h_state->n_builds;
       prunes0[r] = (long long)b->ctx[r]->h_state->n_prunes;
+      b->ctx[r]->prune_pending = false;  // by the block's first pair launch
     }
     relres_status s = batch_graph(b, sp, d_vel, blk, done);
     if (s != RELRES_OK) return s;
@@ -1838,6 +1893,7 @@ relres_status relres_step(relres_ctx* c, int n_steps, double dt_fs, double* d_po
   while (done < n_steps) {
     const int blk = std::min(kBlockSteps, n_steps - done);
     const long long builds0 = c->h_state->n_builds, prunes0 = (long long)c->h_state->n_prunes;
+    c->prune_pending = false;  // by the block's first pair launch
     if (c->use_graphs) {
       s = step_graph(c, sp, d_vel, blk, done);
       if (s != RELRES_OK) return s;
@@ -1873,7 +1929,8 @@ relres_status relres_set_step_counter(relres_ctx* c, long long step) {
 
 relres_status relres_get_stats(relres_ctx* c, relres_stats* o) {
   if (!c || !o) return RELRES_ERR_ARG;
-  relres_status s = read_state(c);
+  relres_status s = finish_prune(c);  // counted with its build
+  if (s == RELRES_OK) s = read_state(c);
   if (s != RELRES_OK) return s;
   std::memset(o, 0, sizeof(*o));
   o->n_atoms = c->n;

@@ -233,7 +233,8 @@ __global__ void k_gather_g(int nslots, const int* __restrict__ perm, const doubl
 // dL/dx = FG part + CG part (hybrids), caller order, FP64 out
 template <typename R>
 __global__ void k_sum_gx(int n, const GVec<R>* __restrict__ gx_fg, const GVec<R>* __restrict__ gx_cg,
-                         int with_cg, double* __restrict__ out) {
+                         int with_cg, const DevState* st, double* __restrict__ out) {
+  if (*(volatile const unsigned*)&st->flags & F_BADPOS) return;  // the call fails: no output
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     R a[3], b[3] = {R(0), R(0), R(0)};
     ld3(gx_fg, i, a);
@@ -299,7 +300,8 @@ static cudaError_t launch_grad_t(relres_ctx* c, const double* d_grad_forces, dou
     k_pair_grad<R, kThreads><<<nb_cg + nb_fg, kThreads, smem, c->stream>>>(a);
   RELRES_LAUNCHED(c);
   if (d_grad_pos) {
-    k_sum_gx<R><<<grid_for(c->n), kThreads, 0, c->stream>>>(c->n, xfg, xcg, do_cg ? 1 : 0, d_grad_pos);
+    k_sum_gx<R><<<grid_for(c->n), kThreads, 0, c->stream>>>(c->n, xfg, xcg, do_cg ? 1 : 0, c->d_state,
+                                                                 d_grad_pos);
     RELRES_LAUNCHED(c);
   }
   return cudaGetLastError();

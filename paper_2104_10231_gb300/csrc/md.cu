@@ -130,7 +130,7 @@ __global__ void k_convert(int n, const double* __restrict__ pos, const int* __re
   }
   if (__syncthreads_or(rebuild) && threadIdx.x == 0) atomicOr(&st->flags, F_REBUILD);
   if (__syncthreads_or(reprune) && threadIdx.x == 0) atomicOr(&st->flags, F_PRUNE);
-  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&st->flags, F_NONFINITE);
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&st->flags, F_NONFINITE | F_BADPOS);
 }
 
 // A 64-bit fixed-point coordinate as a double in [0, L): u L 2^-64, with u
@@ -514,9 +514,21 @@ struct FinishArgs {
   ForceT<R>* f_tot;
   double* f_out;       // FP64 copy in caller order
   int with_out;
+  int host_call;
   long long* acc;
   DevState* st;
 };
+
+// End of a force evaluation that is a call of its own: the lists are those of
+// these positions now (one thread, after the pair kernel).
+__device__ __forceinline__ void close_host_call(DevState* st) {
+  const unsigned f = *(volatile unsigned*)&st->flags;
+  if ((f & F_REBUILD) && !(f & F_BADPOS)) st->n_builds += 1;
+  atomicAnd(&st->flags, ~unsigned(F_REBUILD | F_PRUNE));
+}
+__device__ __forceinline__ bool bad_positions(const DevState* st) {
+  return (*(volatile const unsigned*)&st->flags & F_BADPOS) != 0u;
+}
 
 // Total force per atom: FG part + CG part + the slots of its bonded terms;
 // kinetic energy of u + c F for the thermostat.
@@ -524,6 +536,8 @@ template <typename R>
 __global__ void __launch_bounds__(kThreads) k_finish(FinishArgs<R> a) {
   R ke = R(0);
   bool bad = false;
+  const bool with_out = a.with_out && !(a.host_call && bad_positions(a.st));
+  if (a.host_call && blockIdx.x == 0 && threadIdx.x == 0) close_host_call(a.st);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < a.n) {
     const int t = a.type[i];
@@ -550,7 +564,7 @@ __global__ void __launch_bounds__(kThreads) k_finish(FinishArgs<R> a) {
     }
     bad = !(isfinite(f[0]) && isfinite(f[1]) && isfinite(f[2]));
     save_force(a.f_tot, i, f);
-    if (a.with_out) {
+    if (with_out) {
       a.f_out[3 * i] = double(f[0]);
       a.f_out[3 * i + 1] = double(f[1]);
       a.f_out[3 * i + 2] = double(f[2]);
@@ -602,6 +616,7 @@ struct SegArgs {
   ForceT<R>* f_tot;
   double* f_out;
   int with_out;
+  int host_call;
   long long* acc;
   DevState* st;
 };
@@ -617,6 +632,8 @@ __global__ void __launch_bounds__(kThreads) k_finish_seg(SegArgs<R> a) {
   const Sc3<R> sc = a.sc;
   // the terms are the prototype's (atoms from `base`): shifted onto this segment
   const GPosOff xg{a.xfx, a0 - base};
+  const bool with_out = a.with_out && !(a.host_call && bad_positions(a.st));
+  if (a.host_call && blockIdx.x == 0 && threadIdx.x == 0) close_host_call(a.st);
   R e = R(0);
   for (int q = threadIdx.x; q < nb + na + nd; q += blockDim.x) {
     if (q < nb) {
@@ -677,7 +694,7 @@ __global__ void __launch_bounds__(kThreads) k_finish_seg(SegArgs<R> a) {
     }
     bad = !(isfinite(f[0]) && isfinite(f[1]) && isfinite(f[2]));
     save_force(a.f_tot, i, f);
-    if (a.with_out) {
+    if (with_out) {
       a.f_out[3 * i] = double(f[0]);
       a.f_out[3 * i + 1] = double(f[1]);
       a.f_out[3 * i + 2] = double(f[2]);
@@ -1209,7 +1226,9 @@ __global__ void __launch_bounds__(kThreads) k_sum_batch(const SumArgs<R>* __rest
 }
 
 // Energies and virial of relres_compute (one thread); clears the accumulators.
-__global__ void k_reduce_out(long long* acc, double* energy, int with_e, double* virial, int with_w) {
+__global__ void k_reduce_out(long long* acc, double* energy, int with_e, double* virial, int with_w,
+                             const DevState* st) {
+  if (bad_positions(st)) with_e = with_w = 0;
   const double efg = acc_value(acc[kAccFg], acc[kNAcc + kAccFg]), ecg = acc_value(acc[kAccCg], acc[kNAcc + kAccCg]);
   const double eb = double(acc[kAccEb]) / kFix;
   if (with_e) {
@@ -1245,6 +1264,8 @@ __global__ void k_call_start(DevState* st, int reset_ab) {
 }
 
 __global__ void k_flags_and(DevState* st, unsigned keep) { st->flags &= keep; }
+__global__ void k_flags_or(DevState* st, unsigned set) { st->flags |= set; }
+__global__ void k_close_call(DevState* st) { close_host_call(st); }
 
 // FP32 path: caller's FP64 velocities -> float-float state
 __global__ void k_vel_in(int n3, const double* __restrict__ vel, float2* __restrict__ uff) {
@@ -1415,7 +1436,7 @@ static cudaError_t launch_bonded_t(relres_ctx* c, bool ev) {
 }
 
 template <typename R>
-static cudaError_t launch_finish_t(relres_ctx* c, double* d_forces_out, const double* vel) {
+static cudaError_t launch_finish_t(relres_ctx* c, double* d_forces_out, const double* vel, bool host_call) {
   const int with_cg = (c->has_cg && c->n_h > 0) ? 1 : 0;
   FinishArgs<R> a{c->n,
                   static_cast<const ForceT<R>*>(c->d_f_fg),
@@ -1436,6 +1457,7 @@ static cudaError_t launch_finish_t(relres_ctx* c, double* d_forces_out, const do
                   static_cast<ForceT<R>*>(c->d_f_tot),
                   d_forces_out ? d_forces_out : static_cast<double*>(c->d_dummy),
                   d_forces_out ? 1 : 0,
+                  host_call ? 1 : 0,
                   c->d_acc,
                   c->d_state};
   k_finish<R><<<(c->n + kThreads - 1) / kThreads, kThreads, 0, c->stream>>>(a);
@@ -1444,7 +1466,8 @@ static cudaError_t launch_finish_t(relres_ctx* c, double* d_forces_out, const do
 }
 
 template <typename R>
-static cudaError_t launch_finish_seg_t(relres_ctx* c, bool ev, double* d_forces_out, const double* vel) {
+static cudaError_t launch_finish_seg_t(relres_ctx* c, bool ev, double* d_forces_out, const double* vel,
+                                       bool host_call) {
   const double k = std::is_same<R, float>::value ? 4294967296.0 : 18446744073709551616.0;
   SegArgs<R> a{};
   a.seg = c->d_seg;
@@ -1469,6 +1492,7 @@ static cudaError_t launch_finish_seg_t(relres_ctx* c, bool ev, double* d_forces_
   a.f_tot = static_cast<ForceT<R>*>(c->d_f_tot);
   a.f_out = d_forces_out ? d_forces_out : static_cast<double*>(c->d_dummy);
   a.with_out = d_forces_out ? 1 : 0;
+  a.host_call = host_call ? 1 : 0;
   a.acc = c->d_acc;
   a.st = c->d_state;
   const size_t smem = size_t(c->seg_slots) * (std::is_same<R, float>::value ? 16 : 24);
@@ -1480,22 +1504,22 @@ static cudaError_t launch_finish_seg_t(relres_ctx* c, bool ev, double* d_forces_
   return cudaGetLastError();
 }
 
-cudaError_t launch_finish(relres_ctx* c, bool ev, double* d_forces_out, const double* d_vel) {
+cudaError_t launch_finish(relres_ctx* c, bool ev, double* d_forces_out, const double* d_vel, bool host_call) {
   if (c->seg_ok && c->use_seg)
-    return c->fp64 ? launch_finish_seg_t<double>(c, ev, d_forces_out, d_vel)
-                   : launch_finish_seg_t<float>(c, ev, d_forces_out, d_vel);
+    return c->fp64 ? launch_finish_seg_t<double>(c, ev, d_forces_out, d_vel, host_call)
+                   : launch_finish_seg_t<float>(c, ev, d_forces_out, d_vel, host_call);
   if (c->fp64) {
     const cudaError_t e = launch_bonded_t<double>(c, ev);
-    return e != cudaSuccess ? e : launch_finish_t<double>(c, d_forces_out, d_vel);
+    return e != cudaSuccess ? e : launch_finish_t<double>(c, d_forces_out, d_vel, host_call);
   }
   const cudaError_t e = launch_bonded_t<float>(c, ev);
-  return e != cudaSuccess ? e : launch_finish_t<float>(c, d_forces_out, d_vel);
+  return e != cudaSuccess ? e : launch_finish_t<float>(c, d_forces_out, d_vel, host_call);
 }
 
 cudaError_t launch_reduce_out(relres_ctx* c, double* d_energy, double* d_virial) {
   double* dd = static_cast<double*>(c->d_dummy);
   k_reduce_out<<<1, 1, 0, c->stream>>>(c->d_acc, d_energy ? d_energy : dd, d_energy ? 1 : 0,
-                                       d_virial ? d_virial : dd, d_virial ? 1 : 0);
+                                       d_virial ? d_virial : dd, d_virial ? 1 : 0, c->d_state);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
@@ -1664,7 +1688,7 @@ static cudaError_t launch_sum_t(relres_ctx* c, const StepParams& sp, int k, cons
 cudaError_t launch_end_of_step(relres_ctx* c, const StepParams& sp, int k, bool ev, double* d_vel) {
   if (step_segments(c))
     return c->fp64 ? launch_sum_t<double>(c, sp, k, d_vel) : launch_sum_t<float>(c, sp, k, d_vel);
-  cudaError_t e = launch_finish(c, ev, nullptr, d_vel);
+  cudaError_t e = launch_finish(c, ev, nullptr, d_vel, false);
   return e != cudaSuccess ? e : launch_thermo(c, sp, k);
 }
 
@@ -1687,6 +1711,18 @@ cudaError_t launch_call_start(relres_ctx* c, bool reset_ab) {
 
 cudaError_t launch_flags_and(relres_ctx* c, unsigned keep) {
   k_flags_and<<<1, 1, 0, c->stream>>>(c->d_state, keep);
+  RELRES_LAUNCHED(c);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_flags_or(relres_ctx* c, unsigned set) {
+  k_flags_or<<<1, 1, 0, c->stream>>>(c->d_state, set);
+  RELRES_LAUNCHED(c);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_close_call(relres_ctx* c) {
+  k_close_call<<<1, 1, 0, c->stream>>>(c->d_state);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }

@@ -1074,6 +1074,7 @@ __global__ void __launch_bounds__(kListThreads) k_rebuild(const unsigned* gate, 
                                                           const __grid_constant__ PruneArgs p, int prune,
                                                           unsigned* bar) {
   const unsigned f = *(volatile const unsigned*)gate;
+  if (f & F_NONFINITE) return;  // no lists from such positions
   const int bid = blockIdx.x, nblk = gridDim.x;
   if (f & F_REBUILD) {
     bin_body(bid, nblk, b.n, gate, b.xfx, b.type, b.hyb_mask, b.gf.n0, b.gf.n1, b.gf.n2, b.gf.rank_of, b.gf.count,

@@ -95,6 +95,7 @@ enum : unsigned {
   F_DIRTY = 16u,        // incoming positions differ from the cached state
   F_BADCELL = 32u,      // a computed cell index was out of range (access skipped)
   F_PRUNE = 64u,        // an atom moved more than delta/2 since the last pruning pass
+  F_BADPOS = 512u,      // a non-finite incoming position (with F_NONFINITE)
   F_BARRIER = 256u,     // a grid-wide barrier of the fused rebuild ran out of time
   F_VDIRTY = 128u,      // incoming velocities differ from the ones returned last
 };
@@ -303,6 +304,9 @@ struct relres_ctx {
   // pruning pass, same layout and capacity; the pair kernels walk these
   double prune_delta = relres::kPruneDelta;  // <= 0: no pruning (pair kernels walk the lists above)
   bool prune_on = false;                     // prune_delta > 0 and the inner lists are allocated
+  // the last host build left its pruning pass to the next pair launch (F_PRUNE
+  // is set on the device); whoever else reads the pruned lists runs it first
+  bool prune_pending = false;
   int* d_nbr_fg_in = nullptr;
   int* d_cnt_fg_in = nullptr;
   int* d_nbr_cg_in = nullptr;
@@ -459,7 +463,10 @@ cudaError_t launch_pairs(relres_ctx* c, bool ev, int which = 3);
 // whether this context's pair launches prune (pruning on, one thread per
 // slot); otherwise a separate pruning pass precedes them when it is due
 bool pairs_prune(const relres_ctx* c);
-cudaError_t launch_finish(relres_ctx* c, bool ev, double* d_forces_out, const double* d_vel);
+// `host_call`: this evaluation is a call of its own (not an MD step): the
+// kernel closes it by counting and clearing the list flags, and leaves the
+// outputs alone if a position was not finite.
+cudaError_t launch_finish(relres_ctx* c, bool ev, double* d_forces_out, const double* d_vel, bool host_call);
 cudaError_t launch_reduce_out(relres_ctx* c, double* d_energy, double* d_virial);
 // backward pass of the pair interaction (grad.cu): per-type-pair totals into
 // d_gc, dL/dx (FP64, caller order) into d_grad_pos if non-null
@@ -486,6 +493,9 @@ inline void* vel_state(relres_ctx* c, double* d_vel) {
   return c->fp64 ? static_cast<void*>(d_vel) : static_cast<void*>(c->d_uff);
 }
 cudaError_t launch_flags_and(relres_ctx* c, unsigned keep);
+cudaError_t launch_flags_or(relres_ctx* c, unsigned set);
+// end of a call that refreshed the lists: counts a rebuild, clears the list flags
+cudaError_t launch_close_call(relres_ctx* c);
 
 // ---- batched launches (relres_batch_step): one launch of a kernel class
 // covers every replica.  d_args holds one argument struct per replica and

@@ -1,0 +1,124 @@
+"""Force evaluations as calls of their own (relres_compute, relres_backward):
+lists refreshed on the device without a host round trip.  Positions past the
+rebuild trigger, lists that overflow inside the evaluation, pruning left over
+by a build, and non-finite positions, which leave the outputs alone."""
+import numpy as np
+import pytest
+
+from oracle import core as O
+from paper_2104_10231_gb300 import relres as R
+from paper_2104_10231_gb300 import systems as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch as T
+
+    assert T.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2104_10231_gb300.build import build_library
+
+    build_library()
+    R.load()
+    return T
+
+
+def _dev(torch, a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+
+def _reference(s, pos):
+    fr, e, _ = O.pair_forces(pos, s.box, s.types, O.table_for(s), s.n_types, s.excl)
+    fb, _ = O.bonded(pos, s.box, s.topo)
+    return fr + fb, e
+
+
+def _err(f, ref):
+    return np.abs(f - ref).max() / np.sqrt((ref * ref).sum(1).mean())
+
+
+# a shift of every atom by more than half the skin rebuilds without changing
+# the physics; 25 000 atoms take the launches chosen by timing
+@pytest.mark.parametrize("precision", [R.RELRES_PREC_FP32, R.RELRES_PREC_FP64])
+@pytest.mark.parametrize("n_mol", [250, 1000])
+@pytest.mark.parametrize("config", [-1, 3])
+def test_moved_positions_rebuild_inside_the_evaluation(torch, precision, n_mol, config):
+    s = S.neopentane(n_mol=n_mol, seed=4)
+    ctx = R.Context(R.params_for(s, precision), R.topology_for(s))
+    ctx.set_pair_config(config)
+    ctx.build_neighbors(_dev(torch, s.pos), s.box)
+    ref, e0 = _reference(s, s.pos)
+    tol = 1e-5 if precision == R.RELRES_PREC_FP32 else 1e-10
+    builds = ctx.stats()["n_builds"]
+    for k, shift in enumerate((0.0, 0.4, 1.5, 1.6, 7.0)):
+        x = _dev(torch, s.pos + shift)
+        f, e = torch.empty_like(x), torch.zeros(4, dtype=torch.float64, device="cuda")
+        ctx.compute(x, f, e)
+        torch.cuda.synchronize()
+        assert _err(f.cpu().numpy(), ref) <= tol, shift
+        assert abs(float(e[0] + e[1]) - e0) <= 1e-7 * abs(e0)
+    st = ctx.stats()
+    assert st["n_builds"] == builds + 2  # at 1.5 (from 0) and 7.0 (from 1.5)
+    assert st["n_prunes"] >= st["n_builds"]
+    ctx.close()
+
+
+def test_overflow_inside_an_evaluation_grows_the_lists(torch):
+    s = S.neopentane(n_mol=300, seed=5)
+    ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP32), R.topology_for(s))
+    ctx.build_neighbors(_dev(torch, s.pos * 1.0), s.box)
+    f = _dev(torch, s.pos)
+    ctx.compute(_dev(torch, s.pos), f)
+    ctx.set_list_caps(1, 1)  # grown at once to what these positions need
+    # half of the liquid pushed into half of the box: far longer lists
+    pos = s.pos.copy()
+    mol = s.mol
+    centre = np.stack([s.pos[mol == m].mean(0) for m in range(mol.max() + 1)])
+    pos += (np.floor(centre / s.box * 2) / 2 * -1)[mol] * s.box * np.array([0.0, 0.0, 0.97])
+    x = _dev(torch, pos)
+    e = torch.zeros(4, dtype=torch.float64, device="cuda")
+    ctx.compute(x, f, e)
+    torch.cuda.synchronize()
+    ref, _ = _reference(s, np.mod(pos, s.box))
+    assert _err(f.cpu().numpy(), ref) <= 1e-5
+    ctx.close()
+
+
+def test_nonfinite_positions_leave_outputs_and_lists_alone(torch):
+    s = S.neopentane(n_mol=300, seed=6)
+    ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP32), R.topology_for(s))
+    good = _dev(torch, s.pos)
+    ctx.build_neighbors(good, s.box)
+    f = torch.empty_like(good)
+    ctx.compute(good, f)
+    want = f.cpu().numpy()
+    bad = good.clone()
+    bad[7, 1] = float("nan")
+    e = torch.full((4,), 3.0, dtype=torch.float64, device="cuda")
+    f.fill_(5.0)
+    g = torch.full_like(good, 9.0)
+    for call in (lambda: ctx.compute(bad, f, e), lambda: ctx.backward(bad, None, 1.0, g)):
+        with pytest.raises(R.RelresError) as ei:
+            call()
+        assert ei.value.status == 5 and "position" in str(ei.value)
+    torch.cuda.synchronize()
+    assert float(f.min()) == float(f.max()) == 5.0 and float(e.min()) == 3.0 and float(g.min()) == 9.0
+    ctx.compute(good, f)
+    torch.cuda.synchronize()
+    assert np.abs(f.cpu().numpy() - want).max() <= 1e-5 * np.abs(want).max()
+    assert ctx.stats()["n_builds"] == 1
+    ctx.close()
+
+
+def test_backward_right_after_a_build_reads_pruned_lists(torch):
+    s = S.propane()
+    ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP64), R.make_topology(s.types, s.mass_by_type, s.excl, None))
+    x = _dev(torch, s.pos)
+    ctx.build_neighbors(x, s.box)
+    g = torch.empty_like(x)
+    ctx.backward(x, None, 1.0, g)
+    torch.cuda.synchronize()
+    fr, _, _ = O.pair_forces(s.pos, s.box, s.types, O.table_for(s), s.n_types, s.excl)
+    assert _err(g.cpu().numpy(), -fr) <= 1e-10
+    ctx.close()
