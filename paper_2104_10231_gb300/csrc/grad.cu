@@ -17,10 +17,9 @@
 //
 // One launch walks both lists (CG blocks first) like the force kernel; the
 // lists are those of the last force evaluation (nothing of the forward pass
-// is stored besides them).  Per-type-pair sums are kept per thread in
-// registers (the atom's own type is fixed, the partner's type selects the
-// accumulator), reduced per block in shared memory and added to FP64 totals
-// with atomics.
+// is stored besides them).  Per-type-pair sums are kept per thread (the atom's
+// own type is fixed, the partner's type selects the accumulator), reduced per
+// block in shared memory and added to FP64 totals with atomics.
 #include "common.cuh"
 
 namespace relres {
@@ -129,77 +128,104 @@ struct GradLaunch {
   double* gc;  // [nt*nt][4]: dL/dC12_FG, dL/dC6_FG, dL/dC12_CG, dL/dC6_CG
 };
 
-template <typename R, bool CG>
+constexpr int kGradThreads = 128;
+
+// 1/r from r^2 to about one rounding: the estimate and a Newton step (FP32),
+// the refined reciprocal square root (FP64)
+__device__ __forceinline__ float inv_r(float r2) {
+  const float y = rsqrtf(r2);
+  return fmaf(0.5f * y, fmaf(-r2 * y, y, 1.f), y);
+}
+__device__ __forceinline__ double inv_r(double r2) { return rsqrt_d(r2, float(r2)); }
+
+// One slot's walk, its list shared by T lanes (lane q takes chunks q, q + T,
+// ...): with one thread per slot a launch lasts as long as one list's chain of
+// loads, 77 us at 20 000 atoms.  The partner's type selects one of the
+// thread's accumulators in shared memory (s_acc[2 t + b][thread]: C12 and C6
+// sums of partner type t).
+template <typename R, bool CG, int T>
 __device__ __forceinline__ void grad_walk(const GradWalk<R>& W, int blk, const BasisTab<R>* tab,
-                                          const GradLaunch<R>& a, double* s_gc) {
-  const int s = blk * blockDim.x + threadIdx.x;
-  R acc12[RELRES_MAX_TYPES], acc6[RELRES_MAX_TYPES];
-#pragma unroll
-  for (int t = 0; t < RELRES_MAX_TYPES; ++t) acc12[t] = acc6[t] = R(0);
+                                          const GradLaunch<R>& a, double* s_gc, R (*s_acc)[kGradThreads]) {
+  const int s = (blk * kGradThreads + threadIdx.x) / T, q = threadIdx.x % T;
+  const bool own = s < W.nslots;
+  R gi[3] = {R(0), R(0), R(0)}, gx[3] = {R(0), R(0), R(0)};
   int ti = 0;
-  if (s < W.nslots) {
+  for (int t = 0; t < 2 * a.nt; ++t) s_acc[t][threadIdx.x] = R(0);
+  if (own) {
     const auto pi = W.pos[s];
     ti = gtype(pi);
-    R gi[3], gx[3] = {R(0), R(0), R(0)};
     ld3(W.g, s, gi);
-    const int m = W.cnt[s];
-    for (int k = 0; k < m; ++k) {
-      const int j = W.nbr[((size_t(k >> 2) * W.nslots + s) << 2) + (k & 3)];
-      const auto pj = W.pos[j];
-      const int tj = gtype(pj);
-      const BasisTab<R>& T = tab[ti * a.nt + tj];
-      R d[3];
-      diff3(pi, pj, a.sx, a.sy, a.sz, d);
-      const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-      const R rcut = CG ? T.rcp : T.rsp;
-      if (!(r2 < rcut * rcut)) continue;
-      const R r = sqrt(r2);
-      const R ri = R(1) / r;
-      R p[2], p1[2], p2[2];
-      basis<R, CG>(T, r, ri, p, p1, p2);
-      const R c12 = CG ? T.c12c : T.c12f, c6 = CG ? T.c6c : T.c6f;
-      const R u1 = c12 * p1[0] - c6 * p1[1];
-      const R u2 = c12 * p2[0] - c6 * p2[1];
-      R gj[3];
-      ld3(W.g, j, gj);
-      R rh[3], w[3];
-      R rw = R(0), gir = R(0);
+    const int m = W.cnt[s], nch = (m + 3) >> 2;
+    const int4* nb4 = reinterpret_cast<const int4*>(W.nbr) + s;
+    int4 jj = make_int4(s, s, s, s);
+    if (q < nch) jj = nb4[size_t(q) * W.nslots];
+    for (int ch = q; ch < nch; ch += T) {
+      int4 jn = jj;
+      if (ch + T < nch) jn = nb4[size_t(ch + T) * W.nslots];
+      const int rem = m - 4 * ch;  // >= 1
+      const int j[4] = {jj.x, rem > 1 ? jj.y : s, rem > 2 ? jj.z : s, rem > 3 ? jj.w : s};
+      GPos<R> pj[4];
+      R gj[4][3];
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        rh[q] = d[q] * ri;
-        w[q] = gi[q] - gj[q];
-        rw += rh[q] * w[q];
-        gir += gi[q] * rh[q];
+      for (int e = 0; e < 4; ++e) {
+        pj[e] = W.pos[j[e]];
+        ld3(W.g, j[e], gj[e]);
       }
 #pragma unroll
-      for (int q = 0; q < 3; ++q)
-        gx[q] += a.g_energy * u1 * rh[q] - (u2 * rw * rh[q] + u1 * ri * (w[q] - rw * rh[q]));
-      const R e12 = R(0.5) * a.g_energy * p[0] - p1[0] * gir;
-      const R e6 = R(0.5) * a.g_energy * p[1] - p1[1] * gir;
+      for (int e = 0; e < 4; ++e) {
+        const int tj = gtype(pj[e]);
+        const BasisTab<R>& B = tab[ti * a.nt + tj];
+        R d[3];
+        diff3(pi, pj[e], a.sx, a.sy, a.sz, d);
+        const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        const R rcut = CG ? B.rcp : B.rsp;
+        if (!(rem > e && r2 < rcut * rcut)) continue;
+        const R ri = inv_r(r2), r = r2 * ri;
+        R p[2], p1[2], p2[2];
+        basis<R, CG>(B, r, ri, p, p1, p2);
+        const R c12 = CG ? B.c12c : B.c12f, c6 = CG ? B.c6c : B.c6f;
+        const R u1 = c12 * p1[0] - c6 * p1[1];
+        const R u2 = c12 * p2[0] - c6 * p2[1];
+        R rh[3], w[3];
+        R rw = R(0), gir = R(0);
 #pragma unroll
-      for (int t = 0; t < RELRES_MAX_TYPES; ++t) {
-        acc12[t] += t == tj ? e12 : R(0);
-        acc6[t] += t == tj ? e6 : R(0);
+        for (int c = 0; c < 3; ++c) {
+          rh[c] = d[c] * ri;
+          w[c] = gi[c] - gj[e][c];
+          rw += rh[c] * w[c];
+          gir += gi[c] * rh[c];
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          gx[c] += a.g_energy * u1 * rh[c] - (u2 * rw * rh[c] + u1 * ri * (w[c] - rw * rh[c]));
+        s_acc[2 * tj][threadIdx.x] += R(0.5) * a.g_energy * p[0] - p1[0] * gir;
+        s_acc[2 * tj + 1][threadIdx.x] += R(0.5) * a.g_energy * p[1] - p1[1] * gir;
       }
+      jj = jn;
     }
-    st3(W.gx, W.perm[s], gx);
   }
-  // per-type-pair sums: shared-memory FP64 atomics per block, then global
-  if (s < W.nslots) {
+  // the slot's lanes together (T divides 32: whole slots per warp)
 #pragma unroll
-    for (int t = 0; t < RELRES_MAX_TYPES; ++t) {
-      if (t < a.nt && acc12[t] != R(0)) atomicAdd(&s_gc[(ti * a.nt + t) * 2], double(acc12[t]));
-      if (t < a.nt && acc6[t] != R(0)) atomicAdd(&s_gc[(ti * a.nt + t) * 2 + 1], -double(acc6[t]));
-    }
+  for (int o = T / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) gx[c] += __shfl_xor_sync(0xffffffffu, gx[c], o);
+  if (own && q == 0) st3(W.gx, W.perm[s], gx);
+  // per-type-pair sums: shared-memory FP64 atomics per block, then global
+  for (int t = 0; t < 2 * a.nt; ++t) {
+    double v = double(s_acc[t][threadIdx.x]);
+#pragma unroll
+    for (int o = T / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (own && q == 0 && v != 0.0) atomicAdd(&s_gc[ti * a.nt * 2 + t], (t & 1) ? -v : v);
   }
 }
 
-template <typename R, int BS>
-__global__ void __launch_bounds__(BS) k_pair_grad(GradLaunch<R> a) {
+template <typename R, int T>
+__global__ void __launch_bounds__(kGradThreads) k_pair_grad(GradLaunch<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nrow = a.nt * a.nt;
-  BasisTab<R>* tab = reinterpret_cast<BasisTab<R>*>(smem_raw);
-  double* s_gc = reinterpret_cast<double*>(smem_raw + ((sizeof(BasisTab<R>) * nrow + 15) / 16) * 16);
+  double* s_gc = reinterpret_cast<double*>(smem_raw);
+  R(*s_acc)[kGradThreads] = reinterpret_cast<R(*)[kGradThreads]>(s_gc + 2 * nrow);
+  BasisTab<R>* tab = reinterpret_cast<BasisTab<R>*>(s_acc + 2 * a.nt);
   {
     const int words = nrow * int(sizeof(BasisTab<R>) / sizeof(int));
     const int* src = reinterpret_cast<const int*>(a.tab);
@@ -210,9 +236,9 @@ __global__ void __launch_bounds__(BS) k_pair_grad(GradLaunch<R> a) {
   __syncthreads();
   const bool cg = int(blockIdx.x) < a.nblk_cg;
   if (cg)
-    grad_walk<R, true>(a.cg, blockIdx.x, tab, a, s_gc);
+    grad_walk<R, true, T>(a.cg, blockIdx.x, tab, a, s_gc, s_acc);
   else
-    grad_walk<R, false>(a.fg, blockIdx.x - a.nblk_cg, tab, a, s_gc);
+    grad_walk<R, false, T>(a.fg, blockIdx.x - a.nblk_cg, tab, a, s_gc, s_acc);
   __syncthreads();
   const int off = cg ? 2 : 0;
   for (int q = threadIdx.x; q < 2 * nrow; q += blockDim.x)
@@ -250,6 +276,20 @@ static int grid_for(int n) {
   return b < 1 ? 1 : (b > 152 * 8 ? 152 * 8 : b);
 }
 
+// Threads per slot by the slots of both lists.  Measured on neopentane-like
+// liquids (1.2 slots an atom), us per launch with 8 / 4 / 1 threads (one
+// register accumulator per type and 64-thread blocks before: last column):
+//   FP32   1 715 atoms  11.1 /  16.1 /  47.7    65.9
+//         10 000        16.9 /  17.8 /  49.1    73.3
+//         20 000        33.1 /  22.8 /  50.7    76.1
+//         90 000       107.4 /  82.7 /  71.5    82.7
+//        320 000       373.8 / 289.9 / 238.9   315.3
+//   FP64   1 715        64.6 / 103.7 / 362     397
+//         20 000         378 /   299 / 530     506
+static int grad_lanes(long long slots, bool fp64) {
+  return slots <= 14000 ? 8 : (fp64 || slots <= 75000 ? 4 : 1);
+}
+
 template <typename R>
 static cudaError_t launch_grad_t(relres_ctx* c, const double* d_grad_forces, double g_energy, double* d_grad_pos) {
   using V = GVec<R>;
@@ -285,19 +325,20 @@ static cudaError_t launch_grad_t(relres_ctx* c, const double* d_grad_forces, dou
   }
   a.fg = GradWalk<R>{c->n, pfg, walk_nbr_fg(c), walk_cnt_fg(c), c->d_perm_fg, gfg, xfg};
   a.cg = do_cg ? GradWalk<R>{c->n_h, pcg, walk_nbr_cg(c), walk_cnt_cg(c), c->d_perm_cg, gcg, xcg} : a.fg;
-  // small systems: 64-thread blocks, so that the launch covers every SM
-  const int bs = c->n < 200000 ? 64 : kThreads;
-  const int nb_fg = (c->n + bs - 1) / bs;
-  const int nb_cg = do_cg ? (c->n_h + bs - 1) / bs : 0;
+  const int lanes = grad_lanes(pair_slots(c), c->fp64), per = kGradThreads / lanes;
+  const int nb_fg = (c->n + per - 1) / per;
+  const int nb_cg = do_cg ? (c->n_h + per - 1) / per : 0;
   a.nblk_cg = nb_cg;
   const int nrow = c->n_types * c->n_types;
-  const size_t smem = ((sizeof(BasisTab<R>) * nrow + 15) / 16) * 16 + sizeof(double) * 2 * nrow;
+  const size_t smem = sizeof(double) * 2 * nrow + sizeof(R) * 2 * c->n_types * kGradThreads + sizeof(BasisTab<R>) * nrow;
   const cudaError_t ez = cudaMemsetAsync(c->d_gc, 0, sizeof(double) * 4 * nrow, c->stream);
   if (ez != cudaSuccess) return ez;
-  if (bs == 64)
-    k_pair_grad<R, 64><<<nb_cg + nb_fg, 64, smem, c->stream>>>(a);
+  if (lanes == 8)
+    k_pair_grad<R, 8><<<nb_cg + nb_fg, kGradThreads, smem, c->stream>>>(a);
+  else if (lanes == 4)
+    k_pair_grad<R, 4><<<nb_cg + nb_fg, kGradThreads, smem, c->stream>>>(a);
   else
-    k_pair_grad<R, kThreads><<<nb_cg + nb_fg, kThreads, smem, c->stream>>>(a);
+    k_pair_grad<R, 1><<<nb_cg + nb_fg, kGradThreads, smem, c->stream>>>(a);
   RELRES_LAUNCHED(c);
   if (d_grad_pos) {
     k_sum_gx<R><<<grid_for(c->n), kThreads, 0, c->stream>>>(c->n, xfg, xcg, do_cg ? 1 : 0, c->d_state,
