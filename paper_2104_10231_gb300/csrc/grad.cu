@@ -46,17 +46,6 @@ __device__ __forceinline__ void st3(double* a, int i, const double v[3]) {
   a[3 * i + 1] = v[1];
   a[3 * i + 2] = v[2];
 }
-__device__ __forceinline__ void diff3(const int4& a, const int4& b, float sx, float sy, float sz, float d[3]) {
-  d[0] = dfix32(a.x, b.x, sx);
-  d[1] = dfix32(a.y, b.y, sy);
-  d[2] = dfix32(a.z, b.z, sz);
-}
-__device__ __forceinline__ void diff3(const Pos64& a, const Pos64& b, double sx, double sy, double sz,
-                                      double d[3]) {
-  d[0] = dfix64(a.x, b.x, sx);
-  d[1] = dfix64(a.y, b.y, sy);
-  d[2] = dfix64(a.z, b.z, sz);
-}
 __device__ __forceinline__ int gtype(const int4& p) { return p.w; }
 __device__ __forceinline__ int gtype(const Pos64& p) { return int(p.t); }
 
@@ -68,12 +57,17 @@ __device__ __forceinline__ void poly3(const R (&g)[5], R d, R& f, R& f1, R& f2) 
   f2 = (R(12) * g[4] * d + R(6) * g[3]) * d + R(2) * g[2];
 }
 
+// One pair: difference vector, r, and the powers 1/r, r^-2, r^-12, r^-6.
+template <typename R>
+struct PairGeo {
+  R d[3], r2, r, ri, r2i, v[2];
+};
+
 // phi, phi', phi'' of both bases (b = 0: r^-12, b = 1: r^-6) for one part.
 template <typename R, bool CG>
-__device__ __forceinline__ void basis(const BasisTab<R>& T, R r, R ri, R (&p)[2], R (&p1)[2], R (&p2)[2]) {
-  const R r2i = ri * ri;
-  const R v6 = r2i * r2i * r2i;
-  const R v[2] = {v6 * v6, v6};
+__device__ __forceinline__ void basis(const BasisTab<R>& T, const PairGeo<R>& G, R (&p)[2], R (&p1)[2], R (&p2)[2]) {
+  const R r = G.r, ri = G.ri, r2i = G.r2i;
+  const R (&v)[2] = G.v;
   const R kk[2] = {R(12), R(6)};
 #pragma unroll
   for (int b = 0; b < 2; ++b) {
@@ -124,19 +118,48 @@ struct GradLaunch {
   const BasisTab<R>* tab;
   int nt;
   R sx, sy, sz;
+  float sxl, syl, szl;  // FP32: lo parts of L / 2^32
   R g_energy;
   double* gc;  // [nt*nt][4]: dL/dC12_FG, dL/dC6_FG, dL/dC12_CG, dL/dC6_CG
 };
 
 constexpr int kGradThreads = 128;
 
-// 1/r from r^2 to about one rounding: the estimate and a Newton step (FP32),
-// the refined reciprocal square root (FP64)
-__device__ __forceinline__ float inv_r(float r2) {
-  const float y = rsqrtf(r2);
-  return fmaf(0.5f * y, fmaf(-r2 * y, y, 1.f), y);
+// The geometry of one pair.  FP32: the second derivative goes as r^-14, so the
+// distance and its powers are formed in float-float from the exact integer
+// differences and rounded once; FP32 all the way amplified the roundings of
+// r^2 about sevenfold.
+__device__ __forceinline__ void geometry(const int4& a, const int4& b, const GradLaunch<float>& L, PairGeo<float>& G) {
+  const ff ex = ff_fixed_diff32(a.x, b.x, ff{L.sx, L.sxl}), ey = ff_fixed_diff32(a.y, b.y, ff{L.sy, L.syl}),
+           ez = ff_fixed_diff32(a.z, b.z, ff{L.sz, L.szl});
+  const ff r2 = ff_add(ff_add(ff_mul(ex, ex), ff_mul(ey, ey)), ff_mul(ez, ez));
+  G.d[0] = ex.hi;
+  G.d[1] = ey.hi;
+  G.d[2] = ez.hi;
+  G.r2 = r2.hi;
+  const float y = rcp_approx(r2.hi);
+  const float e = fmaf(-r2.lo, y, fmaf(-r2.hi, y, 1.f)), ye = y * e;
+  const ff i2 = ff_quick(y, fmaf(ye, e, ye));
+  const ff i6 = ff_mul(ff_mul(i2, i2), i2);
+  G.r2i = ff_val(i2);
+  G.v[0] = ff_val(ff_mul(i6, i6));
+  G.v[1] = ff_val(i6);
+  const float z = rsqrtf(r2.hi);
+  G.ri = fmaf(0.5f * z, fmaf(-r2.lo * z, z, fmaf(-r2.hi * z, z, 1.f)), z);
+  G.r = fmaf(r2.hi, G.ri, r2.lo * G.ri);
 }
-__device__ __forceinline__ double inv_r(double r2) { return rsqrt_d(r2, float(r2)); }
+__device__ __forceinline__ void geometry(const Pos64& a, const Pos64& b, const GradLaunch<double>& L,
+                                         PairGeo<double>& G) {
+  G.d[0] = dfix64(a.x, b.x, L.sx);
+  G.d[1] = dfix64(a.y, b.y, L.sy);
+  G.d[2] = dfix64(a.z, b.z, L.sz);
+  G.r2 = G.d[0] * G.d[0] + G.d[1] * G.d[1] + G.d[2] * G.d[2];
+  G.ri = rsqrt_d(G.r2, float(G.r2));
+  G.r = G.r2 * G.ri;
+  G.r2i = G.ri * G.ri;
+  G.v[1] = G.r2i * G.r2i * G.r2i;
+  G.v[0] = G.v[1] * G.v[1];
+}
 
 // One slot's walk, its list shared by T lanes (lane q takes chunks q, q + T,
 // ...): with one thread per slot a launch lasts as long as one list's chain of
@@ -175,14 +198,13 @@ __device__ __forceinline__ void grad_walk(const GradWalk<R>& W, int blk, const B
       for (int e = 0; e < 4; ++e) {
         const int tj = gtype(pj[e]);
         const BasisTab<R>& B = tab[ti * a.nt + tj];
-        R d[3];
-        diff3(pi, pj[e], a.sx, a.sy, a.sz, d);
-        const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        PairGeo<R> G;
+        geometry(pi, pj[e], a, G);
         const R rcut = CG ? B.rcp : B.rsp;
-        if (!(rem > e && r2 < rcut * rcut)) continue;
-        const R ri = inv_r(r2), r = r2 * ri;
+        if (!(rem > e && G.r2 < rcut * rcut)) continue;
+        const R ri = G.ri;
         R p[2], p1[2], p2[2];
-        basis<R, CG>(B, r, ri, p, p1, p2);
+        basis<R, CG>(B, G, p, p1, p2);
         const R c12 = CG ? B.c12c : B.c12f, c6 = CG ? B.c6c : B.c6f;
         const R u1 = c12 * p1[0] - c6 * p1[1];
         const R u2 = c12 * p2[0] - c6 * p2[1];
@@ -190,7 +212,7 @@ __device__ __forceinline__ void grad_walk(const GradWalk<R>& W, int blk, const B
         R rw = R(0), gir = R(0);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          rh[c] = d[c] * ri;
+          rh[c] = G.d[c] * ri;
           w[c] = gi[c] - gj[e][c];
           rw += rh[c] * w[c];
           gir += gi[c] * rh[c];
@@ -310,6 +332,9 @@ static cudaError_t launch_grad_t(relres_ctx* c, const double* d_grad_forces, dou
   a.sx = R(c->box[0] / unit);
   a.sy = R(c->box[1] / unit);
   a.sz = R(c->box[2] / unit);
+  a.sxl = float(c->box[0] / unit - double(a.sx));
+  a.syl = float(c->box[1] / unit - double(a.sy));
+  a.szl = float(c->box[2] / unit - double(a.sz));
   a.nt = c->n_types;
   a.tab = static_cast<const BasisTab<R>*>(c->d_basis);
   a.g_energy = R(g_energy);
