@@ -332,7 +332,8 @@ relres_status relres_get_stats(relres_ctx* ctx, relres_stats* out);
  * differentiable form treats them as variables.  n_types, is_hybrid, mixing,
  * precision, shift, skin, every radius and the set of type pairs with
  * eps^CG > 0 must stay as at relres_create (RELRES_ERR_ARG otherwise, the
- * context unchanged).  Waits for the context stream.  Cached forces are
+ * context unchanged).  Waits for the context stream; new tables follow on it
+ * in one transfer, none if the values are those in place.  Cached forces are
  * dropped (the next relres_step recomputes them).
  */
 relres_status relres_set_params(relres_ctx* ctx, const relres_params* p);

@@ -338,6 +338,54 @@ size_t force_bytes(const relres_ctx* c) { return size_t(c->n) * (c->fp64 ? 24 : 
 
 
 
+// The type-pair tables (force, energy and gradient rows) in one device
+// allocation, filled from a pinned copy by one transfer on the context stream.
+struct TablePart {
+  const void* src;
+  size_t bytes;
+  void** dst;
+};
+void table_parts(relres_ctx* c, TablePart (&t)[3]) {
+  if (c->fp64)
+    t[0] = {c->tab_d.data(), sizeof(PairTab<double>) * c->tab_d.size(), &c->d_tab};
+  else
+    t[0] = {c->rows_f.data(), sizeof(PairRowF) * c->rows_f.size(), &c->d_tab};
+  t[1] = {c->rows_e.data(), sizeof(PairRowE) * c->rows_e.size(), &c->d_tabe};
+  if (c->fp64)
+    t[2] = {c->basis_d.data(), sizeof(BasisTab<double>) * c->basis_d.size(), &c->d_basis};
+  else
+    t[2] = {c->basis_f.data(), sizeof(BasisTab<float>) * c->basis_f.size(), &c->d_basis};
+}
+size_t table_room(size_t bytes) { return (bytes + 255) / 256 * 256; }
+
+cudaError_t alloc_tables(relres_ctx* c) {
+  TablePart t[3];
+  table_parts(c, t);
+  c->table_bytes = 0;
+  for (const TablePart& q : t) c->table_bytes += table_room(q.bytes);
+  cudaError_t e = cudaMalloc(&c->d_tables, c->table_bytes);
+  if (e == cudaSuccess) e = cudaMallocHost(&c->h_tables, c->table_bytes);
+  if (e != cudaSuccess) return e;
+  size_t off = 0;
+  for (const TablePart& q : t) {
+    *q.dst = static_cast<unsigned char*>(c->d_tables) + off;
+    off += table_room(q.bytes);
+  }
+  return cudaSuccess;
+}
+
+// (the stream must have finished with the last upload)
+cudaError_t upload_tables(relres_ctx* c) {
+  TablePart t[3];
+  table_parts(c, t);
+  size_t off = 0;
+  for (const TablePart& q : t) {
+    std::memcpy(static_cast<unsigned char*>(c->h_tables) + off, q.src, q.bytes);
+    off += table_room(q.bytes);
+  }
+  return cudaMemcpyAsync(c->d_tables, c->h_tables, c->table_bytes, cudaMemcpyHostToDevice, c->stream);
+}
+
 }  // namespace
 
 extern "C" {
@@ -377,23 +425,10 @@ relres_status relres_create(relres_ctx** out, const relres_params* p, void* cuda
   }
   for (int t = 0; t < c->n_types; ++t)
     if (c->has_cg && c->is_hybrid[t]) c->hyb_mask |= 1 << t;
-  const size_t tb = c->fp64 ? sizeof(PairTab<double>) * c->tab_d.size() : sizeof(PairRowF) * c->rows_f.size();
-  cudaError_t ce = cudaMalloc(&c->d_tab, tb);
-  if (ce == cudaSuccess)
-    ce = cudaMemcpy(c->d_tab, c->fp64 ? static_cast<const void*>(c->tab_d.data())
-                                      : static_cast<const void*>(c->rows_f.data()),
-                    tb, cudaMemcpyHostToDevice);
-  if (ce == cudaSuccess) ce = cudaMalloc(&c->d_tabe, sizeof(PairRowE) * c->rows_e.size());
-  if (ce == cudaSuccess)
-    ce = cudaMemcpy(c->d_tabe, c->rows_e.data(), sizeof(PairRowE) * c->rows_e.size(), cudaMemcpyHostToDevice);
   build_basis_tables(c->recs, p->shift, &c->basis_f, &c->basis_d);
-  const size_t bb = c->fp64 ? sizeof(BasisTab<double>) * c->basis_d.size()
-                            : sizeof(BasisTab<float>) * c->basis_f.size();
-  if (ce == cudaSuccess) ce = cudaMalloc(&c->d_basis, bb);
-  if (ce == cudaSuccess)
-    ce = cudaMemcpy(c->d_basis, c->fp64 ? static_cast<const void*>(c->basis_d.data())
-                                        : static_cast<const void*>(c->basis_f.data()),
-                    bb, cudaMemcpyHostToDevice);
+  cudaError_t ce = alloc_tables(c);
+  if (ce == cudaSuccess) ce = upload_tables(c);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(c->stream);
   if (ce == cudaSuccess) ce = cudaMalloc(&c->d_gc, sizeof(double) * 4 * c->recs.size());
   if (ce == cudaSuccess) ce = cudaMalloc(&c->d_state, sizeof(DevState));
   if (ce == cudaSuccess) ce = cudaMemset(c->d_state, 0, sizeof(DevState));
@@ -1206,22 +1241,20 @@ relres_status relres_set_params(relres_ctx* c, const relres_params* p) {
         (a.eps_cg > 0.0) != (b.eps_cg > 0.0))
       return fail(c, RELRES_ERR_ARG, "relres_set_params: radii and the set of CG pairs must not change");
   }
+  // values already in place (a backward pass after its forward pass): nothing to upload
+  bool same = true;
+  for (int t = 0; t < c->n_types; ++t) same = same && p->eps_fg[t] == c->eps_fg[t] && p->sig_fg[t] == c->sig_fg[t];
+  for (size_t k = 0; k < recs.size(); ++k)
+    same = same && recs[k].eps_cg == c->recs[k].eps_cg && recs[k].sig_cg == c->recs[k].sig_cg;
   CK(cudaStreamSynchronize(c->stream));
-  c->recs = recs;
-  c->eps_fg.assign(p->eps_fg, p->eps_fg + p->n_types);
-  c->sig_fg.assign(p->sig_fg, p->sig_fg + p->n_types);
-  build_kernel_tables(c->recs, &c->tab_f, &c->tab_d);
-  pack_pair_rows(c->tab_f, c->tab_d, &c->rows_f, &c->rows_e);
-  build_basis_tables(c->recs, p->shift, &c->basis_f, &c->basis_d);
-  if (c->fp64) {
-    CK(cudaMemcpy(c->d_tab, c->tab_d.data(), sizeof(PairTab<double>) * c->tab_d.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->d_basis, c->basis_d.data(), sizeof(BasisTab<double>) * c->basis_d.size(),
-                  cudaMemcpyHostToDevice));
-  } else {
-    CK(cudaMemcpy(c->d_tab, c->rows_f.data(), sizeof(PairRowF) * c->rows_f.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->d_tabe, c->rows_e.data(), sizeof(PairRowE) * c->rows_e.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->d_basis, c->basis_f.data(), sizeof(BasisTab<float>) * c->basis_f.size(),
-                  cudaMemcpyHostToDevice));
+  if (!same) {
+    c->recs = recs;
+    c->eps_fg.assign(p->eps_fg, p->eps_fg + p->n_types);
+    c->sig_fg.assign(p->sig_fg, p->sig_fg + p->n_types);
+    build_kernel_tables(c->recs, &c->tab_f, &c->tab_d);
+    pack_pair_rows(c->tab_f, c->tab_d, &c->rows_f, &c->rows_e);
+    build_basis_tables(c->recs, p->shift, &c->basis_f, &c->basis_d);
+    CK(upload_tables(c));
   }
   c->forces_valid = false;
   return RELRES_OK;
@@ -2019,8 +2052,8 @@ void relres_destroy(relres_ctx* c) {
   drop_step_graph(c);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->body_stream) cudaStreamDestroy(c->body_stream);
-  dfree(c->d_tab);
-  dfree(c->d_tabe);
+  dfree(c->d_tables);  // d_tab, d_tabe, d_basis
+  if (c->h_tables) cudaFreeHost(c->h_tables);
   dfree(c->d_cdt);
   dfree(c->d_mass);
   dfree(c->d_type);
@@ -2076,7 +2109,6 @@ void relres_destroy(relres_ctx* c) {
   dfree(c->d_f_bond);
   dfree(c->d_tf);
   dfree(c->d_seg);
-  dfree(c->d_basis);
   dfree(c->d_gc);
   dfree(c->d_g_fg);
   dfree(c->d_g_cg);

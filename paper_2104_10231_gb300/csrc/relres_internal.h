@@ -229,7 +229,10 @@ struct relres_ctx {
   double* d_zero_n3 = nullptr;
   int grad_n = 0;             // atoms the gradient buffers were allocated for
 
-  // device tables
+  // device tables: one allocation and its pinned source
+  void* d_tables = nullptr;
+  void* h_tables = nullptr;
+  size_t table_bytes = 0;
   void* d_tab = nullptr;  // PairRowF (FP32) or PairTab<double> [n_types^2]
   void* d_tabe = nullptr; // PairRowE[n_types^2] (energies of the FP32 path)
   double* d_cdt = nullptr;   // per type: (dt/2m) * ftm2v  (set per step call)

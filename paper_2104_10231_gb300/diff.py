@@ -80,6 +80,11 @@ class RelResPair:
                              sig_cg=np.asarray(sig_cg, np.float64).reshape(-1), shift=self.shift,
                              precision=self.precision)
 
+    def _params_eq13(self, eps_fg, sig_fg):
+        """FG parameters with CG ones that the library derives by Eq. 13."""
+        return R.make_params(eps_fg, sig_fg, self.is_hybrid, self.radii, self.skin, mixing=self.mixing,
+                             group_comp=self.group_comp, shift=self.shift, precision=self.precision)
+
     def set_params(self, eps_fg, sig_fg, eps_cg, sig_cg):
         self.ctx.set_params(self._params(eps_fg, sig_fg, eps_cg, sig_cg))
 
@@ -113,17 +118,18 @@ class RelResPair:
 
 
 def _host(t):
-    return t.detach().to("cpu", dtype=torch.float64).numpy()
+    # a copy: the backward pass needs these values, whatever happens to the leaves until then
+    return t.detach().to("cpu", dtype=torch.float64).numpy().copy()
 
 
 class _RelResPairFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, owner, pos, eps_fg, sig_fg, eps_cg, sig_cg):
-        params = [_host(t) for t in (eps_fg, sig_fg, eps_cg, sig_cg)]
-        owner.set_params(*params)
+        params = owner._params(*[_host(t) for t in (eps_fg, sig_fg, eps_cg, sig_cg)])
+        owner.ctx.set_params(params)
         pos = pos.detach().contiguous()
         f = torch.empty_like(pos)
-        e = torch.zeros(4, dtype=torch.float64, device=pos.device)
+        e = torch.empty(4, dtype=torch.float64, device=pos.device)
         owner.ctx.compute(pos, f, e)
         ctx.owner = owner
         ctx.params = params
@@ -136,7 +142,7 @@ class _RelResPairFn(torch.autograd.Function):
     def backward(ctx, g_energy, g_forces):
         (pos,) = ctx.saved_tensors
         owner = ctx.owner
-        owner.set_params(*ctx.params)
+        owner.ctx.set_params(ctx.params)
         ge = 0.0 if g_energy is None else float(g_energy)
         gf = None if g_forces is None else g_forces.detach().to(torch.float64).contiguous()
         gx = torch.empty_like(pos)
@@ -152,15 +158,14 @@ class _RelResPairEq13Fn(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, owner, pos, eps_fg, sig_fg):
-        ef, sf = _host(eps_fg), _host(sig_fg)
-        ec, sc = owner.cg_from_fg(ef, sf)
-        owner.set_params(ef, sf, ec, sc)
+        params = owner._params_eq13(_host(eps_fg), _host(sig_fg))
+        owner.ctx.set_params(params)
         pos = pos.detach().contiguous()
         f = torch.empty_like(pos)
-        e = torch.zeros(4, dtype=torch.float64, device=pos.device)
+        e = torch.empty(4, dtype=torch.float64, device=pos.device)
         owner.ctx.compute(pos, f, e)
         ctx.owner = owner
-        ctx.params = [ef, sf, ec, sc]
+        ctx.params = params
         ctx.save_for_backward(pos)
         ctx.param_meta = [(t.dtype, t.device, t.shape) for t in (eps_fg, sig_fg)]
         return e[3], f
@@ -169,15 +174,12 @@ class _RelResPairEq13Fn(torch.autograd.Function):
     def backward(ctx, g_energy, g_forces):
         (pos,) = ctx.saved_tensors
         owner = ctx.owner
-        ef, sf, ec, sc = ctx.params
-        owner.set_params(ef, sf, ec, sc)
+        owner.ctx.set_params(ctx.params)
         ge = 0.0 if g_energy is None else float(g_energy)
         gf = None if g_forces is None else g_forces.detach().to(torch.float64).contiguous()
         gx = torch.empty_like(pos)
         out = owner.ctx.backward(pos, gf, ge, gx)
-        p = R.make_params(ef, sf, owner.is_hybrid, owner.radii, owner.skin, mixing=owner.mixing,
-                          group_comp=owner.group_comp, shift=owner.shift, precision=owner.precision)
-        d_eps, d_sig = R.relres_chain_cg_grads(p, out["eps_cg"], out["sig_cg"], out["eps_fg"], out["sig_fg"])
+        d_eps, d_sig = R.relres_chain_cg_grads(ctx.params, out["eps_cg"], out["sig_cg"], out["eps_fg"], out["sig_fg"])
         grads = [torch.as_tensor(g.reshape(shape), dtype=dtype, device=device)
                  for g, (dtype, device, shape) in zip((d_eps, d_sig), ctx.param_meta)]
         return (None, gx, *grads)
