@@ -78,35 +78,32 @@ __device__ __forceinline__ double poly4(const double* g, double d) {
 }
 
 // Eq. 20 as the sum of its FG and CG parts (see PairTab); returns -u'(r)/r
-// in *fr and u(r) in *u.
+// in *fr and u(r) in *u.  Reciprocals as in the FP64 pair launches (rcp_d,
+// rsqrt_d); a pair is inside at most one region of each part.
 __device__ __forceinline__ void relres_pair(const PairTab<double>& T, double r2, double* fr, double* u) {
   double f = 0.0, e = 0.0;
-  if (r2 < T.rsp2) {  // FG part
-    if (r2 < T.rsm2) {
-      const double r2i = 1.0 / r2, r6i = r2i * r2i * r2i;
-      f += r6i * (T.f12f * r6i - T.f6f) * r2i;
-      e += r6i * (T.c12f * r6i - T.c6f) - T.e_fg_shift;
+  const float r2f = float(r2);
+  const bool fg = r2 < T.rsp2, cg = r2 < T.rcp2;  // CG: zero table entries for pairs without it
+  const bool core = r2 < T.rsm2, lj = cg && !fg && r2 < T.rcm2;
+  if (core || lj) {  // Lennard-Jones, FG below r_s- or CG between the shells
+    const double r2i = rcp_d(r2, r2f), r6i = r2i * r2i * r2i;
+    f = r6i * ((core ? T.f12f : T.f12c) * r6i - (core ? T.f6f : T.f6c)) * r2i;
+    e = r6i * ((core ? T.c12f : T.c12c) * r6i - (core ? T.c6f : T.c6c)) - (core ? T.e_fg_shift : T.gam_cm);
+    if (core && cg) e += T.e_cg_close;
+  } else if (fg || cg) {  // a smoothing shell: both parts at r_s, CG at r_c
+    const double ri = rsqrt_d(r2, r2f), r = r2 * ri;
+    if (fg) {
+      const double d = r - T.rsm, d2 = d * d;
+      f = -poly4(T.fgd, d) * ri;
+      e = poly5(T.fg, d) - T.e_fg_shift;
+      if (cg) {
+        f -= d2 * (T.ond4 * d + T.ond3) * ri;
+        e += T.on0 + d2 * d * (T.on4 * d + T.on3) - T.gam_cm;
+      }
     } else {
-      const double r = sqrt(r2), d = r - T.rsm;
-      f += -poly4(T.fgd, d) / r;
-      e += poly5(T.fg, d) - T.e_fg_shift;
-    }
-  }
-  if (r2 < T.rcp2) {  // CG part (zero table entries for pairs without CG)
-    if (r2 < T.rsm2) {
-      e += T.e_cg_close;
-    } else if (r2 < T.rsp2) {
-      const double r = sqrt(r2), d = r - T.rsm, d2 = d * d;
-      f += -(d2 * (T.ond4 * d + T.ond3)) / r;
-      e += T.on0 + d2 * d * (T.on4 * d + T.on3) - T.gam_cm;
-    } else if (r2 < T.rcm2) {
-      const double r2i = 1.0 / r2, r6i = r2i * r2i * r2i;
-      f += r6i * (T.f12c * r6i - T.f6c) * r2i;
-      e += r6i * (T.c12c * r6i - T.c6c) - T.gam_cm;
-    } else {
-      const double r = sqrt(r2), d = r - T.rcm;
-      f += -poly4(T.cgod, d) / r;
-      e += poly5(T.cgo, d) - T.gam_cm;
+      const double d = r - T.rcm;
+      f = -poly4(T.cgod, d) * ri;
+      e = poly5(T.cgo, d) - T.gam_cm;
     }
   }
   *fr = f;
@@ -151,10 +148,35 @@ __device__ __forceinline__ double min_image(double d, double l, double il) {
   return fma(-l, t - 6755399441055744.0, d);
 }
 
+// one thread's sums: force, then energy and virial
+constexpr int kSums = 3 + kNQ;
 struct StaticSums {
-  double f[3] = {0.0, 0.0, 0.0};
-  double q[kNQ] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  double v[kSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
 };
+
+// The sums over a warp, each left in one pair of lanes: at every level a lane
+// passes on the half of its values that its partner keeps (12 FP64 additions a
+// lane; ten butterflies take 50).  Returns this lane's value, its index in k
+// (-1: none).
+__device__ __forceinline__ double warp_sums(const StaticSums& S, int lane, int& k) {
+  static_assert(kSums == 10, "split as 5 + 5, 3 + 2, 2 + 1, 1 + 1");
+  const bool a = lane & 16, b = lane & 8, c = lane & 4, d = lane & 2;
+  double x[6], y[4], z[2];
+#pragma unroll
+  for (int q = 0; q < 5; ++q)
+    x[q] = (a ? S.v[q + 5] : S.v[q]) + __shfl_xor_sync(0xffffffffu, a ? S.v[q] : S.v[q + 5], 16);
+  x[5] = 0.0;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) y[q] = (b ? x[q + 3] : x[q]) + __shfl_xor_sync(0xffffffffu, b ? x[q] : x[q + 3], 8);
+  y[3] = 0.0;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) z[q] = (c ? y[q + 2] : y[q]) + __shfl_xor_sync(0xffffffffu, c ? y[q] : y[q + 2], 4);
+  double t = (d ? z[1] : z[0]) + __shfl_xor_sync(0xffffffffu, d ? z[0] : z[1], 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  const int in = 2 * int(c) + int(d);
+  k = in < (b ? 2 : 3) ? 5 * int(a) + 3 * int(b) + in : -1;
+  return t;
+}
 
 // One queued pair (i, j): excluded partners are skipped here, where few
 // candidates are left.
@@ -169,40 +191,43 @@ __device__ __forceinline__ void static_pair(const double* __restrict__ pos, cons
   double fr, u;
   relres_pair(tab[ti * nt + type[j]], dx * dx + dy * dy + dz * dz, &fr, &u);
   const double fx = fr * dx, fy = fr * dy, fz = fr * dz;
-  S.f[0] += fx;
-  S.f[1] += fy;
-  S.f[2] += fz;
-  S.q[0] += u;
-  S.q[1] += fx * dx;
-  S.q[2] += fy * dy;
-  S.q[3] += fz * dz;
-  S.q[4] += fx * dy;
-  S.q[5] += fx * dz;
-  S.q[6] += fy * dz;
+  S.v[0] += fx;
+  S.v[1] += fy;
+  S.v[2] += fz;
+  S.v[3] += u;
+  S.v[4] += fx * dx;
+  S.v[5] += fy * dy;
+  S.v[6] += fz * dz;
+  S.v[7] += fx * dy;
+  S.v[8] += fx * dz;
+  S.v[9] += fy * dz;
 }
 
 // One warp per atom.  The FP32 test of a partner is ~20 instructions (n^2 of
 // them: the floor of large n); the FP64 evaluation of the few percent that
 // pass runs with full lanes from the queue, at the FP64 rate (1.66 FMA per
 // clock and SM).  Against one thread per atom evaluating every partner in
-// FP64: 18.5 -> 0.14 ms per call at 3993 propane-like atoms, where 16 blocks
+// FP64: 18.5 -> 0.094 ms per call at 3993 propane-like atoms, where 16 blocks
 // of 256 had left most SMs without work and 95 % of the FP64 arithmetic went
-// to pairs out of range.
+// to pairs out of range (0.14 ms, and 0.76 against 0.43 ms at 14 739 atoms,
+// without the four partners in flight, the refined reciprocals and the split
+// sums; held to 80 registers the loop is not unrolled: 0.20 and 1.5 ms).
 __global__ void __launch_bounds__(kStaticThreads)
     k_allpairs_static(int n, int nt, const double* __restrict__ pos, const int* __restrict__ type, double l0,
                       double l1, double l2, const int* __restrict__ eoff, const int* __restrict__ eidx, int with_excl,
                       StaticReach reach, double* __restrict__ forces, StaticScratch* scratch) {
-  constexpr int kWarps = kStaticThreads / 32;
+  constexpr int kWarps = kStaticThreads / 32, kUnroll = 4;
   __shared__ float s_reach[kWarps][kCodes];
-  __shared__ int s_queue[kWarps][64];
-  __shared__ double s_sum[kWarps * kNQ];
+  __shared__ int s_queue[kWarps][32 + 32 * kUnroll];
+  __shared__ double s_sum[kWarps][kNQ];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = blockIdx.x * kWarps + w;
   StaticSums S;
+  bool bad_i = false;
   if (i < n) {
     const float4 ai = scratch->atom[i];
     const int ci = __float_as_int(ai.w);
-    const bool bad_i = ci == kCodeBadType;
+    bad_i = ci == kCodeBadType;
     if (!bad_i) {
       const int ti = type[i];
       if (lane < kCodes) {
@@ -218,40 +243,54 @@ __global__ void __launch_bounds__(kStaticThreads)
       const int e0 = with_excl ? eoff[i] : 0, e1 = with_excl ? eoff[i + 1] : 0;
       const float fl0 = float(l0), fl1 = float(l1), fl2 = float(l2);
       int waiting = 0;
-      for (int base = 0; base < n; base += 32) {
-        const int j = base + lane;
-        bool near = false;
-        if (j < n && j != i) {
-          const float4 aj = scratch->atom[j];
-          const float dx = nearest(ai.x, aj.x, fl0), dy = nearest(ai.y, aj.y, fl1), dz = nearest(ai.z, aj.z, fl2);
-          near = dx * dx + dy * dy + dz * dz < s_reach[w][__float_as_int(aj.w)];
+      float4 next[kUnroll];  // four partners a lane in flight
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) next[u] = scratch->atom[min(32 * u + lane, n - 1)];
+      for (int base = 0; base < n; base += 32 * kUnroll) {
+        float4 at[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+          at[u] = next[u];
+          next[u] = scratch->atom[min(base + 32 * (kUnroll + u) + lane, n - 1)];
         }
-        const unsigned b = __ballot_sync(0xffffffffu, near);
-        if (b == 0u) continue;
-        if (near) s_queue[w][waiting + __popc(b & ((1u << lane) - 1u))] = j;
-        waiting += __popc(b);
+        bool near[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+          const int j = base + 32 * u + lane;
+          const float dx = nearest(ai.x, at[u].x, fl0), dy = nearest(ai.y, at[u].y, fl1),
+                      dz = nearest(ai.z, at[u].z, fl2);
+          near[u] = j < n && j != i && dx * dx + dy * dy + dz * dz < s_reach[w][__float_as_int(at[u].w)];
+        }
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+          const unsigned b = __ballot_sync(0xffffffffu, near[u]);
+          if (near[u]) s_queue[w][waiting + __popc(b & ((1u << lane) - 1u))] = base + 32 * u + lane;
+          waiting += __popc(b);
+        }
         __syncwarp();
-        if (waiting >= 32) {
+        while (waiting >= 32) {
           waiting -= 32;
-          const int jq = s_queue[w][waiting + lane];
-          __syncwarp();
-          static_pair(pos, type, xi, yi, zi, ti, nt, jq, l0, l1, l2, il0, il1, il2, eidx, e0, e1, scratch->tab, S);
+          static_pair(pos, type, xi, yi, zi, ti, nt, s_queue[w][waiting + lane], l0, l1, l2, il0, il1, il2, eidx, e0, e1,
+                      scratch->tab, S);
         }
+        __syncwarp();
       }
       if (lane < waiting)
         static_pair(pos, type, xi, yi, zi, ti, nt, s_queue[w][lane], l0, l1, l2, il0, il1, il2, eidx, e0, e1,
                     scratch->tab, S);
     }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) S.f[q] = warp_sum(S.f[q]);
-    if (lane < 3)
-      forces[3 * i + lane] =
-          bad_i ? __longlong_as_double(0x7ff8000000000000LL) : (lane == 0 ? S.f[0] : (lane == 1 ? S.f[1] : S.f[2]));
   }
-  block_sum<double, kNQ>(S.q, s_sum);
-  if (threadIdx.x == 0)
+  int k;
+  const double t = warp_sums(S, lane, k);
+  if (k >= 0 && k < 3 && i < n) forces[3 * i + k] = bad_i ? __longlong_as_double(0x7ff8000000000000LL) : t;
+  if (k >= 3) s_sum[w][k - 3] = t;
+  __syncthreads();
+  if (threadIdx.x < kNQ) {
+    double v = 0.0;
 #pragma unroll
-    for (int q = 0; q < kNQ; ++q) scratch->partial[q][blockIdx.x] = 0.5 * S.q[q];
+    for (int q = 0; q < kWarps; ++q) v += s_sum[q][threadIdx.x];
+    scratch->partial[threadIdx.x][blockIdx.x] = 0.5 * v;
+  }
 }
 
 // Block q sums the q-th of the energy and virial partial sums (fixed order).
