@@ -906,8 +906,11 @@ __device__ __forceinline__ void drift_seg_block(const DriftSegArgs<R>& a, int bi
 #pragma unroll
     for (int q = 0; q < 3; ++q) sx[3 * threadIdx.x + q] = x[q];
   }
-  if (__syncthreads_or(rebuild) && threadIdx.x == 0) atomicOr(&a.d.st->flags, F_REBUILD);
-  if (__syncthreads_or(reprune) && threadIdx.x == 0) atomicOr(&a.d.st->flags, F_PRUNE);
+  if (__any_sync(0xffffffffu, rebuild || reprune)) {
+    const unsigned f = (__any_sync(0xffffffffu, rebuild) ? F_REBUILD : 0u) | (__any_sync(0xffffffffu, reprune) ? F_PRUNE : 0u);
+    if ((threadIdx.x & 31) == 0) atomicOr(&a.d.st->flags, f);
+  }
+  __syncthreads();
   // bonded terms of the segment from the new positions (the records name the
   // prototype's atoms, base .. base + a1 - a0 - 1: the same local indices)
   const SPos xs{sx, base};
@@ -1017,22 +1020,30 @@ __device__ void csvr_draws(double n_f, unsigned long long seed, unsigned long lo
   r1 = gauss(seed, c);
   s = 2.0 * gamma_mt(0.5 * (n_f - 1.0), seed, c);
 }
-// e = exp(-dt / tau), computed once per call on the host
-__device__ double csvr_alpha(double ke, double e, double n_f, double kt, double r1, double s) {
-  const double kn = ke + (1.0 - e) * (kt / n_f * (r1 * r1 + s) - ke) +
-                    2.0 * r1 * sqrt(e * (1.0 - e) * ke * kt / n_f);
-  return sqrt(kn / ke);
+// With e = exp(-dt / tau) (computed once per call on the host) the rescaled
+// kinetic energy is K' = e K + A + B sqrt(K), where A and B hold the random
+// numbers and the target; they are formed with the draws, so the end of a step
+// (one thread, on the critical path of every step) is left with alpha = sqrt(K' / K) = sqrt(e + (A / sqrt K + B) / sqrt K).
+__device__ __forceinline__ double csvr_alpha(double ke, double e, double ca, double cb) {
+  const float kf = float(ke);
+  if (kf > 1e-30f && kf < 1e30f) {
+    const double rk = rsqrt_d(ke, kf);
+    const double x = fma(fma(ca, rk, cb), rk, e);
+    if (x > 1e-30) return x * rsqrt_d(x, float(x));
+    return sqrt(x);
+  }
+  return sqrt(e + (ca + cb * sqrt(ke)) / ke);
 }
 
-// Draws for the steps st->step + k, k < count (one thread each).
-__global__ void k_csvr_draws(double n_f, unsigned long long seed, int count, const DevState* st,
+// (A, B) of the steps st->step + k, k < count (one thread each).
+__global__ void k_csvr_draws(double n_f, double kt, double e, unsigned long long seed, int count, const DevState* st,
                              double* draws) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   double r1, s;
   csvr_draws(n_f, seed, st->step + (unsigned long long)k, r1, s);
-  draws[2 * k] = r1;
-  draws[2 * k + 1] = s;
+  draws[2 * k] = (1.0 - e) * (kt / n_f) * (r1 * r1 + s);
+  draws[2 * k + 1] = 2.0 * r1 * sqrt(e * (1.0 - e) * (kt / n_f));
 }
 
 // total of an accumulator and the finer one beside it
@@ -1042,13 +1053,13 @@ __device__ __forceinline__ double acc_value(long long hi, long long fine) {
 
 // End of a step (one thread): thermostat factor from the kinetic energy,
 // thermo row on energy steps, counters, and the accumulators cleared for the
-// next step.  `draw` points at this step's (r1, s).  The accumulators are read
+// next step.  ca, cb: this step's thermostat terms (k_csvr_draws).  The accumulators are read
 // through volatile loads (other blocks of the calling kernel added to them).
-__device__ void end_of_step(volatile long long* acc, const StepParams& sp, DevState* st, double r1, double s) {
+__device__ void end_of_step(volatile long long* acc, const StepParams& sp, DevState* st, double ca, double cb) {
   const bool ev = st->ev != 0;
   const double ke = double(acc[kAccKe]) / kFix;
   double alpha = 1.0;
-  if (sp.t_target > 0.0 && ke > 0.0) alpha = csvr_alpha(ke, sp.csvr_e, sp.n_f, sp.kt, r1, s);
+  if (sp.t_target > 0.0 && ke > 0.0) alpha = csvr_alpha(ke, sp.csvr_e, ca, cb);
   st->alpha = alpha;
   st->a = alpha;
   st->b = alpha + 1.0;
@@ -1168,10 +1179,10 @@ __device__ __forceinline__ R sum_atom(const SumArgs<R>& a, int i, SumIn<R>& in, 
 template <typename R>
 __device__ __forceinline__ void sum_block(const SumArgs<R>& a, int bid, int nblk, int k) {
   // this step's thermostat draws, read early (the last block uses them)
-  double r1 = 0.0, rs = 0.0;
+  double ca = 0.0, cb = 0.0;
   if (threadIdx.x == 0 && a.sp.t_target > 0.0) {
-    r1 = a.draw[2 * k];
-    rs = a.draw[2 * k + 1];
+    ca = a.draw[2 * k];
+    cb = a.draw[2 * k + 1];
   }
   // launched as a programmatic dependent of the pair kernel: wait for its
   // forces, then let the next drift launch (its early loads read nothing that
@@ -1195,7 +1206,7 @@ __device__ __forceinline__ void sum_block(const SumArgs<R>& a, int bid, int nblk
     sum_load(a, i, in);
     ke += sum_atom(a, i, in, bad);
   }
-  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&a.st->flags, F_NONFINITE);
+  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&a.st->flags, F_NONFINITE);
   double v[1] = {double(ke)};
   __shared__ double sh_k[kThreads / 32];
   block_sum<double, 1>(v, sh_k);
@@ -1206,7 +1217,7 @@ __device__ __forceinline__ void sum_block(const SumArgs<R>& a, int bid, int nblk
     if (ticket == unsigned(nblk - 1)) {
       __threadfence();
       a.st->done_blocks = 0u;
-      end_of_step(a.acc, a.sp, a.st, r1, rs);
+      end_of_step(a.acc, a.sp, a.st, ca, cb);
     }
   }
 }
@@ -1526,7 +1537,8 @@ cudaError_t launch_reduce_out(relres_ctx* c, double* d_energy, double* d_virial)
 
 cudaError_t launch_csvr_draws(relres_ctx* c, const StepParams& sp, int count) {
   if (!(sp.t_target > 0.0) || count <= 0) return cudaSuccess;
-  k_csvr_draws<<<(count + 127) / 128, 128, 0, c->stream>>>(sp.n_f, sp.seed, count, c->d_state, c->d_draws);
+  k_csvr_draws<<<(count + 127) / 128, 128, 0, c->stream>>>(sp.n_f, sp.kt, sp.csvr_e, sp.seed, count,
+                                                                c->d_state, c->d_draws);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
