@@ -1084,12 +1084,7 @@ static relres_status record_pairs(relres_ctx* c, bool ev, bool graph, cudaGraphC
 static relres_status record_block(relres_ctx* c, const StepParams& sp, double* d_vel, int blk, int done,
                                   bool graph) {
   const unsigned* gate = &c->d_state->flags;
-  const size_t xb = sizeof(unsigned long long) * 3 * size_t(c->n), vb = sizeof(double) * 3 * size_t(c->n);
-  CK(cudaMemcpyAsync(c->d_snap_x, c->d_xfx, xb, cudaMemcpyDeviceToDevice, c->stream));
-  CK(cudaMemcpyAsync(c->d_snap_v, vel_state(c, d_vel), vb, cudaMemcpyDeviceToDevice, c->stream));
-  CK(cudaMemcpyAsync(c->d_snap_f, c->d_f_tot, force_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
-  CK(cudaMemcpyAsync(c->d_snap_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToDevice, c->stream));
-  CK(launch_csvr_draws(c, sp, blk));
+  CK(launch_block_start(c, sp, d_vel, blk));
   for (int k = 0; k < blk; ++k) {
     c->cur_step = done + k;
     // energy steps are known here: the device sets DevState::ev by the same rule
@@ -1385,7 +1380,6 @@ static relres_status step_begin(relres_ctx* c, int n_steps, double dt_fs, double
   relres_status s = RELRES_OK;
   if (cached) {
     const bool try_u = !c->fp64 && dt_fs == c->io_dt;
-    CK(launch_flags_and(c, ~(unsigned)(F_DIRTY | F_VDIRTY)));
     CK(launch_check_io(c, d_pos, try_u ? d_vel : nullptr));
     s = read_state(c);
     if (s != RELRES_OK) return s;
@@ -1408,12 +1402,14 @@ static relres_status step_begin(relres_ctx* c, int n_steps, double dt_fs, double
     fresh = true;
   }
   CK(upload_type_consts(c, dt_fs));
-  CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAccAll, c->stream));
   // Everything that follows runs on the context stream, after these launches.
   // Without a force evaluation above, the state read at the start is still
   // current for the block accounting (the set-up above changes no count), so
-  // no further round trip is needed; after one, read it again.
-  return fresh ? read_state(c) : RELRES_OK;
+  // no further round trip is needed; after one, clear what it left in the
+  // accumulators (launch_call_start cleared them before) and read it again.
+  if (!fresh) return RELRES_OK;
+  CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAccAll, c->stream));
+  return read_state(c);
 }
 
 // After a block has run: status, timing and launch accounting; on a list
@@ -1526,7 +1522,7 @@ struct relres_batch {
   int mode = -1;                 // relres_batch_set_mode
   std::vector<int> shared;       // replicas in the shared launches of the captured graph
   std::vector<char> is_shared;   // [nrep]
-  BatchLaunch bl_pair, bl_pair_ev, bl_drift, bl_sum;
+  BatchLaunch bl_start, bl_pair, bl_pair_ev, bl_drift, bl_sum;
   RebuildBatch rebuild;
   DevState** d_states = nullptr;  // [nrep]
 };
@@ -1609,8 +1605,8 @@ static void batch_drop_graph(relres_batch* b) {
 }
 
 // The shared-launch part of one block of steps, captured on the batch stream
-// (tables uploaded beforehand): per replica the rollback snapshot and the
-// thermostat draws, then per step the batched drift, the work list of
+// (tables uploaded beforehand): the batched block start (rollback snapshots
+// and thermostat draws), then per step the batched drift, the work list of
 // replicas whose trigger fired with one conditional node holding the six
 // batched rebuild kernels, the batched pair kernel and the batched force sum.
 static relres_status capture_shared(relres_batch* b, const std::vector<relres_ctx*>& cs,
@@ -1620,23 +1616,7 @@ static relres_status capture_shared(relres_batch* b, const std::vector<relres_ct
   const bool fp64 = cs[0]->fp64;
   const int acc = cs[0]->force_acc;
   cudaError_t e = cudaSuccess;
-  for (int q = 0; q < ns && e == cudaSuccess; ++q) {
-    relres_ctx* c = cs[q];
-    const size_t xb = sizeof(unsigned long long) * 3 * size_t(c->n), vb = sizeof(double) * 3 * size_t(c->n);
-    e = cudaMemcpyAsync(c->d_snap_x, c->d_xfx, xb, cudaMemcpyDeviceToDevice, b->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_snap_v, vel_state(c, vel[q]), vb, cudaMemcpyDeviceToDevice, b->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_snap_f, c->d_f_tot, force_bytes(c), cudaMemcpyDeviceToDevice, b->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(c->d_snap_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToDevice, b->stream);
-    if (e == cudaSuccess) {
-      const cudaStream_t own = c->stream;
-      const long long n0 = c->n_launches;  // counted per executed block in k_parent
-      c->stream = b->stream;
-      e = launch_csvr_draws(c, sp[q], blk);
-      c->stream = own;
-      c->n_launches = n0;
-    }
-  }
+  e = launch_block_start_batch(b->stream, b->bl_start, ns);
   relres_status s = RELRES_OK;
   for (int k = 0; k < blk && e == cudaSuccess && s == RELRES_OK; ++k) {
     const bool ev_step = sp[0].thermo_every > 0 && ((done + k + 1) % sp[0].thermo_every) == 0;
@@ -1695,6 +1675,7 @@ static relres_status batch_graph(relres_batch* b, const std::vector<StepParams>&
   cudaError_t e = cudaSuccess;
   if (ns > 0) {
     e = prepare_pairs_batch(cs, &b->bl_pair, &b->bl_pair_ev);
+    if (e == cudaSuccess) e = prepare_block_start_batch(cs, ssp, svel.data(), blk, &b->bl_start);
     if (e == cudaSuccess) e = prepare_drift_batch(cs, ssp, svel.data(), &b->bl_drift);
     if (e == cudaSuccess) e = prepare_sum_batch(cs, ssp, svel.data(), &b->bl_sum);
     if (e == cudaSuccess) e = prepare_rebuild_batch(cs, &b->rebuild);
@@ -1743,8 +1724,9 @@ static relres_status batch_graph(relres_batch* b, const std::vector<StepParams>&
   }
   if (ns > 0 && s == RELRES_OK && e == cudaSuccess) {
     s = capture_shared(b, cs, ssp, svel, blk, done);
-    // every shared replica takes part in the step's drift, work-list, pair and force-sum launches
-    for (int q = 0; q < ns; ++q) b->k_parent[shared[q]] = 4LL * blk + (ssp[q].t_target > 0.0 ? 1 : 0);
+    // every shared replica takes part in the block's start and the steps' drift, work-list, pair and force-sum
+    // launches
+    for (int q = 0; q < ns; ++q) b->k_parent[shared[q]] = 4LL * blk + 1;
   }
   for (int r : joins)
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_join[r], 0);
@@ -1902,6 +1884,7 @@ void relres_batch_destroy(relres_batch* b) {
   batch_drop_graph(b);
   free_batch(&b->bl_pair);
   free_batch(&b->bl_pair_ev);
+  free_batch(&b->bl_start);
   free_batch(&b->bl_drift);
   free_batch(&b->bl_sum);
   free_rebuild_batch(&b->rebuild);

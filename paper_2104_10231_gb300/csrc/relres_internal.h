@@ -486,7 +486,8 @@ cudaError_t launch_drift(relres_ctx* c, const StepParams& sp, double* d_vel, boo
 // bookkeeping (k_sum with the thermostat in its last block, or the
 // finish + k_thermo pair where there are no segments)
 cudaError_t launch_end_of_step(relres_ctx* c, const StepParams& sp, int k, bool ev, double* d_vel);
-cudaError_t launch_csvr_draws(relres_ctx* c, const StepParams& sp, int count);
+// start of a block of `count` steps: rollback snapshot and thermostat draws
+cudaError_t launch_block_start(relres_ctx* c, const StepParams& sp, double* d_vel, int count);
 cudaError_t launch_thermo(relres_ctx* c, const StepParams& sp, int k);
 cudaError_t launch_call_start(relres_ctx* c, bool reset_ab);
 // FP32 path: caller's velocities -> the float-float state (start of a call)
@@ -521,6 +522,9 @@ cudaError_t upload_batch(BatchLaunch* b, const void* args, size_t bytes, const s
 void free_batch(BatchLaunch* b);
 cudaError_t prepare_pairs_batch(const std::vector<relres_ctx*>& cs, BatchLaunch* b, BatchLaunch* b_ev);
 cudaError_t launch_pairs_batch(cudaStream_t s, bool fp64, int acc, bool ev, const BatchLaunch& b, int nrep);
+cudaError_t prepare_block_start_batch(const std::vector<relres_ctx*>& cs, const std::vector<StepParams>& sp,
+                                      double* const* d_vel, int count, BatchLaunch* b);
+cudaError_t launch_block_start_batch(cudaStream_t s, const BatchLaunch& b, int nrep);
 cudaError_t prepare_drift_batch(const std::vector<relres_ctx*>& cs, const std::vector<StepParams>& sp,
                                 double* const* d_vel, BatchLaunch* b);
 cudaError_t launch_drift_batch(cudaStream_t s, bool fp64, bool ev, const BatchLaunch& b, int nrep);
