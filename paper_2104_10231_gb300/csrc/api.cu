@@ -1951,7 +1951,7 @@ relres_status relres_get_stats(relres_ctx* c, relres_stats* o) {
   std::memset(o, 0, sizeof(*o));
   o->n_atoms = c->n;
   o->n_hybrid = c->n_h;
-  o->pair_tpa = c->fp64 ? fp64_lanes(c) : kPairConfigs[c->pair_cfg].tpa;
+  o->pair_tpa = c->fp64 ? std::min(8, fp64_lanes(c, false)) : kPairConfigs[c->pair_cfg].tpa;
   o->pair_block = c->fp64 ? kFp64Block : kPairConfigs[c->pair_cfg].bs;
   o->cap_fg = c->cap_fg;
   o->cap_cg = c->cap_cg;

@@ -12,8 +12,10 @@
 // evaluate 32 of them at a time, nearly always of one region, ~22 FP64
 // instructions each.  Against one thread per list entry by entry, and eight
 // per slot with the pruning as a pass of its own below 20 000 slots: 200 ->
-// 163 us per step at 25 000 neopentane-like atoms, 65 -> 44 us at 648
-// propane-like ones (185 -> 16 us the launch with energies).  The potential is C2 at the region limits, so a pair that
+// 119 us per step at 25 000 neopentane-like atoms, 65 -> 30 us at 648
+// propane-like ones (a launch with energies 185 -> 12 us).  What is left
+// there is the FP64 rate, then the latency of one warp's rounds: fetching the
+// partners of the next pass ahead, or two chains per sum, gave 0 to 1 %.  The potential is C2 at the region limits, so a pair that
 // FP32 puts on the other side of one (1e-7 of r^2) changes nothing above 1e-13.
 //
 // The terms of a slot are stored by their rank in its list and added in list
@@ -335,22 +337,41 @@ static int make_launch64(const relres_ctx* c, int which, int per, bool prune, La
   return a.nblk_cg + (do_fg ? (c->n + per - 1) / per : 0);
 }
 
+// F<EV, T>(...) for the threads per slot of a launch
+#define RELRES_LANES64(F, ...)             \
+  if (ev) {                                \
+    if (lanes == 32)                       \
+      F<true, 32>(__VA_ARGS__);            \
+    else if (lanes == 16)                  \
+      F<true, 16>(__VA_ARGS__);            \
+    else                                   \
+      F<true, 4>(__VA_ARGS__);             \
+  } else if (lanes == 32) {                \
+    F<false, 32>(__VA_ARGS__);             \
+  } else if (lanes == 16) {                \
+    F<false, 16>(__VA_ARGS__);             \
+  } else if (lanes == 8) {                 \
+    F<false, 8>(__VA_ARGS__);              \
+  } else {                                 \
+    F<false, 4>(__VA_ARGS__);              \
+  }
+
+template <bool EV, int T>
+static void launch64(cudaStream_t s, const Launch64& a, int grid) {
+  k_pair64<EV, T><<<grid, kFp64Block, smem64<EV>(a.nt), s>>>(a);
+}
+template <bool EV, int T>
+static void launch64_batch(cudaStream_t s, const BatchLaunch& b, int nrep) {
+  k_pair64_batch<EV, T>
+      <<<b.nblk, kFp64Block, smem64<EV>(b.nt), s>>>(static_cast<const Launch64*>(b.d_args), b.d_off, nrep);
+}
+
 cudaError_t launch_pairs_f64(relres_ctx* c, bool ev, int which) {
-  const int lanes = fp64_lanes(c);
+  const int lanes = fp64_lanes(c, ev);
   Launch64 a;
   const int grid = make_launch64(c, which, kFp64Block / lanes, pairs_prune(c), &a);
   if (grid == 0) return cudaSuccess;
-  const size_t smem = ev ? smem64<true>(a.nt) : smem64<false>(a.nt);
-  if (lanes == kFp64LanesSmall) {
-    if (ev)
-      k_pair64<true, kFp64LanesSmall><<<grid, kFp64Block, smem, c->stream>>>(a);
-    else
-      k_pair64<false, kFp64LanesSmall><<<grid, kFp64Block, smem, c->stream>>>(a);
-  } else if (ev) {
-    k_pair64<true, kFp64Lanes><<<grid, kFp64Block, smem, c->stream>>>(a);
-  } else {
-    k_pair64<false, kFp64Lanes><<<grid, kFp64Block, smem, c->stream>>>(a);
-  }
+  RELRES_LANES64(launch64, c->stream, a, grid)
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
@@ -359,34 +380,25 @@ cudaError_t launch_pairs_f64(relres_ctx* c, bool ev, int which) {
 cudaError_t prepare_pairs_batch_f64(const std::vector<relres_ctx*>& cs, BatchLaunch* b, BatchLaunch* b_ev) {
   long long slots = 0;
   for (const relres_ctx* c : cs) slots += pair_slots(c);
-  const int lanes = fp64_lanes_for(slots);
-  std::vector<Launch64> args(cs.size());
-  std::vector<int> off(cs.size() + 1, 0);
-  b->nt = 1;
-  for (size_t r = 0; r < cs.size(); ++r) {
-    off[r + 1] = off[r] + make_launch64(cs[r], 3, kFp64Block / lanes, cs[r]->prune_on, &args[r]);
-    b->nt = std::max(b->nt, cs[r]->n_types);
+  for (BatchLaunch* l : {b, b_ev}) {
+    l->lanes = fp64_lanes_for(slots, l == b_ev);
+    l->nt = 1;
+    std::vector<Launch64> args(cs.size());
+    std::vector<int> off(cs.size() + 1, 0);
+    for (size_t r = 0; r < cs.size(); ++r) {
+      off[r + 1] = off[r] + make_launch64(cs[r], 3, kFp64Block / l->lanes, cs[r]->prune_on, &args[r]);
+      l->nt = std::max(l->nt, cs[r]->n_types);
+    }
+    l->nblk = off.back();
+    const cudaError_t e = upload_batch(l, args.data(), sizeof(Launch64) * args.size(), off);
+    if (e != cudaSuccess) return e;
   }
-  b->nblk = b_ev->nblk = off.back();
-  b->lanes = b_ev->lanes = lanes;
-  b_ev->nt = b->nt;
-  const cudaError_t e = upload_batch(b, args.data(), sizeof(Launch64) * args.size(), off);
-  return e != cudaSuccess ? e : upload_batch(b_ev, args.data(), sizeof(Launch64) * args.size(), off);
+  return cudaSuccess;
 }
 
 void launch_pairs_batch_f64(cudaStream_t s, bool ev, const BatchLaunch& b, int nrep) {
-  const auto* args = static_cast<const Launch64*>(b.d_args);
-  const size_t smem = ev ? smem64<true>(b.nt) : smem64<false>(b.nt);
-  if (b.lanes == kFp64LanesSmall) {
-    if (ev)
-      k_pair64_batch<true, kFp64LanesSmall><<<b.nblk, kFp64Block, smem, s>>>(args, b.d_off, nrep);
-    else
-      k_pair64_batch<false, kFp64LanesSmall><<<b.nblk, kFp64Block, smem, s>>>(args, b.d_off, nrep);
-  } else if (ev) {
-    k_pair64_batch<true, kFp64Lanes><<<b.nblk, kFp64Block, smem, s>>>(args, b.d_off, nrep);
-  } else {
-    k_pair64_batch<false, kFp64Lanes><<<b.nblk, kFp64Block, smem, s>>>(args, b.d_off, nrep);
-  }
+  const int lanes = b.lanes;
+  RELRES_LANES64(launch64_batch, s, b, nrep)
 }
 
 }  // namespace relres

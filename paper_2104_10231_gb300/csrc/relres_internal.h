@@ -582,12 +582,21 @@ inline int fp32_lanes(const relres_ctx* c, bool ev) { return fp32_lanes_for(pair
 // FP64 pair launches (pair64.cu): threads per slot, and one warp per block (a
 // launch is a few blocks per SM long, and the last ones decide: 152.7 against
 // 163.1 us per step with 128-thread blocks at 25 000 neopentane-like atoms).
-// Eight threads per slot below four warps of them per SM; us per step there
-// and above with 16 / 8 / 4 / 2 threads: 10 000 atoms - / 87 / - / -, 20 000
-// atoms 158 / - / 117 / 134, 40 000 atoms 244 / - / 202 / 211.
-constexpr int kFp64LanesSmall = 8, kFp64Lanes = 4, kFp64Block = 32;
-inline int fp64_lanes_for(long long slots) { return slots < 4LL * 32 * kPartSMs ? kFp64LanesSmall : kFp64Lanes; }
-inline int fp64_lanes(const relres_ctx* c) { return fp64_lanes_for(pair_slots(c)); }
+// The fewer the slots, the more threads take one, so that every SM has a few
+// warps; us per step with 32 / 16 / 8 / 4 threads, forces only: 864 slots
+// 29.5 / 33.3 / 39.6 / -, 2058 slots 35.4 / 35.3 / 38.4 / -, 6000 slots 57 /
+// 49.4 / 48.0 / -, 12 000 slots 90 / 75 / 67 / -, 30 000 slots - / - / 134 /
+// 119; steps with energies, ten sums per slot instead of three: 864 slots 40 /
+// 45 / 59 / -, 2058 slots 45 / 47 / 56 / -, 6000 slots 70 / 64 / 69 / -,
+// 12 000 slots 109 / 93 / 103 / -, 30 000 slots - / - / 190 / 178.
+// The force bits are the same for all of them.
+constexpr int kFp64Block = 32;
+inline int fp64_lanes_for(long long slots, bool ev) {
+  if (slots < (ev ? 24 : 12) * kPartSMs) return 32;
+  if (slots < (ev ? 128 : 32) * kPartSMs) return 16;
+  return slots < 128 * kPartSMs ? 8 : 4;
+}
+inline int fp64_lanes(const relres_ctx* c, bool ev) { return fp64_lanes_for(pair_slots(c), ev); }
 
 // the lists the pair kernels walk: the pruned ones when pruning is on
 inline const int* walk_nbr_fg(const relres_ctx* c) { return c->prune_on ? c->d_nbr_fg_in : c->d_nbr_fg; }

@@ -141,3 +141,36 @@ def test_fp64_batch_keeps_the_bits_of_each_replica_alone(torch):
     batch.close()
     for c, _, _ in alone + both:
         c.close()
+
+
+def test_fp64_lanes_by_size_keep_the_bits(torch):
+    """32, 16 and 8 threads per slot alone (energy steps 32, 32 and 16), four in one batch."""
+    systems = [S.propane(), S.neopentane(n_mol=400, seed=41), S.neopentane(n_mol=1000, seed=42),
+               S.neopentane(n_mol=2000, seed=43)]
+
+    def run(batched):
+        ctxs, ps, vs, ths = [], [], [], []
+        for s in systems:
+            ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP64), R.topology_for(s))
+            ps.append(_dev(torch, s.pos))
+            vs.append(_dev(torch, s.vel))
+            ths.append(torch.zeros((6, R.RELRES_THERMO_COLS), dtype=torch.float64, device="cuda"))
+            ctx.build_neighbors(ps[-1], s.box)
+            ctxs.append(ctx)
+        if batched:
+            b = R.Batch(ctxs)
+            b.step(30, 1.0, ps, vs, [0.0] * 4, 100.0, [1] * 4, thermo_every=5, d_thermo=ths)
+            assert b.n_shared() == 4
+            b.close()
+        else:
+            for c, p, v, th in zip(ctxs, ps, vs, ths):
+                c.step(30, 1.0, p, v, thermo_every=5, d_thermo=th)
+        torch.cuda.synchronize()
+        for c in ctxs:
+            c.close()
+        return [[x.cpu().numpy() for x in (p, v, th)] for p, v, th in zip(ps, vs, ths)]
+
+    for (p0, v0, t0), (p1, v1, t1) in zip(run(False), run(True)):
+        assert np.array_equal(p0, p1) and np.array_equal(v0, v1)
+        # pair energies summed in groups of 32 / T slots and rounded to 2^-52 kcal/mol per group or better
+        assert np.abs(t0 - t1).max() <= 1e-12 * np.abs(t0).max()
