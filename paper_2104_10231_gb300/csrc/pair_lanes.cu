@@ -64,9 +64,11 @@ __device__ __forceinline__ void add_pair(const int4& d, float fr, const SmemTabs
   }
 }
 
-// Queued pairs of one warp: fewer than 32 wait between two rounds, and a round
-// adds at most four per lane.
-constexpr int kQueue = 32 + 4 * 32;
+// Queued pairs of one warp, of two classes: the plain Lennard-Jones range from
+// the front, the switching ranges from the back, so that the warps that
+// evaluate them run one range's arithmetic.  Fewer than 32 of a class wait
+// between two rounds, and a round adds at most four per lane.
+constexpr int kQueue = 2 * 31 + 4 * 32;
 struct PairQueue {
   int4 d[kQueue];   // coordinate differences and type-pair row
   float fr[kQueue]; // force factor
@@ -94,7 +96,7 @@ __device__ __forceinline__ void walk_lanes(const ListWalk& L, int blk, const Sme
   Acc A;
   int kept = 0;
   int4 buf = make_int4(ss, ss, ss, ss);
-  int waiting = 0;
+  int waiting = 0, waiting2 = 0;  // of the Lennard-Jones range, of the others
   if constexpr (EV) {
 #pragma unroll
     for (int k = 0; k < kNQ; ++k) tot->v[k][threadIdx.x] = 0;
@@ -164,15 +166,19 @@ __device__ __forceinline__ void walk_lanes(const ListWalk& L, int blk, const Sme
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int row = row0 + p[e].w;
-          const bool need = r2[e] < (CG ? S.row[row].cg.a.y : S.row[row].fg.a.y) && s < j[e];
-          const unsigned b = __ballot_sync(0xffffffffu, need);
+          const PairRow& R = S.row[row];
+          const bool need = r2[e] < (CG ? R.cg.a.y : R.fg.a.y) && s < j[e];
+          const bool lj = CG ? r2[e] >= R.cg.a.x && r2[e] < R.cg.a.w * R.cg.a.w : r2[e] < R.fg.b.x * R.fg.b.x;
+          const unsigned b = __ballot_sync(0xffffffffu, need && lj), b2 = __ballot_sync(0xffffffffu, need && !lj);
           if (need) {
-            const int k = waiting + __popc(b & ((1u << lane) - 1u));
+            const int k = lj ? waiting + __popc(b & ((1u << lane) - 1u))
+                             : kQueue - 1 - waiting2 - __popc(b2 & ((1u << lane) - 1u));
             Q.d[k] = make_int4(int(unsigned(pi.x) - unsigned(p[e].x)), int(unsigned(pi.y) - unsigned(p[e].y)),
                                int(unsigned(pi.z) - unsigned(p[e].z)), row);
             Q.fr[k] = fr[e];
           }
           waiting += __popc(b);
+          waiting2 += __popc(b2);
         }
       }
       jj = jn;
@@ -181,10 +187,15 @@ __device__ __forceinline__ void walk_lanes(const ListWalk& L, int blk, const Sme
       __syncwarp();
       PairQueue& Q = queue[threadIdx.x >> 5];
       const int least = r < rounds ? 32 : 1;
-      while (waiting >= least) {
-        const int take = min(waiting, 32);
-        waiting -= take;
-        if (lane < take) add_pair<CG>(Q.d[waiting + lane], Q.fr[waiting + lane], S, a, tot);
+      while (max(waiting, waiting2) >= least) {
+        const bool lj = waiting >= least;
+        const int left = lj ? waiting : waiting2, take = min(left, 32), at = left - take + lane;
+        if (lj)
+          waiting -= take;
+        else
+          waiting2 -= take;
+        const int k = lj ? at : kQueue - 1 - at;
+        if (lane < take) add_pair<CG>(Q.d[k], Q.fr[k], S, a, tot);
       }
       __syncwarp();
     }
@@ -275,15 +286,16 @@ __device__ __forceinline__ void lanes_block(const PairLaunch& a, int bid) {
   }
 }
 
-// energy steps: 80 registers a thread (six blocks per SM), forces only: 64
+// energy steps: 96 registers a thread (five blocks per SM; at six they spill, 7 %
+// slower at 20 000 atoms, at four 9 % slower), forces only: 64
 template <bool EV, int T, int ACC>
-__global__ void __launch_bounds__(kLaneThreads, EV ? 6 : 8) k_pair_lanes(PairLaunch a) {
+__global__ void __launch_bounds__(kLaneThreads, EV ? 5 : 8) k_pair_lanes(PairLaunch a) {
   grid_dependents_launch();  // as k_pair
   lanes_block<EV, T, ACC>(a, blockIdx.x);
 }
 
 template <bool EV, int T, int ACC>
-__global__ void __launch_bounds__(kLaneThreads, EV ? 6 : 8)
+__global__ void __launch_bounds__(kLaneThreads, EV ? 5 : 8)
     k_pair_lanes_batch(const PairLaunch* __restrict__ args, const int* __restrict__ off, int nrep) {
   const int r = batch_replica(off, nrep, blockIdx.x);
   lanes_block<EV, T, ACC>(args[r], int(blockIdx.x) - off[r]);
