@@ -282,9 +282,9 @@ __device__ __forceinline__ double angle_forces(const BondedArgs& B, const X& xfx
   dvec(xfx, an.x, an.y, sc, r1);
   dvec(xfx, an.z, an.y, sc, r2);
   const double q1 = dot3(r1, r1), q2 = dot3(r2, r2), qq = q1 * q2;
-  const double i12 = rsqrt_d(qq, float(qq));  // 1 / (|r1| |r2|)
+  const double i12 = rsqrt_d(qq, float(qq)), iqq = i12 * i12;  // 1 / (|r1| |r2|) and its square
   cross3(r1, r2, n);
-  const double nn = dot3(n, n) * (i12 * i12);  // sin^2 theta
+  const double nn = dot3(n, n) * iqq;  // sin^2 theta
   const double c = dot3(r1, r2) * i12;
   const double si = nn > 1e-12 ? rsqrt_d(nn, float(nn)) : 1e6;  // 1 / sin theta
   const double s = nn * si;
@@ -294,7 +294,7 @@ __device__ __forceinline__ double angle_forces(const BondedArgs& B, const X& xfx
   const double dth = (fabs(sd) <= 0.25 && cd > 0.0) ? asin_small(sd) : atan2(sd, cd);
   const double pref = 2.0 * k * dth * si;
   const double a12 = pref * i12, pc = pref * c;
-  const double b1 = pc * rcp_d(q1, float(q1)), b2 = pc * rcp_d(q2, float(q2));
+  const double pq = pc * iqq, b1 = pq * q2, b2 = pq * q1;  // pc / q1, pc / q2
 #pragma unroll
   for (int w = 0; w < 3; ++w) {
     f[0][w] = a12 * r2[w] - b1 * r1[w];

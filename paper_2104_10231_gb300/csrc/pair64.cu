@@ -12,16 +12,19 @@
 // evaluate 32 of them at a time, nearly always of one region, ~22 FP64
 // instructions each.  Against one thread per list entry by entry, and eight
 // per slot with the pruning as a pass of its own below 20 000 slots: 200 ->
-// 119 us per step at 25 000 neopentane-like atoms, 65 -> 30 us at 648
+// 116 us per step at 25 000 neopentane-like atoms, 65 -> 27 us at 648
 // propane-like ones (a launch with energies 185 -> 12 us).  What is left
 // there is the FP64 rate, then the latency of one warp's rounds: fetching the
-// partners of the next pass ahead, or two chains per sum, gave 0 to 1 %.  The potential is C2 at the region limits, so a pair that
+// partners of the next pass ahead gave 0 to 1 %.  The potential is C2 at the region limits, so a pair that
 // FP32 puts on the other side of one (1e-7 of r^2) changes nothing above 1e-13.
 //
 // The terms of a slot are stored by their rank in its list and added in list
-// order, one rounded product after the other.  Entries past the cutoff are no
-// terms, so the forces (and, per slot, energy and virial) are the same bits
-// for every T, with and without pruning.
+// order to four sums by rank modulo four (one chain of a hundred additions by
+// three lanes was a quarter of a 648-atom launch: a scheduler's FP64 unit
+// takes a warp instruction every 65 cycles).  Entries past the cutoff are no
+// terms (a CG pair below r_s- is none either: its constant energy is summed
+// apart), so the forces are the same bits for every T, with and without
+// energies and pruning.
 #include "common.cuh"
 #include "fbits.h"
 #include "pair.cuh"
@@ -61,7 +64,7 @@ struct Launch64 {
 
 // regions, in the order the entries are sorted by
 enum { kCore = 0, kShell = 1, kFgRegions = 2 };                      // FG: LJ below r_s-, switching off
-enum { kLj = 0, kOff = 1, kOn = 2, kClose = 3, kCgRegions = 4 };     // CG: kClose has an energy only
+enum { kLj = 0, kOff = 1, kOn = 2, kCgRegions = 3 };                 // CG: below r_s- an energy only
 
 // values of a term: force, then (energy steps) energy and virial
 constexpr int kTermF = 3, kTermEv = 3 + kNQ;
@@ -80,11 +83,6 @@ struct WarpTerms {
 template <bool CG, bool EV>
 __device__ __forceinline__ void term64(int region, const PairTab<double>& T, double r2, float r2f, double& fr,
                                        double& e) {
-  if (CG && region == kClose) {
-    fr = 0.0;
-    e = T.e_cg_close;
-    return;
-  }
   if (region == (CG ? int(kLj) : int(kCore))) {
     const double r2i = rcp_d(r2, r2f);
     const double r6i = r2i * r2i * r2i;
@@ -113,9 +111,10 @@ template <bool CG, bool EV, int T, bool PRN>
 __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0, const PairTab<double>* tab,
                                                      const float4* thr, WarpTerms<EV>& W, const Launch64& a) {
   constexpr int NV = EV ? kTermEv : kTermF;
-  constexpr int NL = (NV + T - 1) / T;  // values summed by one lane: q, q + T, ...
-  constexpr int NR = CG ? (EV ? int(kCgRegions) : int(kClose)) : int(kFgRegions);
-  const int lane = threadIdx.x & 31, sl = lane / T, q = lane % T;
+  constexpr int NG = T / 4;              // four lanes, one per chain, sum value g, g + NG, ...
+  constexpr int NL = (NV + NG - 1) / NG;  // values of one lane
+  constexpr int NR = CG ? int(kCgRegions) : int(kFgRegions);
+  const int lane = threadIdx.x & 31, sl = lane / T, q = lane % T, chain = q & 3, g = q >> 2;
   const int s = slot0 + sl;
   const bool own = s < L.nslots;
   const int ss = own ? s : 0;  // a valid slot for the loads of the other lanes
@@ -139,7 +138,8 @@ __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0,
   double f[NL];
 #pragma unroll
   for (int k = 0; k < NL; ++k) f[k] = 0.0;
-  int kept = 0;
+  double close = 0.0;  // energy of the CG pairs below r_s-
+  int kept = 0, done = 0;  // entries kept, terms added
   for (int r = 0; r < rounds; ++r) {
     const int ch = r * T + q;
     int4 jn = jj;
@@ -155,10 +155,10 @@ __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0,
       r2[e] = rem > e ? dx * dx + dy * dy + dz * dz : 3.0e38f;
       const float4 t = thr[row0 + p.w];
       if (CG)
-        region[e] = !(r2[e] < t.w) ? -1 : (r2[e] < t.x ? (EV ? int(kClose) : -1)
-                                                        : (r2[e] < t.y ? int(kOn) : (r2[e] < t.z ? int(kLj) : int(kOff))));
+        region[e] = !(r2[e] < t.w) || r2[e] < t.x ? -1 : (r2[e] < t.y ? int(kOn) : (r2[e] < t.z ? int(kLj) : int(kOff)));
       else
         region[e] = !(r2[e] < t.y) ? -1 : (r2[e] < t.x ? int(kCore) : int(kShell));
+      if (CG && EV && r2[e] < t.x) close += tab[row0 + p.w].e_cg_close;
     }
     // rank of each term in its slot's list order, and place in the sorted entries
     unsigned in[4];
@@ -210,10 +210,35 @@ __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0,
       }
     }
     __syncwarp();
+    // four threads a slot: the sums of a round take as many additions as with
+    // one chain a value, and its loads are issued together (forces only: 119.7
+    // -> 116.4 us per step at 25 000 atoms) or a value of every lane at a time
+    // (with energies, ten values a lane: 188 -> 174 us)
+    const int k0 = (chain - done) & 3;
+    if constexpr (T == 4 && !EV) {
 #pragma unroll
-    for (int v = 0; v < NL; ++v)
-      if (q + v * T < NV)
-        for (int k = 0; k < terms; ++k) f[v] += W.v[q + v * T][4 * T * sl + k];
+      for (int v = 0; v < NL; ++v) {
+        const double* const t = W.v[v] + 16 * sl + k0;
+        double x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = k0 + 4 * u < terms ? t[4 * u] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) f[v] += x[u];
+      }
+    } else if constexpr (T == 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (__any_sync(0xffffffffu, k0 + 4 * u < terms)) {
+#pragma unroll
+          for (int v = 0; v < NL; ++v) f[v] += k0 + 4 * u < terms ? W.v[v][16 * sl + k0 + 4 * u] : 0.0;
+        }
+    } else {
+      for (int k = k0; k < terms; k += 4)
+#pragma unroll
+        for (int v = 0; v < NL; ++v)
+          if (g + v * NG < NV) f[v] += W.v[g + v * NG][4 * T * sl + k];
+    }
+    done += terms;
     if constexpr (PRN) {
       int at = kept;
       unsigned b[4];
@@ -232,11 +257,25 @@ __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0,
     }
     jj = jn;
   }
-  if (own) {
-    const int i = L.perm[s];
+#pragma unroll
+  for (int v = 0; v < NL; ++v) {
+    f[v] += __shfl_xor_sync(0xffffffffu, f[v], 1);
+    f[v] += __shfl_xor_sync(0xffffffffu, f[v], 2);
+  }
+  if constexpr (CG && EV) {
+#pragma unroll
+    for (int o = T / 2; o > 0; o >>= 1) close += __shfl_xor_sync(0xffffffffu, close, o);
 #pragma unroll
     for (int v = 0; v < NL; ++v)
-      if (q + v * T < kTermF) L.f_out[3 * size_t(i) + q + v * T] = f[v];
+      if (g + v * NG == kTermF) f[v] += close;
+  }
+  if (own) {
+    const int i = L.perm[s];
+    if (chain == 0) {
+#pragma unroll
+      for (int v = 0; v < NL; ++v)
+        if (g + v * NG < kTermF) L.f_out[3 * size_t(i) + g + v * NG] = f[v];
+    }
     if (PRN && q == 0) {
       L.cnt_in[s] = kept;
       if (!CG) a.ref_p[i] = pi;
@@ -248,7 +287,7 @@ __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0,
     __syncwarp();
 #pragma unroll
     for (int v = 0; v < NL; ++v)
-      if (q + v * T < NV) W.v[q + v * T][sl] = own ? f[v] : 0.0;
+      if (chain == 0 && g + v * NG < NV) W.v[g + v * NG][sl] = own ? f[v] : 0.0;
     __syncwarp();
     if (lane < kNQ) {
       double t = 0.0;
