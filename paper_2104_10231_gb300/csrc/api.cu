@@ -1506,7 +1506,7 @@ struct relres_batch {
   std::vector<relres_ctx*> ctx;
   cudaStream_t stream = nullptr;
   std::vector<cudaStream_t> fork;
-  cudaEvent_t ev_fork = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_ctx = nullptr;
   std::vector<cudaEvent_t> ev_join;
   cudaGraphExec_t exec = nullptr;
   bool valid = false;
@@ -1775,6 +1775,7 @@ relres_status relres_batch_create(relres_batch** out, relres_ctx* const* ctxs, i
   b->fork.assign(n_ctx, nullptr);
   b->ev_join.assign(n_ctx, nullptr);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_ctx, cudaEventDisableTiming);
   for (int r = 0; r < n_ctx && e == cudaSuccess; ++r) {
     e = cudaStreamCreateWithFlags(&b->fork[r], cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_join[r], cudaEventDisableTiming);
@@ -1801,6 +1802,16 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
       return batch_fail(b, s, "replica " + std::to_string(r) + ": " + b->ctx[r]->err);
   }
   if (n_steps == 0) return RELRES_OK;
+  // the graphs follow what the contexts' own streams hold (the start of this call among it)
+  for (int r = 0; r < nr; ++r) {
+    const cudaStream_t cs = b->ctx[r]->stream;
+    bool seen = cs == b->stream;
+    for (int q = 0; q < r && !seen; ++q) seen = b->ctx[q]->stream == cs;
+    if (seen) continue;
+    cudaError_t e = cudaEventRecord(b->ev_ctx, cs);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_ctx);
+    if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
+  }
   int done = 0, retries = 0;
   while (done < n_steps) {
     const int blk = std::min(kBlockSteps, n_steps - done);
@@ -1894,6 +1905,7 @@ void relres_batch_destroy(relres_batch* b) {
   for (cudaEvent_t ev : b->ev_join)
     if (ev) cudaEventDestroy(ev);
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+  if (b->ev_ctx) cudaEventDestroy(b->ev_ctx);
   if (b->own_stream) cudaStreamDestroy(b->stream);
   delete b;
 }
