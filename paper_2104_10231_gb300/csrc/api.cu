@@ -105,6 +105,12 @@ relres_status setup_grid(relres_ctx* c, Grid* g, double rlist) {
   return RELRES_OK;
 }
 
+// h_state is current once the stream has been waited for
+static relres_status fetch_state(relres_ctx* c, cudaStream_t stream) {
+  CK(cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, stream));
+  return RELRES_OK;
+}
+
 relres_status read_state(relres_ctx* c) {
   CK(cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
@@ -1343,10 +1349,12 @@ static relres_status rollback_block(relres_ctx* c, double* d_vel) {
   return RELRES_OK;
 }
 
-// ---- relres_step in three phases (shared with relres_batch_step)
+// ---- relres_step in phases (shared with relres_batch_step, which issues each
+// phase for every replica before it waits for one)
 
-// Validation, forces at the incoming positions, autotuning, per-call constants.
-static relres_status step_begin(relres_ctx* c, int n_steps, double dt_fs, double* d_pos, double* d_vel,
+// Validation, and the comparison of the incoming arrays with the last ones
+// (out->cached: its result is in the state on its way to the host).
+static relres_status step_check(relres_ctx* c, int n_steps, double dt_fs, double* d_pos, double* d_vel,
                                 double t_target, double tau_fs, uint64_t seed, int thermo_every, double* d_thermo,
                                 StepParams* out) {
   if (!c->have_lists) return fail(c, RELRES_ERR_STATE, "relres_build_neighbors first");
@@ -1366,7 +1374,16 @@ static relres_status step_begin(relres_ctx* c, int n_steps, double dt_fs, double
   *out = sp;
   if (n_steps == 0) return RELRES_OK;
   if (c->n < 2 && t_target > 0.0) return fail(c, RELRES_ERR_ARG, "the thermostat needs at least 2 atoms");
+  out->cached = c->io_valid && c->forces_valid;
+  out->try_u = out->cached && !c->fp64 && dt_fs == c->io_dt;
+  c->io_valid = false;  // until this call has returned its arrays
+  if (!out->cached) return RELRES_OK;
+  CK(launch_check_io(c, d_pos, out->try_u ? d_vel : nullptr));
+  return fetch_state(c, c->stream);
+}
 
+// Forces at the incoming positions, autotuning, per-call constants.
+static relres_status step_begin(relres_ctx* c, const StepParams& sp, double* d_pos, double* d_vel) {
   // The state at the call's start.  After a relres_step, a call given the
   // arrays that step returned (compared word for word on the device)
   // continues from its end state: the forces are reused and, in FP32 mode
@@ -1374,18 +1391,13 @@ static relres_status step_begin(relres_ctx* c, int n_steps, double dt_fs, double
   // thermostat factors (the trajectory is then the bits of one longer call).
   // Otherwise the positions are read and the forces evaluated, and the
   // velocities are read (u = v, a = b = 1).
-  const bool cached = c->io_valid && c->forces_valid;
-  c->io_valid = false;  // until this call has returned its arrays
   bool dirty = true, keep_u = false;
   relres_status s = RELRES_OK;
-  if (cached) {
-    const bool try_u = !c->fp64 && dt_fs == c->io_dt;
-    CK(launch_check_io(c, d_pos, try_u ? d_vel : nullptr));
-    s = read_state(c);
-    if (s != RELRES_OK) return s;
+  if (sp.cached) {
+    CK(cudaStreamSynchronize(c->stream));  // step_check
     const unsigned fl = c->h_state->flags;
     dirty = (fl & F_DIRTY) != 0;
-    keep_u = try_u && !dirty && !(fl & F_VDIRTY);
+    keep_u = sp.try_u && !dirty && !(fl & F_VDIRTY);
   }
   if (!keep_u) CK(launch_vel_in(c, d_vel));  // FP32: the float-float velocity state of the call
   CK(launch_call_start(c, !keep_u));
@@ -1401,7 +1413,7 @@ static relres_status step_begin(relres_ctx* c, int n_steps, double dt_fs, double
     if (s != RELRES_OK) return s;
     fresh = true;
   }
-  CK(upload_type_consts(c, dt_fs));
+  CK(upload_type_consts(c, sp.dt));
   // Everything that follows runs on the context stream, after these launches.
   // Without a force evaluation above, the state read at the start is still
   // current for the block accounting (the set-up above changes no count), so
@@ -1474,13 +1486,10 @@ static void step_end(relres_ctx* c, int n_steps, double dt_fs) {
   c->io_dt = dt_fs;
 }
 
-// Positions and velocities back to the caller, then the counters (batches).
-static relres_status write_back_and_end(relres_ctx* c, int n_steps, double* d_pos, double* d_vel, double dt_fs) {
+// Positions and velocities back to the caller, the state on its way to the host (batches).
+static relres_status write_back(relres_ctx* c, double* d_pos, double* d_vel, double dt_fs) {
   CK(launch_write_back(c, d_pos, d_vel, dt_fs));
-  relres_status s = read_state(c);
-  if (s != RELRES_OK) return s;
-  step_end(c, n_steps, dt_fs);
-  return RELRES_OK;
+  return fetch_state(c, c->stream);
 }
 
 // ---- batches of independent replicas: one CUDA graph per block of steps
@@ -1796,12 +1805,17 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
   const int nr = int(b->ctx.size());
   std::vector<StepParams> sp(nr);
   for (int r = 0; r < nr; ++r) {
-    relres_status s = step_begin(b->ctx[r], n_steps, dt_fs, d_pos[r], d_vel[r], t_target[r], tau_fs, seed[r],
+    relres_status s = step_check(b->ctx[r], n_steps, dt_fs, d_pos[r], d_vel[r], t_target[r], tau_fs, seed[r],
                                  thermo_every, d_thermo ? d_thermo[r] : nullptr, &sp[r]);
     if (s != RELRES_OK)
       return batch_fail(b, s, "replica " + std::to_string(r) + ": " + b->ctx[r]->err);
   }
   if (n_steps == 0) return RELRES_OK;
+  for (int r = 0; r < nr; ++r) {
+    relres_status s = step_begin(b->ctx[r], sp[r], d_pos[r], d_vel[r]);
+    if (s != RELRES_OK)
+      return batch_fail(b, s, "replica " + std::to_string(r) + ": " + b->ctx[r]->err);
+  }
   // the graphs follow what the contexts' own streams hold (the start of this call among it)
   for (int r = 0; r < nr; ++r) {
     const cudaStream_t cs = b->ctx[r]->stream;
@@ -1824,14 +1838,14 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
     relres_status s = batch_graph(b, sp, d_vel, blk, done);
     if (s != RELRES_OK) return s;
     cudaError_t e = cudaGraphLaunch(b->exec, b->stream);
+    for (int r = 0; r < nr && e == cudaSuccess && s == RELRES_OK; ++r) s = fetch_state(b->ctx[r], b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e == cudaSuccess && s != RELRES_OK) return batch_fail(b, s, "status read");
     if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
     std::vector<unsigned> flags(nr);
     bool overflow = false;
     for (int r = 0; r < nr; ++r) {
       relres_ctx* c = b->ctx[r];
-      s = read_state(c);
-      if (s != RELRES_OK) return batch_fail(b, s, "replica " + std::to_string(r) + ": " + c->err);
       const long long kpr = (!b->is_shared[r] && c->prune_on && !pairs_prune(c)) ? 1 : 0;
       // a rebuild body of kRebuildKernels kernels runs per rebuild (the shared
       // launches' batched kernels are counted for every replica they rebuild)
@@ -1842,7 +1856,10 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
         return batch_fail(b, RELRES_ERR_CUDA, "replica " + std::to_string(r) + ": out-of-range cell index");
       if (flags[r] & F_NONFINITE) {
         for (int q = 0; q < nr; ++q) rollback_block(b->ctx[q], d_vel[q]);
-        for (int q = 0; q < nr; ++q) write_back_and_end(b->ctx[q], 0, d_pos[q], d_vel[q], dt_fs);
+        for (int q = 0; q < nr; ++q) {
+          if (write_back(b->ctx[q], d_pos[q], d_vel[q], dt_fs) != RELRES_OK) continue;
+          if (cudaStreamSynchronize(b->ctx[q]->stream) == cudaSuccess) step_end(b->ctx[q], 0, dt_fs);
+        }
         return batch_fail(b, RELRES_ERR_NONFINITE, "replica " + std::to_string(r) + ": non-finite force");
       }
       overflow |= (flags[r] & (F_OVERFLOW_FG | F_OVERFLOW_CG)) != 0;
@@ -1867,8 +1884,13 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
     done += blk;
   }
   for (int r = 0; r < nr; ++r) {
-    relres_status s = write_back_and_end(b->ctx[r], n_steps, d_pos[r], d_vel[r], dt_fs);
+    relres_status s = write_back(b->ctx[r], d_pos[r], d_vel[r], dt_fs);
     if (s != RELRES_OK) return batch_fail(b, s, "replica " + std::to_string(r) + ": " + b->ctx[r]->err);
+  }
+  for (int r = 0; r < nr; ++r) {
+    const cudaError_t e = cudaStreamSynchronize(b->ctx[r]->stream);
+    if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
+    step_end(b->ctx[r], n_steps, dt_fs);
   }
   return RELRES_OK;
 }
@@ -1915,8 +1937,10 @@ relres_status relres_step(relres_ctx* c, int n_steps, double dt_fs, double* d_po
                           double* d_thermo) {
   if (!c) return RELRES_ERR_ARG;
   StepParams sp{};
-  relres_status s = step_begin(c, n_steps, dt_fs, d_pos, d_vel, t_target, tau_fs, seed, thermo_every, d_thermo, &sp);
+  relres_status s = step_check(c, n_steps, dt_fs, d_pos, d_vel, t_target, tau_fs, seed, thermo_every, d_thermo, &sp);
   if (s != RELRES_OK || n_steps == 0) return s;
+  s = step_begin(c, sp, d_pos, d_vel);
+  if (s != RELRES_OK) return s;
   int done = 0, retries = 0;
   while (done < n_steps) {
     const int blk = std::min(kBlockSteps, n_steps - done);

@@ -170,6 +170,7 @@ struct StepParams {
   unsigned long long seed;
   int thermo_every;
   double* thermo;  // device [rows][RELRES_THERMO_COLS] or null
+  bool cached, try_u;  // the call may continue from the last one's positions, velocity state (step_check)
 };
 
 // Cell grid of one list.  Full cells are at least one list radius wide (nf
