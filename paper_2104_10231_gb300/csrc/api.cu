@@ -107,12 +107,12 @@ relres_status setup_grid(relres_ctx* c, Grid* g, double rlist) {
 
 // h_state is current once the stream has been waited for
 static relres_status fetch_state(relres_ctx* c, cudaStream_t stream) {
-  CK(cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, stream));
+  CK(launch_post_state(c, stream));
   return RELRES_OK;
 }
 
 relres_status read_state(relres_ctx* c) {
-  CK(cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
+  CK(launch_post_state(c, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   return RELRES_OK;
 }
@@ -295,7 +295,8 @@ bool tunes_by_timing(const relres_ctx* c) {
   return c->tune_mode < 0 && !c->fp64 && fp32_lanes(c, false) == 1 && c->n >= 20000;
 }
 
-// Forces at the positions already converted into d_xfx (F_tot, FP64 copy optional).
+// Forces at the positions that launch_convert has just put into d_xfx, which
+// also cleared the accumulators (F_tot, FP64 copy optional).
 relres_status forces_now(relres_ctx* c, int ev_mode, double* d_forces, double* d_energy,
                          double* d_virial) {
   if (!c->tuned && tunes_by_timing(c)) {  // on lists that are ready
@@ -312,10 +313,10 @@ relres_status forces_now(relres_ctx* c, int ev_mode, double* d_forces, double* d
     const relres_status s = autotune_pairs(c);
     if (s != RELRES_OK) return s;
   }
-  for (bool retry = true; retry;) {
+  for (bool retry = true, again = false; retry; again = true) {
     relres_status s = refresh_lists(c, !pairs_prune(c));
     if (s != RELRES_OK) return s;
-    CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAccAll, c->stream));
+    if (again) CK(cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * kNAccAll, c->stream));
     TIMED(ev_mode == 1 ? RELRES_T_PAIR_EV : RELRES_T_PAIR, launch_pairs(c, ev_mode == 1));
     TIMED(RELRES_T_FINISH, launch_finish(c, ev_mode == 1, d_forces, nullptr, true));
     if (ev_mode == 1) TIMED(RELRES_T_THERMO, launch_reduce_out(c, d_energy, d_virial));

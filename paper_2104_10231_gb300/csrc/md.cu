@@ -110,7 +110,9 @@ __global__ void k_convert(int n, const double* __restrict__ pos, const int* __re
                           unsigned long long* __restrict__ xfx, BoxConsts b, int have_lists,
                           const int* rank_fg, const int* rank_cg, int with_cg, int4* pos_fg,
                           int4* pos_cg, int fp64, Pos64* pos_fg64, Pos64* pos_cg64, const int4* ref,
-                          float thr2, const int4* ref_p, float thr2_p, int prune, DevState* st) {
+                          float thr2, const int4* ref_p, float thr2_p, int prune, DevState* st, long long* acc) {
+  if (blockIdx.x == 0)  // empty accumulators for the evaluation that follows
+    for (int q = threadIdx.x; q < kNAccAll; q += blockDim.x) acc[q] = 0;
   const double il0 = b.inv_l0, il1 = b.inv_l1, il2 = b.inv_l2;
   const Sc3<float> s{b.s32_0, b.s32_1, b.s32_2};
   bool rebuild = false, reprune = false, bad = false;
@@ -1326,6 +1328,14 @@ __global__ void k_flags_and(DevState* st, unsigned keep) { st->flags &= keep; }
 __global__ void k_flags_or(DevState* st, unsigned set) { st->flags |= set; }
 __global__ void k_close_call(DevState* st) { close_host_call(st); }
 
+// The state to the host's pinned copy, written by a kernel: a copy of these
+// few words as a transfer of its own starts 5 us behind the kernel before it,
+// this one follows like any launch.
+__global__ void k_post_state(const DevState* __restrict__ st, DevState* __restrict__ host) {
+  for (int w = threadIdx.x; w < int(sizeof(DevState) / 8); w += blockDim.x)
+    reinterpret_cast<unsigned long long*>(host)[w] = reinterpret_cast<const unsigned long long*>(st)[w];
+}
+
 // FP32 path: caller's FP64 velocities -> float-float state
 __global__ void k_vel_in(int n3, const double* __restrict__ vel, float2* __restrict__ uff) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n3; k += gridDim.x * blockDim.x) {
@@ -1444,7 +1454,7 @@ cudaError_t launch_convert(relres_ctx* c, const double* d_pos) {
       c->n, d_pos, c->d_type, c->d_xfx, b, c->have_lists ? 1 : 0, c->d_rank_fg, c->d_rank_cg,
       (c->has_cg && c->n_h > 0) ? 1 : 0, c->d_pos_fg, c->d_pos_cg, c->fp64 ? 1 : 0, p64(c, c->d_pos_fg64),
       p64(c, c->d_pos_cg64), c->d_ref, trigger_thr2(c), c->prune_on ? c->d_ref_p : c->d_ref, prune_thr2(c),
-      c->prune_on ? 1 : 0, c->d_state);
+      c->prune_on ? 1 : 0, c->d_state, c->d_acc);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
@@ -1801,6 +1811,12 @@ cudaError_t launch_thermo(relres_ctx* c, const StepParams& sp, int k) {
 
 cudaError_t launch_call_start(relres_ctx* c, bool reset_ab) {
   k_call_start<<<1, 32, 0, c->stream>>>(c->d_state, c->d_acc, reset_ab ? 1 : 0);
+  RELRES_LAUNCHED(c);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_post_state(relres_ctx* c, cudaStream_t stream) {
+  k_post_state<<<1, 32, 0, stream>>>(c->d_state, c->h_state);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }

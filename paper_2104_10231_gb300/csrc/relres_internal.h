@@ -497,6 +497,8 @@ cudaError_t launch_vel_in(relres_ctx* c, const double* d_vel);
 inline void* vel_state(relres_ctx* c, double* d_vel) {
   return c->fp64 ? static_cast<void*>(d_vel) : static_cast<void*>(c->d_uff);
 }
+// d_state to h_state, once the stream has been waited for
+cudaError_t launch_post_state(relres_ctx* c, cudaStream_t stream);
 cudaError_t launch_flags_and(relres_ctx* c, unsigned keep);
 cudaError_t launch_flags_or(relres_ctx* c, unsigned set);
 // end of a call that refreshed the lists: counts a rebuild, clears the list flags
