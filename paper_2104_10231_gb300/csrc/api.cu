@@ -105,14 +105,8 @@ relres_status setup_grid(relres_ctx* c, Grid* g, double rlist) {
   return RELRES_OK;
 }
 
-// h_state is current once the stream has been waited for
-static relres_status fetch_state(relres_ctx* c, cudaStream_t stream) {
-  CK(launch_post_state(c, stream));
-  return RELRES_OK;
-}
-
 relres_status read_state(relres_ctx* c) {
-  CK(launch_post_state(c, c->stream));
+  CK(launch_post_state(c));
   CK(cudaStreamSynchronize(c->stream));
   return RELRES_OK;
 }
@@ -1353,9 +1347,8 @@ static relres_status rollback_block(relres_ctx* c, double* d_vel) {
 // ---- relres_step in phases (shared with relres_batch_step, which issues each
 // phase for every replica before it waits for one)
 
-// Validation, and the comparison of the incoming arrays with the last ones
-// (out->cached: its result is in the state on its way to the host).
-static relres_status step_check(relres_ctx* c, int n_steps, double dt_fs, double* d_pos, double* d_vel,
+// Validation, and whether the call may continue from the last one's end.
+static relres_status step_check(relres_ctx* c, int n_steps, double dt_fs, const double* d_pos, const double* d_vel,
                                 double t_target, double tau_fs, uint64_t seed, int thermo_every, double* d_thermo,
                                 StepParams* out) {
   if (!c->have_lists) return fail(c, RELRES_ERR_STATE, "relres_build_neighbors first");
@@ -1378,12 +1371,12 @@ static relres_status step_check(relres_ctx* c, int n_steps, double dt_fs, double
   out->cached = c->io_valid && c->forces_valid;
   out->try_u = out->cached && !c->fp64 && dt_fs == c->io_dt;
   c->io_valid = false;  // until this call has returned its arrays
-  if (!out->cached) return RELRES_OK;
-  CK(launch_check_io(c, d_pos, out->try_u ? d_vel : nullptr));
-  return fetch_state(c, c->stream);
+  return RELRES_OK;
 }
 
-// Forces at the incoming positions, autotuning, per-call constants.
+// Forces at the incoming positions, autotuning, per-call constants; behind
+// launch_check_io and launch_call_start, whose stream has been waited for if
+// sp.cached (h_state holds what the comparison found).
 static relres_status step_begin(relres_ctx* c, const StepParams& sp, double* d_pos, double* d_vel) {
   // The state at the call's start.  After a relres_step, a call given the
   // arrays that step returned (compared word for word on the device)
@@ -1395,13 +1388,11 @@ static relres_status step_begin(relres_ctx* c, const StepParams& sp, double* d_p
   bool dirty = true, keep_u = false;
   relres_status s = RELRES_OK;
   if (sp.cached) {
-    CK(cudaStreamSynchronize(c->stream));  // step_check
     const unsigned fl = c->h_state->flags;
     dirty = (fl & F_DIRTY) != 0;
     keep_u = sp.try_u && !dirty && !(fl & F_VDIRTY);
   }
   if (!keep_u) CK(launch_vel_in(c, d_vel));  // FP32: the float-float velocity state of the call
-  CK(launch_call_start(c, !keep_u));
   bool fresh = false;  // host state read after the last device work that changes it
   if (dirty) {
     CK(launch_convert(c, d_pos));
@@ -1454,13 +1445,13 @@ static relres_status block_end(relres_ctx* c, double* d_pos, double* d_vel, doub
     s = rollback_block(c, d_vel);
     if (s != RELRES_OK) return s;
     if (fl & F_NONFINITE) {
-      CK(launch_write_back(c, d_pos, d_vel, dt_fs));
+      CK(launch_write_back(c, d_pos, d_vel));
       CK(cudaStreamSynchronize(c->stream));
       c->forces_valid = true;
       return fail(c, RELRES_ERR_NONFINITE, "non-finite force during relres_step");
     }
     if (++*retries > 8) {
-      CK(launch_write_back(c, d_pos, d_vel, dt_fs));  // the caller's copy of the restored state
+      CK(launch_write_back(c, d_pos, d_vel));  // the caller's copy of the restored state
       CK(cudaStreamSynchronize(c->stream));
       return fail(c, RELRES_ERR_LIST_OVERFLOW, "repeated list overflow");
     }
@@ -1485,12 +1476,6 @@ static void step_end(relres_ctx* c, int n_steps, double dt_fs) {
   c->forces_valid = true;
   c->io_valid = true;
   c->io_dt = dt_fs;
-}
-
-// Positions and velocities back to the caller, the state on its way to the host (batches).
-static relres_status write_back(relres_ctx* c, double* d_pos, double* d_vel, double dt_fs) {
-  CK(launch_write_back(c, d_pos, d_vel, dt_fs));
-  return fetch_state(c, c->stream);
 }
 
 // ---- batches of independent replicas: one CUDA graph per block of steps
@@ -1535,7 +1520,23 @@ struct relres_batch {
   BatchLaunch bl_start, bl_pair, bl_pair_ev, bl_drift, bl_sum;
   RebuildBatch rebuild;
   DevState** d_states = nullptr;  // [nrep]
+  void* d_call = nullptr;         // fill_call_table, and the pinned copy it is written in
+  void* h_call = nullptr;
 };
+
+// The batch's stream behind what the contexts' own streams hold.
+static cudaError_t batch_follow(relres_batch* b) {
+  cudaError_t e = cudaSuccess;
+  for (size_t r = 0; r < b->ctx.size() && e == cudaSuccess; ++r) {
+    const cudaStream_t cs = b->ctx[r]->stream;
+    bool seen = cs == b->stream;
+    for (size_t q = 0; q < r && !seen; ++q) seen = b->ctx[q]->stream == cs;
+    if (seen) continue;
+    e = cudaEventRecord(b->ev_ctx, cs);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_ctx);
+  }
+  return e;
+}
 
 static relres_status batch_fail(relres_batch* b, relres_status s, const std::string& m) {
   b->err = m;
@@ -1812,21 +1813,27 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
       return batch_fail(b, s, "replica " + std::to_string(r) + ": " + b->ctx[r]->err);
   }
   if (n_steps == 0) return RELRES_OK;
+  // the call's boundary kernels for all replicas at once
+  cudaError_t e = cudaSuccess;
+  const size_t tb = call_table_bytes(nr);
+  if (!b->d_call) e = cudaMalloc(&b->d_call, tb);
+  if (e == cudaSuccess && !b->h_call) e = cudaMallocHost(&b->h_call, tb);
+  if (e == cudaSuccess) {
+    fill_call_table(b->ctx.data(), nr, sp.data(), d_pos, d_vel, b->h_call);
+    e = cudaMemcpyAsync(b->d_call, b->h_call, tb, cudaMemcpyHostToDevice, b->stream);
+  }
+  if (e == cudaSuccess) e = batch_follow(b);  // the caller's arrays
+  if (e == cudaSuccess) e = launch_call_batch(b->stream, b->d_call, b->ctx.data(), nr, kCallCheck);
+  if (e == cudaSuccess) e = launch_call_batch(b->stream, b->d_call, b->ctx.data(), nr, kCallStart);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+  if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
   for (int r = 0; r < nr; ++r) {
     relres_status s = step_begin(b->ctx[r], sp[r], d_pos[r], d_vel[r]);
     if (s != RELRES_OK)
       return batch_fail(b, s, "replica " + std::to_string(r) + ": " + b->ctx[r]->err);
   }
-  // the graphs follow what the contexts' own streams hold (the start of this call among it)
-  for (int r = 0; r < nr; ++r) {
-    const cudaStream_t cs = b->ctx[r]->stream;
-    bool seen = cs == b->stream;
-    for (int q = 0; q < r && !seen; ++q) seen = b->ctx[q]->stream == cs;
-    if (seen) continue;
-    cudaError_t e = cudaEventRecord(b->ev_ctx, cs);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_ctx);
-    if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
-  }
+  e = batch_follow(b);  // what the contexts' set-up has launched
+  if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
   int done = 0, retries = 0;
   while (done < n_steps) {
     const int blk = std::min(kBlockSteps, n_steps - done);
@@ -1838,10 +1845,9 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
     }
     relres_status s = batch_graph(b, sp, d_vel, blk, done);
     if (s != RELRES_OK) return s;
-    cudaError_t e = cudaGraphLaunch(b->exec, b->stream);
-    for (int r = 0; r < nr && e == cudaSuccess && s == RELRES_OK; ++r) s = fetch_state(b->ctx[r], b->stream);
+    e = cudaGraphLaunch(b->exec, b->stream);
+    if (e == cudaSuccess) e = launch_call_batch(b->stream, b->d_call, b->ctx.data(), nr, kCallStatus);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e == cudaSuccess && s != RELRES_OK) return batch_fail(b, s, "status read");
     if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
     std::vector<unsigned> flags(nr);
     bool overflow = false;
@@ -1858,8 +1864,8 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
       if (flags[r] & F_NONFINITE) {
         for (int q = 0; q < nr; ++q) rollback_block(b->ctx[q], d_vel[q]);
         for (int q = 0; q < nr; ++q) {
-          if (write_back(b->ctx[q], d_pos[q], d_vel[q], dt_fs) != RELRES_OK) continue;
-          if (cudaStreamSynchronize(b->ctx[q]->stream) == cudaSuccess) step_end(b->ctx[q], 0, dt_fs);
+          if (launch_write_back(b->ctx[q], d_pos[q], d_vel[q]) != cudaSuccess) continue;
+          if (read_state(b->ctx[q]) == RELRES_OK) step_end(b->ctx[q], 0, dt_fs);
         }
         return batch_fail(b, RELRES_ERR_NONFINITE, "replica " + std::to_string(r) + ": non-finite force");
       }
@@ -1884,15 +1890,11 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
     }
     done += blk;
   }
-  for (int r = 0; r < nr; ++r) {
-    relres_status s = write_back(b->ctx[r], d_pos[r], d_vel[r], dt_fs);
-    if (s != RELRES_OK) return batch_fail(b, s, "replica " + std::to_string(r) + ": " + b->ctx[r]->err);
-  }
-  for (int r = 0; r < nr; ++r) {
-    const cudaError_t e = cudaStreamSynchronize(b->ctx[r]->stream);
-    if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
-    step_end(b->ctx[r], n_steps, dt_fs);
-  }
+  e = launch_call_batch(b->stream, b->d_call, b->ctx.data(), nr, kCallFinish);
+  if (e == cudaSuccess) e = launch_call_batch(b->stream, b->d_call, b->ctx.data(), nr, kCallStatus);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+  if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
+  for (int r = 0; r < nr; ++r) step_end(b->ctx[r], n_steps, dt_fs);
   return RELRES_OK;
 }
 
@@ -1923,6 +1925,8 @@ void relres_batch_destroy(relres_batch* b) {
   free_batch(&b->bl_sum);
   free_rebuild_batch(&b->rebuild);
   if (b->d_states) cudaFree(b->d_states);
+  if (b->d_call) cudaFree(b->d_call);
+  if (b->h_call) cudaFreeHost(b->h_call);
   for (cudaStream_t st : b->fork)
     if (st) cudaStreamDestroy(st);
   for (cudaEvent_t ev : b->ev_join)
@@ -1940,6 +1944,9 @@ relres_status relres_step(relres_ctx* c, int n_steps, double dt_fs, double* d_po
   StepParams sp{};
   relres_status s = step_check(c, n_steps, dt_fs, d_pos, d_vel, t_target, tau_fs, seed, thermo_every, d_thermo, &sp);
   if (s != RELRES_OK || n_steps == 0) return s;
+  if (sp.cached) CK(launch_check_io(c, sp, d_pos, d_vel));
+  CK(launch_call_start(c, sp));
+  if (sp.cached) CK(cudaStreamSynchronize(c->stream));
   s = step_begin(c, sp, d_pos, d_vel);
   if (s != RELRES_OK) return s;
   int done = 0, retries = 0;
@@ -1958,7 +1965,7 @@ relres_status relres_step(relres_ctx* c, int n_steps, double dt_fs, double* d_po
     // behind the last block the positions and velocities go back to the
     // caller, so that one status read covers both (a block that fails or is
     // retried restores the state, and the caller's copy is written again)
-    if (done + blk == n_steps) CK(launch_write_back(c, d_pos, d_vel, dt_fs));
+    if (done + blk == n_steps) CK(launch_write_back(c, d_pos, d_vel));
     bool retry = false;
     s = block_end(c, d_pos, d_vel, dt_fs, builds0, prunes0, c->use_graphs, &retries, &retry);
     if (s != RELRES_OK) return s;

@@ -147,16 +147,27 @@ __device__ __forceinline__ double back_to_double(unsigned long long u, double l6
 // The caller's positions (and velocities, when vel is not NULL) against the
 // ones the last relres_step returned, word for word: F_DIRTY / F_VDIRTY when
 // any differs.
-__global__ void k_check_io(int n3, const unsigned long long* __restrict__ pos,
-                           const unsigned long long* __restrict__ pos_ret, const unsigned long long* __restrict__ vel,
-                           const unsigned long long* __restrict__ vel_ret, DevState* st) {
+struct CheckIo {
+  int n3;  // 0: nothing to compare
+  const unsigned long long* pos;
+  const unsigned long long* pos_ret;
+  const unsigned long long* vel;
+  const unsigned long long* vel_ret;
+  DevState* st;
+};
+
+__device__ __forceinline__ void check_io(const CheckIo& a, int bid, int nblk) {
   bool dp = false, dv = false;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n3; k += gridDim.x * blockDim.x) {
-    dp |= pos[k] != pos_ret[k];
-    if (vel != nullptr) dv |= vel[k] != vel_ret[k];
+  for (int k = bid * kThreads + threadIdx.x; k < a.n3; k += nblk * kThreads) {
+    dp |= a.pos[k] != a.pos_ret[k];
+    if (a.vel != nullptr) dv |= a.vel[k] != a.vel_ret[k];
   }
-  if (__syncthreads_or(dp) && threadIdx.x == 0) atomicOr(&st->flags, F_DIRTY);
-  if (__syncthreads_or(dv) && threadIdx.x == 0) atomicOr(&st->flags, F_VDIRTY);
+  if (__syncthreads_or(dp) && threadIdx.x == 0) atomicOr(&a.st->flags, F_DIRTY);
+  if (__syncthreads_or(dv) && threadIdx.x == 0) atomicOr(&a.st->flags, F_VDIRTY);
+}
+
+__global__ void __launch_bounds__(kThreads) k_check_io(const __grid_constant__ CheckIo a) {
+  check_io(a, blockIdx.x, gridDim.x);
 }
 
 // ----------------------------------------------------------------- bonded
@@ -1303,14 +1314,33 @@ __global__ void k_reduce_out(long long* acc, double* energy, int with_e, double*
   for (int q = 0; q < kNAccAll; ++q) acc[q] = 0;
 }
 
-// Start of a relres_step call: its step and thermo-row counters, empty
-// accumulators, the flags of k_check_io cleared for the next call, and (unless
-// the call continues the velocity state of the last one) the factors of the
-// first drift for velocities read from the caller, u = v: a = b = 1.
-__global__ void k_call_start(DevState* st, long long* acc, int reset_ab) {
-  for (int q = threadIdx.x; q < kNAccAll; q += blockDim.x) acc[q] = 0;
+// Start of a relres_step call: the state (with the flags of k_check_io) to the
+// host's pinned copy, then the call's step and thermo-row counters, empty
+// accumulators, those flags cleared for the next call, and (unless the call
+// continues the velocity state of the last one) the factors of the first drift
+// for velocities read from the caller, u = v: a = b = 1.  One warp.
+struct CallStart {
+  DevState* st;
+  DevState* host;
+  long long* acc;
+  int try_u;  // the velocity state continues if the arrays are the ones returned last
+};
+
+// The state to the host's pinned copy, written by a kernel: a copy of these
+// few words as a transfer of its own starts 5 us behind the kernel before it,
+// this one follows like any launch.
+__device__ __forceinline__ void post_state(const DevState* st, DevState* host) {
+  for (int w = threadIdx.x; w < int(sizeof(DevState) / 8); w += 32)
+    reinterpret_cast<unsigned long long*>(host)[w] = reinterpret_cast<const unsigned long long*>(st)[w];
+}
+
+__device__ __forceinline__ void call_start(const CallStart& a) {
+  post_state(a.st, a.host);
+  for (int q = threadIdx.x; q < kNAccAll; q += 32) a.acc[q] = 0;
+  __syncwarp();
   if (threadIdx.x != 0) return;
-  if (reset_ab) {
+  DevState* const st = a.st;
+  if (!a.try_u || (st->flags & (F_DIRTY | F_VDIRTY)) != 0u) {
     st->a = 1.0;
     st->b = 1.0;
     st->a_hi = 1.f;
@@ -1324,17 +1354,13 @@ __global__ void k_call_start(DevState* st, long long* acc, int reset_ab) {
   st->flags &= ~unsigned(F_DIRTY | F_VDIRTY);
 }
 
+__global__ void __launch_bounds__(32) k_call_start(const __grid_constant__ CallStart a) { call_start(a); }
+
 __global__ void k_flags_and(DevState* st, unsigned keep) { st->flags &= keep; }
 __global__ void k_flags_or(DevState* st, unsigned set) { st->flags |= set; }
 __global__ void k_close_call(DevState* st) { close_host_call(st); }
 
-// The state to the host's pinned copy, written by a kernel: a copy of these
-// few words as a transfer of its own starts 5 us behind the kernel before it,
-// this one follows like any launch.
-__global__ void k_post_state(const DevState* __restrict__ st, DevState* __restrict__ host) {
-  for (int w = threadIdx.x; w < int(sizeof(DevState) / 8); w += blockDim.x)
-    reinterpret_cast<unsigned long long*>(host)[w] = reinterpret_cast<const unsigned long long*>(st)[w];
-}
+__global__ void __launch_bounds__(32) k_post_state(const DevState* st, DevState* host) { post_state(st, host); }
 
 // FP32 path: caller's FP64 velocities -> float-float state
 __global__ void k_vel_in(int n3, const double* __restrict__ vel, float2* __restrict__ uff) {
@@ -1354,39 +1380,81 @@ __device__ __forceinline__ double force_component(const double* f, int, int, int
 // End of a call: positions and velocities to the caller, and copies of both.
 // One component per thread, so that every array is read and written in whole
 // lines (one atom per thread: 9.3 us at 140 000 atoms, 36 us at a million).
+struct FinishMd {
+  int n3;
+  const DevState* st;
+  const void* vel_u;  // VelT<R>
+  const void* f_tot;  // ForceT<R>
+  const int* type;
+  const double* cdt;
+  const float2* cdt_ff;
+  const unsigned long long* xfx;
+  BoxConsts b;
+  double* vel_out;
+  double* pos_out;
+  double* pos_ret;
+  double* vel_ret;
+};
+
 template <typename R>
-__global__ void k_finish_md(int n3, const DevState* st, const VelT<R>* vel_u,
-                            const ForceT<R>* __restrict__ f_tot, const int* __restrict__ type,
-                            const double* __restrict__ cdt, const float2* __restrict__ cdt_ff,
-                            const unsigned long long* __restrict__ xfx, BoxConsts b, double* vel_out,
-                            double* __restrict__ pos_out, double* __restrict__ pos_ret, double* __restrict__ vel_ret) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n3; k += gridDim.x * blockDim.x) {
+__device__ __forceinline__ void finish_md(const FinishMd& a, int bid, int nblk) {
+  for (int k = bid * kThreads + threadIdx.x; k < a.n3; k += nblk * kThreads) {
     const int i = k / 3, q = k - 3 * i;
-    const int t = type[i];
-    const R f = force_component(f_tot, i, q, k);
+    const int t = a.type[i];
+    const R f = force_component(static_cast<const ForceT<R>*>(a.f_tot), i, q, k);
     double v;
     if constexpr (std::is_same<R, float>::value) {
       // v = a u + (b - 1) c F in float-float, returned as the double nearest
       // to hi + lo: the parts converted exactly with integer operations, one
       // FP64 addition
-      const ff ca{st->a_hi, st->a_lo};
-      const ff cb1 = ff_add(ff{st->b_hi, st->b_lo}, ff{-1.f, 0.f});
-      const float2 cc = cdt_ff[t];
+      const ff ca{a.st->a_hi, a.st->a_lo};
+      const ff cb1 = ff_add(ff{a.st->b_hi, a.st->b_lo}, ff{-1.f, 0.f});
+      const float2 cc = a.cdt_ff[t];
       const ff cbc = ff_mul(cb1, ff{cc.x, cc.y});
-      const float2 u = vel_u[k];
+      const float2 u = static_cast<const VelT<R>*>(a.vel_u)[k];
       const ff w = ff_add(ff_mul(ca, ff{u.x, u.y}), ff_mul_f(cbc, f));
       v = double_of_float(w.hi) + double_of_float(w.lo);
     } else {
-      const double ca = st->a, cb1 = st->b - 1.0;
-      v = fma(ca, vel_d(vel_u, k), double(R(cb1 * cdt[t]) * f));
+      const double ca = a.st->a, cb1 = a.st->b - 1.0;
+      v = fma(ca, vel_d(static_cast<const VelT<R>*>(a.vel_u), k), double(R(cb1 * a.cdt[t]) * f));
     }
-    vel_out[k] = v;
-    if (vel_ret) vel_ret[k] = v;
-    const double x = q == 0 ? back_to_double(xfx[k], b.l64_0, b.l0)
-                            : (q == 1 ? back_to_double(xfx[k], b.l64_1, b.l1) : back_to_double(xfx[k], b.l64_2, b.l2));
-    pos_out[k] = x;
-    if (pos_ret) pos_ret[k] = x;
+    a.vel_out[k] = v;
+    if (a.vel_ret) a.vel_ret[k] = v;
+    const double x = q == 0 ? back_to_double(a.xfx[k], a.b.l64_0, a.b.l0)
+                            : (q == 1 ? back_to_double(a.xfx[k], a.b.l64_1, a.b.l1) : back_to_double(a.xfx[k], a.b.l64_2, a.b.l2));
+    a.pos_out[k] = x;
+    if (a.pos_ret) a.pos_ret[k] = x;
   }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kThreads) k_finish_md(const __grid_constant__ FinishMd a) {
+  finish_md<R>(a, blockIdx.x, gridDim.x);
+}
+
+// Batches: the three kernels at a call's boundaries for every replica at once
+// (blockIdx.y), from a table filled at the start of the call.
+struct CallArgs {
+  CheckIo check;
+  CallStart start;
+  FinishMd finish;
+  int fp64;
+};
+__global__ void __launch_bounds__(kThreads) k_check_io_batch(const CallArgs* __restrict__ t) {
+  check_io(t[blockIdx.y].check, blockIdx.x, gridDim.x);
+}
+__global__ void __launch_bounds__(32) k_call_start_batch(const CallArgs* __restrict__ t) {
+  call_start(t[blockIdx.x].start);
+}
+__global__ void __launch_bounds__(32) k_post_state_batch(const CallArgs* __restrict__ t) {
+  post_state(t[blockIdx.x].start.st, t[blockIdx.x].start.host);
+}
+__global__ void __launch_bounds__(kThreads) k_finish_md_batch(const CallArgs* __restrict__ t) {
+  const CallArgs& a = t[blockIdx.y];
+  if (a.fp64)
+    finish_md<double>(a.finish, blockIdx.x, gridDim.x);
+  else
+    finish_md<float>(a.finish, blockIdx.x, gridDim.x);
 }
 
 // ----------------------------------------------------------------- launchers
@@ -1459,13 +1527,56 @@ cudaError_t launch_convert(relres_ctx* c, const double* d_pos) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_check_io(relres_ctx* c, const double* d_pos, const double* d_vel) {
-  const int n3 = 3 * c->n;
-  k_check_io<<<std::max(1, std::min((n3 + kThreads - 1) / kThreads, 152 * 8)), kThreads, 0, c->stream>>>(
-      n3, reinterpret_cast<const unsigned long long*>(d_pos), reinterpret_cast<const unsigned long long*>(c->d_pos_ret),
-      reinterpret_cast<const unsigned long long*>(d_vel), reinterpret_cast<const unsigned long long*>(c->d_vel_ret),
-      c->d_state);
+static CheckIo check_args(relres_ctx* c, const StepParams& sp, const double* d_pos, const double* d_vel) {
+  auto words = [](const double* p) { return reinterpret_cast<const unsigned long long*>(p); };
+  return CheckIo{sp.cached ? 3 * c->n : 0, words(d_pos), words(c->d_pos_ret), sp.try_u ? words(d_vel) : nullptr,
+                 words(c->d_vel_ret), c->d_state};
+}
+static CallStart start_args(relres_ctx* c, const StepParams& sp) {
+  return CallStart{c->d_state, c->h_state, c->d_acc, sp.try_u ? 1 : 0};
+}
+static FinishMd finish_args(relres_ctx* c, double* d_pos, double* d_vel) {
+  return FinishMd{3 * c->n, c->d_state, vel_state(c, d_vel), c->d_f_tot, c->d_type, c->d_cdt, c->d_cdt_ff, c->d_xfx,
+                  box_consts(c, 0.0), d_vel, d_pos, c->d_pos_ret, c->fp64 ? nullptr : c->d_vel_ret};
+}
+
+cudaError_t launch_check_io(relres_ctx* c, const StepParams& sp, const double* d_pos, const double* d_vel) {
+  k_check_io<<<std::max(1, std::min((3 * c->n + kThreads - 1) / kThreads, 152 * 8)), kThreads, 0, c->stream>>>(
+      check_args(c, sp, d_pos, d_vel));
   RELRES_LAUNCHED(c);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_call_start(relres_ctx* c, const StepParams& sp) {
+  k_call_start<<<1, 32, 0, c->stream>>>(start_args(c, sp));
+  RELRES_LAUNCHED(c);
+  return cudaGetLastError();
+}
+
+size_t call_table_bytes(int nrep) { return sizeof(CallArgs) * size_t(nrep); }
+
+void fill_call_table(relres_ctx* const* cs, int nrep, const StepParams* sp, double* const* d_pos,
+                     double* const* d_vel, void* host) {
+  CallArgs* const t = static_cast<CallArgs*>(host);
+  for (int r = 0; r < nrep; ++r) {
+    t[r].check = check_args(cs[r], sp[r], d_pos[r], d_vel[r]);
+    t[r].start = start_args(cs[r], sp[r]);
+    t[r].finish = finish_args(cs[r], d_pos[r], d_vel[r]);
+    t[r].fp64 = cs[r]->fp64 ? 1 : 0;
+  }
+}
+
+cudaError_t launch_call_batch(cudaStream_t s, const void* table, relres_ctx* const* cs, int nrep, CallPhase phase) {
+  const CallArgs* const t = static_cast<const CallArgs*>(table);
+  int most = 1;
+  for (int r = 0; r < nrep; ++r) most = std::max(most, cs[r]->n);
+  // a component per thread of the largest replica, at most 16 blocks per SM in all
+  const int nx = std::max(1, std::min((3 * most + kThreads - 1) / kThreads, 152 * 16 / nrep));
+  if (phase == kCallCheck) k_check_io_batch<<<dim3(nx, nrep), kThreads, 0, s>>>(t);
+  if (phase == kCallStart) k_call_start_batch<<<nrep, 32, 0, s>>>(t);
+  if (phase == kCallStatus) k_post_state_batch<<<nrep, 32, 0, s>>>(t);
+  if (phase == kCallFinish) k_finish_md_batch<<<dim3(nx, nrep), kThreads, 0, s>>>(t);
+  for (int r = 0; r < nrep; ++r) RELRES_LAUNCHED(cs[r]);
   return cudaGetLastError();
 }
 
@@ -1809,14 +1920,8 @@ cudaError_t launch_thermo(relres_ctx* c, const StepParams& sp, int k) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_call_start(relres_ctx* c, bool reset_ab) {
-  k_call_start<<<1, 32, 0, c->stream>>>(c->d_state, c->d_acc, reset_ab ? 1 : 0);
-  RELRES_LAUNCHED(c);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_post_state(relres_ctx* c, cudaStream_t stream) {
-  k_post_state<<<1, 32, 0, stream>>>(c->d_state, c->h_state);
+cudaError_t launch_post_state(relres_ctx* c) {
+  k_post_state<<<1, 32, 0, c->stream>>>(c->d_state, c->h_state);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
@@ -1910,17 +2015,11 @@ cudaError_t launch_sum_batch(cudaStream_t s, bool fp64, int k, const BatchLaunch
   return cudaGetLastError();
 }
 
-cudaError_t launch_write_back(relres_ctx* c, double* d_pos, double* d_vel, double dt) {
-  (void)dt;
-  const BoxConsts b = box_consts(c, 0.0);
+cudaError_t launch_write_back(relres_ctx* c, double* d_pos, double* d_vel) {
   if (c->fp64)
-    k_finish_md<double><<<grid_for(3 * c->n), kThreads, 0, c->stream>>>(
-        3 * c->n, c->d_state, static_cast<const double*>(vel_state(c, d_vel)), static_cast<const double*>(c->d_f_tot),
-        c->d_type, c->d_cdt, c->d_cdt_ff, c->d_xfx, b, d_vel, d_pos, c->d_pos_ret, nullptr);
+    k_finish_md<double><<<grid_for(3 * c->n), kThreads, 0, c->stream>>>(finish_args(c, d_pos, d_vel));
   else
-    k_finish_md<float><<<grid_for(3 * c->n), kThreads, 0, c->stream>>>(
-        3 * c->n, c->d_state, static_cast<const float2*>(vel_state(c, d_vel)), static_cast<const float4*>(c->d_f_tot),
-        c->d_type, c->d_cdt, c->d_cdt_ff, c->d_xfx, b, d_vel, d_pos, c->d_pos_ret, c->d_vel_ret);
+    k_finish_md<float><<<grid_for(3 * c->n), kThreads, 0, c->stream>>>(finish_args(c, d_pos, d_vel));
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }

@@ -439,8 +439,8 @@ namespace relres {
 
 // positions
 cudaError_t launch_convert(relres_ctx* c, const double* d_pos);
-cudaError_t launch_check_io(relres_ctx* c, const double* d_pos, const double* d_vel);
-cudaError_t launch_write_back(relres_ctx* c, double* d_pos, double* d_vel, double dt);
+cudaError_t launch_check_io(relres_ctx* c, const StepParams& sp, const double* d_pos, const double* d_vel);
+cudaError_t launch_write_back(relres_ctx* c, double* d_pos, double* d_vel);
 
 // neighbour lists; gate: device flag word (rebuild only if F_REBUILD set) or null
 cudaError_t launch_rebuild(relres_ctx* c, const unsigned* gate);
@@ -490,7 +490,15 @@ cudaError_t launch_end_of_step(relres_ctx* c, const StepParams& sp, int k, bool 
 // start of a block of `count` steps: rollback snapshot and thermostat draws
 cudaError_t launch_block_start(relres_ctx* c, const StepParams& sp, double* d_vel, int count);
 cudaError_t launch_thermo(relres_ctx* c, const StepParams& sp, int k);
-cudaError_t launch_call_start(relres_ctx* c, bool reset_ab);
+// the state to h_state, then the start of a call
+cudaError_t launch_call_start(relres_ctx* c, const StepParams& sp);
+// the same kernels and the status read for all replicas of a batch, from a
+// table of call_table_bytes that fill_call_table writes on the host
+enum CallPhase { kCallCheck, kCallStart, kCallStatus, kCallFinish };
+size_t call_table_bytes(int nrep);
+void fill_call_table(relres_ctx* const* cs, int nrep, const StepParams* sp, double* const* d_pos,
+                     double* const* d_vel, void* host);
+cudaError_t launch_call_batch(cudaStream_t s, const void* table, relres_ctx* const* cs, int nrep, CallPhase phase);
 // FP32 path: caller's velocities -> the float-float state (start of a call)
 cudaError_t launch_vel_in(relres_ctx* c, const double* d_vel);
 // the velocity state of a call: the float-float array (FP32) or the caller's (FP64)
@@ -498,7 +506,7 @@ inline void* vel_state(relres_ctx* c, double* d_vel) {
   return c->fp64 ? static_cast<void*>(d_vel) : static_cast<void*>(c->d_uff);
 }
 // d_state to h_state, once the stream has been waited for
-cudaError_t launch_post_state(relres_ctx* c, cudaStream_t stream);
+cudaError_t launch_post_state(relres_ctx* c);
 cudaError_t launch_flags_and(relres_ctx* c, unsigned keep);
 cudaError_t launch_flags_or(relres_ctx* c, unsigned set);
 // end of a call that refreshed the lists: counts a rebuild, clears the list flags

@@ -122,3 +122,39 @@ def test_backward_right_after_a_build_reads_pruned_lists(torch):
     fr, _, _ = O.pair_forces(s.pos, s.box, s.types, O.table_for(s), s.n_types, s.excl)
     assert _err(g.cpu().numpy(), -fr) <= 1e-10
     ctx.close()
+
+
+def test_batch_calls_continue_or_read_the_arrays_as_each_replica_alone(torch):
+    """Second and third calls with one replica's positions changed, another's velocities, another left alone, an
+    FP64 one, then all with another time step: the bits of every context stepped by itself."""
+    systems = [S.neopentane(n_mol=200, seed=51), S.propane(), S.neopentane(n_mol=120, seed=52), S.propane(seed=53)]
+    prec = [R.RELRES_PREC_FP32] * 3 + [R.RELRES_PREC_FP64]
+
+    def run(batched):
+        ctxs, ps, vs = [], [], []
+        for s, q in zip(systems, prec):
+            ctxs.append(R.Context(R.params_for(s, q), R.topology_for(s)))
+            ps.append(_dev(torch, s.pos))
+            vs.append(_dev(torch, s.vel))
+            ctxs[-1].build_neighbors(ps[-1], s.box)
+        temps, seeds = [s.temperature for s in systems], [3, 4, 5, 6]
+        batch = R.Batch(ctxs) if batched else None
+        for call, dt in enumerate((1.0, 1.0, 0.5)):
+            if call == 1:
+                ps[0] += 0.01
+                vs[1] *= 0.9
+                vs[3] *= 1.1
+            if batched:
+                batch.step(7, dt, ps, vs, temps, 100.0, seeds)
+            else:
+                for c, p, v, t, sd in zip(ctxs, ps, vs, temps, seeds):
+                    c.step(7, dt, p, v, t_target=t, tau_fs=100.0, seed=sd)
+        torch.cuda.synchronize()
+        if batched:
+            batch.close()
+        for c in ctxs:
+            c.close()
+        return [x.cpu().numpy() for x in ps + vs]
+
+    for a, b in zip(run(False), run(True)):
+        assert np.array_equal(a, b)
