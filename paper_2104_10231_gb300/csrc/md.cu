@@ -1814,29 +1814,6 @@ static size_t drift_seg_smem(const relres_ctx* c) {
   return seg_pos_bytes(c->seg_atoms) + size_t(c->seg_slots) * (std::is_same<R, float>::value ? 16 : 24);
 }
 
-// A launch that may overlap the tail of the previous kernel of the stream
-// (programmatic dependent launch) when pdl is set: the kernel waits for that
-// kernel (grid_dependency_wait) before reading what it writes.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(bool pdl, void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
-                              Args... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
-// Programmatic dependent launches only without timing events between the
-// kernels (an event between them would stand in the way).
-static bool pdl_ok(const relres_ctx* c) { return c->use_pdl && !c->timing; }
-
 template <typename R>
 static cudaError_t launch_drift_t(relres_ctx* c, const StepParams& sp, double* d_vel, bool ev, bool after_sum) {
   if (step_segments(c)) {

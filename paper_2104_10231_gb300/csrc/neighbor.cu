@@ -1073,6 +1073,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned* flags) {
 __global__ void __launch_bounds__(kListThreads) k_rebuild(const unsigned* gate, const __grid_constant__ BuildArgs b,
                                                           const __grid_constant__ PruneArgs p, int prune,
                                                           unsigned* bar) {
+  grid_dependents_launch();  // the pair kernel waits for this grid to finish
   const unsigned f = *(volatile const unsigned*)gate;
   if (f & F_NONFINITE) return;  // no lists from such positions
   const int bid = blockIdx.x, nblk = gridDim.x;

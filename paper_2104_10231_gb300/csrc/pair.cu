@@ -125,6 +125,7 @@ __device__ __forceinline__ void pair_block(const PairLaunch& a, int bid) {
   PairRow* const row = reinterpret_cast<PairRow*>(smem_raw);
   copy_words(row, a.tab, a.nt * a.nt * int(sizeof(PairRow) / sizeof(int)));
   const SmemTabs S{row, nullptr};
+  after_rebuild();
   __syncthreads();
   const bool cg = bid < a.nblk_cg;
   const int blk = cg ? bid : bid - a.nblk_cg;
@@ -145,9 +146,6 @@ __device__ __forceinline__ void pair_block(const PairLaunch& a, int bid) {
 
 template <int TPA, int BS, int ACC>
 __global__ void __launch_bounds__(BS, pair_min_blocks(BS)) k_pair(PairLaunch a) {
-  // the force sum that follows may start launching once every block of this
-  // grid runs (it waits for this grid to finish before reading the forces)
-  grid_dependents_launch();
   pair_block<TPA, ACC>(a, blockIdx.x);
 }
 
@@ -170,7 +168,7 @@ static void launch_forces(relres_ctx* c, const PairLaunch& a, int grid, size_t s
   switch (c->pair_cfg) {
 #define RELRES_PAIR_CASE(k, T, B) \
   case k:                         \
-    k_pair<T, B, ACC><<<grid, B, smem, c->stream>>>(a); \
+    launch_pdl(pair_pdl(c, grid, B), k_pair<T, B, ACC>, grid, B, smem, c->stream, a); \
     break;
     RELRES_PAIR_CASE(0, 1, 256)
     RELRES_PAIR_CASE(1, 1, 128)
@@ -235,7 +233,7 @@ static cudaError_t launch_pairs_f32(relres_ctx* c, bool ev, int which) {
   const int grid = make_pair_launch(c, which, per, pairs_prune(c), &a);
   if (grid == 0) return cudaSuccess;
   if (lanes) {
-    launch_pairs_lanes(c->stream, c->force_acc, a, ev, lanes, grid);
+    launch_pairs_lanes(c->stream, c->force_acc, a, ev, lanes, grid, pair_pdl(c, grid, kLaneThreads));
   } else {
     const size_t smem = pair_smem(c->n_types);
     if (c->force_acc == RELRES_ACC_FP32)

@@ -158,6 +158,16 @@ struct SmemTabs {
   const PairRowEnergy* rowe;  // energy steps
 };
 
+// Between a pair kernel's tables and its lists: waits for the kernel before it
+// (the rebuild, see pair_pdl), then lets the force sum that follows start
+// launching once every block of this grid is here (it waits for this grid to
+// finish before reading the forces).  In this order, so that nothing behind
+// this kernel runs while the lists may still change.
+__device__ __forceinline__ void after_rebuild() {
+  grid_dependency_wait();
+  grid_dependents_launch();
+}
+
 // copies n words from global to shared memory with the whole block
 __device__ __forceinline__ void copy_words(void* dst, const void* src, int n) {
   for (int w = threadIdx.x; w < n; w += blockDim.x) static_cast<int*>(dst)[w] = static_cast<const int*>(src)[w];
@@ -242,7 +252,7 @@ __device__ __forceinline__ float pair_term(const int4& pi, const int4& pj, bool 
 // ---- pair_lanes.cu: FP32 launches of kLaneThreads-thread blocks, `lanes`
 // threads per slot (1, 4 or 8; forces only: 4 or 8)
 constexpr int kLaneThreads = 128;
-void launch_pairs_lanes(cudaStream_t s, int acc, const PairLaunch& a, bool ev, int lanes, int grid);
+void launch_pairs_lanes(cudaStream_t s, int acc, const PairLaunch& a, bool ev, int lanes, int grid, bool pdl);
 void launch_pairs_lanes_batch(cudaStream_t s, int acc, bool ev, const BatchLaunch& b, int nrep);
 
 // ---- pair64.cu: FP64 contexts

@@ -314,6 +314,7 @@ __device__ __forceinline__ void block64(const Launch64& a, int bid) {
   copy_words(tab, a.tab, nrow * int(sizeof(PairTab<double>) / sizeof(int)));
   for (int k = threadIdx.x; k < nrow; k += kFp64Block)
     thr[k] = make_float4(float(a.tab[k].rsm2), float(a.tab[k].rsp2), float(a.tab[k].rcm2), float(a.tab[k].rcp2));
+  after_rebuild();
   __syncwarp();
   const bool cg = bid < a.nblk_cg;
   const int slot0 = (cg ? bid : bid - a.nblk_cg) * (32 / T);
@@ -333,7 +334,6 @@ __device__ __forceinline__ void block64(const Launch64& a, int bid) {
 
 template <bool EV, int T>
 __global__ void __launch_bounds__(kFp64Block) k_pair64(Launch64 a) {
-  grid_dependents_launch();  // as k_pair
   block64<EV, T>(a, blockIdx.x);
 }
 
@@ -396,8 +396,8 @@ static int make_launch64(const relres_ctx* c, int which, int per, bool prune, La
   }
 
 template <bool EV, int T>
-static void launch64(cudaStream_t s, const Launch64& a, int grid) {
-  k_pair64<EV, T><<<grid, kFp64Block, smem64<EV>(a.nt), s>>>(a);
+static void launch64(cudaStream_t s, const Launch64& a, int grid, bool pdl) {
+  launch_pdl(pdl, k_pair64<EV, T>, grid, kFp64Block, smem64<EV>(a.nt), s, a);
 }
 template <bool EV, int T>
 static void launch64_batch(cudaStream_t s, const BatchLaunch& b, int nrep) {
@@ -410,7 +410,7 @@ cudaError_t launch_pairs_f64(relres_ctx* c, bool ev, int which) {
   Launch64 a;
   const int grid = make_launch64(c, which, kFp64Block / lanes, pairs_prune(c), &a);
   if (grid == 0) return cudaSuccess;
-  RELRES_LANES64(launch64, c->stream, a, grid)
+  RELRES_LANES64(launch64, c->stream, a, grid, pair_pdl(c, grid, kFp64Block))
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }

@@ -270,6 +270,7 @@ __device__ __forceinline__ void lanes_block(const PairLaunch& a, int bid) {
     tot = reinterpret_cast<PairTotals*>(carve(sizeof(PairTotals)));
   }
   float4* stage = T > 1 ? reinterpret_cast<float4*>(carve(sizeof(float4) * kLaneThreads)) : nullptr;
+  after_rebuild();
   const bool cg = bid < a.nblk_cg;
   const int blk = cg ? bid : bid - a.nblk_cg;
   const bool prn = a.prune_on && (*(volatile const unsigned*)a.gate & (F_REBUILD | F_PRUNE)) != 0u;
@@ -290,7 +291,6 @@ __device__ __forceinline__ void lanes_block(const PairLaunch& a, int bid) {
 // slower at 20 000 atoms, at four 9 % slower), forces only: 64
 template <bool EV, int T, int ACC>
 __global__ void __launch_bounds__(kLaneThreads, EV ? 5 : 8) k_pair_lanes(PairLaunch a) {
-  grid_dependents_launch();  // as k_pair
   lanes_block<EV, T, ACC>(a, blockIdx.x);
 }
 
@@ -302,8 +302,8 @@ __global__ void __launch_bounds__(kLaneThreads, EV ? 5 : 8)
 }
 
 template <bool EV, int T, int ACC>
-static void launch_one(cudaStream_t s, const PairLaunch& a, int grid) {
-  k_pair_lanes<EV, T, ACC><<<grid, kLaneThreads, lanes_smem<EV, T>(a.nt), s>>>(a);
+static void launch_one(cudaStream_t s, const PairLaunch& a, int grid, bool pdl) {
+  launch_pdl(pdl, k_pair_lanes<EV, T, ACC>, grid, kLaneThreads, lanes_smem<EV, T>(a.nt), s, a);
 }
 template <bool EV, int T, int ACC>
 static void launch_batch(cudaStream_t s, const BatchLaunch& b, int nrep) {
@@ -331,8 +331,8 @@ static void launch_batch(cudaStream_t s, const BatchLaunch& b, int nrep) {
     F<true, 1, RELRES_ACC_FP64>(__VA_ARGS__);                     \
   }
 
-void launch_pairs_lanes(cudaStream_t s, int acc, const PairLaunch& a, bool ev, int lanes, int grid) {
-  RELRES_LANES(launch_one, s, a, grid)
+void launch_pairs_lanes(cudaStream_t s, int acc, const PairLaunch& a, bool ev, int lanes, int grid, bool pdl) {
+  RELRES_LANES(launch_one, s, a, grid, pdl)
 }
 
 void launch_pairs_lanes_batch(cudaStream_t s, int acc, bool ev, const BatchLaunch& b, int nrep) {

@@ -590,6 +590,40 @@ inline int fp32_lanes_for(long long slots, int acc, bool ev) {
 }
 inline int fp32_lanes(const relres_ctx* c, bool ev) { return fp32_lanes_for(pair_slots(c), c->force_acc, ev); }
 
+// A launch that may overlap the tail of the previous kernel of the stream
+// (programmatic dependent launch) when pdl is set: the kernel waits for that
+// kernel (grid_dependency_wait) before reading what it writes.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(bool pdl, void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
+                              Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// Programmatic dependent launches only without timing events between the
+// kernels (an event between them would stand in the way).
+inline bool pdl_ok(const relres_ctx* c) { return c->use_pdl && !c->timing; }
+// Pair launches of small systems follow the rebuild kernel that way: launched
+// and with their tables in place while it still looks at the flags (a graph
+// without the fused kernel has a conditional node there, which nothing may
+// follow early).  Forces of a frame, without / with: 44.5 / 42.1 us at 648
+// atoms, 44.1 / 41.4 at 1 715, FP64 62.3 / 58.5; an FP64 MD step of 648 atoms
+// 26.5 / 25.8 us.  Above 256 threads per SM it costs more than it hides (MD
+// steps, without / with: 5 184 atoms FP64 50.5 / 58.6 us, 20 000 atoms FP32
+// 25.1 / 27.8 us).
+inline bool pair_pdl(const relres_ctx* c, int grid, int block) {
+  return pdl_ok(c) && c->use_fused && (long long)grid * block <= 256 * kPartSMs;
+}
+
 // FP64 pair launches (pair64.cu): threads per slot, and one warp per block (a
 // launch is a few blocks per SM long, and the last ones decide: 152.7 against
 // 163.1 us per step with 128-thread blocks at 25 000 neopentane-like atoms).
