@@ -1010,28 +1010,43 @@ __device__ double gauss(unsigned long long key, unsigned long long& c) {
   const double u1 = uniform01(key, c), u2 = uniform01(key, c);
   return sqrt(-2.0 * log(u1)) * cos(6.283185307179586 * u2);
 }
-// Marsaglia & Tsang (2000) gamma(shape, 1) for shape >= 1
-__device__ double gamma_mt(double shape, unsigned long long key, unsigned long long& c) {
-  const double d = shape - 1.0 / 3.0, k = 1.0 / sqrt(9.0 * d);
+// Bussi-Donadio-Parrinello (2007) velocity rescaling.  The two random
+// numbers of step `step` (a normal deviate r1 and a chi-square deviate s with
+// n_f - 1 degrees of freedom, drawn as twice a gamma(n_f/2 - 1/2) deviate by
+// Marsaglia & Tsang (2000): d = shape - 1/3, k = 1 / sqrt(9 d), from the host)
+// depend only on the seed and the step, so a block of steps has them drawn
+// in parallel ahead of time.  Four lanes of a warp share a step: the normal
+// deviates of r1 and of the gamma deviate's first trial and the logarithm of
+// its acceptance test are formed side by side (counters 0-1, 2-3 and 4 of the
+// step), each lane ends with both numbers, and a rejected trial (one in a
+// thousand and less) goes on serially.
+__device__ void csvr_draws(double d, double k, unsigned long long seed, unsigned long long step, double& r1,
+                           double& s) {
+  const int lane = threadIdx.x & 31, j = lane & 3, base = lane & ~3;
+  const unsigned long long c0 = step << 20;
+  unsigned long long c = c0 + (j == 0 ? 0 : (j == 1 ? 2 : 4));
+  const double u1 = uniform01(seed, c), u2 = uniform01(seed, c);
+  const double lu = log(u1);
+  const double g = sqrt(-2.0 * lu) * cos(6.283185307179586 * u2);
+  r1 = __shfl_sync(0xffffffffu, g, base);
+  double x = __shfl_sync(0xffffffffu, g, base + 1);
+  double lt = __shfl_sync(0xffffffffu, lu, base + 2);
+  c = c0 + 4;
   for (int it = 0; it < 1000; ++it) {
-    const double x = gauss(key, c);
+    if (it > 0) x = gauss(seed, c);
     double v = 1.0 + k * x;
     if (v <= 0.0) continue;
     v = v * v * v;
-    if (log(uniform01(key, c)) < 0.5 * x * x + d - d * v + d * log(v)) return d * v;
+    if (it > 0)
+      lt = log(uniform01(seed, c));
+    else
+      ++c;
+    if (lt < 0.5 * x * x + d - d * v + d * log(v)) {
+      s = 2.0 * (d * v);
+      return;
+    }
   }
-  return d;
-}
-// Bussi-Donadio-Parrinello (2007) velocity rescaling.  The two random
-// numbers of step `step` (a normal deviate r1 and a chi-square deviate s with
-// n_f - 1 degrees of freedom, drawn as twice a gamma(n_f/2 - 1/2) deviate)
-// depend only on the seed and the step, so a block of steps has them drawn
-// in parallel ahead of time.
-__device__ void csvr_draws(double n_f, unsigned long long seed, unsigned long long step, double& r1,
-                           double& s) {
-  unsigned long long c = step << 20;
-  r1 = gauss(seed, c);
-  s = 2.0 * gamma_mt(0.5 * (n_f - 1.0), seed, c);
+  s = 2.0 * d;
 }
 // With e = exp(-dt / tau) (computed once per call on the host) the rescaled
 // kinetic energy is K' = e K + A + B sqrt(K), where A and B hold the random
@@ -1049,19 +1064,22 @@ __device__ __forceinline__ double csvr_alpha(double ke, double e, double ca, dou
 }
 
 // Start of a block of steps: the rollback snapshot of positions, velocity
-// state, forces and DevState, and beside it (block 0) the thermostat terms
-// (A, B) of the steps st->step + k, k < count, one thread each.  One launch:
-// four copies and then the draws, one after the other, took 18 us of a 122 us
-// one-step call at 140 000 atoms.
+// state, forces and DevState, and beside it (the first blocks) the thermostat
+// terms (A, B) of the steps st->step + k, k < count, 32 steps to a block.  One
+// launch: four copies and then the draws, one after the other, took 18 us of a
+// 122 us one-step call at 140 000 atoms, draws of one thread a step beside the
+// copies 9.8 us, as here 6.2 us.
 struct BlockStart {
   const unsigned long long* src[3];
   unsigned long long* dst[3];
   long long words[3];  // 8-byte words
   const DevState* st;
   DevState* snap;
-  double n_f, kt, e;
+  double gd, gk;         // gamma deviate (csvr_draws)
+  double scale_a, scale_b;  // A = scale_a (r1^2 + s), B = scale_b r1
   unsigned long long seed;
-  int count;  // 0: no thermostat
+  int count;   // 0: no thermostat
+  int ndraw;   // blocks that draw (at least one: it copies DevState)
   double* draws;
 };
 
@@ -1077,21 +1095,26 @@ __device__ __forceinline__ void copy_words64(unsigned long long* dst, const unsi
   }
 }
 
+constexpr int kDrawSteps = 32;  // steps per drawing block, four lanes each
+
 __device__ __forceinline__ void block_start(const BlockStart& a, int bid, int nblk) {
-  if (bid == 0) {
-    const int k = threadIdx.x;
+  if (bid < a.ndraw) {
     constexpr int kWords = int(sizeof(DevState) / 8);
-    static_assert(sizeof(DevState) % 8 == 0 && kBlockSteps <= kThreads, "one block");
-    for (int w = k; w < kWords; w += kThreads)
-      reinterpret_cast<unsigned long long*>(a.snap)[w] = reinterpret_cast<const unsigned long long*>(a.st)[w];
-    if (k >= a.count) return;
+    static_assert(sizeof(DevState) % 8 == 0 && 4 * kDrawSteps <= kThreads, "whole words, one block");
+    if (bid == 0)
+      for (int w = threadIdx.x; w < kWords; w += kThreads)
+        reinterpret_cast<unsigned long long*>(a.snap)[w] = reinterpret_cast<const unsigned long long*>(a.st)[w];
+    const int k = kDrawSteps * bid + int(threadIdx.x >> 2);
+    if (a.count == 0 || threadIdx.x >= 4 * kDrawSteps) return;  // whole warps
     double r1, s;
-    csvr_draws(a.n_f, a.seed, a.st->step + (unsigned long long)k, r1, s);
-    a.draws[2 * k] = (1.0 - a.e) * (a.kt / a.n_f) * (r1 * r1 + s);
-    a.draws[2 * k + 1] = 2.0 * r1 * sqrt(a.e * (1.0 - a.e) * (a.kt / a.n_f));
+    csvr_draws(a.gd, a.gk, a.seed, a.st->step + (unsigned long long)k, r1, s);
+    if (k >= a.count || (threadIdx.x & 3) != 0) return;
+    a.draws[2 * k] = a.scale_a * (r1 * r1 + s);
+    a.draws[2 * k + 1] = 2.0 * r1 * a.scale_b;
     return;
   }
-  const long long first = (long long)(bid - 1) * kThreads + threadIdx.x, stride = (long long)(nblk - 1) * kThreads;
+  const long long first = (long long)(bid - a.ndraw) * kThreads + threadIdx.x,
+                  stride = (long long)(nblk - a.ndraw) * kThreads;
 #pragma unroll
   for (int q = 0; q < 3; ++q) copy_words64(a.dst[q], a.src[q], a.words[q], first, stride);
 }
@@ -1379,7 +1402,8 @@ __device__ __forceinline__ double force_component(const double* f, int, int, int
 
 // End of a call: positions and velocities to the caller, and copies of both.
 // One component per thread, so that every array is read and written in whole
-// lines (one atom per thread: 9.3 us at 140 000 atoms, 36 us at a million).
+// lines (140 000 atoms: 7.4 us, one atom per thread 9.3; a million atoms: 37 us
+// either way, 60 % of the copy rate).
 struct FinishMd {
   int n3;
   const DevState* st;
@@ -1398,32 +1422,40 @@ struct FinishMd {
 
 template <typename R>
 __device__ __forceinline__ void finish_md(const FinishMd& a, int bid, int nblk) {
+  const VelT<R>* vel_u = static_cast<const VelT<R>*>(a.vel_u);  // FP64: also written (vel_out)
+  const ForceT<R>* __restrict__ f_tot = static_cast<const ForceT<R>*>(a.f_tot);
+  const int* __restrict__ type = a.type;
+  const unsigned long long* __restrict__ xfx = a.xfx;
+  double* const vel_out = a.vel_out;
+  double* const vel_ret = a.vel_ret;
+  double* __restrict__ const pos_out = a.pos_out;
+  double* __restrict__ const pos_ret = a.pos_ret;
+  const ff ca{a.st->a_hi, a.st->a_lo}, cb1 = ff_add(ff{a.st->b_hi, a.st->b_lo}, ff{-1.f, 0.f});
+  const double da = a.st->a, db1 = a.st->b - 1.0;
   for (int k = bid * kThreads + threadIdx.x; k < a.n3; k += nblk * kThreads) {
     const int i = k / 3, q = k - 3 * i;
-    const int t = a.type[i];
-    const R f = force_component(static_cast<const ForceT<R>*>(a.f_tot), i, q, k);
+    const int t = type[i];
+    const R f = force_component(f_tot, i, q, k);
+    const unsigned long long ux = xfx[k];
     double v;
     if constexpr (std::is_same<R, float>::value) {
       // v = a u + (b - 1) c F in float-float, returned as the double nearest
       // to hi + lo: the parts converted exactly with integer operations, one
       // FP64 addition
-      const ff ca{a.st->a_hi, a.st->a_lo};
-      const ff cb1 = ff_add(ff{a.st->b_hi, a.st->b_lo}, ff{-1.f, 0.f});
       const float2 cc = a.cdt_ff[t];
       const ff cbc = ff_mul(cb1, ff{cc.x, cc.y});
-      const float2 u = static_cast<const VelT<R>*>(a.vel_u)[k];
+      const float2 u = vel_u[k];
       const ff w = ff_add(ff_mul(ca, ff{u.x, u.y}), ff_mul_f(cbc, f));
       v = double_of_float(w.hi) + double_of_float(w.lo);
     } else {
-      const double ca = a.st->a, cb1 = a.st->b - 1.0;
-      v = fma(ca, vel_d(static_cast<const VelT<R>*>(a.vel_u), k), double(R(cb1 * a.cdt[t]) * f));
+      v = fma(da, vel_d(vel_u, k), double(R(db1 * a.cdt[t]) * f));
     }
-    a.vel_out[k] = v;
-    if (a.vel_ret) a.vel_ret[k] = v;
-    const double x = q == 0 ? back_to_double(a.xfx[k], a.b.l64_0, a.b.l0)
-                            : (q == 1 ? back_to_double(a.xfx[k], a.b.l64_1, a.b.l1) : back_to_double(a.xfx[k], a.b.l64_2, a.b.l2));
-    a.pos_out[k] = x;
-    if (a.pos_ret) a.pos_ret[k] = x;
+    const double x = q == 0 ? back_to_double(ux, a.b.l64_0, a.b.l0)
+                            : (q == 1 ? back_to_double(ux, a.b.l64_1, a.b.l1) : back_to_double(ux, a.b.l64_2, a.b.l2));
+    vel_out[k] = v;
+    if (vel_ret) vel_ret[k] = v;
+    pos_out[k] = x;
+    if (pos_ret) pos_ret[k] = x;
   }
 }
 
@@ -1701,6 +1733,10 @@ cudaError_t launch_reduce_out(relres_ctx* c, double* d_energy, double* d_virial)
   return cudaGetLastError();
 }
 
+static int block_start_draws(int count) { return std::max(1, (count + kDrawSteps - 1) / kDrawSteps); }
+// blocks of a snapshot of n atoms: 8 words of each array per thread
+static int block_start_copies(int n) { return std::max(1, std::min((3 * n / 8 + kThreads - 1) / kThreads, 152 * 8)); }
+
 static BlockStart block_start_args(relres_ctx* c, const StepParams& sp, double* d_vel, int count) {
   BlockStart a{};
   const long long n3 = 3LL * c->n;
@@ -1714,20 +1750,20 @@ static BlockStart block_start_args(relres_ctx* c, const StepParams& sp, double* 
   a.words[2] = c->fp64 ? n3 : 2LL * c->n;
   a.st = c->d_state;
   a.snap = c->d_snap_state;
-  a.n_f = sp.n_f;
-  a.kt = sp.kt;
-  a.e = sp.csvr_e;
+  const double unit = sp.kt / sp.n_f;
+  a.gd = 0.5 * (sp.n_f - 1.0) - 1.0 / 3.0;
+  a.gk = 1.0 / std::sqrt(9.0 * a.gd);
+  a.scale_a = (1.0 - sp.csvr_e) * unit;
+  a.scale_b = std::sqrt(sp.csvr_e * (1.0 - sp.csvr_e) * unit);
   a.seed = sp.seed;
   a.count = sp.t_target > 0.0 ? count : 0;
+  a.ndraw = block_start_draws(count);
   a.draws = c->d_draws;
   return a;
 }
 
-// blocks of a snapshot of n atoms: the draws, and 8 words of each array per thread
-static int block_start_blocks(int n) { return 1 + std::max(1, std::min((3 * n / 8 + kThreads - 1) / kThreads, 152 * 8)); }
-
 cudaError_t launch_block_start(relres_ctx* c, const StepParams& sp, double* d_vel, int count) {
-  k_block_start<<<block_start_blocks(c->n), kThreads, 0, c->stream>>>(block_start_args(c, sp, d_vel, count));
+  k_block_start<<<block_start_draws(count) + block_start_copies(c->n), kThreads, 0, c->stream>>>(block_start_args(c, sp, d_vel, count));
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
@@ -1735,11 +1771,12 @@ cudaError_t launch_block_start(relres_ctx* c, const StepParams& sp, double* d_ve
 cudaError_t prepare_block_start_batch(const std::vector<relres_ctx*>& cs, const std::vector<StepParams>& sp,
                                       double* const* d_vel, int count, BatchLaunch* b) {
   std::vector<BlockStart> args(cs.size());
-  b->nblk = 1;
+  int copies = 1;
   for (size_t r = 0; r < cs.size(); ++r) {
     args[r] = block_start_args(cs[r], sp[r], d_vel[r], count);
-    b->nblk = std::max(b->nblk, std::min(block_start_blocks(cs[r]->n), 17));
+    copies = std::max(copies, std::min(block_start_copies(cs[r]->n), 16));
   }
+  b->nblk = block_start_draws(count) + copies;
   return upload_batch(b, args.data(), sizeof(BlockStart) * args.size(), {0, int(cs.size())});
 }
 
@@ -1994,9 +2031,9 @@ cudaError_t launch_sum_batch(cudaStream_t s, bool fp64, int k, const BatchLaunch
 
 cudaError_t launch_write_back(relres_ctx* c, double* d_pos, double* d_vel) {
   if (c->fp64)
-    k_finish_md<double><<<grid_for(3 * c->n), kThreads, 0, c->stream>>>(finish_args(c, d_pos, d_vel));
+    k_finish_md<double><<<(3 * c->n + kThreads - 1) / kThreads, kThreads, 0, c->stream>>>(finish_args(c, d_pos, d_vel));
   else
-    k_finish_md<float><<<grid_for(3 * c->n), kThreads, 0, c->stream>>>(finish_args(c, d_pos, d_vel));
+    k_finish_md<float><<<(3 * c->n + kThreads - 1) / kThreads, kThreads, 0, c->stream>>>(finish_args(c, d_pos, d_vel));
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
