@@ -82,7 +82,7 @@ def workload_config(args, n_atoms, box):
         "l2": "inputs larger than L2 (neighbour lists ~0.5 GB, state 64 MB)",
         "parallelism": "replicas only (one independent system per GPU)",
         "thermo_every": args.thermo_every,
-        "execution": "stream launches" if args.no_graphs else "CUDA graph per 100 steps, conditional rebuild node",
+        "execution": "stream launches" if args.no_graphs else "CUDA graph per 100 steps, cooperative rebuild kernel",
         "lists": (f"rebuilt at skin/2 = 1 A displacement; pair kernels walk lists pruned to the cutoff + "
                   f"{args.prune} A, re-pruned at {args.prune / 2} A displacement") if args.prune > 0 else
                  "rebuilt at skin/2 = 1 A displacement; pair kernels walk the full lists",

@@ -441,7 +441,7 @@ relres_status relres_set_prune(relres_ctx* ctx, double delta);
  * one CUDA graph launch.  Where the replicas allow it (relres_batch_get_info)
  * each step is one drift, one pair and one force-sum launch covering every
  * replica (each kernel finds its replica from a table of block offsets), with
- * each replica's list rebuild a conditional node opened by one decide kernel;
+ * the list rebuilds of the replicas that need one behind one conditional node;
  * otherwise every replica's block sits on its own branch of the graph.
  * Results are bit-identical to stepping each context alone with the same
  * arguments.  If any replica's list overflows, every replica returns to the
