@@ -315,8 +315,8 @@ relres_status forces_now(relres_ctx* c, int ev_mode, double* d_forces, double* d
     TIMED(RELRES_T_FINISH, launch_finish(c, ev_mode == 1, d_forces, nullptr, true));
     if (ev_mode == 1) TIMED(RELRES_T_THERMO, launch_reduce_out(c, d_energy, d_virial));
     c->prune_pending = false;
-    s = read_state(c);
-    if (s != RELRES_OK) return s;
+    if (ev_mode != 1) CK(launch_post_state(c));  // launch_reduce_out has done it
+    CK(cudaStreamSynchronize(c->stream));
     s = flush_timing(c);
     if (s != RELRES_OK) return s;
     s = check_evaluation(c, &retry);

@@ -1316,25 +1316,34 @@ __global__ void __launch_bounds__(kThreads) k_sum_batch(const SumArgs<R>* __rest
   sum_block<R>(args[r], int(blockIdx.x) - off[r], off[r + 1] - off[r], k);
 }
 
-// Energies and virial of relres_compute (one thread); clears the accumulators.
-__global__ void k_reduce_out(long long* acc, double* energy, int with_e, double* virial, int with_w,
-                             const DevState* st) {
+// The state to the host's pinned copy, written by a kernel: a copy of these
+// few words as a transfer of its own starts 5 us behind the kernel before it,
+// this one follows like any launch.
+__device__ __forceinline__ void post_state(const DevState* st, DevState* host) {
+  for (int w = threadIdx.x; w < int(sizeof(DevState) / 8); w += 32)
+    reinterpret_cast<unsigned long long*>(host)[w] = reinterpret_cast<const unsigned long long*>(st)[w];
+}
+
+// Energies and virial of relres_compute (one warp: lane 0 the energies, lanes
+// 1-6 the virial), the accumulators cleared, and the state to the host.
+__global__ void __launch_bounds__(32) k_reduce_out(long long* acc, double* energy, int with_e, double* virial,
+                                                   int with_w, const DevState* st, DevState* host) {
   if (bad_positions(st)) with_e = with_w = 0;
-  const double efg = acc_value(acc[kAccFg], acc[kNAcc + kAccFg]), ecg = acc_value(acc[kAccCg], acc[kNAcc + kAccCg]);
-  const double eb = double(acc[kAccEb]) / kFix;
-  if (with_e) {
+  const int q = threadIdx.x;
+  if (q == 0 && with_e) {
+    const double efg = acc_value(acc[kAccFg], acc[kNAcc + kAccFg]), ecg = acc_value(acc[kAccCg], acc[kNAcc + kAccCg]);
+    const double eb = double(acc[kAccEb]) / kFix;
     energy[0] = efg;
     energy[1] = ecg;
     energy[2] = eb;
     energy[3] = efg + ecg + eb;
   }
-  if (with_w)
-#pragma unroll
-    for (int q = 1; q < kNQ; ++q)
-      virial[q - 1] =
-          acc_value(acc[kAccFg + q] + acc[kAccCg + q], acc[kNAcc + kAccFg + q] + acc[kNAcc + kAccCg + q]);
-#pragma unroll
-  for (int q = 0; q < kNAccAll; ++q) acc[q] = 0;
+  if (q >= 1 && q < kNQ && with_w)
+    virial[q - 1] =
+        acc_value(acc[kAccFg + q] + acc[kAccCg + q], acc[kNAcc + kAccFg + q] + acc[kNAcc + kAccCg + q]);
+  __syncwarp();
+  for (int k = q; k < kNAccAll; k += 32) acc[k] = 0;
+  post_state(st, host);
 }
 
 // Start of a relres_step call: the state (with the flags of k_check_io) to the
@@ -1348,14 +1357,6 @@ struct CallStart {
   long long* acc;
   int try_u;  // the velocity state continues if the arrays are the ones returned last
 };
-
-// The state to the host's pinned copy, written by a kernel: a copy of these
-// few words as a transfer of its own starts 5 us behind the kernel before it,
-// this one follows like any launch.
-__device__ __forceinline__ void post_state(const DevState* st, DevState* host) {
-  for (int w = threadIdx.x; w < int(sizeof(DevState) / 8); w += 32)
-    reinterpret_cast<unsigned long long*>(host)[w] = reinterpret_cast<const unsigned long long*>(st)[w];
-}
 
 __device__ __forceinline__ void call_start(const CallStart& a) {
   post_state(a.st, a.host);
@@ -1727,8 +1728,8 @@ cudaError_t launch_finish(relres_ctx* c, bool ev, double* d_forces_out, const do
 
 cudaError_t launch_reduce_out(relres_ctx* c, double* d_energy, double* d_virial) {
   double* dd = static_cast<double*>(c->d_dummy);
-  k_reduce_out<<<1, 1, 0, c->stream>>>(c->d_acc, d_energy ? d_energy : dd, d_energy ? 1 : 0,
-                                       d_virial ? d_virial : dd, d_virial ? 1 : 0, c->d_state);
+  k_reduce_out<<<1, 32, 0, c->stream>>>(c->d_acc, d_energy ? d_energy : dd, d_energy ? 1 : 0,
+                                        d_virial ? d_virial : dd, d_virial ? 1 : 0, c->d_state, c->h_state);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }

@@ -349,6 +349,7 @@ struct relres_ctx {
   bool use_seg = true;  // the fused kernel where segments exist (relres_set_option)
   // force sum and drift as programmatic dependent launches (untimed steps)
   bool use_pdl = true;
+  int rebuild_per_sm = 0;  // blocks of k_rebuild an SM holds (0: not asked yet)
   // reductions: 64-bit fixed-point accumulators (kNAccAll), cleared by their reader
   long long* d_acc = nullptr;
   double* d_draws = nullptr;  // CSVR random numbers of the current block of steps, 2 per step
