@@ -175,7 +175,7 @@ typedef struct relres_stats {
   int pair_tpa, pair_block;      /* forces-only pair kernel: threads per atom and block size of its launch
                                     configuration (small FP32 systems left to configuration -1 run
                                     configuration 0 with several lanes per atom, and FP64 systems below
-                                    5000 atoms run 16 or 32 where this says 8: the same force bits) */
+                                    8500 atoms and CG sites run 16 or 32 where this says 8: the same force bits) */
   double prune_delta;            /* pruning margin in Angstrom (0: pruning off) */
   long long n_prunes;            /* pruning passes since create (each build is followed by one) */
   double mean_fg_pruned, mean_cg_pruned;  /* mean pruned list length over all passes */

@@ -630,16 +630,16 @@ inline bool pair_pdl(const relres_ctx* c, int grid, int block) {
 // 163.1 us per step with 128-thread blocks at 25 000 neopentane-like atoms).
 // The fewer the slots, the more threads take one, so that every SM has a few
 // warps; us per step with 32 / 16 / 8 / 4 threads, forces only: 864 slots
-// 29.5 / 33.3 / 39.6 / -, 2058 slots 35.4 / 35.3 / 38.4 / -, 6000 slots 57 /
-// 49.4 / 48.0 / -, 12 000 slots 90 / 75 / 67 / -, 30 000 slots - / - / 134 /
-// 119; steps with energies, ten sums per slot instead of three: 864 slots 40 /
-// 45 / 59 / -, 2058 slots 45 / 47 / 56 / -, 6000 slots 70 / 64 / 69 / -,
-// 12 000 slots 109 / 93 / 103 / -, 30 000 slots - / - / 190 / 178.
-// The force bits are the same for all of them.
+// 25.7 / 29.6 / 36.9 / 50.8, 2058 slots 30.7 / 31.5 / 36.1 / 47.2, 6000 slots
+// 48.4 / 42.6 / 44.9 / 54.8, 12 000 slots 73.3 / 64.4 / 62.3 / 64.6, 30 000
+// slots 145 / 123 / 126 / 116; steps with energies, ten sums per slot instead
+// of three, with 32 / 16 / 4: 864 slots 36.2 / 41.6 / 76.1, 2058 slots 41.8 /
+// 45.3 / 71.4, 6000 slots 64.1 / 62.4 / 86.9, 12 000 slots 98.9 / 91.3 / 96.9,
+// 30 000 slots 206 / 183 / 174.  The force bits are the same for all of them.
 constexpr int kFp64Block = 32;
 inline int fp64_lanes_for(long long slots, bool ev) {
-  if (slots < (ev ? 24 : 12) * kPartSMs) return 32;
-  if (slots < (ev ? 128 : 32) * kPartSMs) return 16;
+  if (slots < (ev ? 24 : 16) * kPartSMs) return 32;
+  if (slots < (ev ? 128 : 56) * kPartSMs) return 16;
   return slots < 128 * kPartSMs ? 8 : 4;
 }
 inline int fp64_lanes(const relres_ctx* c, bool ev) { return fp64_lanes_for(pair_slots(c), ev); }

@@ -112,7 +112,7 @@ def test_overlapping_atoms_keep_their_energy(torch):
 
 
 def test_fp64_batch_keeps_the_bits_of_each_replica_alone(torch):
-    """FP64 replicas that alone take eight lanes per list and together four."""
+    """FP64 replicas that alone take eight lanes per list or more and together four."""
     systems = [S.neopentane(n_mol=1000, seed=31), S.propane(n_mol=1000, box=53.0, seed=32),
                S.neopentane(n_mol=2000, seed=33), S.neopentane(n_mol=400, seed=34)]
     temps, seeds = [s.temperature for s in systems], [5, 6, 7, 8]
@@ -144,7 +144,7 @@ def test_fp64_batch_keeps_the_bits_of_each_replica_alone(torch):
 
 
 def test_fp64_lanes_by_size_keep_the_bits(torch):
-    """32, 16 and 8 threads per slot alone (energy steps 32, 32 and 16), four in one batch."""
+    """32, 32, 16 and 8 threads per slot alone (energy steps 32, 32, 16 and 16), four in one batch."""
     systems = [S.propane(), S.neopentane(n_mol=400, seed=41), S.neopentane(n_mol=1000, seed=42),
                S.neopentane(n_mol=2000, seed=43)]
 
