@@ -1123,7 +1123,7 @@ __global__ void __launch_bounds__(kThreads) k_block_start(const __grid_constant_
   block_start(a, blockIdx.x, gridDim.x);
 }
 __global__ void __launch_bounds__(kThreads) k_block_start_batch(const BlockStart* __restrict__ args) {
-  block_start(args[blockIdx.y], blockIdx.x, gridDim.x);
+  block_start(args[blockIdx.x], blockIdx.y, gridDim.y);
 }
 
 // total of an accumulator and the finer one beside it
@@ -1466,7 +1466,8 @@ __global__ void __launch_bounds__(kThreads) k_finish_md(const __grid_constant__ 
 }
 
 // Batches: the three kernels at a call's boundaries for every replica at once
-// (blockIdx.y), from a table filled at the start of the call.
+// (blockIdx.x: no limit on their number in practice), from a table filled at
+// the start of the call.
 struct CallArgs {
   CheckIo check;
   CallStart start;
@@ -1474,7 +1475,7 @@ struct CallArgs {
   int fp64;
 };
 __global__ void __launch_bounds__(kThreads) k_check_io_batch(const CallArgs* __restrict__ t) {
-  check_io(t[blockIdx.y].check, blockIdx.x, gridDim.x);
+  check_io(t[blockIdx.x].check, blockIdx.y, gridDim.y);
 }
 __global__ void __launch_bounds__(32) k_call_start_batch(const CallArgs* __restrict__ t) {
   call_start(t[blockIdx.x].start);
@@ -1483,11 +1484,11 @@ __global__ void __launch_bounds__(32) k_post_state_batch(const CallArgs* __restr
   post_state(t[blockIdx.x].start.st, t[blockIdx.x].start.host);
 }
 __global__ void __launch_bounds__(kThreads) k_finish_md_batch(const CallArgs* __restrict__ t) {
-  const CallArgs& a = t[blockIdx.y];
+  const CallArgs& a = t[blockIdx.x];
   if (a.fp64)
-    finish_md<double>(a.finish, blockIdx.x, gridDim.x);
+    finish_md<double>(a.finish, blockIdx.y, gridDim.y);
   else
-    finish_md<float>(a.finish, blockIdx.x, gridDim.x);
+    finish_md<float>(a.finish, blockIdx.y, gridDim.y);
 }
 
 // ----------------------------------------------------------------- launchers
@@ -1605,10 +1606,10 @@ cudaError_t launch_call_batch(cudaStream_t s, const void* table, relres_ctx* con
   for (int r = 0; r < nrep; ++r) most = std::max(most, cs[r]->n);
   // a component per thread of the largest replica, at most 16 blocks per SM in all
   const int nx = std::max(1, std::min((3 * most + kThreads - 1) / kThreads, 152 * 16 / nrep));
-  if (phase == kCallCheck) k_check_io_batch<<<dim3(nx, nrep), kThreads, 0, s>>>(t);
+  if (phase == kCallCheck) k_check_io_batch<<<dim3(nrep, nx), kThreads, 0, s>>>(t);
   if (phase == kCallStart) k_call_start_batch<<<nrep, 32, 0, s>>>(t);
   if (phase == kCallStatus) k_post_state_batch<<<nrep, 32, 0, s>>>(t);
-  if (phase == kCallFinish) k_finish_md_batch<<<dim3(nx, nrep), kThreads, 0, s>>>(t);
+  if (phase == kCallFinish) k_finish_md_batch<<<dim3(nrep, nx), kThreads, 0, s>>>(t);
   for (int r = 0; r < nrep; ++r) RELRES_LAUNCHED(cs[r]);
   return cudaGetLastError();
 }
@@ -1782,7 +1783,7 @@ cudaError_t prepare_block_start_batch(const std::vector<relres_ctx*>& cs, const 
 }
 
 cudaError_t launch_block_start_batch(cudaStream_t s, const BatchLaunch& b, int nrep) {
-  k_block_start_batch<<<dim3(b.nblk, nrep), kThreads, 0, s>>>(static_cast<const BlockStart*>(b.d_args));
+  k_block_start_batch<<<dim3(nrep, b.nblk), kThreads, 0, s>>>(static_cast<const BlockStart*>(b.d_args));
   return cudaGetLastError();
 }
 
