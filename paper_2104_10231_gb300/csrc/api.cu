@@ -130,11 +130,14 @@ relres_status alloc_lists(relres_ctx* c) {
   // pruned lists: same layout and capacity (a pruned list is never longer)
   c->prune_on = c->prune_delta > 0.0;
   if (c->prune_on) {
+    // empty until the first pruning pass
     CK(dalloc(&c->d_nbr_fg_in, size_t(c->cap_fg) * c->n));
     CK(dalloc(&c->d_cnt_fg_in, size_t(c->n)));
+    CK(cudaMemsetAsync(c->d_cnt_fg_in, 0, sizeof(int) * c->n, c->stream));
     if (c->has_cg && c->n_h > 0) {
       CK(dalloc(&c->d_nbr_cg_in, size_t(c->cap_cg) * c->n_h));
       CK(dalloc(&c->d_cnt_cg_in, size_t(c->n_h)));
+      CK(cudaMemsetAsync(c->d_cnt_cg_in, 0, sizeof(int) * c->n_h, c->stream));
     }
   } else {
     dfree(c->d_nbr_fg_in);
@@ -266,6 +269,8 @@ relres_status refresh_lists(relres_ctx* c, bool prune) {
 relres_status check_evaluation(relres_ctx* c, bool* retry) {
   *retry = false;
   const unsigned fl = c->h_state->flags;
+  // a pruning pass left over by a build has run, unless the positions were bad
+  if (!(fl & F_BADPOS)) c->prune_pending = false;
   if (fl & F_BADCELL) return fail(c, RELRES_ERR_CUDA, "cell binning produced an out-of-range index");
   if (fl & F_BARRIER) return barrier_timeout(c);
   if (fl & F_NONFINITE) {
@@ -297,7 +302,6 @@ relres_status forces_now(relres_ctx* c, int ev_mode, double* d_forces, double* d
     relres_status s = refresh_lists(c, true);
     if (s != RELRES_OK) return s;
     CK(launch_close_call(c));
-    c->prune_pending = false;
     s = read_state(c);
     bool retry;
     if (s == RELRES_OK) s = check_evaluation(c, &retry);
@@ -314,7 +318,6 @@ relres_status forces_now(relres_ctx* c, int ev_mode, double* d_forces, double* d
     TIMED(ev_mode == 1 ? RELRES_T_PAIR_EV : RELRES_T_PAIR, launch_pairs(c, ev_mode == 1));
     TIMED(RELRES_T_FINISH, launch_finish(c, ev_mode == 1, d_forces, nullptr, true));
     if (ev_mode == 1) TIMED(RELRES_T_THERMO, launch_reduce_out(c, d_energy, d_virial));
-    c->prune_pending = false;
     if (ev_mode != 1) CK(launch_post_state(c));  // launch_reduce_out has done it
     CK(cudaStreamSynchronize(c->stream));
     s = flush_timing(c);
@@ -1322,7 +1325,6 @@ relres_status relres_backward(relres_ctx* c, const double* d_pos, const double* 
     if (s != RELRES_OK) return s;
     CK(launch_pair_grad(c, d_grad_forces, grad_energy, d_grad_pos));
     CK(launch_close_call(c));
-    c->prune_pending = false;
     CK(cudaMemcpyAsync(gc.data(), c->d_gc, sizeof(double) * gc.size(), cudaMemcpyDeviceToHost, c->stream));
     s = read_state(c);
     if (s != RELRES_OK) return s;

@@ -121,6 +121,7 @@ struct GradLaunch {
   float sxl, syl, szl;  // FP32: lo parts of L / 2^32
   R g_energy;
   double* gc;  // [nt*nt][4]: dL/dC12_FG, dL/dC6_FG, dL/dC12_CG, dL/dC6_CG
+  const unsigned* flags;  // F_BADPOS: the rebuild kernel left the lists alone, no walk
 };
 
 constexpr int kGradThreads = 128;
@@ -244,6 +245,7 @@ __device__ __forceinline__ void grad_walk(const GradWalk<R>& W, int blk, const B
 template <typename R, int T>
 __global__ void __launch_bounds__(kGradThreads) k_pair_grad(GradLaunch<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (*(volatile const unsigned*)a.flags & F_BADPOS) return;
   const int nrow = a.nt * a.nt;
   double* s_gc = reinterpret_cast<double*>(smem_raw);
   R(*s_acc)[kGradThreads] = reinterpret_cast<R(*)[kGradThreads]>(s_gc + 2 * nrow);
@@ -339,6 +341,7 @@ static cudaError_t launch_grad_t(relres_ctx* c, const double* d_grad_forces, dou
   a.tab = static_cast<const BasisTab<R>*>(c->d_basis);
   a.g_energy = R(g_energy);
   a.gc = c->d_gc;
+  a.flags = &c->d_state->flags;
   const GPos<R>* pfg;
   const GPos<R>* pcg;
   if constexpr (std::is_same<R, float>::value) {

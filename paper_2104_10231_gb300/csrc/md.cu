@@ -533,11 +533,15 @@ struct FinishArgs {
 };
 
 // End of a force evaluation that is a call of its own: the lists are those of
-// these positions now (one thread, after the pair kernel).
+// these positions now (one thread, after the pair kernel).  After a non-finite
+// position they are still those of the call before: the displacement triggers
+// are worked out again from the next positions, but a pruning pass that was
+// due may be one that a build left over, so it stays due.
 __device__ __forceinline__ void close_host_call(DevState* st) {
   const unsigned f = *(volatile unsigned*)&st->flags;
-  if ((f & F_REBUILD) && !(f & F_BADPOS)) st->n_builds += 1;
-  atomicAnd(&st->flags, ~unsigned(F_REBUILD | F_PRUNE));
+  const bool bad = (f & F_BADPOS) != 0u;
+  if ((f & F_REBUILD) && !bad) st->n_builds += 1;
+  atomicAnd(&st->flags, bad ? ~unsigned(F_REBUILD) : ~unsigned(F_REBUILD | F_PRUNE));
 }
 __device__ __forceinline__ bool bad_positions(const DevState* st) {
   return (*(volatile const unsigned*)&st->flags & F_BADPOS) != 0u;

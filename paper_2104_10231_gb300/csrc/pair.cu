@@ -126,6 +126,7 @@ __device__ __forceinline__ void pair_block(const PairLaunch& a, int bid) {
   copy_words(row, a.tab, a.nt * a.nt * int(sizeof(PairRow) / sizeof(int)));
   const SmemTabs S{row, nullptr};
   after_rebuild();
+  if (lists_unpruned(a)) return;
   __syncthreads();
   const bool cg = bid < a.nblk_cg;
   const int blk = cg ? bid : bid - a.nblk_cg;

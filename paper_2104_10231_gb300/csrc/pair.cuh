@@ -168,6 +168,14 @@ __device__ __forceinline__ void after_rebuild() {
   grid_dependents_launch();
 }
 
+// A launch whose lists were to be pruned by a pass of their own (or that walks
+// the full lists) behind a non-finite position: the pass did not run, so the
+// pruned lists may never have been written.  The call fails without reading
+// these forces.
+__device__ __forceinline__ bool lists_unpruned(const PairLaunch& a) {
+  return !a.prune_on && (*(volatile const unsigned*)a.gate & F_BADPOS) != 0u;
+}
+
 // copies n words from global to shared memory with the whole block
 __device__ __forceinline__ void copy_words(void* dst, const void* src, int n) {
   for (int w = threadIdx.x; w < n; w += blockDim.x) static_cast<int*>(dst)[w] = static_cast<const int*>(src)[w];

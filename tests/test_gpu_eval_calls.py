@@ -111,6 +111,50 @@ def test_nonfinite_positions_leave_outputs_and_lists_alone(torch):
     ctx.close()
 
 
+# A build leaves the pruning pass to the next evaluation; a non-finite position
+# ends that evaluation before it, and the one after it prunes.  Configuration 3
+# has the pass run by the rebuild kernel instead of the pair launch; 40 008
+# atoms and hybrids is above the sizes whose launch shape goes without timing.
+@pytest.mark.parametrize("precision", [R.RELRES_PREC_FP32, R.RELRES_PREC_FP64])
+@pytest.mark.parametrize("first", ["backward", "compute", "config", "tuned"])
+def test_nonfinite_positions_right_after_a_build(torch, precision, first):
+    s = S.neopentane(n_mol=6668 if first == "tuned" else 400, seed=8)
+    ctx = R.Context(R.params_for(s, precision), R.make_topology(s.types, s.mass_by_type, s.excl, None))
+    good = _dev(torch, s.pos)
+    bad = good.clone()
+    bad[s.n_atoms // 2, 2] = float("inf")
+    ctx.build_neighbors(good, s.box)
+    if first == "config":
+        ctx.set_pair_config(3)
+    f, g = torch.full_like(good, 5.0), torch.full_like(good, 9.0)
+    e = torch.full((4,), 3.0, dtype=torch.float64, device="cuda")
+    with pytest.raises(R.RelresError) as ei:
+        if first == "backward":
+            ctx.backward(bad, None, 1.0, g)
+        else:
+            ctx.compute(bad, f, e if first == "compute" else None)
+    assert ei.value.status == 5 and "position" in str(ei.value)
+    torch.cuda.synchronize()
+    assert float(f.min()) == float(f.max()) == 5.0 and float(e.max()) == 3.0 and float(g.max()) == 9.0
+    # a little further on, within the margin of both lists
+    x = good + 0.2
+    if first == "backward":
+        ctx.backward(x, None, 1.0, g)
+        f = -g
+    else:
+        ctx.compute(x, f, e)
+    torch.cuda.synchronize()
+    ref, e0, _ = O.pair_forces(s.pos, s.box, s.types, O.table_for(s), s.n_types, s.excl)
+    assert _err(f.cpu().numpy(), ref) <= (1e-5 if precision == R.RELRES_PREC_FP32 else 1e-10)
+    if first != "backward":
+        assert abs(float(e[3]) - e0) <= 1e-7 * abs(e0)
+    assert ctx.stats()["n_builds"] == 1
+    lists = [set(map(tuple, ctx.get_list(w).tolist())) for w in range(4)]
+    # (no hybrid pairs between the two radii in some of these lattices)
+    assert lists[2] and lists[2] < lists[0] and lists[3] and lists[3] <= lists[1]
+    ctx.close()
+
+
 def test_backward_right_after_a_build_reads_pruned_lists(torch):
     s = S.propane()
     ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP64), R.make_topology(s.types, s.mass_by_type, s.excl, None))
