@@ -122,6 +122,7 @@ int round_cap(double x, int limit) {
 
 relres_status alloc_lists(relres_ctx* c) {
   ++c->buf_gen;
+  c->prune_pending = false;  // nothing in them to prune
   // list offsets are 32-bit inside the list kernel
   if (double(c->cap_fg) * c->n >= 2147483648.0 || double(c->cap_cg) * c->n_h >= 2147483648.0)
     return fail(c, RELRES_ERR_NOMEM, "neighbour list larger than 2^31 entries");
@@ -152,6 +153,7 @@ relres_status barrier_timeout(relres_ctx* c) {
   CK(launch_flags_and(c, ~(unsigned)F_BARRIER));
   CK(cudaMemsetAsync(c->d_bar, 0, 2 * sizeof(unsigned), c->stream));
   c->have_lists = false;  // left unfinished
+  c->prune_pending = false;
   return fail(c, RELRES_ERR_CUDA, "the list rebuild's grid-wide barrier timed out");
 }
 
@@ -248,7 +250,7 @@ static bool timed_now(const relres_ctx* c, int cls) {
 // The pruning pass left over by the last host build, for a reader of the
 // pruned lists other than a pair launch (at the current positions).
 relres_status finish_prune(relres_ctx* c) {
-  if (!c->prune_pending) return RELRES_OK;
+  if (!c->prune_pending || !c->have_lists) return RELRES_OK;
   CK(launch_prune(c, nullptr));
   CK(launch_flags_and(c, ~(unsigned)F_PRUNE));
   c->prune_pending = false;
@@ -788,6 +790,7 @@ relres_status relres_set_topology(relres_ctx* c, const relres_topology* t) {
   CK(cudaMemset(c->d_f_cg, 0, fb));
   c->have_topo = true;
   c->have_lists = false;
+  c->prune_pending = false;
   c->consts_dt = 0.0;  // masses may have changed
   if (c->tune_mode < 0) untune(c);  // the pair launches go with the size
   c->forces_valid = false;

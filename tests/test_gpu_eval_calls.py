@@ -155,6 +155,30 @@ def test_nonfinite_positions_right_after_a_build(torch, precision, first):
     ctx.close()
 
 
+@pytest.mark.parametrize("n_mol", [300, 1200])
+def test_new_topology_after_a_build_and_before_an_evaluation(torch, n_mol):
+    """The pruning pass left over by the first build goes with its lists."""
+    s0, s = S.neopentane(n_mol=600, seed=9), S.neopentane(n_mol=n_mol, seed=10)
+    ctx = R.Context(R.params_for(s0, R.RELRES_PREC_FP32), R.topology_for(s0))
+    ctx.build_neighbors(_dev(torch, s0.pos), s0.box)
+    ctx.set_topology(R.topology_for(s))
+    assert ctx.stats()["n_prunes"] == 0
+    for call in (lambda: ctx.get_list(2), lambda: ctx.compute(_dev(torch, s.pos), _dev(torch, s.pos))):
+        with pytest.raises(R.RelresError) as ei:
+            call()
+        assert ei.value.status == 6
+    x = _dev(torch, s.pos)
+    ctx.build_neighbors(x, s.box)
+    f, e = torch.empty_like(x), torch.zeros(4, dtype=torch.float64, device="cuda")
+    ctx.compute(x, f, e)
+    torch.cuda.synchronize()
+    ref, e0 = _reference(s, s.pos)
+    assert _err(f.cpu().numpy(), ref) <= 1e-5 and abs(float(e[0] + e[1]) - e0) <= 1e-7 * abs(e0)
+    st = ctx.stats()
+    assert st["n_prunes"] == 1 and st["n_atoms"] == s.n_atoms
+    ctx.close()
+
+
 def test_backward_right_after_a_build_reads_pruned_lists(torch):
     s = S.propane()
     ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP64), R.make_topology(s.types, s.mass_by_type, s.excl, None))
