@@ -1891,6 +1891,8 @@ relres_status relres_batch_step(relres_batch* b, int n_steps, double dt_fs, doub
         }
         if (s != RELRES_OK) return batch_fail(b, s, "replica " + std::to_string(r) + ": " + c->err);
       }
+      e = batch_follow(b);  // what the rebuilds have launched behind their last status read
+      if (e != cudaSuccess) return batch_fail(b, RELRES_ERR_CUDA, cudaGetErrorString(e));
       continue;
     }
     done += blk;

@@ -1384,8 +1384,8 @@ __device__ __forceinline__ void call_start(const CallStart& a) {
 
 __global__ void __launch_bounds__(32) k_call_start(const __grid_constant__ CallStart a) { call_start(a); }
 
-__global__ void k_flags_and(DevState* st, unsigned keep) { st->flags &= keep; }
-__global__ void k_flags_or(DevState* st, unsigned set) { st->flags |= set; }
+__global__ void k_flags_and(DevState* st, unsigned keep) { atomicAnd(&st->flags, keep); }
+__global__ void k_flags_or(DevState* st, unsigned set) { atomicOr(&st->flags, set); }
 __global__ void k_close_call(DevState* st) { close_host_call(st); }
 
 __global__ void __launch_bounds__(32) k_post_state(const DevState* st, DevState* host) { post_state(st, host); }

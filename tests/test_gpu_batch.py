@@ -181,3 +181,50 @@ def test_mixed_precision_batch_takes_graph_branches_and_matches_solo(torch):
     batch.close()
     for c, _, _ in solo + both:
         c.close()
+
+
+@pytest.mark.parametrize("mode", [-1, 0])
+def test_a_list_overflow_in_one_replica_restarts_the_block_of_all(torch, mode):
+    """Contexts on streams of their own, the batch on another; the last replica's lists are sized for its first
+    positions and overflow at a rebuild inside a block.  That replica ends with the bits of stepping it alone (the
+    same block restarts there); the others run their block again on the lists that the first attempt left, so they
+    agree up to rounding: force errors of 1e-5 kcal/mol/A move an atom by 5e-5 A in 600 fs, grown tenfold or less."""
+    systems = [S.neopentane(n_mol=300, seed=61), S.propane(seed=62), S.neopentane(n_mol=500, seed=31)]
+    temps, seeds = [200.0, 230.0, 260.0], [7, 8, 4]
+
+    def run(batched):
+        ctxs, ps, vs = [], [], []
+        for s in systems:
+            p = torch.tensor(s.pos, dtype=torch.float64, device="cuda")
+            v = torch.tensor(s.vel, dtype=torch.float64, device="cuda")
+            torch.cuda.synchronize()
+            ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP32), R.topology_for(s), stream=torch.cuda.Stream())
+            ctx.set_pair_config(0)
+            ctx.build_neighbors(p, s.box)
+            ctxs.append(ctx)
+            ps.append(p)
+            vs.append(v)
+        st = ctxs[2].stats()
+        ctxs[2].set_list_caps(st["max_fg"], st["max_cg"])
+        st = ctxs[2].stats()
+        if batched:
+            b = R.Batch(ctxs, stream=torch.cuda.Stream())
+            b.set_mode(mode)
+            b.step(300, 2.0, ps, vs, temps, 100.0, seeds)
+            b.close()
+        else:
+            for c, p, v, t, sd in zip(ctxs, ps, vs, temps, seeds):
+                c.step(300, 2.0, p, v, t_target=t, tau_fs=100.0, seed=sd)
+        torch.cuda.synchronize()
+        end = ctxs[2].stats()
+        assert end["cap_fg"] > st["cap_fg"] or end["cap_cg"] > st["cap_cg"]  # it did overflow
+        for c in ctxs:
+            assert c.stats()["n_steps"] == 300
+            c.close()
+        return [(p.cpu().numpy(), v.cpu().numpy()) for p, v in zip(ps, vs)]
+
+    alone, both = run(False), run(True)
+    assert np.array_equal(alone[2][0], both[2][0]) and np.array_equal(alone[2][1], both[2][1])
+    for s, (p0, _), (p1, _) in zip(systems[:2], alone, both):
+        d = p0 - p1
+        assert np.abs(d - s.box * np.rint(d / s.box)).max() <= 1e-2
