@@ -313,7 +313,9 @@ relres_status relres_compute(relres_ctx* ctx, const double* d_pos, double* d_for
  * replace the velocity state.
  * On RELRES_ERR_NONFINITE or RELRES_ERR_LIST_OVERFLOW the state is rolled
  * back to the last completed block of steps (blocks of up to 100 steps),
- * d_pos/d_vel receive it, and the error is returned.
+ * d_pos/d_vel receive it, and the error is returned; also when the blocks of
+ * the list rebuild waited for one another in vain (RELRES_ERR_CUDA, "barrier
+ * timed out"), after which the lists have to be built again.
  * Errors: RELRES_ERR_STATE, RELRES_ERR_LIST_OVERFLOW, RELRES_ERR_NONFINITE,
  * RELRES_ERR_ARG, RELRES_ERR_CUDA.
  */
@@ -482,6 +484,17 @@ relres_status relres_measure_rates(void* d_scratch, size_t scratch_bytes, void* 
  * Errors: RELRES_ERR_ARG (null pointer, n < 0), RELRES_ERR_CUDA.
  */
 relres_status relres_eval_recip(const double* d_x, float* d_out32, double* d_out64, int n, void* cuda_stream);
+
+/*
+ * Failure injection (tests of the error path): in the next list rebuild that
+ * relres_compute, relres_backward or a captured step of relres_step runs on
+ * the device, the grid-wide barrier counts from a value that its blocks do not
+ * reach, so their bounded wait (half a second) runs out.  That call returns
+ * RELRES_ERR_CUDA and leaves its outputs alone (relres_step: as described
+ * there); relres_build_neighbors then makes the context whole.  Synchronous.
+ * Errors: RELRES_ERR_ARG (null context), RELRES_ERR_CUDA.
+ */
+relres_status relres_stall_rebuild(relres_ctx* ctx);
 
 typedef struct relres_batch relres_batch;
 relres_status relres_batch_create(relres_batch** out, relres_ctx* const* ctxs, int n_ctx, void* cuda_stream);

@@ -149,11 +149,18 @@ relres_status alloc_lists(relres_ctx* c) {
   return RELRES_OK;
 }
 
+// The rebuild stopped at a barrier: its cell counts go back to zero, as every
+// build starts from, and the lists, left unfinished, are allocated and built
+// again by relres_build_neighbors.
 relres_status barrier_timeout(relres_ctx* c) {
+  c->have_lists = false;
+  c->prune_pending = false;
+  c->forces_valid = false;
+  c->cap_fg = c->cap_cg = 0;
   CK(launch_flags_and(c, ~(unsigned)F_BARRIER));
   CK(cudaMemsetAsync(c->d_bar, 0, 2 * sizeof(unsigned), c->stream));
-  c->have_lists = false;  // left unfinished
-  c->prune_pending = false;
+  for (const Grid* g : {&c->gfg, &c->gcg})
+    if (g->d_count) CK(cudaMemsetAsync(g->d_count, 0, sizeof(int) * g->ncell, c->stream));
   return fail(c, RELRES_ERR_CUDA, "the list rebuild's grid-wide barrier timed out");
 }
 
@@ -1445,7 +1452,13 @@ static relres_status block_end(relres_ctx* c, double* d_pos, double* d_vel, doub
   }
   const unsigned fl = c->h_state->flags;
   if (fl & F_BADCELL) return fail(c, RELRES_ERR_CUDA, "cell binning produced an out-of-range index");
-  if (fl & F_BARRIER) return barrier_timeout(c);
+  if (fl & F_BARRIER) {  // the steps since ran on unfinished lists: back to the block start
+    s = rollback_block(c, d_vel);
+    if (s != RELRES_OK) return s;
+    CK(launch_write_back(c, d_pos, d_vel));
+    CK(cudaStreamSynchronize(c->stream));
+    return barrier_timeout(c);
+  }
   if (fl & (F_OVERFLOW_FG | F_OVERFLOW_CG | F_NONFINITE)) {
     s = rollback_block(c, d_vel);
     if (s != RELRES_OK) return s;
@@ -1991,6 +2004,15 @@ relres_status relres_set_step_counter(relres_ctx* c, long long step) {
                      cudaMemcpyHostToDevice, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   c->step_counter = (unsigned long long)step;
+  return RELRES_OK;
+}
+
+relres_status relres_stall_rebuild(relres_ctx* c) {
+  if (!c) return RELRES_ERR_ARG;
+  // a count of arrivals that no grid reaches
+  const unsigned bar[2] = {0x40000000u, 0u};
+  CK(cudaStreamSynchronize(c->stream));
+  CK(cudaMemcpy(c->d_bar, bar, sizeof bar, cudaMemcpyHostToDevice));
   return RELRES_OK;
 }
 

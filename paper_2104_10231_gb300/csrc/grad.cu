@@ -121,7 +121,7 @@ struct GradLaunch {
   float sxl, syl, szl;  // FP32: lo parts of L / 2^32
   R g_energy;
   double* gc;  // [nt*nt][4]: dL/dC12_FG, dL/dC6_FG, dL/dC12_CG, dL/dC6_CG
-  const unsigned* flags;  // F_BADPOS: the rebuild kernel left the lists alone, no walk
+  const unsigned* flags;  // F_NOLISTS: no walk
 };
 
 constexpr int kGradThreads = 128;
@@ -245,7 +245,7 @@ __device__ __forceinline__ void grad_walk(const GradWalk<R>& W, int blk, const B
 template <typename R, int T>
 __global__ void __launch_bounds__(kGradThreads) k_pair_grad(GradLaunch<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (*(volatile const unsigned*)a.flags & F_BADPOS) return;
+  if (*(volatile const unsigned*)a.flags & F_NOLISTS) return;
   const int nrow = a.nt * a.nt;
   double* s_gc = reinterpret_cast<double*>(smem_raw);
   R(*s_acc)[kGradThreads] = reinterpret_cast<R(*)[kGradThreads]>(s_gc + 2 * nrow);
@@ -284,7 +284,7 @@ __global__ void k_gather_g(int nslots, const int* __restrict__ perm, const doubl
 template <typename R>
 __global__ void k_sum_gx(int n, const GVec<R>* __restrict__ gx_fg, const GVec<R>* __restrict__ gx_cg,
                          int with_cg, const DevState* st, double* __restrict__ out) {
-  if (*(volatile const unsigned*)&st->flags & F_BADPOS) return;  // the call fails: no output
+  if (*(volatile const unsigned*)&st->flags & F_NOLISTS) return;  // the call fails: no output
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     R a[3], b[3] = {R(0), R(0), R(0)};
     ld3(gx_fg, i, a);

@@ -539,12 +539,12 @@ struct FinishArgs {
 // due may be one that a build left over, so it stays due.
 __device__ __forceinline__ void close_host_call(DevState* st) {
   const unsigned f = *(volatile unsigned*)&st->flags;
-  const bool bad = (f & F_BADPOS) != 0u;
+  const bool bad = (f & F_NOLISTS) != 0u;
   if ((f & F_REBUILD) && !bad) st->n_builds += 1;
   atomicAnd(&st->flags, bad ? ~unsigned(F_REBUILD) : ~unsigned(F_REBUILD | F_PRUNE));
 }
-__device__ __forceinline__ bool bad_positions(const DevState* st) {
-  return (*(volatile const unsigned*)&st->flags & F_BADPOS) != 0u;
+__device__ __forceinline__ bool no_outputs(const DevState* st) {
+  return (*(volatile const unsigned*)&st->flags & F_NOLISTS) != 0u;
 }
 
 // Total force per atom: FG part + CG part + the slots of its bonded terms;
@@ -553,7 +553,7 @@ template <typename R>
 __global__ void __launch_bounds__(kThreads) k_finish(FinishArgs<R> a) {
   R ke = R(0);
   bool bad = false;
-  const bool with_out = a.with_out && !(a.host_call && bad_positions(a.st));
+  const bool with_out = a.with_out && !(a.host_call && no_outputs(a.st));
   if (a.host_call && blockIdx.x == 0 && threadIdx.x == 0) close_host_call(a.st);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < a.n) {
@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(kThreads) k_finish_seg(SegArgs<R> a) {
   const Sc3<R> sc = a.sc;
   // the terms are the prototype's (atoms from `base`): shifted onto this segment
   const GPosOff xg{a.xfx, a0 - base};
-  const bool with_out = a.with_out && !(a.host_call && bad_positions(a.st));
+  const bool with_out = a.with_out && !(a.host_call && no_outputs(a.st));
   if (a.host_call && blockIdx.x == 0 && threadIdx.x == 0) close_host_call(a.st);
   R e = R(0);
   for (int q = threadIdx.x; q < nb + na + nd; q += blockDim.x) {
@@ -1332,7 +1332,7 @@ __device__ __forceinline__ void post_state(const DevState* st, DevState* host) {
 // 1-6 the virial), the accumulators cleared, and the state to the host.
 __global__ void __launch_bounds__(32) k_reduce_out(long long* acc, double* energy, int with_e, double* virial,
                                                    int with_w, const DevState* st, DevState* host) {
-  if (bad_positions(st)) with_e = with_w = 0;
+  if (no_outputs(st)) with_e = with_w = 0;
   const int q = threadIdx.x;
   if (q == 0 && with_e) {
     const double efg = acc_value(acc[kAccFg], acc[kNAcc + kAccFg]), ecg = acc_value(acc[kAccCg], acc[kNAcc + kAccCg]);

@@ -1045,8 +1045,9 @@ cudaError_t launch_prune(relres_ctx* c, const unsigned* gate) {
 // 160 000, 282 / 276 at 1 000 000.
 
 // Grid-wide barrier: bar[0] counts arrivals, bar[1] is the generation.  The
-// wait is bounded (about a second); a block that gives up sets F_BARRIER, and
-// every block leaves at its next barrier.  Returns whether to go on.
+// wait is bounded (0.3 s in a small grid, 0.6 s in one that fills the GPU); a
+// block that gives up sets F_BARRIER, and every block leaves at its next
+// barrier.  Returns whether to go on.
 __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned* flags) {
   __shared__ int s_go;
   __syncthreads();
@@ -1075,7 +1076,7 @@ __global__ void __launch_bounds__(kListThreads) k_rebuild(const unsigned* gate, 
                                                           unsigned* bar) {
   grid_dependents_launch();  // the pair kernel waits for this grid to finish
   const unsigned f = *(volatile const unsigned*)gate;
-  if (f & F_NONFINITE) return;  // no lists from such positions
+  if (f & (F_NONFINITE | F_BARRIER)) return;  // no lists from such positions, or on top of unfinished ones
   const int bid = blockIdx.x, nblk = gridDim.x;
   if (f & F_REBUILD) {
     bin_body(bid, nblk, b.n, gate, b.xfx, b.type, b.hyb_mask, b.gf.n0, b.gf.n1, b.gf.n2, b.gf.rank_of, b.gf.count,

@@ -169,11 +169,11 @@ __device__ __forceinline__ void after_rebuild() {
 }
 
 // A launch whose lists were to be pruned by a pass of their own (or that walks
-// the full lists) behind a non-finite position: the pass did not run, so the
-// pruned lists may never have been written.  The call fails without reading
-// these forces.
+// the full lists) behind a non-finite position or an unfinished rebuild: the
+// pass did not run, so the pruned lists may never have been written.  The call
+// fails without reading these forces.
 __device__ __forceinline__ bool lists_unpruned(const PairLaunch& a) {
-  return !a.prune_on && (*(volatile const unsigned*)a.gate & F_BADPOS) != 0u;
+  return !a.prune_on && (*(volatile const unsigned*)a.gate & F_NOLISTS) != 0u;
 }
 
 // copies n words from global to shared memory with the whole block

@@ -98,6 +98,9 @@ enum : unsigned {
   F_BADPOS = 512u,      // a non-finite incoming position (with F_NONFINITE)
   F_BARRIER = 256u,     // a grid-wide barrier of the fused rebuild ran out of time
   F_VDIRTY = 128u,      // incoming velocities differ from the ones returned last
+  // the lists are not those of the positions: nothing that the rebuild kernel
+  // was to write is read, and the call leaves its outputs alone
+  F_NOLISTS = F_BADPOS | F_BARRIER,
 };
 
 struct DevState {
@@ -354,7 +357,8 @@ struct relres_ctx {
   long long* d_acc = nullptr;
   double* d_draws = nullptr;  // CSVR random numbers of the current block of steps, 2 per step
   relres::DevState* d_state = nullptr;
-  unsigned* d_bar = nullptr;   // grid-wide barrier of the fused rebuild: arrivals, generation
+  // grid-wide barrier of the fused rebuild: arrivals, generation
+  unsigned* d_bar = nullptr;
   // step graphs rebuild in one kernel (else behind a conditional node: the
   // concurrent branches of a batch graph)
   bool use_fused = true;

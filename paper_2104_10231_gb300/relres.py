@@ -39,7 +39,7 @@ EXPORTED = ["relres_prepare_table", "relres_cg_params", "relres_chain_cg_grads",
             "relres_batch_last_error", "relres_batch_destroy", "relres_set_timing_sampled",
             "relres_set_list_caps", "relres_set_prune", "relres_measure_rates", "relres_get_list",
             "relres_eval_recip", "relres_set_force_accumulation", "relres_batch_get_info",
-            "relres_batch_set_mode"]
+            "relres_batch_set_mode", "relres_stall_rebuild"]
 RELRES_STATIC_MAX_ATOMS = 16384
 RELRES_BATCH_SHARED_MAX_ATOMS = 16384
 TIMING_CLASSES = ["drift", "rebuild", "lists", "pair", "finish", "thermo", "pair_ev", "prune"]
@@ -130,6 +130,7 @@ def load():
     L.relres_measure_rates.argtypes = [vp, C.c_size_t, vp, C.POINTER(relres_rates)]
     L.relres_get_list.argtypes = [vp, C.c_int, _ip, _ip, C.c_longlong, C.POINTER(C.c_longlong)]
     L.relres_eval_recip.argtypes = [vp, vp, vp, C.c_int, vp]
+    L.relres_stall_rebuild.argtypes = [vp]
     L.relres_set_graphs.argtypes = [vp, C.c_int]
     L.relres_set_params.argtypes = [vp, C.POINTER(relres_params)]
     L.relres_set_pair_config.argtypes = [vp, C.c_int]

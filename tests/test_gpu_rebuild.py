@@ -1,0 +1,115 @@
+"""The list rebuild inside one kernel (its phases separated by a grid-wide
+barrier with a bounded wait): the error path when the wait runs out."""
+import time
+
+import numpy as np
+import pytest
+
+from oracle import core as O
+from paper_2104_10231_gb300 import relres as R
+from paper_2104_10231_gb300 import systems as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch as T
+
+    assert T.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2104_10231_gb300.build import build_library
+
+    build_library()
+    R.load()
+    return T
+
+
+def _dev(torch, a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+
+def _pair_reference(s, pos):
+    fr, e, _ = O.pair_forces(pos, s.box, s.types, O.table_for(s), s.n_types, s.excl)
+    return fr, e
+
+
+def _err(f, ref):
+    return np.abs(f - ref).max() / np.sqrt((ref * ref).sum(1).mean())
+
+
+def _stall(ctx):
+    R._check(R.load().relres_stall_rebuild(ctx.ctx), ctx.ctx)
+
+
+def _whole_again(torch, ctx, s, precision):
+    """After the error the lists have to be built again; then everything is as in a new context."""
+    x = _dev(torch, s.pos)
+    f, e = torch.empty_like(x), torch.zeros(4, dtype=torch.float64, device="cuda")
+    with pytest.raises(R.RelresError) as ei:
+        ctx.compute(x, f, e)
+    assert ei.value.status == 6
+    ctx.stats()
+    ctx.build_neighbors(x, s.box)
+    ref, e0 = _pair_reference(s, s.pos)
+    for shift in (0.0, 1.5, 0.0):  # the second and third rebuild inside the call
+        ctx.compute(_dev(torch, s.pos + shift), f, e)
+        torch.cuda.synchronize()
+        assert _err(f.cpu().numpy(), ref) <= (1e-5 if precision == R.RELRES_PREC_FP32 else 1e-10)
+        assert abs(float(e[3]) - e0) <= 1e-7 * abs(e0)
+
+
+@pytest.mark.parametrize("precision", [R.RELRES_PREC_FP32, R.RELRES_PREC_FP64])
+@pytest.mark.parametrize("call", ["compute", "backward", "config"])
+def test_barrier_that_runs_out_of_time_in_an_evaluation(torch, precision, call):
+    s = S.neopentane(n_mol=500, seed=14)
+    ctx = R.Context(R.params_for(s, precision), R.make_topology(s.types, s.mass_by_type, s.excl, None))
+    if call == "config":
+        ctx.set_pair_config(3)
+    x = _dev(torch, s.pos)
+    ctx.build_neighbors(x, s.box)
+    _stall(ctx)
+    out = torch.full_like(x, 5.0)
+    e = torch.full((4,), 3.0, dtype=torch.float64, device="cuda")
+    moved = x + 1.5  # past half the skin
+    t0 = time.perf_counter()
+    with pytest.raises(R.RelresError) as ei:
+        if call == "backward":
+            ctx.backward(moved, None, 1.0, out)
+        else:
+            ctx.compute(moved, out, e)
+    assert time.perf_counter() - t0 < 20.0
+    assert ei.value.status == 2 and "barrier" in str(ei.value)
+    torch.cuda.synchronize()
+    assert float(out.min()) == float(out.max()) == 5.0 and float(e.min()) == float(e.max()) == 3.0
+    _whole_again(torch, ctx, s, precision)
+    ctx.close()
+
+
+@pytest.mark.parametrize("precision", [R.RELRES_PREC_FP32, R.RELRES_PREC_FP64])
+def test_barrier_that_runs_out_of_time_in_a_step_returns_the_block_start(torch, precision):
+    """The first rebuild of a run comes within its first block of 100 steps; the call gives back the arrays that it
+    was given, through 64-bit fixed point (2^-64 of the box) and, in FP32 mode, float-float (2^-47)."""
+    s = S.neopentane(n_mol=500, seed=31)
+    ctx = R.Context(R.params_for(s, precision), R.topology_for(s))
+    p, v = _dev(torch, np.mod(s.pos, s.box)), _dev(torch, s.vel)
+    ctx.build_neighbors(p, s.box)
+    ctx.step(1, 2.0, p, v, t_target=260.0, tau_fs=100.0, seed=4)
+    p0, v0 = p.cpu().numpy(), v.cpu().numpy()
+    _stall(ctx)
+    with pytest.raises(R.RelresError) as ei:
+        ctx.step(100, 2.0, p, v, t_target=260.0, tau_fs=100.0, seed=4)
+    assert ei.value.status == 2 and "barrier" in str(ei.value)
+    torch.cuda.synchronize()
+    assert np.abs(p.cpu().numpy() - p0).max() <= 1e-12 * s.box.max()
+    assert np.abs(v.cpu().numpy() - v0).max() <= 1e-13 * np.abs(v0).max()
+    # on from there as a new context goes from the same arrays
+    p2, v2 = _dev(torch, p.cpu().numpy()), _dev(torch, v.cpu().numpy())
+    new = R.Context(R.params_for(s, precision), R.topology_for(s))
+    for c, q, w in ((ctx, p, v), (new, p2, v2)):
+        c.build_neighbors(q, s.box)
+        R.relres_set_step_counter(c.ctx, 1)
+        c.step(100, 2.0, q, w, t_target=260.0, tau_fs=100.0, seed=4)
+    torch.cuda.synchronize()
+    assert np.array_equal(p.cpu().numpy(), p2.cpu().numpy()) and np.array_equal(v.cpu().numpy(), v2.cpu().numpy())
+    ctx.close()
+    new.close()
