@@ -948,6 +948,10 @@ struct PruneArgs {
 
 constexpr int kPruneThreads = 256;
 
+// One slot's pruned list from its full one; returns its length.  RO: nothing
+// writes the positions during this kernel (k_prune), so they may go through the
+// read-only path; in k_rebuild other blocks wrote them before the last barrier.
+template <bool RO>
 __device__ __forceinline__ int prune_slot(const PruneList& L, int s, float sx, float sy, float sz) {
   const int4 pi = L.pos[s];
   const int m = L.cnt[s];
@@ -964,7 +968,7 @@ __device__ __forceinline__ int prune_slot(const PruneList& L, int s, float sx, f
     const int j[4] = {jj.x, rem > 1 ? jj.y : s, rem > 2 ? jj.z : s, rem > 3 ? jj.w : s};
     int4 p[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) p[q] = __ldg(L.pos + j[q]);
+    for (int q = 0; q < 4; ++q) p[q] = RO ? __ldg(L.pos + j[q]) : L.pos[j[q]];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float dx = dfix32(pi.x, p[q].x, sx), dy = dfix32(pi.y, p[q].y, sy), dz = dfix32(pi.z, p[q].z, sz);
@@ -984,9 +988,9 @@ __global__ void __launch_bounds__(kPruneThreads) k_prune(const unsigned* gate, P
   const int s = blk * kPruneThreads + threadIdx.x;
   unsigned long long kept = 0ull;
   if (is_cg) {
-    if (s < a.cg.nslots) kept = prune_slot(a.cg, s, a.sx, a.sy, a.sz);
+    if (s < a.cg.nslots) kept = prune_slot<true>(a.cg, s, a.sx, a.sy, a.sz);
   } else if (s < a.fg.nslots) {
-    kept = prune_slot(a.fg, s, a.sx, a.sy, a.sz);
+    kept = prune_slot<true>(a.fg, s, a.sx, a.sy, a.sz);
     a.ref_p[a.perm_fg[s]] = a.fg.pos[s];
   }
   __shared__ unsigned long long sh[kPruneThreads / 32];
@@ -1105,10 +1109,10 @@ __global__ void __launch_bounds__(kListThreads) k_rebuild(const unsigned* gate, 
     unsigned long long kept_cg = 0ull, kept_fg = 0ull;
     for (int s = bid * kListThreads + threadIdx.x; s < n_cg + p.fg.nslots; s += nblk * kListThreads) {
       if (s < n_cg) {
-        kept_cg += prune_slot(p.cg, s, p.sx, p.sy, p.sz);
+        kept_cg += prune_slot<false>(p.cg, s, p.sx, p.sy, p.sz);
       } else {
         const int sf = s - n_cg;
-        kept_fg += prune_slot(p.fg, sf, p.sx, p.sy, p.sz);
+        kept_fg += prune_slot<false>(p.fg, sf, p.sx, p.sy, p.sz);
         p.ref_p[p.perm_fg[sf]] = p.fg.pos[sf];
       }
     }

@@ -1,5 +1,6 @@
 """The list rebuild inside one kernel (its phases separated by a grid-wide
-barrier with a bounded wait): the error path when the wait runs out."""
+barrier with a bounded wait): rebuilds, pruning and overflows that come with a
+backward pass, and the error path when the wait runs out."""
 import time
 
 import numpy as np
@@ -35,6 +36,63 @@ def _pair_reference(s, pos):
 
 def _err(f, ref):
     return np.abs(f - ref).max() / np.sqrt((ref * ref).sum(1).mean())
+
+
+def _backward(torch, ctx, s, pos):
+    """Gradients of E for the box and lists of ctx at pos: dL/dx = -F, and the parameter gradients."""
+    x = _dev(torch, pos)
+    g = torch.empty_like(x)
+    out = ctx.backward(x, None, 1.0, g)
+    torch.cuda.synchronize()
+    return g.cpu().numpy(), out
+
+
+# shifts of the whole liquid leave the physics alone; the second and the last
+# are past half the skin
+@pytest.mark.parametrize("precision", [R.RELRES_PREC_FP32, R.RELRES_PREC_FP64])
+@pytest.mark.parametrize("n_mol", [250, 2000, 12000])
+def test_backward_rebuilds_and_prunes_at_moved_positions(torch, precision, n_mol):
+    s = S.neopentane(n_mol=n_mol, seed=12)
+    ctx = R.Context(R.params_for(s, precision), R.make_topology(s.types, s.mass_by_type, s.excl, None))
+    ctx.build_neighbors(_dev(torch, s.pos), s.box)
+    ref, _ = _pair_reference(s, s.pos)
+    first = None
+    for shift in (0.0, 1.5, 1.7, 9.0):
+        g, out = _backward(torch, ctx, s, s.pos + shift)
+        assert _err(g, -ref) <= (1e-5 if precision == R.RELRES_PREC_FP32 else 1e-10), shift
+        first = first or out
+        # sums over all pairs of terms rounded to FP32 (FP64) once each
+        tol = 1e-5 if precision == R.RELRES_PREC_FP32 else 1e-11
+        for k, v in first.items():
+            assert np.abs(out[k] - v).max() <= tol * np.abs(v).max(), (shift, k)
+    st = ctx.stats()
+    assert st["n_builds"] == 3 and st["n_prunes"] >= 3
+    # the pruned lists of the rebuild kernel are those of a new context at the same positions
+    got = [set(map(tuple, ctx.get_list(w).tolist())) for w in (2, 3)]
+    ctx.close()
+    new = R.Context(R.params_for(s, precision), R.make_topology(s.types, s.mass_by_type, s.excl, None))
+    new.build_neighbors(_dev(torch, s.pos + 9.0), s.box)
+    want = [set(map(tuple, new.get_list(w).tolist())) for w in (2, 3)]
+    new.close()
+    assert got == want
+
+
+@pytest.mark.parametrize("precision", [R.RELRES_PREC_FP32, R.RELRES_PREC_FP64])
+def test_backward_grows_lists_that_overflow(torch, precision):
+    s = S.neopentane(n_mol=300, seed=5)
+    ctx = R.Context(R.params_for(s, precision), R.make_topology(s.types, s.mass_by_type, s.excl, None))
+    ctx.build_neighbors(_dev(torch, s.pos), s.box)
+    ctx.set_list_caps(1, 1)  # grown at once to what these positions need
+    caps = ctx.stats()
+    # half of the liquid pushed into half of the box: far longer lists
+    centre = np.stack([s.pos[s.mol == m].mean(0) for m in range(s.mol.max() + 1)])
+    pos = s.pos - np.floor(centre / s.box * 2)[s.mol] / 2 * s.box * np.array([0.0, 0.0, 0.97])
+    g, _ = _backward(torch, ctx, s, pos)
+    ref, _ = _pair_reference(s, np.mod(pos, s.box))
+    assert _err(g, -ref) <= (1e-5 if precision == R.RELRES_PREC_FP32 else 1e-10)
+    st = ctx.stats()
+    assert st["cap_fg"] > caps["cap_fg"] and st["cap_cg"] > caps["cap_cg"]
+    ctx.close()
 
 
 def _stall(ctx):
