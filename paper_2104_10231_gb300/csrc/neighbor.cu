@@ -20,6 +20,7 @@
 // The pair kernels walk pruned copies of the lists (k_prune below, or the pair
 // kernel's own pruning walk).
 #include "common.cuh"
+#include "grid.h"
 
 namespace relres {
 
@@ -1128,15 +1129,21 @@ __global__ void __launch_bounds__(kListThreads) k_rebuild(const unsigned* gate, 
 
 cudaError_t launch_rebuild_fused(relres_ctx* c, bool prune) {
   cudaError_t e = cudaSuccess;
-  if (c->rebuild_per_sm == 0)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->rebuild_per_sm, k_rebuild, kListThreads, 0);
+  if (c->rebuild_per_sm == 0) {
+    int dev = 0;
+    e = cudaGetDevice(&dev);
+    // the SMs that this process may use, which can be fewer than the part has
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->rebuild_per_sm, k_rebuild, kListThreads, 0);
+  }
   if (e != cudaSuccess) return e;
   BuildArgs b = build_args(c, &c->d_state->flags);
   PruneArgs p = prune_args(c);
   const unsigned* gate = &c->d_state->flags;
   int with_prune = prune ? 1 : 0;
   void* args[] = {&gate, &b, &p, &with_prune, &c->d_bar};
-  const int nb = std::max(1, std::min(b.ncell_cg + b.gf.ncell_full, kPartSMs * c->rebuild_per_sm));
+  const int nb = cooperative_blocks(b.ncell_cg + b.gf.ncell_full, c->sm_count, c->rebuild_per_sm);
   e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_rebuild), dim3(nb),
                                   dim3(kListThreads), args, 0, c->stream);
   if (e != cudaSuccess) return e;

@@ -353,6 +353,7 @@ struct relres_ctx {
   // force sum and drift as programmatic dependent launches (untimed steps)
   bool use_pdl = true;
   int rebuild_per_sm = 0;  // blocks of k_rebuild an SM holds (0: not asked yet)
+  int sm_count = 0;        // SMs of the device (asked with rebuild_per_sm)
   // reductions: 64-bit fixed-point accumulators (kNAccAll), cleared by their reader
   long long* d_acc = nullptr;
   double* d_draws = nullptr;  // CSVR random numbers of the current block of steps, 2 per step
@@ -569,6 +570,8 @@ constexpr long long kRebuildKernels = 6;
 // MD steps take the segmented drift + bonded kernel and k_sum
 inline bool step_segments(const relres_ctx* c) { return c->seg_ok && c->use_seg; }
 
+// SMs of the part that launch shapes are tuned to (a launch that needs every
+// block resident asks the device instead)
 constexpr int kPartSMs = 152;
 
 // slots of both lists
