@@ -15,8 +15,10 @@
 // 116 us per step at 25 000 neopentane-like atoms, 65 -> 27 us at 648
 // propane-like ones (a launch with energies 185 -> 12 us).  What is left
 // there is the FP64 rate, then the latency of one warp's rounds: fetching the
-// partners of the next pass ahead gave 0 to 1 %.  The potential is C2 at the region limits, so a pair that
-// FP32 puts on the other side of one (1e-7 of r^2) changes nothing above 1e-13.
+// partners of the next pass ahead gave 0 to 1 %.  A pair whose FP32 distance
+// is too close to a region limit to tell the side (kNear) is kept whatever the
+// side, and the FP64 distance decides when it is evaluated: the regions are
+// those of an FP64 comparison (without the full shift the energy jumps at r_c+).
 //
 // The terms of a slot are stored by their rank in its list and added in list
 // order to four sums by rank modulo four (one chain of a hundred additions by
@@ -56,6 +58,7 @@ struct Launch64 {
   int nt;
   double sx, sy, sz;  // L / 2^64
   float fx, fy, fz;   // L / 2^32
+  float near;         // share of r^2 within which FP32 does not decide a region
   const unsigned* gate;
   int prune_on;
   int4* ref_p;
@@ -65,6 +68,20 @@ struct Launch64 {
 // regions, in the order the entries are sorted by
 enum { kCore = 0, kShell = 1, kFgRegions = 2 };                      // FG: LJ below r_s-, switching off
 enum { kLj = 0, kOff = 1, kOn = 2, kCgRegions = 3 };                 // CG: below r_s- an energy only
+
+// beside the place of an entry: the region is left to the FP64 distance
+constexpr int kNear = 0x80;
+
+// the region of a pair by its FP64 squared distance; past the cutoff (and, for
+// the CG part, below r_s-) none: kOutside, kClose
+enum { kOutside = 8, kClose = 9 };
+template <bool CG>
+__device__ __forceinline__ int region64(const PairTab<double>& T, double r2) {
+  if (!CG) return !(r2 < T.rsp2) ? int(kOutside) : (r2 < T.rsm2 ? int(kCore) : int(kShell));
+  if (!(r2 < T.rcp2)) return kOutside;
+  if (r2 < T.rsm2) return kClose;
+  return r2 < T.rsp2 ? int(kOn) : (r2 < T.rcm2 ? int(kLj) : int(kOff));
+}
 
 // values of a term: force, then (energy steps) energy and virial
 constexpr int kTermF = 3, kTermEv = 3 + kNQ;
@@ -88,6 +105,11 @@ __device__ __forceinline__ void term64(int region, const PairTab<double>& T, dou
     const double r6i = r2i * r2i * r2i;
     fr = r6i * ((CG ? T.f12c : T.f12f) * r6i - (CG ? T.f6c : T.f6f)) * r2i;
     if (EV) e = r6i * ((CG ? T.c12c : T.c12f) * r6i - (CG ? T.c6c : T.c6f)) - (CG ? T.gam_cm : T.e_fg_shift);
+    return;
+  }
+  if (region >= kOutside) {
+    fr = 0.0;
+    if (EV) e = CG && region == kClose ? T.e_cg_close : 0.0;
     return;
   }
   const double ri = rsqrt_d(r2, r2f);
@@ -147,18 +169,24 @@ __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0,
     const int rem = m - 4 * ch;  // <= 0 past the list
     const int j[4] = {rem > 0 ? jj.x : ss, rem > 1 ? jj.y : ss, rem > 2 ? jj.z : ss, rem > 3 ? jj.w : ss};
     float r2[4];
-    int region[4];
+    int region[4], near[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int4 p = __ldg(L.pos32 + j[e]);
       const float dx = dfix32(pi.x, p.x, a.fx), dy = dfix32(pi.y, p.y, a.fy), dz = dfix32(pi.z, p.z, a.fz);
       r2[e] = rem > e ? dx * dx + dy * dy + dz * dz : 3.0e38f;
       const float4 t = thr[row0 + p.w];
-      if (CG)
+      const float w = a.near * r2[e];
+      float gap = fminf(fabsf(r2[e] - t.x), fabsf(r2[e] - t.y));
+      if (CG) {
+        gap = fminf(gap, fminf(fabsf(r2[e] - t.z), fabsf(r2[e] - t.w)));
         region[e] = !(r2[e] < t.w) || r2[e] < t.x ? -1 : (r2[e] < t.y ? int(kOn) : (r2[e] < t.z ? int(kLj) : int(kOff)));
-      else
+      } else {
         region[e] = !(r2[e] < t.y) ? -1 : (r2[e] < t.x ? int(kCore) : int(kShell));
-      if (CG && EV && r2[e] < t.x) close += tab[row0 + p.w].e_cg_close;
+      }
+      near[e] = gap <= w ? kNear : 0;
+      if (near[e]) region[e] = max(region[e], 0);
+      if (CG && EV && r2[e] < t.x && !near[e]) close += tab[row0 + p.w].e_cg_close;
     }
     // rank of each term in its slot's list order, and place in the sorted entries
     unsigned in[4];
@@ -184,7 +212,7 @@ __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0,
       if (region[e] >= 0) {
         W.j[place[e]] = j[e];
         W.r2[place[e]] = r2[e];
-        W.at[place[e]] = (unsigned short)((region[e] << 8) | (4 * T * sl + rank));
+        W.at[place[e]] = (unsigned short)(((region[e] | near[e]) << 8) | (4 * T * sl + rank));
         ++rank;
       }
     __syncwarp();
@@ -193,8 +221,12 @@ __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0,
       const Pos64 p = L.pos[W.j[k]];
       const double dx = dfix64(W.px[from], p.x, a.sx), dy = dfix64(W.py[from], p.y, a.sy),
                    dz = dfix64(W.pz[from], p.z, a.sz);
+      const PairTab<double>& T2 = tab[W.row0[from] + int(p.t)];
+      const double r2d = fma(dz, dz, fma(dy, dy, dx * dx));
+      int reg = W.at[k] >> 8;
+      if (reg & kNear) reg = region64<CG>(T2, r2d);
       double fr, en = 0.0;
-      term64<CG, EV>(W.at[k] >> 8, tab[W.row0[from] + int(p.t)], fma(dz, dz, fma(dy, dy, dx * dx)), W.r2[k], fr, en);
+      term64<CG, EV>(reg, T2, r2d, W.r2[k], fr, en);
       const double tx = fr * dx, ty = fr * dy, tz = fr * dz;
       W.v[0][at] = tx;
       W.v[1][at] = ty;
@@ -344,8 +376,21 @@ __global__ void __launch_bounds__(kFp64Block)
   block64<EV, T>(args[r], int(blockIdx.x) - off[r]);
 }
 
+// The FP32 squared distance of a pair and the FP64 one differ by less than this
+// share of it at any region limit: each difference is rounded three times (the
+// conversion, the box scale and its product) and the sum of squares three more,
+// the limit once, 10 x 2^-24; the upper 32 bits of two coordinates are off by
+// less than 2^-32 of the box each way, sqrt(3) of that in the distance.
+static float near_share(const relres_ctx* c) {
+  double rmin = c->tab_d[0].rsm;
+  for (const PairTab<double>& t : c->tab_d) rmin = std::min(rmin, t.rsm);
+  const double l = std::max(c->box[0], std::max(c->box[1], c->box[2]));
+  return float(1e-6 + 4.0 / 4294967296.0 * l / std::max(rmin, 1e-3));
+}
+
 static int make_launch64(const relres_ctx* c, int which, int per, bool prune, Launch64* out) {
   Launch64 a{};
+  a.near = near_share(c);
   a.sx = c->box[0] / 18446744073709551616.0;
   a.sy = c->box[1] / 18446744073709551616.0;
   a.sz = c->box[2] / 18446744073709551616.0;
