@@ -271,7 +271,8 @@ __device__ __forceinline__ void lanes_block(const PairLaunch& a, int bid) {
   }
   float4* stage = T > 1 ? reinterpret_cast<float4*>(carve(sizeof(float4) * kLaneThreads)) : nullptr;
   after_rebuild();
-  if (lists_unpruned(a)) return;
+  // (forces only: these launches prune as they walk wherever pruning is on)
+  if (EV && lists_unpruned(a)) return;
   const bool cg = bid < a.nblk_cg;
   const int blk = cg ? bid : bid - a.nblk_cg;
   const bool prn = a.prune_on && (*(volatile const unsigned*)a.gate & (F_REBUILD | F_PRUNE)) != 0u;
