@@ -445,9 +445,14 @@ relres_status relres_set_prune(relres_ctx* ctx, double delta);
  * replica (each kernel finds its replica from a table of block offsets), with
  * the list rebuilds of the replicas that need one behind one conditional node;
  * otherwise every replica's block sits on its own branch of the graph.
- * Results are bit-identical to stepping each context alone with the same
- * arguments.  If any replica's list overflows, every replica returns to the
- * block start and the block is repeated with larger lists.  cuda_stream: the
+ * Positions, velocities and the thermo rows of FP32 contexts are bit-identical
+ * to stepping each context alone with the same arguments; pair energies and
+ * virial in the rows of FP64 contexts agree to rounding (each warp adds those
+ * of its lists before they join the exact sums, and a batch may have more
+ * lists to a warp).  If any replica's list overflows, every replica returns to
+ * the block start and the block is repeated with larger lists; the replicas
+ * whose lists had room repeat it on the lists that they have by then, so from
+ * there on they too agree to rounding.  cuda_stream: the
  * stream the graphs run on (NULL: the batch creates its own).  Errors name the
  * replica (relres_batch_last_error).  Per-class kernel timing is not recorded
  * in batches.
