@@ -384,6 +384,7 @@ def ours(args):
               "pruning_launch_fraction": roof_f["p_prune"],
               "mean_list": stf["mean_fg"], "mean_list_pruned": roof_f["mean_fg_walked"], "rebuilds": stf["n_builds"]}
     ctx_stats = st1
+    pair_launch = R.relres_get_pair_launch(ctx.ctx)
     ctx.close()
 
     # roofline of the dominant kernel: the RelRes pair kernel (FG and CG lists,
@@ -439,7 +440,7 @@ def ours(args):
                                               "0 or 1 list rebuilds, this one the long-run share"},
                   "prune_delta": ctx_stats["prune_delta"], "prunes_in_timed_region": prunes,
                   "mean_fg_walked": roof["mean_fg_walked"], "mean_cg_walked": roof["mean_cg_walked"]},
-        "pair_launch": {"threads_per_atom": ctx_stats["pair_tpa"], "block": ctx_stats["pair_block"],
+        "pair_launch": {"threads_per_atom": pair_launch[0], "block": pair_launch[1],
                         "chosen_by": "autotuner (first relres_step)",
                         "force_accumulation": ["FP32", "compensated float-float", "FP64"][ctx_stats["force_acc"]]},
         "gpu_launches": ctx_stats["n_launches"] - st0["n_launches"],

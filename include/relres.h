@@ -172,10 +172,10 @@ typedef struct relres_stats {
   long long n_steps;             /* MD steps since create (also the thermostat counter) */
   int has_cg;                    /* 1 if any hybrid pair has eps^CG > 0 */
   long long n_launches;          /* CUDA kernels this context has launched */
-  int pair_tpa, pair_block;      /* forces-only pair kernel: threads per atom and block size of its launch
-                                    configuration (small FP32 systems left to configuration -1 run
-                                    configuration 0 with several lanes per atom, and FP64 systems below
-                                    8500 atoms and CG sites run 16 or 32 where this says 8: the same force bits) */
+  int pair_tpa, pair_block;      /* launch configuration of the forces-only pair kernel (threads per atom and block
+                                    size, FP64 contexts: 4 or 8 and 32); systems that do not fill the GPU run it
+                                    with more threads per atom and the same force bits, which
+                                    relres_get_pair_launch reports */
   double prune_delta;            /* pruning margin in Angstrom (0: pruning off) */
   long long n_prunes;            /* pruning passes since create (each build is followed by one) */
   double mean_fg_pruned, mean_cg_pruned;  /* mean pruned list length over all passes */
@@ -328,6 +328,16 @@ relres_status relres_set_step_counter(relres_ctx* ctx, long long step);
 
 /* Statistics of the last build and counters (host struct). */
 relres_status relres_get_stats(relres_ctx* ctx, relres_stats* out);
+
+/*
+ * Shape of the pair launches as they run, at the present size, precision,
+ * configuration and accumulation: *threads that share one atom's list and
+ * threads per *block, of launches with forces only (with_energies 0) or with
+ * energies and virial.  Where configuration -1 chooses by timing and has not
+ * yet done so (relres_set_pair_config): the shape of configuration 0.
+ * Errors: RELRES_ERR_ARG (null pointer), RELRES_ERR_STATE (no lists yet).
+ */
+relres_status relres_get_pair_launch(relres_ctx* ctx, int with_energies, int* threads, int* block);
 
 /*
  * Replace the LJ parameters of a context (eps_fg, sig_fg and the CG pair

@@ -2007,6 +2007,19 @@ relres_status relres_set_step_counter(relres_ctx* c, long long step) {
   return RELRES_OK;
 }
 
+relres_status relres_get_pair_launch(relres_ctx* c, int with_energies, int* threads, int* block) {
+  if (!c || !threads || !block) return RELRES_ERR_ARG;
+  if (!c->have_lists) return fail(c, RELRES_ERR_STATE, "relres_build_neighbors first");
+  if (!c->tuned && !tunes_by_timing(c)) {  // a rule decides, no launch to time
+    const relres_status s = autotune_pairs(c);
+    if (s != RELRES_OK) return s;
+  }
+  const PairShape shape = pair_shape(c, with_energies != 0);
+  *threads = shape.threads;
+  *block = shape.block;
+  return RELRES_OK;
+}
+
 relres_status relres_stall_rebuild(relres_ctx* c) {
   if (!c) return RELRES_ERR_ARG;
   // a count of arrivals that no grid reaches

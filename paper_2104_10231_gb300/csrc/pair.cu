@@ -226,12 +226,21 @@ static int make_pair_launch(const relres_ctx* c, int which, int per, bool prune_
   return nb_cg + nb_fg;
 }
 
+// threads per slot of pair_lanes.cu for this launch (0: this file's kernels)
+static int launch_lanes(const relres_ctx* c, bool ev) { return ev ? fp32_lanes(c, true) : c->pair_lanes; }
+
+PairShape pair_shape(const relres_ctx* c, bool ev) {
+  if (c->fp64) return PairShape{fp64_lanes(c, ev), kFp64Block};
+  const int lanes = launch_lanes(c, ev);
+  if (lanes) return PairShape{lanes, kLaneThreads};
+  return PairShape{kPairConfigs[c->pair_cfg].tpa, kPairConfigs[c->pair_cfg].bs};
+}
+
 static cudaError_t launch_pairs_f32(relres_ctx* c, bool ev, int which) {
-  const PairConfig& cfg = kPairConfigs[c->pair_cfg];
-  const int lanes = ev ? fp32_lanes(c, true) : c->pair_lanes;  // 0: this file's kernels
+  const int lanes = launch_lanes(c, ev);
+  const PairShape shape = pair_shape(c, ev);
   PairLaunch a;
-  const int per = lanes ? kLaneThreads / lanes : cfg.bs / cfg.tpa;
-  const int grid = make_pair_launch(c, which, per, pairs_prune(c), &a);
+  const int grid = make_pair_launch(c, which, shape.block / shape.threads, pairs_prune(c), &a);
   if (grid == 0) return cudaSuccess;
   if (lanes) {
     launch_pairs_lanes(c->stream, c->force_acc, a, ev, lanes, grid, pair_pdl(c, grid, kLaneThreads));

@@ -451,7 +451,7 @@ static void launch64_batch(cudaStream_t s, const BatchLaunch& b, int nrep) {
 }
 
 cudaError_t launch_pairs_f64(relres_ctx* c, bool ev, int which) {
-  const int lanes = fp64_lanes(c, ev);
+  const int lanes = pair_shape(c, ev).threads;
   Launch64 a;
   const int grid = make_launch64(c, which, kFp64Block / lanes, pairs_prune(c), &a);
   if (grid == 0) return cudaSuccess;

@@ -470,6 +470,11 @@ cudaError_t launch_prune(relres_ctx* c, const unsigned* gate);
 // With pruning on and one thread per slot, a launch that finds F_REBUILD or
 // F_PRUNE set walks the full lists and writes the pruned ones as it goes.
 cudaError_t launch_pairs(relres_ctx* c, bool ev, int which = 3);
+// threads per slot and per block of this context's pair launches
+struct PairShape {
+  int threads, block;
+};
+PairShape pair_shape(const relres_ctx* c, bool ev);
 // whether this context's pair launches prune (pruning on, one thread per
 // slot); otherwise a separate pruning pass precedes them when it is due
 bool pairs_prune(const relres_ctx* c);

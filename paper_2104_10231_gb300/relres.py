@@ -39,7 +39,7 @@ EXPORTED = ["relres_prepare_table", "relres_cg_params", "relres_chain_cg_grads",
             "relres_batch_last_error", "relres_batch_destroy", "relres_set_timing_sampled",
             "relres_set_list_caps", "relres_set_prune", "relres_measure_rates", "relres_get_list",
             "relres_eval_recip", "relres_set_force_accumulation", "relres_batch_get_info",
-            "relres_batch_set_mode", "relres_stall_rebuild"]
+            "relres_batch_set_mode", "relres_stall_rebuild", "relres_get_pair_launch"]
 RELRES_STATIC_MAX_ATOMS = 16384
 RELRES_BATCH_SHARED_MAX_ATOMS = 16384
 TIMING_CLASSES = ["drift", "rebuild", "lists", "pair", "finish", "thermo", "pair_ev", "prune"]
@@ -131,6 +131,7 @@ def load():
     L.relres_get_list.argtypes = [vp, C.c_int, _ip, _ip, C.c_longlong, C.POINTER(C.c_longlong)]
     L.relres_eval_recip.argtypes = [vp, vp, vp, C.c_int, vp]
     L.relres_stall_rebuild.argtypes = [vp]
+    L.relres_get_pair_launch.argtypes = [vp, C.c_int, _ip, _ip]
     L.relres_set_graphs.argtypes = [vp, C.c_int]
     L.relres_set_params.argtypes = [vp, C.POINTER(relres_params)]
     L.relres_set_pair_config.argtypes = [vp, C.c_int]
@@ -355,6 +356,13 @@ def relres_get_stats(ctx):
     st = relres_stats()
     _check(load().relres_get_stats(ctx, C.byref(st)), ctx)
     return st.as_dict()
+
+
+def relres_get_pair_launch(ctx, with_energies=False):
+    """(threads per list, threads per block) of the pair launches as they run."""
+    t, b = C.c_int(), C.c_int()
+    _check(load().relres_get_pair_launch(ctx, 1 if with_energies else 0, C.byref(t), C.byref(b)), ctx)
+    return t.value, b.value
 
 
 def relres_set_timing(ctx, enable):

@@ -84,9 +84,14 @@ def test_energies_and_virial_do_not_depend_on_accumulation_or_pruning(torch, acc
     assert abs(e[0] + e[1] - e0) <= 1e-7 * abs(e0)
     # FP32 products of each pair, summed exactly: a few 2^-24 of the largest component
     assert np.abs(w - w0).max() <= 2e-6 * np.abs(w0[:3]).max()
-    key = (e.tobytes(), w.tobytes())
-    seen = test_energies_and_virial_do_not_depend_on_accumulation_or_pruning.__dict__.setdefault("seen", key)
-    assert seen == key
+    # the bits of the default accumulation and pruning
+    ref = R.Context(R.params_for(s, R.RELRES_PREC_FP32), R.topology_for(s))
+    ref.build_neighbors(p, s.box)
+    e1, w1 = torch.zeros(4, dtype=torch.float64, device="cuda"), torch.zeros(6, dtype=torch.float64, device="cuda")
+    ref.compute(p, f, e1, w1)
+    torch.cuda.synchronize()
+    ref.close()
+    assert np.array_equal(e, e1.cpu().numpy()) and np.array_equal(w, w1.cpu().numpy())
 
 
 def test_overlapping_atoms_keep_their_energy(torch):
@@ -174,3 +179,37 @@ def test_fp64_lanes_by_size_keep_the_bits(torch):
         assert np.array_equal(p0, p1) and np.array_equal(v0, v1)
         # pair energies summed in groups of 32 / T slots and rounded to 2^-52 kcal/mol per group or better
         assert np.abs(t0 - t1).max() <= 1e-12 * np.abs(t0).max()
+
+
+# around the changes of the rules: threads per list of forces-only launches, of launches with energies, and the
+# launch configuration that relres_stats names
+@pytest.mark.parametrize("precision, n_mol, forces, energies, config", [
+    (R.RELRES_PREC_FP64, 400, (32, 32), (32, 32), (8, 32)),       # 2 400 atoms and hybrids
+    (R.RELRES_PREC_FP64, 1000, (16, 32), (16, 32), (8, 32)),      # 6 000
+    (R.RELRES_PREC_FP64, 2000, (8, 32), (16, 32), (8, 32)),       # 12 000
+    (R.RELRES_PREC_FP64, 3300, (4, 32), (4, 32), (4, 32)),        # 19 800
+    (R.RELRES_PREC_FP32, 2000, (8, 128), (8, 128), (1, 256)),     # 12 000
+    (R.RELRES_PREC_FP32, 2001, (4, 128), (8, 128), (1, 256)),
+    (R.RELRES_PREC_FP32, 6666, (4, 128), (4, 128), (1, 256)),     # 39 996
+])
+def test_the_reported_launch_is_the_one_that_runs(torch, precision, n_mol, forces, energies, config):
+    s = S.neopentane(n_mol=n_mol, density=0.5, seed=3)
+    ctx = R.Context(R.params_for(s, precision), R.make_topology(s.types, s.mass_by_type, s.excl, None))
+    with pytest.raises(R.RelresError) as ei:
+        R.relres_get_pair_launch(ctx.ctx)
+    assert ei.value.status == 6
+    p = _dev(torch, s.pos)
+    ctx.build_neighbors(p, s.box)
+    f = torch.empty_like(p)
+    for _ in range(2):  # before and after the first evaluation
+        assert R.relres_get_pair_launch(ctx.ctx) == forces and R.relres_get_pair_launch(ctx.ctx, True) == energies
+        st = ctx.stats()
+        assert (st["pair_tpa"], st["pair_block"]) == config
+        ctx.compute(p, f)
+    if precision == R.RELRES_PREC_FP32:  # a fixed configuration, and accumulations that no lanes share
+        ctx.set_pair_config(4)
+        assert R.relres_get_pair_launch(ctx.ctx) == (4, 256) and R.relres_get_pair_launch(ctx.ctx, True) == energies
+        ctx.set_pair_config(-1)
+        ctx.set_force_accumulation(R.RELRES_ACC_FP64)
+        assert R.relres_get_pair_launch(ctx.ctx)[0] == 1 and R.relres_get_pair_launch(ctx.ctx, True) == (1, 128)
+    ctx.close()

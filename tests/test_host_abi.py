@@ -156,6 +156,7 @@ def test_null_handles_and_bad_arguments_fail_before_any_cuda_call(lib):
     assert lib.relres_measure_rates(None, 0, None, None) == ERR
     assert lib.relres_eval_recip(None, None, None, 4, None) == ERR
     assert lib.relres_stall_rebuild(None) == ERR
+    assert lib.relres_get_pair_launch(None, 0, None, None) == ERR
     assert lib.relres_eval_recip(None, None, None, -1, None) == ERR
     assert lib.relres_eval_recip(None, None, None, 0, None) == R.RELRES_OK
     assert lib.relres_create(None, None, None) == ERR
