@@ -532,8 +532,10 @@ relres_status relres_batch_get_info(relres_batch* batch, int* n_shared);
  * accumulation (at least two); there the launch overhead of separate small
  * systems dominates, while a larger system runs faster with kernels of its
  * own (shared launches read each replica's arguments from device memory).
- * The pair kernel of shared launches runs one thread per atom in 256-thread
- * blocks whatever relres_set_pair_config chose.  Drops the captured graph.
+ * The threads that share an atom's list in the pair kernel of shared launches
+ * go by the list owners of all those replicas together, whatever
+ * relres_set_pair_config chose (the same force bits with compensated sums and
+ * in FP64).  Drops the captured graph.
  * Errors: RELRES_ERR_ARG (unknown mode). */
 #define RELRES_BATCH_SHARED_MAX_ATOMS 16384
 relres_status relres_batch_set_mode(relres_batch* batch, int mode);
@@ -550,8 +552,9 @@ void relres_batch_destroy(relres_batch* batch);
  * owners runs configuration 0 with 4 or 8 lanes per list, which gives the
  * same force bits); config 0..6
  * fixes one (0: one thread per atom, 256 per block; 1, 2: one thread per
- * atom, 128, 512 per block; 3-6: 2, 4, 8, 2 threads per atom).  The choice is reported
- * in relres_stats.  Results agree within rounding (the summation order of an
+ * atom, 128, 512 per block; 3-6: 2, 4, 8, 2 threads per atom).  The choice is
+ * reported in relres_stats, the launch that runs by relres_get_pair_launch.
+ * Results agree within rounding (the summation order of an
  * atom's partners changes with the number of threads).
  */
 relres_status relres_set_pair_config(relres_ctx* ctx, int config);

@@ -1069,10 +1069,9 @@ __device__ __forceinline__ double csvr_alpha(double ke, double e, double ca, dou
 
 // Start of a block of steps: the rollback snapshot of positions, velocity
 // state, forces and DevState, and beside it (the first blocks) the thermostat
-// terms (A, B) of the steps st->step + k, k < count, 32 steps to a block.  One
-// launch: four copies and then the draws, one after the other, took 18 us of a
-// 122 us one-step call at 140 000 atoms, draws of one thread a step beside the
-// copies 9.8 us, as here 6.2 us.
+// terms (A, B) of the steps st->step + k, k < count, 32 steps to a block.  6.2
+// us at 140 000 atoms (9.8 with one thread a step for the draws; 18 as four
+// copies and a launch).
 struct BlockStart {
   const unsigned long long* src[3];
   unsigned long long* dst[3];
@@ -1407,8 +1406,8 @@ __device__ __forceinline__ double force_component(const double* f, int, int, int
 
 // End of a call: positions and velocities to the caller, and copies of both.
 // One component per thread, so that every array is read and written in whole
-// lines (140 000 atoms: 7.4 us, one atom per thread 9.3; a million atoms: 37 us
-// either way, 60 % of the copy rate).
+// lines: 7.4 us at 140 000 atoms (9.3 with an atom per thread), 37 us at a
+// million, 60 % of the copy rate.
 struct FinishMd {
   int n3;
   const DevState* st;

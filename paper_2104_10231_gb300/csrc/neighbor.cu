@@ -229,11 +229,9 @@ __global__ void k_scatter(int n, const unsigned* gate, const int* __restrict__ t
 // 32) take one cell.  An atom's slot is the cell's start plus the number of
 // the cell's atoms with a smaller index (k_scatter left them in arrival
 // order); its sorted position, ranks and reference position are written at
-// once.  Lanes per cell: 8 where cells hold few atoms (x-slabs), else 32.
-// Against one thread per cell with an insertion sort (13 us at 20 000 atoms,
-// 75 us at 250 000 atoms of the FG reference, 110 us for a batch of small
-// boxes with whole cells) and a packing pass: 12 us less per rebuild at 20 000
-// atoms, 120 us less at 250 000, 4.97 -> 4.63 ms per 25 steps of 24 replicas.
+// once.  Lanes per cell: 8 where cells hold few atoms (x-slabs), else 32.  With
+// one thread per cell a rebuild took 12 us more at 20 000 atoms and 120 us more
+// at 250 000 atoms of the FG reference.
 struct OrderGrid {
   int ncell;  // 0: no such list
   const int* start;

@@ -206,12 +206,9 @@ __device__ __forceinline__ void static_pair(const double* __restrict__ pos, cons
 // One warp per atom.  The FP32 test of a partner is ~20 instructions (n^2 of
 // them: the floor of large n); the FP64 evaluation of the few percent that
 // pass runs with full lanes from the queue, at the FP64 rate (1.66 FMA per
-// clock and SM).  Against one thread per atom evaluating every partner in
-// FP64: 18.5 -> 0.094 ms per call at 3993 propane-like atoms, where 16 blocks
-// of 256 had left most SMs without work and 95 % of the FP64 arithmetic went
-// to pairs out of range (0.14 ms, and 0.76 against 0.43 ms at 14 739 atoms,
-// without the four partners in flight, the refined reciprocals and the split
-// sums; held to 80 registers the loop is not unrolled: 0.20 and 1.5 ms).
+// clock and SM).  0.094 ms per call at 3993 propane-like atoms (18.5 with one
+// thread per atom and every partner in FP64), 0.43 ms at 14 739; held to 80
+// registers the loop is not unrolled: 0.20 and 1.5 ms.
 __global__ void __launch_bounds__(kStaticThreads)
     k_allpairs_static(int n, int nt, const double* __restrict__ pos, const int* __restrict__ type, double l0,
                       double l1, double l2, const int* __restrict__ eoff, const int* __restrict__ eidx, int with_excl,

@@ -80,8 +80,7 @@ __device__ __forceinline__ ff cg_energy_ff(const CgE& T, float4 radii2, ff r2) {
 }
 
 // -dU/dr / r of the FG part, every region evaluated and the right one
-// selected (the arithmetic of fg_term, the LJ core chosen by the sign of
-// r - r_s-).  r2 >= r_s+^2 gives 0.
+// selected (the LJ core by the sign of r - r_s-).  r2 >= r_s+^2 gives 0.
 __device__ __forceinline__ float fg_force(const FgRow& T, float r2) {
   const float4 a = T.a, b = T.b;
   const float g4 = a.x;
@@ -96,9 +95,9 @@ __device__ __forceinline__ float fg_force(const FgRow& T, float r2) {
   return r2 < a.y ? fr : 0.f;
 }
 
-// -dU/dr / r of the CG part (the arithmetic of cg_term, the regions below
-// r_s- and r_c- chosen by the signs of r - r_s- and r - r_c-): zero below
-// r_s- (the constant region) and from r_c+ on.
+// -dU/dr / r of the CG part, the regions below r_s- and r_c- chosen by the
+// signs of r - r_s- and r - r_c-: zero below r_s- (the constant region) and
+// from r_c+ on.
 __device__ __forceinline__ float cg_force(const CgRow& T, float r2) {
   const float4 a = T.a, b = T.b, c = T.c;
   const float ri = rsqrtf(r2);

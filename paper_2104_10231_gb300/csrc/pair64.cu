@@ -10,11 +10,9 @@
 // lane), decides each one's region from its FP32 distance, and sorts the
 // entries inside the cutoff by region in shared memory; full warps then
 // evaluate 32 of them at a time, nearly always of one region, ~22 FP64
-// instructions each.  Against one thread per list entry by entry, and eight
-// per slot with the pruning as a pass of its own below 20 000 slots: 200 ->
-// 116 us per step at 25 000 neopentane-like atoms, 65 -> 27 us at 648
-// propane-like ones (a launch with energies 185 -> 12 us).  What is left
-// there is the FP64 rate, then the latency of one warp's rounds: fetching the
+// instructions each: 116 us per step at 25 000 neopentane-like atoms, 26 us at
+// 648 propane-like ones (200 and 65 entry by entry).  What is left is the FP64
+// rate at 25 000 atoms, the latency of one warp's rounds at 648: fetching the
 // partners of the next pass ahead gave 0 to 1 %.  A pair whose FP32 distance
 // is too close to a region limit to tell the side (kNear) is kept whatever the
 // side, and the FP64 distance decides when it is evaluated: the regions are

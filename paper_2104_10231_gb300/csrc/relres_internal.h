@@ -139,7 +139,7 @@ constexpr int kSegAtoms = RELRES_SEG_ATOMS;  // most atoms of a segment (one blo
 // thread per atom.  us per MD step with segments of up to 256 atoms / by this
 // rule (neopentane-like, FP32): 18.1 / 16.9 at 1 715 atoms, 21.8 / 20.6 at
 // 10 000, 27.2 / 26.1 at 20 000, 31.2 / 30.4 at 30 000; at a million atoms
-// segments of 128 gain 3 % of the drift and are not taken.
+// segments of 128 gain 3 % of the drift, 0.5 % of a step, and are not taken.
 inline int seg_atoms_for(int n) { return n <= 2 * 64 * 152 ? 64 : (n <= 2 * 128 * 152 ? 128 : kSegAtoms); }
 // A segment record: atoms [a0, a1), then the bond, angle and dihedral ranges
 // and the first atom of its prototype (a segment whose terms and incident-term

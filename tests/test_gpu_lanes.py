@@ -213,3 +213,23 @@ def test_the_reported_launch_is_the_one_that_runs(torch, precision, n_mol, force
         ctx.set_force_accumulation(R.RELRES_ACC_FP64)
         assert R.relres_get_pair_launch(ctx.ctx)[0] == 1 and R.relres_get_pair_launch(ctx.ctx, True) == (1, 128)
     ctx.close()
+
+
+def test_the_autotuner_times_launches_above_the_sizes_with_a_rule(torch):
+    """42 000 atoms and hybrids: with pruning one thread per list, in blocks that the timing chose; 36 000 take four
+    lanes without timing."""
+    for n_mol, threads in ((6000, 4), (7000, 1)):
+        s = S.neopentane(n_mol=n_mol, seed=2)
+        ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP32), R.topology_for(s))
+        p, v = _dev(torch, s.pos), _dev(torch, s.vel)
+        ctx.build_neighbors(p, s.box)
+        n0 = ctx.stats()["n_launches"]
+        ctx.step(2, s.dt, p, v)
+        st = ctx.stats()
+        launch = R.relres_get_pair_launch(ctx.ctx)
+        assert launch[0] == threads
+        if threads == 1:
+            # three configurations, four launches each
+            assert launch == (1, st["pair_block"]) and launch[1] in (128, 256, 512)
+            assert st["n_launches"] - n0 > 12
+        ctx.close()

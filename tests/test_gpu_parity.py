@@ -304,8 +304,8 @@ def test_every_pair_launch_configuration_matches_oracle(torch):
 
 @pytest.mark.parametrize("prune", [0.5, 0.0])
 def test_fp64_several_threads_per_slot_keep_the_bits(torch, prune):
-    # small FP64 systems walk each slot with eight threads in forces-only
-    # launches; energy launches use one: the forces must be the same bits
+    # small FP64 systems walk each slot with eight threads or more, launches with
+    # energies sum seven more values: the forces must be the same bits
     s = S.propane()
     ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP64), R.topology_for(s))
     ctx.set_prune(prune)
