@@ -10,7 +10,7 @@
 // lane), decides each one's region from its FP32 distance, and sorts the
 // entries inside the cutoff by region in shared memory; full warps then
 // evaluate 32 of them at a time, nearly always of one region, ~22 FP64
-// instructions each: 116 us per step at 25 000 neopentane-like atoms, 26 us at
+// instructions each: 116 us per step at 25 000 neopentane-like atoms, 24 us at
 // 648 propane-like ones (200 and 65 entry by entry).  What is left is the FP64
 // rate at 25 000 atoms, the latency of one warp's rounds at 648: fetching the
 // partners of the next pass ahead gave 0 to 1 %.  A pair whose FP32 distance
@@ -328,20 +328,30 @@ __device__ __forceinline__ unsigned long long walk64(const Walk64& L, int slot0,
   return own && q == 0 ? (unsigned long long)kept : 0ull;
 }
 
-// shared memory of a block (one warp): tables, FP32 radii, terms
-template <bool EV>
+// Whether a launch copies the type-pair rows to shared memory.  It does for up
+// to two types at four threads per slot; else a term's few values come from
+// global memory through the L1 cache, as the copy of every block (one warp; 22
+// KB with eight types) costs more than it saves.  us per step, copied / read in
+// place: 650 atoms (32 threads) of two types 26.1 / 24.2, of eight 51.0 / 24.3;
+// 25 000 atoms (four) of two types 102.8 / 103.1, of four 112.2 / 103.4, of
+// eight 200.9 / 104.2; 100 000 atoms 325.0 / 329.3, 328.2 / 329.6, 665 / 333.
+static bool copies_rows(int lanes, int nt) { return lanes == 4 && nt <= 2; }
+
+// shared memory of a block (one warp): FP32 radii, rows, terms
+template <bool EV, bool COPY>
 static size_t smem64(int nt) {
-  return (sizeof(PairTab<double>) + sizeof(float4)) * size_t(nt) * nt + sizeof(WarpTerms<EV>);
+  return (sizeof(float4) + (COPY ? sizeof(PairTab<double>) : 0)) * size_t(nt) * nt + sizeof(WarpTerms<EV>);
 }
 
-template <bool EV, int T>
+template <bool EV, int T, bool COPY>
 __device__ __forceinline__ void block64(const Launch64& a, int bid) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nrow = a.nt * a.nt;
   float4* const thr = reinterpret_cast<float4*>(smem_raw);
-  PairTab<double>* const tab = reinterpret_cast<PairTab<double>*>(thr + nrow);
-  WarpTerms<EV>& terms = *reinterpret_cast<WarpTerms<EV>*>(tab + nrow);
-  copy_words(tab, a.tab, nrow * int(sizeof(PairTab<double>) / sizeof(int)));
+  PairTab<double>* const rows = reinterpret_cast<PairTab<double>*>(thr + nrow);
+  const PairTab<double>* const tab = COPY ? rows : a.tab;
+  WarpTerms<EV>& terms = *reinterpret_cast<WarpTerms<EV>*>(rows + (COPY ? nrow : 0));
+  if (COPY) copy_words(rows, a.tab, nrow * int(sizeof(PairTab<double>) / sizeof(int)));
   for (int k = threadIdx.x; k < nrow; k += kFp64Block)
     thr[k] = make_float4(float(a.tab[k].rsm2), float(a.tab[k].rsp2), float(a.tab[k].rcm2), float(a.tab[k].rcp2));
   after_rebuild();
@@ -362,16 +372,16 @@ __device__ __forceinline__ void block64(const Launch64& a, int bid) {
   }
 }
 
-template <bool EV, int T>
+template <bool EV, int T, bool COPY>
 __global__ void __launch_bounds__(kFp64Block) k_pair64(Launch64 a) {
-  block64<EV, T>(a, blockIdx.x);
+  block64<EV, T, COPY>(a, blockIdx.x);
 }
 
-template <bool EV, int T>
+template <bool EV, int T, bool COPY>
 __global__ void __launch_bounds__(kFp64Block)
     k_pair64_batch(const Launch64* __restrict__ args, const int* __restrict__ off, int nrep) {
   const int r = batch_replica(off, nrep, blockIdx.x);
-  block64<EV, T>(args[r], int(blockIdx.x) - off[r]);
+  block64<EV, T, COPY>(args[r], int(blockIdx.x) - off[r]);
 }
 
 // The FP32 squared distance of a pair and the FP64 one differ by less than this
@@ -419,33 +429,37 @@ static int make_launch64(const relres_ctx* c, int which, int per, bool prune, La
   return a.nblk_cg + (do_fg ? (c->n + per - 1) / per : 0);
 }
 
-// F<EV, T>(...) for the threads per slot of a launch
-#define RELRES_LANES64(F, ...)             \
+// F<EV, T, COPY>(...) for the threads per slot and types of a launch
+#define RELRES_LANES64(F, NT, ...)         \
   if (ev) {                                \
     if (lanes == 32)                       \
-      F<true, 32>(__VA_ARGS__);            \
+      F<true, 32, false>(__VA_ARGS__);     \
     else if (lanes == 16)                  \
-      F<true, 16>(__VA_ARGS__);            \
+      F<true, 16, false>(__VA_ARGS__);     \
+    else if (copies_rows(lanes, NT))       \
+      F<true, 4, true>(__VA_ARGS__);       \
     else                                   \
-      F<true, 4>(__VA_ARGS__);             \
+      F<true, 4, false>(__VA_ARGS__);      \
   } else if (lanes == 32) {                \
-    F<false, 32>(__VA_ARGS__);             \
+    F<false, 32, false>(__VA_ARGS__);      \
   } else if (lanes == 16) {                \
-    F<false, 16>(__VA_ARGS__);             \
+    F<false, 16, false>(__VA_ARGS__);      \
   } else if (lanes == 8) {                 \
-    F<false, 8>(__VA_ARGS__);              \
+    F<false, 8, false>(__VA_ARGS__);       \
+  } else if (copies_rows(lanes, NT)) {     \
+    F<false, 4, true>(__VA_ARGS__);        \
   } else {                                 \
-    F<false, 4>(__VA_ARGS__);              \
+    F<false, 4, false>(__VA_ARGS__);       \
   }
 
-template <bool EV, int T>
+template <bool EV, int T, bool COPY>
 static void launch64(cudaStream_t s, const Launch64& a, int grid, bool pdl) {
-  launch_pdl(pdl, k_pair64<EV, T>, grid, kFp64Block, smem64<EV>(a.nt), s, a);
+  launch_pdl(pdl, k_pair64<EV, T, COPY>, grid, kFp64Block, smem64<EV, COPY>(a.nt), s, a);
 }
-template <bool EV, int T>
+template <bool EV, int T, bool COPY>
 static void launch64_batch(cudaStream_t s, const BatchLaunch& b, int nrep) {
-  k_pair64_batch<EV, T>
-      <<<b.nblk, kFp64Block, smem64<EV>(b.nt), s>>>(static_cast<const Launch64*>(b.d_args), b.d_off, nrep);
+  k_pair64_batch<EV, T, COPY>
+      <<<b.nblk, kFp64Block, smem64<EV, COPY>(b.nt), s>>>(static_cast<const Launch64*>(b.d_args), b.d_off, nrep);
 }
 
 cudaError_t launch_pairs_f64(relres_ctx* c, bool ev, int which) {
@@ -453,7 +467,7 @@ cudaError_t launch_pairs_f64(relres_ctx* c, bool ev, int which) {
   Launch64 a;
   const int grid = make_launch64(c, which, kFp64Block / lanes, pairs_prune(c), &a);
   if (grid == 0) return cudaSuccess;
-  RELRES_LANES64(launch64, c->stream, a, grid, pair_pdl(c, grid, kFp64Block))
+  RELRES_LANES64(launch64, a.nt, c->stream, a, grid, pair_pdl(c, grid, kFp64Block))
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }
@@ -480,7 +494,7 @@ cudaError_t prepare_pairs_batch_f64(const std::vector<relres_ctx*>& cs, BatchLau
 
 void launch_pairs_batch_f64(cudaStream_t s, bool ev, const BatchLaunch& b, int nrep) {
   const int lanes = b.lanes;
-  RELRES_LANES64(launch64_batch, s, b, nrep)
+  RELRES_LANES64(launch64_batch, b.nt, s, b, nrep)
 }
 
 }  // namespace relres

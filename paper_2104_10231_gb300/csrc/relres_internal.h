@@ -642,12 +642,12 @@ inline bool pair_pdl(const relres_ctx* c, int grid, int block) {
 // 163.1 us per step with 128-thread blocks at 25 000 neopentane-like atoms).
 // The fewer the slots, the more threads take one, so that every SM has a few
 // warps; us per step with 32 / 16 / 8 / 4 threads, forces only: 864 slots
-// 25.7 / 29.6 / 36.9 / 50.8, 2058 slots 30.7 / 31.5 / 36.1 / 47.2, 6000 slots
-// 48.4 / 42.6 / 44.9 / 54.8, 12 000 slots 73.3 / 64.4 / 62.3 / 64.6, 30 000
-// slots 145 / 123 / 126 / 116; steps with energies, ten sums per slot instead
-// of three, with 32 / 16 / 4: 864 slots 36.2 / 41.6 / 76.1, 2058 slots 41.8 /
-// 45.3 / 71.4, 6000 slots 64.1 / 62.4 / 86.9, 12 000 slots 98.9 / 91.3 / 96.9,
-// 30 000 slots 206 / 183 / 174.  The force bits are the same for all of them.
+// 23.1 / 27.0 / 34.6 / 50.2, 2058 slots 27.0 / 28.9 / 34.0 / 45.5, 6000 slots
+// 44.7 / 39.8 / 42.2 / 53.2, 12 000 slots 69.7 / 62.4 / 59.6 / 63.1, 30 000
+// slots 143 / 120 / 122 / 114; steps with energies, ten sums per slot instead
+// of three, with 32 / 16 / 4: 864 slots 30.5 / 36.9 / 75.6, 2058 slots 36.3 /
+// 40.4 / 65.4, 6000 slots 63.1 / 57.7 / 88.9, 12 000 slots 102 / 87.5 / 93.3,
+// 30 000 slots 220 / 180 / 179.  The force bits are the same for all of them.
 constexpr int kFp64Block = 32;
 inline int fp64_lanes_for(long long slots, bool ev) {
   if (slots < (ev ? 24 : 16) * kPartSMs) return 32;

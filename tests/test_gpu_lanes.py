@@ -233,3 +233,44 @@ def test_the_autotuner_times_launches_above_the_sizes_with_a_rule(torch):
             assert launch == (1, st["pair_block"]) and launch[1] in (128, 256, 512)
             assert st["n_launches"] - n0 > 12
         ctx.close()
+
+
+def _with_copied_types(s, copies):
+    """The same system with every type present `copies` times, atoms spread over the copies."""
+    nt = s.n_types
+    pick = np.random.default_rng(0).integers(0, copies, s.n_atoms)
+    comp = np.zeros((nt * copies, nt * copies), np.int32)
+    for q in range(copies):
+        comp[q * nt:(q + 1) * nt, :nt] = np.asarray(s.group_comp).reshape(nt, nt)
+    rep = lambda a: np.tile(np.asarray(a), copies)
+    return s.subset_copy(types=(s.types + nt * pick).astype(np.int32), eps_fg=rep(s.eps_fg), sig_fg=rep(s.sig_fg),
+                         is_hybrid=rep(s.is_hybrid).astype(np.int32), group_comp=comp,
+                         mass_by_type=rep(s.mass_by_type))
+
+
+# 32, 16, 8 and 4 threads per list; up to two types a launch of four copies the
+# parameter rows to shared memory, else they are read in place
+@pytest.mark.parametrize("n_mol", [130, 1000, 2000, 4000])
+@pytest.mark.parametrize("copies", [2, 4])
+def test_fp64_results_do_not_depend_on_where_the_parameters_are_read(torch, n_mol, copies):
+    base = S.neopentane(n_mol=n_mol, density=0.5, seed=3)
+    out = []
+    for s in (base, _with_copied_types(base, copies)):
+        ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP64), R.topology_for(s))
+        p = _dev(torch, s.pos)
+        ctx.build_neighbors(p, s.box)
+        f, g = torch.empty_like(p), torch.empty_like(p)
+        e, w = torch.zeros(4, dtype=torch.float64, device="cuda"), torch.zeros(6, dtype=torch.float64, device="cuda")
+        ctx.compute(p, f)
+        ctx.compute(p, g, e, w)
+        p, v = _dev(torch, s.pos), _dev(torch, s.vel)
+        batch = R.Batch([ctx])  # the same kernels with their arguments in device memory
+        batch.set_mode(1)
+        batch.step(5, 1.0, [p], [v], [0.0], 100.0, [1])
+        torch.cuda.synchronize()
+        batch.close()
+        ctx.close()
+        out.append([x.cpu().numpy() for x in (f, g, e, w, p, v)])
+    assert np.array_equal(out[0][0], out[0][1])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
