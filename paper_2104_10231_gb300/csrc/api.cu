@@ -311,9 +311,9 @@ relres_status forces_now(relres_ctx* c, int ev_mode, double* d_forces, double* d
     relres_status s = refresh_lists(c, true);
     if (s != RELRES_OK) return s;
     CK(launch_close_call(c));
-    s = read_state(c);
+    CK(cudaStreamSynchronize(c->stream));
     bool retry;
-    if (s == RELRES_OK) s = check_evaluation(c, &retry);
+    s = check_evaluation(c, &retry);
     if (s != RELRES_OK) return s;
   }
   if (!c->tuned) {
@@ -1336,8 +1336,7 @@ relres_status relres_backward(relres_ctx* c, const double* d_pos, const double* 
     CK(launch_pair_grad(c, d_grad_forces, grad_energy, d_grad_pos));
     CK(launch_close_call(c));
     CK(cudaMemcpyAsync(gc.data(), c->d_gc, sizeof(double) * gc.size(), cudaMemcpyDeviceToHost, c->stream));
-    s = read_state(c);
-    if (s != RELRES_OK) return s;
+    CK(cudaStreamSynchronize(c->stream));
     s = check_evaluation(c, &retry);
     if (s != RELRES_OK) return s;
   }

@@ -126,28 +126,44 @@ struct GradLaunch {
 
 constexpr int kGradThreads = 128;
 
+// a coordinate difference as hi + lo: the integer difference is hi + lo exactly,
+// the scale's two parts leave 2^-47 of it
+struct Split {
+  float hi, lo;
+};
+__device__ __forceinline__ Split split_diff(int a, int b, float s, float sl) {
+  const int d = int(unsigned(a) - unsigned(b));
+  const float h = __int2float_rn(d), l = __int2float_rn(d - __float2int_rn(h));
+  const float p = __fmul_rn(h, s);
+  return Split{p, fmaf(l, s, fmaf(h, sl, fmaf(h, s, -p)))};
+}
 // The geometry of one pair.  FP32: the second derivative goes as r^-14, so the
-// distance and its powers are formed in float-float from the exact integer
+// distance and its powers are formed as hi + lo from the exact integer
 // differences and rounded once; FP32 all the way amplified the roundings of
-// r^2 about sevenfold.
+// r^2 about sevenfold (and took 77 us where this takes 85, at 100 000 atoms).
 __device__ __forceinline__ void geometry(const int4& a, const int4& b, const GradLaunch<float>& L, PairGeo<float>& G) {
-  const ff ex = ff_fixed_diff32(a.x, b.x, ff{L.sx, L.sxl}), ey = ff_fixed_diff32(a.y, b.y, ff{L.sy, L.syl}),
-           ez = ff_fixed_diff32(a.z, b.z, ff{L.sz, L.szl});
-  const ff r2 = ff_add(ff_add(ff_mul(ex, ex), ff_mul(ey, ey)), ff_mul(ez, ez));
-  G.d[0] = ex.hi;
-  G.d[1] = ey.hi;
-  G.d[2] = ez.hi;
-  G.r2 = r2.hi;
-  const float y = rcp_approx(r2.hi);
-  const float e = fmaf(-r2.lo, y, fmaf(-r2.hi, y, 1.f)), ye = y * e;
-  const ff i2 = ff_quick(y, fmaf(ye, e, ye));
+  const Split x = split_diff(a.x, b.x, L.sx, L.sxl), y = split_diff(a.y, b.y, L.sy, L.syl),
+              z = split_diff(a.z, b.z, L.sz, L.szl);
+  // the leading squares added without error, everything below them in FP32
+  const float xx = __fmul_rn(x.hi, x.hi), yy = __fmul_rn(y.hi, y.hi), zz = __fmul_rn(z.hi, z.hi);
+  const float low = fmaf(2.f * x.hi, x.lo, fmaf(x.hi, x.hi, -xx)) + fmaf(2.f * y.hi, y.lo, fmaf(y.hi, y.hi, -yy)) +
+                    fmaf(2.f * z.hi, z.lo, fmaf(z.hi, z.hi, -zz));
+  const ff s1 = ff_two_sum(xx, yy), s2 = ff_two_sum(s1.hi, zz);
+  const float h = s2.hi, l = low + (s1.lo + s2.lo);
+  G.d[0] = x.hi;
+  G.d[1] = y.hi;
+  G.d[2] = z.hi;
+  G.r2 = h;
+  const float v = rcp_approx(h);
+  const float e = fmaf(-l, v, fmaf(-h, v, 1.f)), ve = v * e;
+  const ff i2 = ff_quick(v, fmaf(ve, e, ve));
   const ff i6 = ff_mul(ff_mul(i2, i2), i2);
   G.r2i = ff_val(i2);
   G.v[0] = ff_val(ff_mul(i6, i6));
   G.v[1] = ff_val(i6);
-  const float z = rsqrtf(r2.hi);
-  G.ri = fmaf(0.5f * z, fmaf(-r2.lo * z, z, fmaf(-r2.hi * z, z, 1.f)), z);
-  G.r = fmaf(r2.hi, G.ri, r2.lo * G.ri);
+  const float q = rsqrtf(h);
+  G.ri = fmaf(0.5f * q, fmaf(-l * q, q, fmaf(-h * q, q, 1.f)), q);
+  G.r = fmaf(h, G.ri, l * G.ri);
 }
 __device__ __forceinline__ void geometry(const Pos64& a, const Pos64& b, const GradLaunch<double>& L,
                                          PairGeo<double>& G) {
@@ -242,8 +258,11 @@ __device__ __forceinline__ void grad_walk(const GradWalk<R>& W, int blk, const B
   }
 }
 
+// FP32: 72 registers a thread, seven blocks per SM (us per launch at six / seven
+// / eight: 24.1 / 24.5 / 25.8 at 20 000 atoms, 82.7 / 85.0 / 90.9 at 100 000,
+// 225 / 208 / 197 at 300 000)
 template <typename R, int T>
-__global__ void __launch_bounds__(kGradThreads) k_pair_grad(GradLaunch<R> a) {
+__global__ void __launch_bounds__(kGradThreads, std::is_same<R, float>::value ? 7 : 1) k_pair_grad(GradLaunch<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (*(volatile const unsigned*)a.flags & F_NOLISTS) return;
   const int nrow = a.nt * a.nt;
@@ -301,17 +320,23 @@ static int grid_for(int n) {
 }
 
 // Threads per slot by the slots of both lists.  Measured on neopentane-like
-// liquids (1.2 slots an atom), us per launch with 8 / 4 / 1 threads (one
-// register accumulator per type and 64-thread blocks before: last column):
-//   FP32   1 715 atoms  11.1 /  16.1 /  47.7    65.9
-//         10 000        16.9 /  17.8 /  49.1    73.3
-//         20 000        33.1 /  22.8 /  50.7    76.1
-//         90 000       107.4 /  82.7 /  71.5    82.7
-//        320 000       373.8 / 289.9 / 238.9   315.3
-//   FP64   1 715        64.6 / 103.7 / 362     397
-//         20 000         378 /   299 / 530     506
+// liquids (1.2 slots an atom), us per launch with 8 / 4 / 2 / 1 threads:
+//   FP32     1 715 atoms  11.6 /  16.5 /  28.5 /  53.1
+//           10 000        18.4 /  18.0 /  26.2 /  44.3
+//           20 000        34.0 /  24.5 /  31.8 /  53.6
+//           35 000        49.1 /  38.8 /  39.6 /  56.5
+//           50 000        60.4 /  52.0 /  48.9 /  61.1
+//          100 000       103.0 /  87.9 /  85.0 /  87.3
+//          150 000       147.6 / 117.6 / 121.1 / 140.1
+//          300 000       299   / 231   / 208   / 221
+//        1 000 000       989   / 754   / 636   / 625
+//   FP64     1 715        56.6 /  91.4 / 178   / 348
+//           20 000       365   / 299   / 352   / 495
+//          100 000      1635   / 1262  / 1261  / 1319
 static int grad_lanes(long long slots, bool fp64) {
-  return slots <= 14000 ? 8 : (fp64 || slots <= 75000 ? 4 : 1);
+  if (slots <= 14000) return 8;
+  if (fp64 || slots <= 50000) return 4;
+  return slots <= 600000 ? 2 : 1;
 }
 
 template <typename R>
@@ -365,6 +390,8 @@ static cudaError_t launch_grad_t(relres_ctx* c, const double* d_grad_forces, dou
     k_pair_grad<R, 8><<<nb_cg + nb_fg, kGradThreads, smem, c->stream>>>(a);
   else if (lanes == 4)
     k_pair_grad<R, 4><<<nb_cg + nb_fg, kGradThreads, smem, c->stream>>>(a);
+  else if (lanes == 2)
+    k_pair_grad<R, 2><<<nb_cg + nb_fg, kGradThreads, smem, c->stream>>>(a);
   else
     k_pair_grad<R, 1><<<nb_cg + nb_fg, kGradThreads, smem, c->stream>>>(a);
   RELRES_LAUNCHED(c);

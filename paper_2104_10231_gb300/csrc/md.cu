@@ -1385,9 +1385,15 @@ __global__ void __launch_bounds__(32) k_call_start(const __grid_constant__ CallS
 
 __global__ void k_flags_and(DevState* st, unsigned keep) { atomicAnd(&st->flags, keep); }
 __global__ void k_flags_or(DevState* st, unsigned set) { atomicOr(&st->flags, set); }
-__global__ void k_close_call(DevState* st) { close_host_call(st); }
 
 __global__ void __launch_bounds__(32) k_post_state(const DevState* st, DevState* host) { post_state(st, host); }
+
+// end of a call that refreshed the lists, and the state to the host
+__global__ void __launch_bounds__(32) k_close_call(DevState* st, DevState* host) {
+  if (threadIdx.x == 0) close_host_call(st);
+  __syncwarp();
+  post_state(st, host);
+}
 
 // FP32 path: caller's FP64 velocities -> float-float state
 __global__ void k_vel_in(int n3, const double* __restrict__ vel, float2* __restrict__ uff) {
@@ -1958,7 +1964,7 @@ cudaError_t launch_flags_or(relres_ctx* c, unsigned set) {
 }
 
 cudaError_t launch_close_call(relres_ctx* c) {
-  k_close_call<<<1, 1, 0, c->stream>>>(c->d_state);
+  k_close_call<<<1, 32, 0, c->stream>>>(c->d_state, c->h_state);
   RELRES_LAUNCHED(c);
   return cudaGetLastError();
 }

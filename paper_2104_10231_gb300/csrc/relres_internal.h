@@ -520,7 +520,8 @@ inline void* vel_state(relres_ctx* c, double* d_vel) {
 cudaError_t launch_post_state(relres_ctx* c);
 cudaError_t launch_flags_and(relres_ctx* c, unsigned keep);
 cudaError_t launch_flags_or(relres_ctx* c, unsigned set);
-// end of a call that refreshed the lists: counts a rebuild, clears the list flags
+// end of a call that refreshed the lists: counts a rebuild, clears the list
+// flags, and the state to h_state (once the stream has been waited for)
 cudaError_t launch_close_call(relres_ctx* c);
 
 // ---- batched launches (relres_batch_step): one launch of a kernel class

@@ -50,7 +50,7 @@ def _backward(torch, ctx, s, pos):
 # shifts of the whole liquid leave the physics alone; the second and the last
 # are past half the skin
 @pytest.mark.parametrize("precision", [R.RELRES_PREC_FP32, R.RELRES_PREC_FP64])
-@pytest.mark.parametrize("n_mol", [250, 2000, 12000])
+@pytest.mark.parametrize("n_mol", [250, 2334, 8334])  # 8, 4 and 2 threads per list in FP32
 def test_backward_rebuilds_and_prunes_at_moved_positions(torch, precision, n_mol):
     s = S.neopentane(n_mol=n_mol, seed=12)
     ctx = R.Context(R.params_for(s, precision), R.make_topology(s.types, s.mass_by_type, s.excl, None))
@@ -75,6 +75,27 @@ def test_backward_rebuilds_and_prunes_at_moved_positions(torch, precision, n_mol
     want = [set(map(tuple, new.get_list(w).tolist())) for w in (2, 3)]
     new.close()
     assert got == want
+
+
+def test_backward_of_a_large_system_with_one_thread_per_list(torch):
+    """600 006 atoms and hybrids in FP32 against FP64 (four threads per list)."""
+    s = S.neopentane(n_mol=100001, density=0.5, seed=12)
+    rng = np.random.default_rng(1)
+    gf = _dev(torch, rng.normal(size=s.pos.shape))
+    out = []
+    for precision in (R.RELRES_PREC_FP32, R.RELRES_PREC_FP64):
+        ctx = R.Context(R.params_for(s, precision), R.make_topology(s.types, s.mass_by_type, s.excl, None))
+        x = _dev(torch, s.pos)
+        ctx.build_neighbors(x, s.box)
+        g = torch.empty_like(x)
+        res = ctx.backward(x, gf, 1.0, g)
+        torch.cuda.synchronize()
+        out.append((g.cpu().numpy(), res))
+        ctx.close()
+    (g0, r0), (g1, r1) = out
+    assert _err(g0, g1) <= 1e-5
+    for k in r1:
+        assert np.abs(r0[k] - r1[k]).max() <= 1e-5 * np.abs(r1[k]).max(), k
 
 
 @pytest.mark.parametrize("precision", [R.RELRES_PREC_FP32, R.RELRES_PREC_FP64])
