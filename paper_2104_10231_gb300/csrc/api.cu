@@ -111,6 +111,14 @@ relres_status read_state(relres_ctx* c) {
   return RELRES_OK;
 }
 
+// the same on a stream that is most likely idle, where a copy is faster
+// (relres_get_stats: 13 against 15 us)
+relres_status copy_state(relres_ctx* c) {
+  CK(cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
+  return RELRES_OK;
+}
+
 // list capacity: a multiple of 8 (the lists are stored in chunks of 4), at
 // most the number of possible partners rounded up
 int round_cap(double x, int limit) {
@@ -2031,7 +2039,7 @@ relres_status relres_stall_rebuild(relres_ctx* c) {
 relres_status relres_get_stats(relres_ctx* c, relres_stats* o) {
   if (!c || !o) return RELRES_ERR_ARG;
   relres_status s = finish_prune(c);  // counted with its build
-  if (s == RELRES_OK) s = read_state(c);
+  if (s == RELRES_OK) s = copy_state(c);
   if (s != RELRES_OK) return s;
   std::memset(o, 0, sizeof(*o));
   o->n_atoms = c->n;
