@@ -288,14 +288,15 @@ __global__ void __launch_bounds__(kGradThreads, std::is_same<R, float>::value ? 
     if (s_gc[q] != 0.0) atomicAdd(&a.gc[(q >> 1) * 4 + off + (q & 1)], s_gc[q]);
 }
 
-// dL/dF (caller order, FP64) into one list's slot order
+// dL/dF (caller order, FP64) into the slot order of the FG list, then of the
+// CG list (n_cg slots, 0 without one)
 template <typename R>
-__global__ void k_gather_g(int nslots, const int* __restrict__ perm, const double* __restrict__ g,
-                           GVec<R>* __restrict__ out) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nslots; s += gridDim.x * blockDim.x) {
-    const int i = perm[s];
+__global__ void k_gather_g(int n_fg, int n_cg, const int* __restrict__ perm_fg, const int* __restrict__ perm_cg,
+                           const double* __restrict__ g, GVec<R>* __restrict__ out_fg, GVec<R>* __restrict__ out_cg) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_fg + n_cg; k += gridDim.x * blockDim.x) {
+    const int s = k < n_fg ? k : k - n_fg, i = (k < n_fg ? perm_fg : perm_cg)[s];
     const R v[3] = {R(g[3 * i]), R(g[3 * i + 1]), R(g[3 * i + 2])};
-    st3(out, s, v);
+    st3(k < n_fg ? out_fg : out_cg, s, v);
   }
 }
 
@@ -348,12 +349,9 @@ static cudaError_t launch_grad_t(relres_ctx* c, const double* d_grad_forces, dou
   V* gcg = static_cast<V*>(c->d_g_cg);
   V* xfg = static_cast<V*>(c->d_gx_fg);
   V* xcg = static_cast<V*>(c->d_gx_cg);
-  k_gather_g<R><<<grid_for(c->n), kThreads, 0, c->stream>>>(c->n, c->d_perm_fg, g, gfg);
+  const int n_cg = do_cg ? c->n_h : 0;
+  k_gather_g<R><<<grid_for(c->n + n_cg), kThreads, 0, c->stream>>>(c->n, n_cg, c->d_perm_fg, c->d_perm_cg, g, gfg, gcg);
   RELRES_LAUNCHED(c);
-  if (do_cg) {
-    k_gather_g<R><<<grid_for(c->n_h), kThreads, 0, c->stream>>>(c->n_h, c->d_perm_cg, g, gcg);
-    RELRES_LAUNCHED(c);
-  }
   const double unit = std::is_same<R, float>::value ? 4294967296.0 : 18446744073709551616.0;
   GradLaunch<R> a{};
   a.sx = R(c->box[0] / unit);
