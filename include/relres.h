@@ -177,7 +177,7 @@ typedef struct relres_stats {
                                     with more threads per atom and the same force bits, which
                                     relres_get_pair_launch reports */
   double prune_delta;            /* pruning margin in Angstrom (0: pruning off) */
-  long long n_prunes;            /* pruning passes since create (each build is followed by one) */
+  long long n_prunes;            /* pruning passes since create (each build that is used is followed by one) */
   double mean_fg_pruned, mean_cg_pruned;  /* mean pruned list length over all passes */
   int step_segments;             /* 1: MD steps evaluate bonded terms per segment of whole molecules
                                     inside the drift kernel; 0: separate bonded-term kernel */
