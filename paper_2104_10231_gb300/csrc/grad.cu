@@ -18,8 +18,8 @@
 // One launch walks both lists (CG blocks first) like the force kernel; the
 // lists are those of the last force evaluation (nothing of the forward pass
 // is stored besides them).  Per-type-pair sums are kept per thread (the atom's
-// own type is fixed, the partner's type selects the accumulator), reduced per
-// block in shared memory and added to FP64 totals with atomics.
+// own type is fixed, the partner's type selects the accumulator), added per warp
+// and pair of types, per block, and to FP64 totals with atomics.
 #include "common.cuh"
 
 namespace relres {
@@ -140,7 +140,7 @@ __device__ __forceinline__ Split split_diff(int a, int b, float s, float sl) {
 // The geometry of one pair.  FP32: the second derivative goes as r^-14, so the
 // distance and its powers are formed as hi + lo from the exact integer
 // differences and rounded once; FP32 all the way amplified the roundings of
-// r^2 about sevenfold (and took 77 us where this takes 85, at 100 000 atoms).
+// r^2 about sevenfold.
 __device__ __forceinline__ void geometry(const int4& a, const int4& b, const GradLaunch<float>& L, PairGeo<float>& G) {
   const Split x = split_diff(a.x, b.x, L.sx, L.sxl), y = split_diff(a.y, b.y, L.sy, L.syl),
               z = split_diff(a.z, b.z, L.sz, L.szl);
@@ -150,9 +150,9 @@ __device__ __forceinline__ void geometry(const int4& a, const int4& b, const Gra
                     fmaf(2.f * z.hi, z.lo, fmaf(z.hi, z.hi, -zz));
   const ff s1 = ff_two_sum(xx, yy), s2 = ff_two_sum(s1.hi, zz);
   const float h = s2.hi, l = low + (s1.lo + s2.lo);
-  G.d[0] = x.hi;
-  G.d[1] = y.hi;
-  G.d[2] = z.hi;
+  G.d[0] = __fadd_rn(x.hi, x.lo);
+  G.d[1] = __fadd_rn(y.hi, y.lo);
+  G.d[2] = __fadd_rn(z.hi, z.lo);
   G.r2 = h;
   const float v = rcp_approx(h);
   const float e = fmaf(-l, v, fmaf(-h, v, 1.f)), ve = v * e;
@@ -178,6 +178,51 @@ __device__ __forceinline__ void geometry(const Pos64& a, const Pos64& b, const G
   G.v[0] = G.v[1] * G.v[1];
 }
 
+// running sums of the per-thread accumulators
+__device__ __forceinline__ void add_to(ff& sum, float v) {
+  const ff t = ff_two_sum(sum.hi, v);
+  sum = ff{t.hi, __fadd_rn(sum.lo, t.lo)};
+}
+__device__ __forceinline__ void add_lane(ff& sum, int o) {
+  const ff other{__shfl_xor_sync(0xffffffffu, sum.hi, o), __shfl_xor_sync(0xffffffffu, sum.lo, o)};
+  add_to(sum, other.hi);
+  sum.lo = __fadd_rn(sum.lo, other.lo);
+}
+__device__ __forceinline__ double total_of(ff sum) { return double(sum.hi) + double(sum.lo); }
+__device__ __forceinline__ void add_to(double& sum, double v) { sum += v; }
+__device__ __forceinline__ void add_lane(double& sum, int o) { sum += __shfl_xor_sync(0xffffffffu, sum, o); }
+__device__ __forceinline__ double total_of(double sum) { return sum; }
+
+// The accumulators of a warp's 32 threads (own type ti, -1 without a slot),
+// added per pair of types: every lane takes one of the 2 nt^2 sums (several
+// lanes one where there are fewer than 32) over the threads of its type, then
+// one shared-memory FP64 atomic per sum.  With an atomic per slot and sum the
+// lanes of a warp waited for one another at the few addresses: 81 us at 100 000
+// atoms of two types where this takes 51, 120 of eight where this takes 78.
+template <typename R>
+__device__ __forceinline__ void add_type_sums(int ti, int nt, const R (*s_acc)[kGradThreads], int* s_type, double* s_gc) {
+  using Sum = typename std::conditional<std::is_same<R, float>::value, ff, double>::type;
+  const int lane = threadIdx.x & 31, first = threadIdx.x & ~31, nsum = 2 * nt * nt;
+  const int share = nt == 1 ? 16 : (nt == 2 ? 4 : 1);  // lanes per sum
+  s_type[threadIdx.x] = ti;
+  __syncwarp();
+  for (int k0 = 0; k0 < nsum; k0 += 32 / share) {
+    const int k = k0 + lane / share, part = lane % share;
+    const int t = k % (2 * nt), want = k / (2 * nt);  // accumulator, own type
+    Sum sum{};
+    if (k < nsum)
+      for (int m = 0; m < 32; m += share) {
+        const int j = first + ((m + part + t * share) & 31);  // (each accumulator from another bank)
+        if (s_type[j] == want) add_to(sum, s_acc[t][j]);
+      }
+    for (int o = share / 2; o > 0; o >>= 1) add_lane(sum, o);
+    if (k < nsum && part == 0) {
+      const double v = total_of(sum);
+      if (v != 0.0) atomicAdd(&s_gc[k], (t & 1) ? -v : v);
+    }
+  }
+}
+
 // One slot's walk, its list shared by T lanes (lane q takes chunks q, q + T,
 // ...): with one thread per slot a launch lasts as long as one list's chain of
 // loads, 77 us at 20 000 atoms.  The partner's type selects one of the
@@ -185,7 +230,7 @@ __device__ __forceinline__ void geometry(const Pos64& a, const Pos64& b, const G
 // sums of partner type t).
 template <typename R, bool CG, int T>
 __device__ __forceinline__ void grad_walk(const GradWalk<R>& W, int blk, const BasisTab<R>* tab,
-                                          const GradLaunch<R>& a, double* s_gc, R (*s_acc)[kGradThreads]) {
+                                          const GradLaunch<R>& a, double* s_gc, R (*s_acc)[kGradThreads], int* s_type) {
   const int s = (blk * kGradThreads + threadIdx.x) / T, q = threadIdx.x % T;
   const bool own = s < W.nslots;
   R gi[3] = {R(0), R(0), R(0)}, gx[3] = {R(0), R(0), R(0)};
@@ -249,22 +294,17 @@ __device__ __forceinline__ void grad_walk(const GradWalk<R>& W, int blk, const B
 #pragma unroll
     for (int c = 0; c < 3; ++c) gx[c] += __shfl_xor_sync(0xffffffffu, gx[c], o);
   if (own && q == 0) st3(W.gx, W.perm[s], gx);
-  // per-type-pair sums: shared-memory FP64 atomics per block, then global
-  for (int t = 0; t < 2 * a.nt; ++t) {
-    double v = double(s_acc[t][threadIdx.x]);
-#pragma unroll
-    for (int o = T / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (own && q == 0 && v != 0.0) atomicAdd(&s_gc[ti * a.nt * 2 + t], (t & 1) ? -v : v);
-  }
+  add_type_sums(own ? ti : -1, a.nt, s_acc, s_type, s_gc);
 }
 
-// FP32: 72 registers a thread, seven blocks per SM (us per launch at six / seven
-// / eight: 24.1 / 24.5 / 25.8 at 20 000 atoms, 82.7 / 85.0 / 90.9 at 100 000,
-// 225 / 208 / 197 at 300 000)
+// FP32: 80 registers a thread, six blocks per SM (us per launch at six / seven /
+// eight: 16.0 / 16.5 / 18.0 at 20 000 atoms, 50.9 / 51.0 / 57.4 at 100 000);
+// FP64: no bound (a bound of one block takes more registers than none)
 template <typename R, int T>
-__global__ void __launch_bounds__(kGradThreads, std::is_same<R, float>::value ? 7 : 1) k_pair_grad(GradLaunch<R> a) {
+__global__ void __launch_bounds__(kGradThreads, std::is_same<R, float>::value ? 6 : 0) k_pair_grad(GradLaunch<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (*(volatile const unsigned*)a.flags & F_NOLISTS) return;
+  __shared__ int s_type[kGradThreads];
   const int nrow = a.nt * a.nt;
   double* s_gc = reinterpret_cast<double*>(smem_raw);
   R(*s_acc)[kGradThreads] = reinterpret_cast<R(*)[kGradThreads]>(s_gc + 2 * nrow);
@@ -279,9 +319,9 @@ __global__ void __launch_bounds__(kGradThreads, std::is_same<R, float>::value ? 
   __syncthreads();
   const bool cg = int(blockIdx.x) < a.nblk_cg;
   if (cg)
-    grad_walk<R, true, T>(a.cg, blockIdx.x, tab, a, s_gc, s_acc);
+    grad_walk<R, true, T>(a.cg, blockIdx.x, tab, a, s_gc, s_acc, s_type);
   else
-    grad_walk<R, false, T>(a.fg, blockIdx.x - a.nblk_cg, tab, a, s_gc, s_acc);
+    grad_walk<R, false, T>(a.fg, blockIdx.x - a.nblk_cg, tab, a, s_gc, s_acc, s_type);
   __syncthreads();
   const int off = cg ? 2 : 0;
   for (int q = threadIdx.x; q < 2 * nrow; q += blockDim.x)
@@ -321,23 +361,24 @@ static int grid_for(int n) {
 }
 
 // Threads per slot by the slots of both lists.  Measured on neopentane-like
-// liquids (1.2 slots an atom), us per launch with 8 / 4 / 2 / 1 threads:
-//   FP32     1 715 atoms  11.6 /  16.5 /  28.5 /  53.1
-//           10 000        18.4 /  18.0 /  26.2 /  44.3
-//           20 000        34.0 /  24.5 /  31.8 /  53.6
-//           35 000        49.1 /  38.8 /  39.6 /  56.5
-//           50 000        60.4 /  52.0 /  48.9 /  61.1
-//          100 000       103.0 /  87.9 /  85.0 /  87.3
-//          150 000       147.6 / 117.6 / 121.1 / 140.1
-//          300 000       299   / 231   / 208   / 221
-//        1 000 000       989   / 754   / 636   / 625
-//   FP64     1 715        56.6 /  91.4 / 178   / 348
-//           20 000       365   / 299   / 352   / 495
-//          100 000      1635   / 1262  / 1261  / 1319
-static int grad_lanes(long long slots, bool fp64) {
-  if (slots <= 14000) return 8;
-  if (fp64 || slots <= 50000) return 4;
-  return slots <= 600000 ? 2 : 1;
+// liquids (1.2 slots an atom), us per launch with 8 / 4 / 2 / 1 threads, of two
+// types and of eight (whose sums at the end of a block take longer):
+//   FP32    10 000 atoms  11.7 /  13.5 /  18.4 /  28.6    24.0 /  25.0 /  30.2 /  40.8
+//           20 000        20.4 /  16.0 /  20.0 /  30.2    40.5 /  28.2 /  32.2 /  42.6
+//           35 000        30.9 /  25.7 /  23.0 /  33.9    62.4 /  50.4 /  36.5 /  46.6
+//           50 000        40.7 /  33.4 /  30.0 /  36.6    85.4 /  65.9 /  53.9 /  51.3
+//          100 000        74.4 /  59.7 /  50.9 /  52.6     156 /   113 /  87.8 /  77.8
+//          200 000         143 /   109 /  91.5 /  88.9     300 /   203 /   152 /   127
+//        1 000 000         684 /   515 /   419 /   376    1457 /   958 /   674 /   527
+//   FP64     5 000        93.0 /   124 /   145 /   284     114 /   141 /   157 /   296
+//           10 000         195 /   176 /   220 /   267     236 /   197 /   237 /   279
+//           20 000         283 /   254 /   288 /   400     350 /   287 /   309 /   416
+//           40 000         493 /   466 /   431 /   510     594 /   524 /   465 /   532
+//          100 000        1430 /  1250 /  1124 /  1152    1662 /  1378 /  1191 /  1273
+static int grad_lanes(long long slots, int nt, bool fp64) {
+  if (slots <= (fp64 ? 9000 : 14000)) return 8;
+  if (slots <= (fp64 ? 35000 : 30000)) return 4;
+  return fp64 || slots <= (nt <= 2 ? 180000 : 70000) ? 2 : 1;
 }
 
 template <typename R>
@@ -376,7 +417,7 @@ static cudaError_t launch_grad_t(relres_ctx* c, const double* d_grad_forces, dou
   }
   a.fg = GradWalk<R>{c->n, pfg, walk_nbr_fg(c), walk_cnt_fg(c), c->d_perm_fg, gfg, xfg};
   a.cg = do_cg ? GradWalk<R>{c->n_h, pcg, walk_nbr_cg(c), walk_cnt_cg(c), c->d_perm_cg, gcg, xcg} : a.fg;
-  const int lanes = grad_lanes(pair_slots(c), c->fp64), per = kGradThreads / lanes;
+  const int lanes = grad_lanes(pair_slots(c), c->n_types, c->fp64), per = kGradThreads / lanes;
   const int nb_fg = (c->n + per - 1) / per;
   const int nb_cg = do_cg ? (c->n_h + per - 1) / per : 0;
   a.nblk_cg = nb_cg;

@@ -116,6 +116,25 @@ def test_fp32_block_copolymer_gradient_matches_oracle(torch):
     _compare(torch, S.block_copolymer(n_chain=20), R.RELRES_PREC_FP32, 2e-5, 1e-4)
 
 
+# the sums over pairs of types: 2 of them over 16 lanes each, 8 over four, 18 and
+# more over one, in up to four passes of a warp; 8 and 4 threads per list
+@pytest.mark.parametrize("n_types", [1, 2, 3, 5, 8])
+@pytest.mark.parametrize("n_mol", [250, 1600])
+def test_parameter_gradients_for_any_number_of_types(torch, n_types, n_mol):
+    base = S.neopentane(n_mol=n_mol, density=0.5, seed=23)
+    rng = np.random.default_rng(n_types)
+    n_hyb = (n_types + 1) // 2
+    centre = rng.integers(0, n_hyb, base.n_atoms)
+    bead = rng.integers(n_hyb, n_types, base.n_atoms) if n_types > 1 else centre
+    hyb = (np.arange(n_types) < n_hyb).astype(np.int32)
+    comp = np.ones((n_types, n_types)) * hyb[:, None]  # (the same CG parameters for all, symmetric to the bit)
+    s = base.subset_copy(types=np.where(np.asarray(base.is_hybrid)[base.types] == 1, centre, bead).astype(np.int32),
+                         eps_fg=rng.uniform(0.05, 0.2, n_types), sig_fg=rng.uniform(3.4, 3.8, n_types), is_hybrid=hyb,
+                         group_comp=comp.astype(np.int32), mass_by_type=rng.uniform(10.0, 20.0, n_types))
+    _compare(torch, s, R.RELRES_PREC_FP64, 1e-9, 1e-9)
+    _compare(torch, s, R.RELRES_PREC_FP32, 2e-5, 1e-4)
+
+
 def test_fp32_snapshots_of_the_20000_atom_liquid(torch):
     # the differentiable workload: seeded snapshots of the 20 000-atom liquid,
     # one context reused across snapshots (lists rebuilt as needed)

@@ -235,7 +235,7 @@ def test_the_autotuner_times_launches_above_the_sizes_with_a_rule(torch):
         ctx.close()
 
 
-def _with_copied_types(s, copies):
+def with_copied_types(s, copies):
     """The same system with every type present `copies` times, atoms spread over the copies."""
     nt = s.n_types
     pick = np.random.default_rng(0).integers(0, copies, s.n_atoms)
@@ -255,7 +255,7 @@ def _with_copied_types(s, copies):
 def test_fp64_results_do_not_depend_on_where_the_parameters_are_read(torch, n_mol, copies):
     base = S.neopentane(n_mol=n_mol, density=0.5, seed=3)
     out = []
-    for s in (base, _with_copied_types(base, copies)):
+    for s in (base, with_copied_types(base, copies)):
         ctx = R.Context(R.params_for(s, R.RELRES_PREC_FP64), R.topology_for(s))
         p = _dev(torch, s.pos)
         ctx.build_neighbors(p, s.box)

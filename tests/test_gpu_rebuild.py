@@ -9,6 +9,7 @@ import pytest
 from oracle import core as O
 from paper_2104_10231_gb300 import relres as R
 from paper_2104_10231_gb300 import systems as S
+from tests.test_gpu_lanes import with_copied_types
 
 pytestmark = pytest.mark.gpu
 
@@ -77,9 +78,10 @@ def test_backward_rebuilds_and_prunes_at_moved_positions(torch, precision, n_mol
     assert got == want
 
 
-def test_backward_of_a_large_system_with_one_thread_per_list(torch):
-    """600 006 atoms and hybrids in FP32 against FP64 (four threads per list)."""
-    s = S.neopentane(n_mol=100001, density=0.5, seed=12)
+@pytest.mark.parametrize("n_mol, copies", [(40000, 1), (14000, 4)])
+def test_backward_of_a_large_system_with_one_thread_per_list(torch, n_mol, copies):
+    """240 000 atoms and hybrids of two types and 84 000 of eight, FP32 against FP64 (two threads per list)."""
+    s = with_copied_types(S.neopentane(n_mol=n_mol, density=0.5, seed=12), copies)
     rng = np.random.default_rng(1)
     gf = _dev(torch, rng.normal(size=s.pos.shape))
     out = []
